@@ -244,9 +244,10 @@ int bie_set_incident_plane_wave(bie_ctx* ctx, const double* dir);
  *                          stalled refinement straight to the full FP64 path
  *   "field.accurate_phase" 1: float-float phases in the mixed field evaluation (default),
  *                          0: FP32 phases with hardware sine/cosine
- *   "field.variant"        mixed field kernel: 2 (default) groups of 16 wavenumbers, 128 points per
- *                          CTA, tiles of 32 quadrature points, FP32 run sums; 1 the same with 64
- *                          points per CTA and 64-point tiles; 0 groups of 8, 128 points,
+ *   "field.variant"        mixed field kernel: 2 (default) groups of 16 wavenumbers taken two at a
+ *                          time in packed FP32, FP32 run sums over 32 quadrature points (for a
+ *                          last group alone at many points the same one group at a time); 1 one
+ *                          group at a time, 64 points per CTA (the same values); 0 groups of 8, 128 points,
  *                          compensated sums per term
  *   "mixed.asm_kb"         FP32 bulk assembly on meshes whose elements carry one boundary
  *                          condition each: 2 (default) wavenumbers per thread, 1, or 0 (the general

@@ -138,8 +138,9 @@ int mlp_adam_api(bie_ctx* c, const float* grad, double lr);
 int mlp_train(bie_ctx* c, const double* k, int64_t nk, const cd* surf, int epochs, float* loss_hist);
 int mlp_predict_api(bie_ctx* c, const double* k, int64_t nk, cd* x0);
 int autotune(bie_ctx* c, const double* k, int64_t nk, const char* cache_path, bie_tune_result* out);
-int field_mixed(bie_ctx* c, const double* kv, int nk, const cd* surf, const double* xp, int64_t M,
+int field_mixed(bie_ctx* c, const double* hk, const double* kv, int nk, const cd* surf, const double* xp, int64_t M,
                 const int32_t* foot_elem, const double* foot, cd* T, void* scratch, size_t scratch_bytes);
+size_t field_mixed_scratch(bie_ctx* c, const double* hk, int nk, int64_t M);
 
 static void free_geometry(bie_ctx* c) {
   void* ptrs[] = {c->nodes, c->elems, c->normals, c->bc, c->qgeo, c->ngeo, c->qshape, c->nshape, c->qgeo32,
@@ -669,7 +670,11 @@ int bie_eval_field(bie_ctx* c, const double* xobs, int64_t M, const double* k, i
   // then spans many waves of resident CTAs, so the last, partial wave costs little
   constexpr int64_t kMaxFieldBatch = 512;
   int64_t kb = std::max<int64_t>(1, std::min<int64_t>(Nk, kMaxFieldBatch));
-  BIE_TRY(ensure_buf(c, c->work3, foot_bytes + kb * perk + kMaxFieldBatch * sizeof(double) + 4096 + 256));
+  size_t scratch_bytes = kb * perk;
+  if (mode == BIE_MODE_MIXED)
+    for (int64_t k0 = 0; k0 < Nk; k0 += kb)
+      scratch_bytes = std::max(scratch_bytes, field_mixed_scratch(c, k + k0, (int)std::min<int64_t>(kb, Nk - k0), M));
+  BIE_TRY(ensure_buf(c, c->work3, foot_bytes + scratch_bytes + kMaxFieldBatch * sizeof(double) + 4096 + 256));
   double* foot = (double*)c->work3.p;
   int32_t* foot_elem = (int32_t*)(foot + 8 * M);
   char* after = (char*)(((uintptr_t)(foot_elem + M) + 255) & ~(uintptr_t)255);
@@ -699,7 +704,7 @@ int bie_eval_field(bie_ctx* c, const double* xobs, int64_t M, const double* k, i
     if (mode == BIE_MODE_FP64)
       BIE_TRY(field64(c, kdev, nk, s, xobs, M, foot_elem, foot, T, scratch));
     else
-      BIE_TRY(field_mixed(c, kdev, nk, s, xobs, M, foot_elem, foot, T, scratch, kb * perk));
+      BIE_TRY(field_mixed(c, k + k0, kdev, nk, s, xobs, M, foot_elem, foot, T, scratch, scratch_bytes));
   }
   BIE_CUDA_TRY(cudaStreamSynchronize(c->stream));
   return BIE_OK;

@@ -629,6 +629,350 @@ __global__ void __launch_bounds__(TP, MINB) k_field32c(const int32_t* __restrict
   }
 }
 
+// ------------------------------------------------------------------------------------------
+// Pairs of wavenumber groups: the evaluation of k_field32c for two consecutive groups of 16
+// wavenumbers at once, wavenumber j of the first group in the low half and of the second in the
+// high half of packed FP32 registers.  Both groups use one float-float geometry of the (point,
+// quadrature point) pair, and every half goes through k_field32c's operations in its order (each
+// group keeps its own start phase and steps by the same rotations), so that the results are the
+// same bit for bit whichever kernel a group takes.
+//
+// Bound: the FMA pipe.  The one-group kernel issues 77.7 slots an evaluation and kept the pipe 61 %
+// busy; here 43.6 slots (46 pipe cycles of packed terms and 8 of geometry an evaluation).  Measured
+// on 23 040 quadrature points: 512 wavenumbers at 16 384 points 477 -> 367 ms, 64 wavenumbers 76.4
+// -> 49 ms (the one-group kernel's 512 CTAs left a nearly empty second wave), 64 at 1000 points on
+// 8000 quadrature points 12.7 -> 5.2 ms, two points at 20 picked wavenumbers 19.2 -> 0.43 ms.
+// ------------------------------------------------------------------------------------------
+constexpr int FPG = 16;      // wavenumbers per group
+constexpr int FPP = 2 * FPG; // per pair
+
+// The pairs of one launch: pair y holds wavenumbers base[y] .. base[y] + n[y] - 1 (n <= FPP) of the
+// call's list, spaced by dk[y] where the launch takes the rotations.
+constexpr int kMaxFieldBatch = 512;  // wavenumbers of one field_mixed call, hence pairs of one launch
+struct PairList {
+  ff dk[kMaxFieldBatch];
+  int16_t base[kMaxFieldBatch];
+  uint8_t n[kMaxFieldBatch];
+};
+
+// Surface values at the quadrature points in the pair kernels' layout: [pair][p][j] two float4,
+// {P re (group 0), P re (group 1), P im, P im} and the same for P'; zero past the last wavenumber.
+// grid (ceil(EQ / 8), pairs), block 128: 16 threads (j) per point.
+__global__ void k_interp_pair(const int32_t* __restrict__ elems, int64_t N, int64_t EQ, int Q,
+                              const double* __restrict__ qshape, const cd* __restrict__ surf,
+                              const __grid_constant__ PairList pairs, float4* __restrict__ PQ) {
+  const int j = threadIdx.x & (FPG - 1);
+  const int kbase = pairs.base[blockIdx.y], nk = pairs.n[blockIdx.y];
+  const int64_t p = blockIdx.x * (int64_t)(blockDim.x / FPG) + threadIdx.x / FPG;
+  if (p >= EQ) return;
+  const int64_t e = p / Q;
+  const int q = (int)(p - e * Q);
+  float v[2][4];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int kk = h * FPG + j;
+    cd a = {0, 0}, b = {0, 0};
+    if (kk < nk) {
+      const cd* P = surf + (int64_t)(kbase + kk) * 2 * N;
+      const cd* Pn = P + N;
+      for (int t = 0; t < 6; ++t) {
+        const int32_t i = elems[6 * e + t];
+        const double sh = qshape[q * 6 + t];
+        a.re += sh * P[i].re; a.im += sh * P[i].im;
+        b.re += sh * Pn[i].re; b.im += sh * Pn[i].im;
+      }
+    }
+    v[h][0] = (float)a.re; v[h][1] = (float)a.im; v[h][2] = (float)b.re; v[h][3] = (float)b.im;
+  }
+  float4* o = PQ + (((int64_t)blockIdx.y * EQ + p) * FPG + j) * 2;
+  o[0] = make_float4(v[0][0], v[1][0], v[0][1], v[1][1]);
+  o[1] = make_float4(v[0][2], v[1][2], v[0][3], v[1][3]);
+}
+
+// Negated surface values at the foot points, {-P0 re (0), -P0 re (1), -P0 im, -P0 im}, the same for P0'.
+__device__ __forceinline__ void foot_values_pair(const int32_t* __restrict__ elems, int64_t N, const cd* __restrict__ surf,
+                                                 const int32_t* __restrict__ foot_elem, const double* __restrict__ foot,
+                                                 int64_t m, int j, int nk, float4* o) {
+  const double fxi = foot[8 * m + 6], feta = foot[8 * m + 7];
+  const double L1 = 1.0 - fxi - feta;
+  const double Nv[6] = {L1 * (2 * L1 - 1), fxi * (2 * fxi - 1), feta * (2 * feta - 1), 4 * L1 * fxi, 4 * fxi * feta,
+                        4 * feta * L1};
+  const int32_t* el = elems + 6 * (int64_t)foot_elem[m];
+  float v[2][4];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int kk = h * FPG + j;
+    double a0 = 0, a1 = 0, b0 = 0, b1 = 0;
+    if (kk < nk) {
+      const cd* P = surf + (int64_t)kk * 2 * N;
+      for (int a = 0; a < 6; ++a) {
+        const cd v2 = P[el[a]], w = P[N + el[a]];
+        a0 += Nv[a] * v2.re; a1 += Nv[a] * v2.im;
+        b0 += Nv[a] * w.re; b1 += Nv[a] * w.im;
+      }
+    }
+    v[h][0] = -(float)a0; v[h][1] = -(float)a1; v[h][2] = -(float)b0; v[h][3] = -(float)b1;
+  }
+  o[0] = make_float4(v[0][0], v[1][0], v[0][1], v[1][1]);
+  o[1] = make_float4(v[0][2], v[1][2], v[0][3], v[1][3]);
+}
+
+struct PairPoint {  // an observation point, its foot point and the foot's normal
+  ff p[3], x0[3], nu0[3];
+};
+__device__ __forceinline__ void load_pair_point(const double* __restrict__ xp, const double* __restrict__ foot, int64_t m,
+                                                PairPoint& o) {
+  for (int d = 0; d < 3; ++d) {
+    o.p[d] = ff_from_double(xp[3 * m + d]);
+    o.x0[d] = ff_from_double(foot[8 * m + d]);
+    o.nu0[d] = ff_from_double(foot[8 * m + 3 + d]);
+  }
+}
+
+// One quadrature point's terms for the pair, added to the run sums pr, pi.  g0..g3: the point's
+// record (13 table values); pq: its surface values [FPG][2]; s0: the foot values, stride ss float4
+// between wavenumbers; nj: wavenumbers of the longer half; sk [FPG]: {k, k, 1/k, 1/k}; skl [FPG]: the low parts of k.  UNI: uniformly
+// spaced groups (phases by rotation), dk the step.
+template <bool UNI, bool ZF>
+__device__ __forceinline__ void pair_terms(const float4 g0, const float4 g1, const float4 g2, const float4 g3,
+                                           const PairPoint& o, const float4* __restrict__ pq,
+                                           const float4* __restrict__ s0, int ss, const float4* __restrict__ sk,
+                                           const float2* __restrict__ skl, int nj, ff dk, float far_r2, f2* pr, f2* pi) {
+  const ff qx = {g0.x, g0.w}, qy = {g0.y, g1.x}, qz = {g0.z, g1.y};
+  const float nx = g1.z, ny = g1.w, nz = g2.x, wj = g2.y;
+  const ff nux = {nx, g2.z}, nuy = {ny, g2.w}, nuz = {nz, g3.x};
+  const ff rpx = ff_diff_lazy(qx, o.p[0]), rpy = ff_diff_lazy(qy, o.p[1]), rpz = ff_diff_lazy(qz, o.p[2]);
+  const ff r0x = ff_diff_lazy(qx, o.x0[0]), r0y = ff_diff_lazy(qy, o.x0[1]), r0z = ff_diff_lazy(qz, o.x0[2]);
+  const ff R0sq = ff_norm2_lazy(r0x, r0y, r0z);
+  float iRp, iR0;
+  const ff Rp = ff_sqrt_lazy(ff_norm2_lazy(rpx, rpy, rpz), iRp);
+  const ff R0 = ff_sqrt_lazy(R0sq, iR0);
+  const ff nr = ff_dot3_lazy(o.nu0, r0x, r0y, r0z);
+  const float ap = wj * iRp, a0 = wj * iR0;
+  const float rnp = ((rpx.hi + rpx.lo) * nx + (rpy.hi + rpy.lo) * ny + (rpz.hi + rpz.lo) * nz) * iRp * iRp;
+  float rn0;
+  if (R0sq.hi > far_r2) {
+    rn0 = (r0x.hi + r0x.lo) * nx + (r0y.hi + r0y.lo) * ny + (r0z.hi + r0z.lo) * nz;
+  } else {
+    const ff nuq[3] = {nux, nuy, nuz};
+    const ff d = ff_dot3_lazy(nuq, r0x, r0y, r0z);
+    rn0 = d.hi + d.lo;
+  }
+  rn0 *= iR0 * iR0;
+  const float nn = o.nu0[0].hi * nx + o.nu0[1].hi * ny + o.nu0[2].hi * nz;
+  const f2 Rph = f2_dup(Rp.hi), R0h = f2_dup(R0.hi), rnp2 = f2_dup(rnp), nrnp2 = f2_dup(-rnp), rn02 = f2_dup(rn0);
+  const f2 nn2 = f2_dup(nn), nnn2 = f2_dup(-nn), ap2 = f2_dup(ap), a02 = f2_dup(a0);
+  f2 cp, sp, c0, s0v, cg, sg;
+  f2 dcp, dsp, dc0, ds0, dcg, dsg, ndsp, nds0, ndsg;
+  if (UNI) {
+    const float4 k4 = sk[0];
+    const float2 kl = skl[0];
+    const f2 nkh = f2_make(-k4.x, -k4.y), nkl = f2_make(-kl.x, -kl.y);
+    cis_ffprod2(nkh, nkl, Rp, cp, sp);
+    cis_ffprod2(nkh, nkl, R0, c0, s0v);
+    cis_ffprod2(nkh, nkl, nr, cg, sg);
+    float a, b;
+    cis_ffprod(dk, Rp, a, b);
+    dcp = f2_dup(a); dsp = f2_dup(b); ndsp = f2_dup(-b);
+    cis_ffprod(dk, R0, a, b);
+    dc0 = f2_dup(a); ds0 = f2_dup(b); nds0 = f2_dup(-b);
+    cis_ffprod(dk, nr, a, b);
+    dcg = f2_dup(a); dsg = f2_dup(b); ndsg = f2_dup(-b);
+    cp = f2_mul(cp, ap2); sp = f2_mul(sp, ap2);
+    c0 = f2_mul(c0, a02); s0v = f2_mul(s0v, a02);
+  }
+#pragma unroll
+  for (int j = 0; j < FPG; ++j) {
+    if (j >= nj) break;  // (uniform over the CTA)
+    const float4 k4 = sk[j];
+    const f2 kh = f2_make(k4.x, k4.y), kinv = f2_make(k4.z, k4.w);
+    if (!UNI) {
+      const float2 kl = skl[j];
+      const f2 nkh = f2_make(-k4.x, -k4.y), nkl = f2_make(-kl.x, -kl.y);
+      cis_ffprod2(nkh, nkl, Rp, cp, sp);
+      cis_ffprod2(nkh, nkl, R0, c0, s0v);
+      cis_ffprod2(nkh, nkl, nr, cg, sg);
+      cp = f2_mul(cp, ap2); sp = f2_mul(sp, ap2);
+      c0 = f2_mul(c0, a02); s0v = f2_mul(s0v, a02);
+    } else if (j > 0) {
+      f2 t = f2_fma(cp, dcp, f2_mul(sp, ndsp));
+      sp = f2_fma(sp, dcp, f2_mul(cp, dsp));
+      cp = t;
+      t = f2_fma(c0, dc0, f2_mul(s0v, nds0));
+      s0v = f2_fma(s0v, dc0, f2_mul(c0, ds0));
+      c0 = t;
+      t = f2_fma(cg, dcg, f2_mul(sg, ndsg));
+      sg = f2_fma(sg, dcg, f2_mul(cg, dsg));
+      cg = t;
+    }
+    const f2 kRp = f2_mul(kh, Rph), kR0 = f2_mul(kh, R0h);
+    const f2 ngdr = f2_sub(c0, cp), gdi = f2_sub(sp, s0v);
+    const f2 ddr = f2_fma(f2_fma(s0v, kR0, c0), rn02, f2_mul(f2_fma(sp, kRp, cp), nrnp2));
+    // -(dG im): kept negated, the sign returned where it enters with a plus
+    const f2 nddi = f2_fma(f2_fma(cp, kRp, f2_neg(sp)), nrnp2, f2_mul(f2_fma(c0, kR0, f2_neg(s0v)), rn02));
+    f2 f = f2_mul(sg, kinv);
+    if (ZF) {  // f's limit nu0.r at k = 0 (kinv 0)
+      float f0, f1;
+      f2_split(f, f0, f1);
+      f = f2_make(k4.z == 0.f ? nr.hi : f0, k4.w == 0.f ? nr.hi : f1);
+    }
+    const f2 dg = f2_mul(f2_mul(kh, sg), nnn2), df = f2_mul(cg, nn2);
+    const float4 z0 = s0[j * ss * 2], z1 = s0[j * ss * 2 + 1], u0 = pq[2 * j], u1 = pq[2 * j + 1];
+    const f2 nP0r = f2_make(z0.x, z0.y), nP0i = f2_make(z0.z, z0.w), nQ0r = f2_make(z1.x, z1.y), nQ0i = f2_make(z1.z, z1.w);
+    const f2 Ptr = f2_fma(nQ0r, f, f2_fma(nP0r, cg, f2_make(u0.x, u0.y)));
+    const f2 Pti = f2_fma(nQ0i, f, f2_fma(nP0i, cg, f2_make(u0.z, u0.w)));
+    const f2 dPr = f2_fma(nQ0r, df, f2_fma(nP0r, dg, f2_make(u1.x, u1.y)));
+    const f2 dPi = f2_fma(nQ0i, df, f2_fma(nP0i, dg, f2_make(u1.z, u1.w)));
+    f2 a = f2_fma(Ptr, ddr, pr[j]);
+    a = f2_fma(Pti, nddi, a);
+    a = f2_fma(ngdr, dPr, a);
+    pr[j] = f2_fma(gdi, dPi, a);
+    a = f2_fma(Ptr, f2_neg(nddi), pi[j]);
+    a = f2_fma(Pti, ddr, a);
+    a = f2_fma(ngdr, dPi, a);
+    pi[j] = f2_fma(f2_neg(gdi), dPr, a);
+  }
+}
+
+// Adds a run sum to a compensated sum (s, c).
+__device__ __forceinline__ void add_run(float run, float& s, float& c) {
+  const ff a = ff_two_sum(s, run);
+  s = a.hi;
+  c += a.lo;
+}
+
+// A CTA of W warps evaluates P points (a power of two up to 32) for one pair.  A lane takes one
+// point and one run of 32 quadrature points at a time; the W 32 / P runs in flight leave their sums
+// in shared memory, and the threads of the CTA add them in the order of the runs to compensated
+// sums that live in T itself between rounds (four floats in the 16 bytes of a value): the order of
+// the additions, hence the result, does not depend on P or W.  DIRECT (P < 32): lanes of a warp are at
+// different quadrature points, which they read from global memory; otherwise each warp stages
+// tiles of 8 points.
+template <bool UNI, bool ZF, bool DIRECT>
+__global__ void __launch_bounds__(384, 1) k_field_pair(const int32_t* __restrict__ elems, int64_t N, int64_t EQ,
+                                                       const float* __restrict__ qtab, const float4* __restrict__ PQ,
+                                                       const cd* __restrict__ surf, const double* __restrict__ xp,
+                                                       int64_t M, const int32_t* __restrict__ foot_elem,
+                                                       const double* __restrict__ foot, const double* __restrict__ kv,
+                                                       const __grid_constant__ PairList pairs, int P_, cd* __restrict__ T,
+                                                       float far_r2) {
+  constexpr int UT = 8;
+  const int P = DIRECT ? P_ : 32;
+  extern __shared__ float4 fp_smem[];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, W = nt >> 5;
+  const int G = 32 / P, pt = lane & (P - 1), rs = lane / P;
+  float4* s0 = fp_smem;                                  // [FPG][2 P]: point t's values at [j][2 t], [j][2 t + 1]
+  float4* sk = s0 + FPG * 2 * P;                         // [FPG]
+  float2* skl = (float2*)(sk + FPG);                     // [FPG]
+  float2* sr = skl + FPG;                                // [W][FPG][2][32]: the runs' sums
+  float4* sg = (float4*)(sr + W * FPG * 2 * 32) + warp * UT * (4 + 2 * FPG);  // this warp's tile: [UT][4]
+  float4* sq = sg + UT * 4;                              // [UT][FPG][2]
+  const int kbase = pairs.base[blockIdx.y], nk = pairs.n[blockIdx.y], nj = min(nk, FPG);
+  const int64_t m0 = (int64_t)blockIdx.x * P;
+  ff dk = {0.f, 0.f};
+  if (UNI) dk = pairs.dk[blockIdx.y];
+  if (tid < FPG) {
+    ff k[2] = {{0.f, 0.f}, {0.f, 0.f}};
+    float ki[2] = {0.f, 0.f};
+    for (int h = 0; h < 2; ++h) {
+      const int kk = h * FPG + tid;
+      if (kk < nk) {
+        k[h] = ff_from_double(kv[kbase + kk]);
+        ki[h] = kinv32(kv[kbase + kk]);
+      }
+    }
+    sk[tid] = make_float4(k[0].hi, k[1].hi, ki[0], ki[1]);
+    skl[tid] = make_float2(k[0].lo, k[1].lo);
+  }
+  for (int e = tid; e < P * FPG; e += nt) {
+    const int t = e & (P - 1), j = e / P;
+    if (m0 + t < M)
+      foot_values_pair(elems, N, surf + (int64_t)kbase * 2 * N, foot_elem, foot, m0 + t, j, nk, s0 + (j * P + t) * 2);
+  }
+  const bool active = m0 + pt < M;
+  PairPoint o;
+  if (active) load_pair_point(xp, foot, m0 + pt, o);
+  __syncthreads();
+  const float4* pqk = PQ + (int64_t)blockIdx.y * EQ * FPG * 2;
+  const int nruns = (int)((EQ + 31) / 32);
+  f2 pr[FPG], pi[FPG];
+  for (int r0 = 0; r0 < nruns; r0 += W * G) {
+#pragma unroll
+    for (int j = 0; j < FPG; ++j) pr[j].v = pi[j].v = 0ull;
+    const int64_t q0 = (int64_t)(r0 + warp * G + rs) * 32;
+    const int cnt = (int)(EQ - q0 < 32 ? EQ - q0 : 32);  // <= 0 past the last run
+    if (DIRECT) {
+      if (active)
+#pragma unroll 1
+        for (int u = 0; u < cnt; ++u) {
+          const int64_t q = q0 + u;
+          float v[13];
+#pragma unroll
+          for (int f = 0; f < 13; ++f) v[f] = __ldg(qtab + f * EQ + q);
+          pair_terms<UNI, ZF>(make_float4(v[0], v[1], v[2], v[3]), make_float4(v[4], v[5], v[6], v[7]),
+                              make_float4(v[8], v[9], v[10], v[11]), make_float4(v[12], 0.f, 0.f, 0.f), o,
+                              pqk + q * FPG * 2, s0 + pt * 2, P, sk, skl, nj, dk, far_r2, pr, pi);
+        }
+    } else {
+#pragma unroll 1
+      for (int t0 = 0; t0 < cnt; t0 += UT) {
+        const int tc = cnt - t0 < UT ? cnt - t0 : UT;
+        __syncwarp();
+        for (int e = lane; e < 13 * UT; e += 32) {
+          const int f = e / UT, u = e - f * UT;
+          if (u < tc) reinterpret_cast<float*>(sg + u * 4)[f] = qtab[f * EQ + q0 + t0 + u];
+        }
+        const float4* src = pqk + (q0 + t0) * FPG * 2;
+        for (int e = lane; e < tc * FPG * 2; e += 32) sq[e] = src[e];
+        __syncwarp();
+        if (active)
+#pragma unroll 1
+          for (int u = 0; u < tc; ++u) {
+            asm volatile("" ::: "memory");  // the foot values stay in shared memory (128 registers otherwise)
+            pair_terms<UNI, ZF>(sg[4 * u], sg[4 * u + 1], sg[4 * u + 2], sg[4 * u + 3], o, sq + u * FPG * 2, s0 + pt * 2, P,
+                                sk, skl, nj, dk, far_r2, pr, pi);
+          }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < FPG; ++j) {
+      float r[2], i[2];
+      f2_split(pr[j], r[0], r[1]);
+      f2_split(pi[j], i[0], i[1]);
+      float2* d = sr + ((warp * FPG + j) * 2) * 32 + lane;
+      d[0] = make_float2(r[0], i[0]);
+      d[32] = make_float2(r[1], i[1]);
+    }
+    __syncthreads();
+    const int have = min(W * G, nruns - r0);
+    for (int e = tid; e < P * FPP; e += nt) {
+      const int t = e & (P - 1), kk = e / P, h = kk / FPG, j = kk - h * FPG;
+      if (kk >= nk || m0 + t >= M) continue;
+      cd* out = T + (int64_t)(kbase + kk) * M + m0 + t;
+      float2* a = reinterpret_cast<float2*>(out);
+      float2 re = make_float2(0.f, 0.f), im = re;
+      if (r0 > 0) { re = a[0]; im = a[1]; }
+      for (int r = 0; r < have; ++r) {
+        const int w = r / G, g = r - w * G;
+        const float2 v = sr[((w * FPG + j) * 2 + h) * 32 + g * P + t];
+        add_run(v.x, re.x, re.y);
+        add_run(v.y, im.x, im.y);
+      }
+      if (r0 + have < nruns) {
+        a[0] = re;
+        a[1] = im;
+      } else {
+        const double inv4pi = 1.0 / (4.0 * kPi);
+        const float4 z = s0[(j * P + t) * 2];
+        const double P0r = -(double)(h ? z.y : z.x), P0i = -(double)(h ? z.w : z.z);
+        const double vr = (double)re.x + (double)re.y, vi = (double)im.x + (double)im.y;
+        *out = {P0r + vr * inv4pi, P0i + vi * inv4pi};
+      }
+    }
+    __syncthreads();
+  }
+}
+
 double far_radius2(bie_ctx* c);
 
 template <int KB, int TP, int MINB, int UT>
@@ -648,82 +992,187 @@ static void launch_field32c(bie_ctx* c, int64_t EQ, const cf* Pq, const cf* Pnq,
 
 int ensure_mixed_tables(bie_ctx* c);
 
-int field_mixed(bie_ctx* c, const double* kv, int nk, const cd* surf, const double* xp, int64_t M,
+// The pairs of `l` (np of them) by k_field_pair.  How the points and runs are laid out: with at least
+// two CTAs of 32 points and 4 warps to an SM (three are resident) that layout; fewer points leave
+// SMs without work, so a CTA takes 12 warps (one CTA fills its SM's registers) and the most points
+// that still give every SM one (M = 3000, 7 wavenumbers: 20 -> 4 ms; M = 1: 3.1 -> 0.1 ms).
+static int launch_pairs(bie_ctx* c, const cd* surf, const double* xp, int64_t M, const int32_t* foot_elem,
+                        const double* foot, const double* kv, const PairList& l, int np, bool uni, cd* T,
+                        bool zero, float4* PQ) {
+  if (np == 0) return BIE_OK;
+  const int64_t EQ = c->E * c->rule.Q;
+  const float far_r2 = (float)far_radius2(c);
+  BIE_LAUNCH(k_interp_pair<<<dim3((unsigned)((EQ + 7) / 8), (unsigned)np), 128, 0, c->stream>>>(
+      c->elems, c->N, EQ, c->rule.Q, c->qshape, surf, l, PQ));
+  int nsm = 0;
+  BIE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
+  int P = 32, W = 4;
+  auto ctas = [&](int p) { return (M + p - 1) / p * np; };
+  if (ctas(32) < 2 * nsm) {
+    W = 12;
+    while (P > 1 && ctas(P) < nsm) P >>= 1;
+  }
+  const size_t smem = (size_t)(FPG * 2 * P + FPG) * sizeof(float4) + FPG * sizeof(float2) +
+                      (size_t)W * FPG * 2 * 32 * sizeof(float2) +
+                      (P == 32 ? (size_t)W * 8 * (4 + 2 * FPG) * sizeof(float4) : 0);
+  const dim3 g((unsigned)((M + P - 1) / P), (unsigned)np);
+  auto go = [&](auto kernel) -> int {
+    BIE_TRY(set_smem_max(kernel));
+    BIE_LAUNCH(kernel<<<g, 32 * W, smem, c->stream>>>(c->elems, c->N, EQ, c->qgeo32, PQ, surf, xp, M, foot_elem, foot, kv, l,
+                                                      P, T, far_r2));
+    return BIE_OK;
+  };
+  if (P == 32) {
+    if (uni) return zero ? go(k_field_pair<true, true, false>) : go(k_field_pair<true, false, false>);
+    return zero ? go(k_field_pair<false, true, false>) : go(k_field_pair<false, false, false>);
+  }
+  if (uni) return zero ? go(k_field_pair<true, true, true>) : go(k_field_pair<true, false, true>);
+  return zero ? go(k_field_pair<false, true, true>) : go(k_field_pair<false, false, true>);
+}
+
+// Segments of a wavenumber list, (start, length): maximal runs of equally spaced wavenumbers (at
+// least 4) take the phase recurrence inside their groups of 16, the rest runs without it (a
+// negative length) -- so that a sweep with the zero-frequency term in front (or any uniform runs
+// inside a list) keeps the recurrence where it applies.
+static std::vector<std::pair<int, int>> field_segments(const double* hk, int nk) {
+  std::vector<std::pair<int, int>> segs;
+  int i = 0, nu_start = -1;
+  while (i < nk) {
+    int L = 1;
+    if (i + 1 < nk) {
+      const double d = hk[i + 1] - hk[i];
+      L = 2;
+      if (!(d > 0.0)) L = 1;
+      else
+        while (i + L < nk && std::fabs(hk[i + L] - (hk[i] + L * d)) <= 1e-12 * std::fabs(hk[i + L])) ++L;
+    }
+    if (L >= 4) {
+      if (nu_start >= 0) { segs.push_back({nu_start, -(i - nu_start)}); nu_start = -1; }
+      segs.push_back({i, L});
+      i += L;
+    } else {
+      if (nu_start < 0) nu_start = i;
+      ++i;
+    }
+  }
+  if (nu_start >= 0) segs.push_back({nu_start, -(nk - nu_start)});
+  return segs;
+}
+
+// Whether a segment's single last group of n <= 16 wavenumbers takes the one-group kernel (k_field32c)
+// instead of a pair with an empty second half, whose packed instructions are half wasted.  The
+// one-group kernel's 128-point CTAs take as long for one point as for the 19456 that give every SM
+// one; measured on 23 040 quadrature points at M = 16 384: 26.2 ms against the pair's 28.3 for
+// n = 16, 19.2 against 13.9 for n = 5 (equal near n = 13); M = 3000, n = 7: 20 against 4 ms.
+static bool scalar_tail(int64_t M, int n) { return M >= 2 * 152 * 128 || (M >= 100 * 152 && n > 12); }
+
+// The pairs of wavenumber groups of a list (uniform segments' and the others'), and the scalar
+// kernel's groups (start, length, segment's step or 0).
+struct FieldPlan {
+  PairList uni, gen;
+  int nuni = 0, ngen = 0;
+  bool zuni = false, zgen = false;  // k = 0 among them
+  struct Tail { int start, n, uniform; double dk; };
+  std::vector<Tail> tails;
+};
+static void field_plan(const double* hk, int nk, int64_t M, FieldPlan& f) {
+  for (const auto& sg : field_segments(hk, nk)) {
+    const int r0 = sg.first, n = sg.second > 0 ? sg.second : -sg.second;
+    const bool uniform = sg.second > 0;
+    const double dk = uniform ? hk[r0 + 1] - hk[r0] : 0.0;
+    for (int i = 0; i < n; i += FPP) {
+      const int m = std::min(FPP, n - i);
+      if (m <= FPG && scalar_tail(M, m)) {
+        f.tails.push_back({r0 + i, m, uniform ? 1 : 0, dk});
+        continue;
+      }
+      PairList& l = uniform ? f.uni : f.gen;
+      int& np = uniform ? f.nuni : f.ngen;
+      l.base[np] = (int16_t)(r0 + i);
+      l.n[np] = (uint8_t)m;
+      l.dk[np] = ff_from_double(dk);
+      ++np;
+      for (int j = 0; j < m; ++j) (uniform ? f.zuni : f.zgen) |= hk[r0 + i + j] == 0.0;
+    }
+  }
+}
+
+// Scratch of field_mixed in bytes for nk wavenumbers at M points.
+size_t field_mixed_scratch(bie_ctx* c, const double* hk, int nk, int64_t M) {
+  const size_t EQ = (size_t)(c->E * c->rule.Q);
+  size_t values = 2 * (size_t)nk * EQ * sizeof(cf);  // P and P' at the quadrature points
+  if (c->field_accurate_phase && c->field_variant == 2) {
+    FieldPlan f;
+    field_plan(hk, nk, M, f);
+    values = (f.tails.empty() ? 0 : 2 * FPG * EQ * sizeof(cf)) + (size_t)std::max(f.nuni, f.ngen) * EQ * FPP * 2 * sizeof(cf);
+  }
+  return values + 512;
+}
+
+// Evaluates nk <= kMaxFieldBatch wavenumbers (hk on the host, kv the same on the device).
+int field_mixed(bie_ctx* c, const double* hk, const double* kv, int nk, const cd* surf, const double* xp, int64_t M,
                 const int32_t* foot_elem, const double* foot, cd* T, void* scratch, size_t scratch_bytes) {
   BIE_TRY(ensure_mixed_tables(c));
   const int64_t EQ = c->E * c->rule.Q;
-  if ((size_t)2 * nk * EQ * sizeof(cf) > scratch_bytes) return fail(BIE_ERR_STATE, "field scratch too small");
+  if (nk > kMaxFieldBatch || field_mixed_scratch(c, hk, nk, M) > scratch_bytes)
+    return fail(BIE_ERR_STATE, "field scratch too small");
+  if (M <= 0) return BIE_OK;
   cf* Pq = (cf*)scratch;
-  cf* Pnq = Pq + (int64_t)nk * EQ;
-  dim3 gi((unsigned)((EQ + 255) / 256), nk);
-  BIE_LAUNCH(k_interp_q32<<<gi, 256, 0, c->stream>>>(c->elems, c->N, c->E, c->rule.Q, c->qshape, surf, Pq, Pnq));
+  auto interp = [&](int start, int n) -> cf* {  // P at the quadrature points from Pq on, returns P'
+    dim3 gi((unsigned)((EQ + 255) / 256), n);
+    cf* Pnq = Pq + (int64_t)n * EQ;
+    BIE_LAUNCH(k_interp_q32<<<gi, 256, 0, c->stream>>>(c->elems, c->N, c->E, c->rule.Q, c->qshape,
+                                                       surf + (int64_t)start * 2 * c->N, Pq, Pnq));
+    return Pnq;
+  };
   TwoPi3f tp;
   const double two_pi = 2.0 * kPi;
   tp.c1 = (float)two_pi;
   tp.c2 = (float)(two_pi - (double)tp.c1);
   tp.c3 = (float)((two_pi - (double)tp.c1 - (double)tp.c2) + 2.4492935982947064e-16);
   tp.inv = (float)(1.0 / two_pi);
-  if (M > 0) {
+  if (!c->field_accurate_phase) {
+    const cf* Pnq = interp(0, nk);
     dim3 gf((unsigned)((M + FT - 1) / FT), nk);
-    if (c->field_accurate_phase) {
-      const int v = c->field_variant;
-      std::vector<double> hk(nk);
-      BIE_CUDA_TRY(cudaMemcpyAsync(hk.data(), kv, nk * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-      BIE_CUDA_TRY(cudaStreamSynchronize(c->stream));
-      // Segments of the wavenumber list, one launch each: maximal runs of equally spaced
-      // wavenumbers (at least 4) take the phase recurrence inside their groups of KB, the rest
-      // runs without it -- so that a sweep with the zero-frequency term in front (or any
-      // uniform runs inside a list) keeps the recurrence where it applies.
-      std::vector<std::pair<int, int>> segs;  // (start, length); a negative length: no recurrence
-      {
-        int i = 0, nu_start = -1;
-        while (i < nk) {
-          int L = 1;
-          if (i + 1 < nk) {
-            const double d = hk[i + 1] - hk[i];
-            L = 2;
-            if (!(d > 0.0)) L = 1;
-            else
-              while (i + L < nk && std::fabs(hk[i + L] - (hk[i] + L * d)) <= 1e-12 * std::fabs(hk[i + L])) ++L;
-          }
-          if (L >= 4) {
-            if (nu_start >= 0) { segs.push_back({nu_start, -(i - nu_start)}); nu_start = -1; }
-            segs.push_back({i, L});
-            i += L;
-          } else {
-            if (nu_start < 0) nu_start = i;
-            ++i;
-          }
-        }
-        if (nu_start >= 0) segs.push_back({nu_start, -(nk - nu_start)});
-      }
-      for (const auto& sg : segs) {
-        const int r0 = sg.first, n = sg.second > 0 ? sg.second : -sg.second;
-        const int uniform = sg.second > 0 ? 1 : 0;
-        const double dkv = uniform ? hk[r0 + 1] - hk[r0] : 0.0;
-        // k = 0 (the zero-frequency term) takes f's limit inside the kernel; launches without it
-        // keep that select out of the inner loop
-        bool zero_s = false;
-        for (int j = 0; j < n; ++j) zero_s |= hk[r0 + j] == 0.0;
-        const ff dkf = ff_from_double(dkv);
-        const double* kr = kv + r0;
-        const cf *Pqr = Pq + (int64_t)r0 * EQ, *Pnqr = Pnq + (int64_t)r0 * EQ;
-        const cd* sr = surf + (int64_t)r0 * 2 * c->N;
-        cd* Tr = T + (int64_t)r0 * M;
-        if (v == 1) {
-          launch_field32c<16, 64, 4, 64>(c, EQ, Pqr, Pnqr, sr, xp, M, foot_elem, foot, kr, n, Tr, tp, uniform, dkf, zero_s);
-        } else if (v == 2) {
-          launch_field32c<16, 128, 3, 32>(c, EQ, Pqr, Pnqr, sr, xp, M, foot_elem, foot, kr, n, Tr, tp, uniform, dkf, zero_s);
-        } else {
-          dim3 gb((unsigned)((M + FT - 1) / FT), (unsigned)((n + FKB - 1) / FKB));
-          BIE_LAUNCH(k_field32b<<<gb, FT, 0, c->stream>>>(c->elems, c->N, EQ, c->qgeo32, Pqr, Pnqr, sr, xp, M, foot_elem,
-                                                          foot, kr, n, Tr, tp, uniform, dkf));
-        }
+    BIE_LAUNCH(k_field32<false><<<gf, FT, 0, c->stream>>>(c->elems, c->N, EQ, c->qgeo32, Pq, Pnq, surf, xp, M, foot_elem,
+                                                          foot, kv, T, tp));
+  } else if (c->field_variant == 2) {
+    FieldPlan f;
+    field_plan(hk, nk, M, f);
+    float4* PQ = (float4*)scratch;
+    if (!f.tails.empty()) PQ = (float4*)(((uintptr_t)(Pq + 2 * FPG * EQ) + 255) & ~(uintptr_t)255);
+    BIE_TRY(launch_pairs(c, surf, xp, M, foot_elem, foot, kv, f.uni, f.nuni, true, T, f.zuni, PQ));
+    BIE_TRY(launch_pairs(c, surf, xp, M, foot_elem, foot, kv, f.gen, f.ngen, false, T, f.zgen, PQ));
+    for (const auto& t : f.tails) {
+      const cf* Pnq = interp(t.start, t.n);
+      bool zero = false;
+      for (int j = 0; j < t.n; ++j) zero |= hk[t.start + j] == 0.0;
+      launch_field32c<16, 128, 3, 32>(c, EQ, Pq, Pnq, surf + (int64_t)t.start * 2 * c->N, xp, M, foot_elem, foot,
+                                      kv + t.start, t.n, T + (int64_t)t.start * M, tp, t.uniform, ff_from_double(t.dk), zero);
+    }
+  } else {
+    const cf* Pnq = interp(0, nk);
+    for (const auto& sg : field_segments(hk, nk)) {  // one launch each
+      const int r0 = sg.first, n = sg.second > 0 ? sg.second : -sg.second;
+      const int uniform = sg.second > 0 ? 1 : 0;
+      const double dkv = uniform ? hk[r0 + 1] - hk[r0] : 0.0;
+      // k = 0 (the zero-frequency term) takes f's limit inside the kernel; launches without it
+      // keep that select out of the inner loop
+      bool zero_s = false;
+      for (int j = 0; j < n; ++j) zero_s |= hk[r0 + j] == 0.0;
+      const ff dkf = ff_from_double(dkv);
+      const double* kr = kv + r0;
+      const cf *Pqr = Pq + (int64_t)r0 * EQ, *Pnqr = Pnq + (int64_t)r0 * EQ;
+      const cd* sr = surf + (int64_t)r0 * 2 * c->N;
+      cd* Tr = T + (int64_t)r0 * M;
+      if (c->field_variant == 1) {
+        launch_field32c<16, 64, 4, 64>(c, EQ, Pqr, Pnqr, sr, xp, M, foot_elem, foot, kr, n, Tr, tp, uniform, dkf, zero_s);
+      } else {
+        dim3 gb((unsigned)((M + FT - 1) / FT), (unsigned)((n + FKB - 1) / FKB));
+        BIE_LAUNCH(k_field32b<<<gb, FT, 0, c->stream>>>(c->elems, c->N, EQ, c->qgeo32, Pqr, Pnqr, sr, xp, M, foot_elem,
+                                                        foot, kr, n, Tr, tp, uniform, dkf));
       }
     }
-    else
-      BIE_LAUNCH(k_field32<false><<<gf, FT, 0, c->stream>>>(c->elems, c->N, EQ, c->qgeo32, Pq, Pnq, surf, xp, M, foot_elem,
-                                                 foot, kv, T, tp));
   }
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
