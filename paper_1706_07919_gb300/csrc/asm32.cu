@@ -50,8 +50,9 @@ __global__ void k_points_to32(const double* __restrict__ g, int64_t n, float* __
 // that the lanes of a warp -- consecutive elements of one colour -- read consecutive floats.
 // Element connectivity in the same order: esort[a * E + t].
 __global__ void k_points_to32_sorted(const double* __restrict__ g, const int32_t* __restrict__ perm,
-                                     const int32_t* __restrict__ elems, int64_t E, int Q, float* __restrict__ o,
-                                     int32_t* __restrict__ esort, float4* __restrict__ aos) {
+                                     const int32_t* __restrict__ elems, bool flip, const uint8_t* __restrict__ bc,
+                                     int64_t E, int Q, float* __restrict__ o, int32_t* __restrict__ esort,
+                                     float4* __restrict__ aos, uint8_t* __restrict__ esoft) {
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= E * Q) return;
   const int64_t t = idx % E;
@@ -74,8 +75,10 @@ __global__ void k_points_to32_sorted(const double* __restrict__ g, const int32_t
   a[1] = make_float4(v[4], v[5], v[6], v[7]);
   a[2] = make_float4(v[8], v[9], v[10], v[11]);
   a[3] = make_float4(v[12], w.lo, 0.f, 0.f);
-  if (q == 0)
+  if (q == 0) {
     for (int a = 0; a < 6; ++a) esort[a * E + t] = elems[6 * e + a];
+    esoft[t] = (uint8_t)((bc[elems[6 * e]] != 0) != flip);  // (flip: bc holds the exchanged conditions)
+  }
 }
 
 // 2 pi as an unevaluated sum of three floats, and 1 / (2 pi).
@@ -245,9 +248,11 @@ __global__ void __launch_bounds__(512) k_asm32_bulk(
 //   kq[k][qq][t] = sum_a N_a(q_qq) known[k][el_t[a]]  (FP32 complex)
 // so that an element whose six nodes share one boundary condition adds its right-hand-side share
 // as sum_q w_q K_q kq_q (K = G on a hard element, -dG/dnu on a soft one) instead of carrying the
-// six nodal sums of both kernels.  grid (ceil(E / 256), nk), block 256.
+// six nodal sums of both kernels.  pair: wavenumbers 2 m and 2 m + 1 interleaved,
+//   kq[2 m][qq][t] as float4 {re, re, im, im} (a last wavenumber alone as without pair).
+// grid (ceil(E / 256), nk), block 256.
 __global__ void k_known_q32(const int32_t* __restrict__ esort, int64_t E, int Q, const float* __restrict__ qshape,
-                            const cd* __restrict__ known, int64_t N, cf* __restrict__ kq) {
+                            const cd* __restrict__ known, int64_t N, cf* __restrict__ kq, int pair) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int kk = blockIdx.y;
   if (t >= E) return;
@@ -262,90 +267,104 @@ __global__ void k_known_q32(const int32_t* __restrict__ esort, int64_t E, int Q,
       sr += sh * kn[a].re;
       si += sh * kn[a].im;
     }
-    kq[((int64_t)kk * Q + qq) * E + t] = {(float)sr, (float)si};
+    if (pair && (kk | 1) < (int)gridDim.y) {
+      float* o = reinterpret_cast<float*>(kq + ((int64_t)(kk & ~1) * Q + 2 * qq) * E + 2 * t) + (kk & 1);
+      o[0] = (float)sr;
+      o[2] = (float)si;
+    } else {
+      kq[((int64_t)kk * Q + qq) * E + t] = {(float)sr, (float)si};
+    }
   }
 }
 
 // Bulk assembly for meshes whose elements each carry one boundary condition on all six nodes
-// (every element of a sound-hard or sound-soft body), KB wavenumbers per thread: the geometry of
-// a (row, quadrature point) pair -- float-float r, R, nu_i.r, r.nu_q -- is formed once and used
-// for KB wavenumbers, each with its own float-float phases (no recurrence: every entry keeps the
-// accuracy of the one-wavenumber kernel).  Per element and wavenumber a lane carries the six nodal
-// sums of the one kernel that enters A (dG/dnu on a hard element, -G on a soft one), the
-// right-hand-side sum against the interpolated known values kq, and the two regularisation sums.
-// A row has ASM_W x QS warps: ASM_W warps take consecutive elements of a colour and, with QS = 2,
-// a second set of ASM_W warps takes the other half of the same elements' quadrature points, so
-// that the registers of KB = 2 fit 16 warps per SM; the halves add into the row one after the
-// other (barrier of the row's warps in between: fixed order, deterministic sums).
-// grid (ceil(N / rows), ceil(nk / KB)); block 32 * rows * ASM_W * QS.  Where a row accumulates:
-//   MODE 0: shared memory, rows * KB * N cf;
+// (every element of a sound-hard or sound-soft body), two wavenumbers per thread in the halves of
+// packed FP32 registers: the geometry of a (row, quadrature point) pair -- float-float r, R, nu_i.r,
+// r.nu_q -- is formed once, and each half goes through the operations of the one-wavenumber kernel
+// below in its order (its own float-float phases, no recurrence: every entry keeps the accuracy of
+// the one-wavenumber kernel; the same entries bit for bit).
+// Per element a lane carries the six nodal sums of the one kernel that enters A (dG/dnu on a hard
+// element, -G on a soft one), the right-hand-side sum against the interpolated known values kq, and
+// the two regularisation sums.  A CTA is one row's 2 ASM_W warps: ASM_W warps take consecutive
+// elements of a colour and a second set of ASM_W warps the other half of the same elements' quadrature
+// points, so that the registers fit 16 warps per SM; the halves add into the row one after the other
+// (a barrier in between: fixed order, deterministic sums).  One row per CTA: four independent CTAs
+// to an SM wait for each other's barriers least.
+// grid (N, ceil(nk / 2)); block 32 * 2 ASM_W.  Where a row accumulates:
+//   MODE 0: shared memory, both wavenumbers' entries side by side, N float4;
 //   MODE 1 (large N): A itself, each row owned by one CTA and the row's warps ordered by the same
 //     barriers (scattered read-modify-writes in L2);
-//   MODE 2 (large N cut into column windows, see build_colouring): shared memory, rows * KB * ws
-//     cf, one window of columns after the other -- the window's elements of every colour, then the
-//     window copied to A -- so that each entry of A is written once.
-template <int KB, int QS, int MODE>
-__global__ void __launch_bounds__(256, 2) k_asm32_bulk_u(
-    const double* __restrict__ nodes, const double* __restrict__ normals, const uint8_t* __restrict__ bc,
+//   MODE 2 (large N cut into column windows, see build_colouring): shared memory, ws float4, one
+//     window of columns after the other -- the window's elements of every colour, then the window
+//     copied to A -- so that each entry of A is written once.
+// Bound: issue slots and dependent latencies at 16 warps (FMA pipe about 60 %).  Measured, 64
+// wavenumbers, the whole assembly: N = 2884 39.8 -> 31.7 ms, N = 1002 7.0 -> 5.6, two wavenumbers at
+// N = 10 272 15.5 -> 12.3; of it packing gave 7 %, the first point's record, condition and nodes
+// loaded together (not one after the other) 5 %, one row instead of two per CTA 10 %.  Three rows of
+// 168 registers (12 warps) measured 33.4, more rows a CTA slower.
+template <int MODE>
+__global__ void __launch_bounds__(32 * 2 * ASM_W, 4) k_asm32_pair(
+    const double* __restrict__ nodes, const double* __restrict__ normals, const uint8_t* __restrict__ esoft, bool flip,
     const int32_t* __restrict__ esort, int64_t N, int64_t E, int Q, const float4* __restrict__ qaos,
     const float* __restrict__ qshape, const int32_t* __restrict__ color_off, int ncolors,
     const double* __restrict__ kv, int nk, const cf* __restrict__ kq, cf* __restrict__ A, int64_t lda,
-    double* __restrict__ rowsum /* [nk][N][6] */, int rows, TwoPi3 tp, float far_r2,
+    double* __restrict__ rowsum /* [nk][N][6] */, float far_r2,
     const int32_t* __restrict__ win_lo, const int32_t* __restrict__ wcol_off, int nwin, int ws) {
   constexpr bool GROW = MODE == 1;
-  constexpr int WR = ASM_W * QS;  // warps per row
-  extern __shared__ cf acc32[];
-  __shared__ float shp[64 * 6];
-  __shared__ double part[8][WR][KB][6];
+  constexpr int QS = 2, WR = ASM_W * QS;  // warps per row
+  extern __shared__ float4 accp[];
+  __shared__ float4 shp[64 * 3];  // shape values, each twice: {N0, N0, N1, N1}, ...
+  __shared__ double part[WR][2][6];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rw = warp / WR, wr = warp % WR, sub = wr % ASM_W, h = wr / ASM_W;
-  const int k0 = blockIdx.y * KB;
-  const int nkb = min(KB, nk - k0);
-  ff k[KB];
-  float kinv[KB];
-#pragma unroll
-  for (int j = 0; j < KB; ++j) {
-    const int kj = min(k0 + j, nk - 1);  // a ragged last group repeats its last wavenumber
-    k[j] = ff_from_double(kv[kj]);
-    kinv[j] = kinv32(kv[kj]);
+  const int wr = warp, sub = wr % ASM_W, h = wr / ASM_W;
+  const int k0 = blockIdx.y * 2;
+  const int nkb = min(2, nk - k0);  // a ragged last group repeats its wavenumber in the second half
+  f2 kh, nkh, nkl, kinv;
+  bool zero;
+  {
+    const ff a = ff_from_double(kv[k0]), b = ff_from_double(kv[k0 + nkb - 1]);
+    kh = f2_make(a.hi, b.hi);
+    nkh = f2_make(-a.hi, -b.hi);
+    nkl = f2_make(-a.lo, -b.lo);
+    const float ia = kinv32(kv[k0]), ib = kinv32(kv[k0 + nkb - 1]);
+    kinv = f2_make(ia, ib);
+    zero = ia == 0.f || ib == 0.f;
   }
-  for (int t = threadIdx.x; t < Q * 6; t += blockDim.x) shp[t] = qshape[t];
-  const int64_t i = (int64_t)blockIdx.x * rows + rw;
-  const bool valid = i < N;
-  // row j of this CTA's row rw: in shared memory, or (GROW) row i of system k0 + j in A
-  auto row_of = [&](int j) -> cf* {
-    if constexpr (GROW) return A + ((int64_t)(k0 + j) * N + i) * lda;
-    else if constexpr (MODE == 2) return acc32 + ((int64_t)rw * KB + j) * ws;
-    else return acc32 + ((int64_t)rw * KB + j) * N;
-  };
+  for (int t = threadIdx.x; t < Q * 3; t += blockDim.x) {
+    const float a = qshape[2 * t], b = qshape[2 * t + 1];
+    shp[t] = make_float4(a, a, b, b);
+  }
+  const int64_t i = blockIdx.x;
+  // the row: in shared memory, or (GROW) row i of system k0 + j in A
+  float4* row = accp;
+  auto grow = [&](int j) -> cf* { return A + ((int64_t)(k0 + j) * N + i) * lda; };
   if constexpr (GROW) {
-    if (valid)
-      for (int j = 0; j < nkb; ++j) {
-        cf* r = row_of(j);
-        for (int64_t c2 = wr * 32 + lane; c2 < N; c2 += 32 * WR) r[c2] = {0.f, 0.f};
-      }
+    for (int j = 0; j < nkb; ++j) {
+      cf* r = grow(j);
+      for (int64_t c2 = threadIdx.x; c2 < N; c2 += 32 * WR) r[c2] = {0.f, 0.f};
+    }
   } else if constexpr (MODE == 0) {
-    for (int64_t t = threadIdx.x; t < (int64_t)rows * KB * N; t += blockDim.x) acc32[t] = {0.f, 0.f};
+    for (int64_t t = threadIdx.x; t < N; t += 32 * WR) row[t] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   __syncthreads();
   const int qlo = h * Q / QS, qhi = (h + 1) * Q / QS;
   ff xi[3], nui[3];
   for (int d = 0; d < 3; ++d) {
-    xi[d] = ff_from_double(valid ? nodes[3 * i + d] : 0.0);
-    nui[d] = ff_from_double(valid ? normals[3 * i + d] : 0.0);
+    xi[d] = ff_from_double(nodes[3 * i + d]);
+    nui[d] = ff_from_double(normals[3 * i + d]);
   }
-  RowSums S[KB];
+  // compensated sums (s, c): alpha, beta and the right-hand side, re and im
+  f2 ss[6], sc[6];
+#pragma unroll
+  for (int t = 0; t < 6; ++t) ss[t].v = sc[t].v = 0ull;
   const int nw = MODE == 2 ? nwin : 1;
   for (int w = 0; w < nw; ++w) {
   int w0 = 0;
   if constexpr (MODE == 2) {  // the row's window accumulator starts at zero
     w0 = win_lo[w];
     const int ww = win_lo[w + 1] - w0;
-    for (int j = 0; j < KB; ++j) {
-      cf* r = row_of(j);
-      for (int c2 = wr * 32 + lane; c2 < ww; c2 += 32 * WR) r[c2] = {0.f, 0.f};
-    }
-    bar_named(1 + rw, 32 * WR);
+    for (int c2 = threadIdx.x; c2 < ww; c2 += 32 * WR) row[c2] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
   }
   for (int col = 0; col < ncolors; ++col) {
     int32_t cbeg, cend;
@@ -356,46 +375,47 @@ __global__ void __launch_bounds__(256, 2) k_asm32_bulk_u(
       cbeg = color_off[col];
       cend = color_off[col + 1];
     }
-    // the same trip count for all warps of the row (the barriers below are the row's)
-    const int iters = valid ? (cend - cbeg + 32 * ASM_W - 1) / (32 * ASM_W) : 0;
+    const int iters = (cend - cbeg + 32 * ASM_W - 1) / (32 * ASM_W);
     for (int it = 0; it < iters; ++it) {
       const int32_t t = cbeg + it * 32 * ASM_W + sub * 32 + lane;
       bool act = t < cend;
+      // the first point's 64-byte record (colour-sorted, point-major: four 16-byte loads), its known
+      // values, the element's condition and nodes: independent loads, issued together
+      const int32_t ts = act ? t : cbeg;
+      const float4* qp = qaos + ((int64_t)qlo * E + ts) * 4;
+      float4 v0 = qp[0], v1 = qp[1], v2 = qp[2], v3 = qp[3];
+      const cf* kqp = kq + (int64_t)k0 * Q * E;
+      auto known = [&](int qq) -> float4 {  // {re, re, im, im} of the two wavenumbers
+        const int64_t at = (int64_t)qq * E + ts;
+        if (nkb == 2) return reinterpret_cast<const float4*>(kqp)[at];
+        const cf v = kqp[at];
+        return make_float4(v.re, v.re, v.im, v.im);
+      };
+      float4 kqn = known(qlo);
+      const bool soft = (esoft[ts] != 0) != flip;
       int32_t el[6];
 #pragma unroll
-      for (int a = 0; a < 6; ++a) {
-        el[a] = act ? esort[a * E + t] : 0;
+      for (int a = 0; a < 6; ++a) el[a] = esort[a * E + ts];
+#pragma unroll
+      for (int a = 0; a < 6; ++a)
         if (el[a] == i) act = false;  // near pair: the near kernel's
-      }
-      float ar[KB][6], ai[KB][6];
+      f2 ar[6], ai[6];
 #pragma unroll
-      for (int j = 0; j < KB; ++j)
-#pragma unroll
-        for (int a = 0; a < 6; ++a) ar[j][a] = ai[j][a] = 0.f;
+      for (int a = 0; a < 6; ++a) ar[a].v = ai[a].v = 0ull;
       if (act) {
-        const bool soft = bc[el[0]] != 0;
-        float sr[KB], si[KB], ear[KB], eai[KB], ebr[KB], ebi[KB];
+        f2 es[6];  // the element's share of the six sums
 #pragma unroll
-        for (int j = 0; j < KB; ++j) sr[j] = si[j] = ear[j] = eai[j] = ebr[j] = ebi[j] = 0.f;
-        // the point's 64-byte record (colour-sorted, point-major: four 16-byte loads); the next
-        // point's is loaded while this one is computed
-        const float4* qp = qaos + ((int64_t)qlo * E + t) * 4;
-        float4 v0 = qp[0], v1 = qp[1], v2 = qp[2], v3 = qp[3];
-        cf kqn[KB];
-#pragma unroll
-        for (int j = 0; j < KB; ++j) kqn[j] = kq[((int64_t)min(k0 + j, nk - 1) * Q + qlo) * E + t];
+        for (int u = 0; u < 6; ++u) es[u].v = 0ull;
+        // (the next point's record and known values are loaded while this one's are used)
         for (int qq = qlo; qq < qhi; ++qq) {
           const float q[P32COUNT] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w, v2.x, v2.y, v2.z, v2.w, v3.x};
-          cf kqc[KB];
-#pragma unroll
-          for (int j = 0; j < KB; ++j) kqc[j] = kqn[j];
+          const float4 kqc = kqn;
           if (qq + 1 < qhi) {
-            const float4* qn = qaos + ((int64_t)(qq + 1) * E + t) * 4;
+            const float4* qn = qaos + ((int64_t)(qq + 1) * E + ts) * 4;
             v0 = qn[0]; v1 = qn[1]; v2 = qn[2]; v3 = qn[3];
-#pragma unroll
-            for (int j = 0; j < KB; ++j) kqn[j] = kq[((int64_t)min(k0 + j, nk - 1) * Q + qq + 1) * E + t];
+            kqn = known(qq + 1);
           }
-          // geometry, shared by the KB wavenumbers
+          // geometry, shared by the two wavenumbers
           // float-float geometry with lazy tails (distance, 1/R, nu_i.r)
           const ff rx = ff_diff_lazy(ff{q[0], q[3]}, xi[0]);
           const ff ry = ff_diff_lazy(ff{q[1], q[4]}, xi[1]);
@@ -416,41 +436,50 @@ __global__ void __launch_bounds__(256, 2) k_asm32_bulk_u(
           const float wj = q[P32W];
           // the weight rides on 1/R and on r.nu/R^3: G and dG/dnu below are w G and w dG/dnu
           const float wiR = wj * invR, wrn = wj * (rnu * invR * invR * invR);
-          float sh[6];
-#pragma unroll
-          for (int a = 0; a < 6; ++a) sh[a] = shp[qq * 6 + a];
-#pragma unroll
-          for (int j = 0; j < KB; ++j) {
-            float c, s;
-            cis_ffprod(k[j], R, c, s);
-            const float kR = k[j].hi * R.hi;
-            const float Gr = c * wiR, Gi = s * wiR;
-            const float dGr = (-c - s * kR) * wrn, dGi = (c * kR - s) * wrn;
-            float cg, sg;
-            cis_ffprod(k[j], nr, cg, sg);
-            const float g = cg, f = kinv[j] != 0.f ? sg * kinv[j] : nr.hi, dg = -k[j].hi * sg * nn, df = cg * nn;
-            ear[j] = __fmaf_rn(g, dGr, __fmaf_rn(-dg, Gr, ear[j]));
-            eai[j] = __fmaf_rn(g, dGi, __fmaf_rn(-dg, Gi, eai[j]));
-            ebr[j] = __fmaf_rn(f, dGr, __fmaf_rn(-df, Gr, ebr[j]));
-            ebi[j] = __fmaf_rn(f, dGi, __fmaf_rn(-df, Gi, ebi[j]));
-            // into A: dG (hard) or -G (soft); into b: G kq (hard) or -dG kq (soft)
-            const float war = soft ? -Gr : dGr, wai = soft ? -Gi : dGi;
-            const float wbr = soft ? -dGr : Gr, wbi = soft ? -dGi : Gi;
-#pragma unroll
-            for (int a = 0; a < 6; ++a) {
-              ar[j][a] = __fmaf_rn(sh[a], war, ar[j][a]);
-              ai[j][a] = __fmaf_rn(sh[a], wai, ai[j][a]);
-            }
-            const cf kqv = kqc[j];
-            sr[j] = __fmaf_rn(wbr, kqv.re, __fmaf_rn(-wbi, kqv.im, sr[j]));
-            si[j] = __fmaf_rn(wbr, kqv.im, __fmaf_rn(wbi, kqv.re, si[j]));
+          f2 c, s, cg, sg;
+          cis_ffprod2(nkh, nkl, R, c, s);
+          cis_ffprod2(nkh, nkl, nr, cg, sg);
+          const f2 kR = f2_mul(kh, f2_dup(R.hi)), wiR2 = f2_dup(wiR);
+          const f2 Gr = f2_mul(c, wiR2), Gi = f2_mul(s, wiR2);
+          const f2 dGr = f2_mul(f2_fma(s, kR, c), f2_dup(-wrn));
+          const f2 dGi = f2_mul(f2_fma(c, kR, f2_neg(s)), f2_dup(wrn));
+          f2 f = f2_mul(sg, kinv);
+          if (zero) {  // f's limit nu_i.r at k = 0
+            float f0, f1, i0, i1;
+            f2_split(f, f0, f1);
+            f2_split(kinv, i0, i1);
+            f = f2_make(i0 != 0.f ? f0 : nr.hi, i1 != 0.f ? f1 : nr.hi);
           }
+          const f2 ndg = f2_mul(f2_mul(kh, sg), f2_dup(nn)), ndf = f2_mul(cg, f2_dup(-nn));
+          es[0] = f2_fma(cg, dGr, f2_fma(ndg, Gr, es[0]));
+          es[1] = f2_fma(cg, dGi, f2_fma(ndg, Gi, es[1]));
+          es[2] = f2_fma(f, dGr, f2_fma(ndf, Gr, es[2]));
+          es[3] = f2_fma(f, dGi, f2_fma(ndf, Gi, es[3]));
+          // into A: dG (hard) or -G (soft); into b: G kq (hard) or -dG kq (soft)
+          f2 war = dGr, wai = dGi, wbr = Gr, wbi = Gi;
+          if (soft) {
+            war = f2_neg(Gr); wai = f2_neg(Gi);
+            wbr = f2_neg(dGr); wbi = f2_neg(dGi);
+          }
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            const float4 sh = shp[qq * 3 + a];
+            const f2 s0 = f2_make(sh.x, sh.y), s1 = f2_make(sh.z, sh.w);
+            ar[2 * a] = f2_fma(s0, war, ar[2 * a]);
+            ai[2 * a] = f2_fma(s0, wai, ai[2 * a]);
+            ar[2 * a + 1] = f2_fma(s1, war, ar[2 * a + 1]);
+            ai[2 * a + 1] = f2_fma(s1, wai, ai[2 * a + 1]);
+          }
+          const f2 kr = f2_make(kqc.x, kqc.y), ki = f2_make(kqc.z, kqc.w);
+          es[4] = f2_fma(wbr, kr, f2_fma(wbi, f2_neg(ki), es[4]));
+          es[5] = f2_fma(wbr, ki, f2_fma(wbi, kr, es[5]));
         }
 #pragma unroll
-        for (int j = 0; j < KB; ++j) {
-          S[j].ar.add(ear[j]); S[j].ai.add(eai[j]);
-          S[j].br.add(ebr[j]); S[j].bi.add(ebi[j]);
-          S[j].sr.add(sr[j]); S[j].si.add(si[j]);
+        for (int u = 0; u < 6; ++u) {  // ksum::add, packed
+          const f2 a = ss[u], b = es[u];
+          const f2 sum = f2_add(a, b), bb = f2_sub(sum, a);
+          sc[u] = f2_add(sc[u], f2_add(f2_sub(a, f2_sub(sum, bb)), f2_sub(b, bb)));
+          ss[u] = sum;
         }
       }
       // scatter into the row: the quadrature halves one after the other
@@ -458,57 +487,217 @@ __global__ void __launch_bounds__(256, 2) k_asm32_bulk_u(
       for (int hh = 0; hh < QS; ++hh) {
         if (act && h == hh) {
 #pragma unroll
-          for (int j = 0; j < KB; ++j) {
-            if (GROW && j >= nkb) break;  // no system behind a ragged group's last slots
-            cf* row = row_of(j);
-#pragma unroll
-            for (int a = 0; a < 6; ++a) {
-              row[el[a] - w0].re += ar[j][a];
-              row[el[a] - w0].im += ai[j][a];
+          for (int a = 0; a < 6; ++a) {
+            if constexpr (GROW) {
+              float r0, r1, i0, i1;
+              f2_split(ar[a], r0, r1);
+              f2_split(ai[a], i0, i1);
+              cf* g = grow(0) + el[a];
+              g->re += r0;
+              g->im += i0;
+              if (nkb == 2) {  // no system behind a ragged group's second half
+                g = grow(1) + el[a];
+                g->re += r1;
+                g->im += i1;
+              }
+            } else {
+              float4* g = row + (el[a] - w0);
+              const float4 v = *g;
+              const f2 r = f2_add(f2_make(v.x, v.y), ar[a]), m = f2_add(f2_make(v.z, v.w), ai[a]);
+              float4 o;
+              f2_split(r, o.x, o.y);
+              f2_split(m, o.z, o.w);
+              *g = o;
             }
           }
         }
-        if (QS > 1) bar_named(1 + rw, 32 * WR);
+        __syncthreads();
       }
     }
-    if (QS == 1) bar_named(1 + rw, 32 * WR);  // the row's warps finish the colour (rows <= 8: ids 1..8)
   }
   if constexpr (MODE == 2) {  // the window to A, then its accumulator is free for the next one
-    bar_named(1 + rw, 32 * WR);
+    __syncthreads();
     const int ww = win_lo[w + 1] - w0;
-    if (valid)
-      for (int j = 0; j < nkb; ++j) {
-        const cf* r = row_of(j);
-        cf* Arow = A + ((int64_t)(k0 + j) * N + i) * lda + w0;
-        for (int c2 = wr * 32 + lane; c2 < ww; c2 += 32 * WR) Arow[c2] = r[c2];
-      }
-    bar_named(1 + rw, 32 * WR);
+    for (int c2 = threadIdx.x; c2 < ww; c2 += 32 * WR) {
+      const float4 v = row[c2];
+      grow(0)[w0 + c2] = cf{v.x, v.z};
+      if (nkb == 2) grow(1)[w0 + c2] = cf{v.y, v.w};
+    }
+    __syncthreads();
   }
   }  // windows
   // reduce the compensated sums across the warp in FP64 (6 values per row and wavenumber)
 #pragma unroll
-  for (int j = 0; j < KB; ++j) {
-    const ksum* v[6] = {&S[j].ar, &S[j].ai, &S[j].br, &S[j].bi, &S[j].sr, &S[j].si};
+  for (int u = 0; u < 6; ++u) {
+    float s2[2], c2[2];
+    f2_split(ss[u], s2[0], s2[1]);
+    f2_split(sc[u], c2[0], c2[1]);
 #pragma unroll
-    for (int u = 0; u < 6; ++u) {
-      double x = (double)v[u]->s + (double)v[u]->c;
+    for (int j = 0; j < 2; ++j) {
+      double x = (double)s2[j] + (double)c2[j];
       for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-      if (lane == 0) part[rw][wr][j][u] = x;
+      if (lane == 0) part[wr][j][u] = x;
     }
   }
   __syncthreads();
-  if (!valid) return;
-  for (int j = 0; j < nkb; ++j) {
-    if constexpr (MODE == 0) {
-      const cf* row = row_of(j);
-      cf* Arow = A + ((int64_t)(k0 + j) * N + i) * lda;
-      for (int64_t c2 = wr * 32 + lane; c2 < N; c2 += 32 * WR) Arow[c2] = row[c2];
+  if constexpr (MODE == 0)
+    for (int64_t c2 = threadIdx.x; c2 < N; c2 += 32 * WR) {
+      const float4 v = row[c2];
+      grow(0)[c2] = cf{v.x, v.z};
+      if (nkb == 2) grow(1)[c2] = cf{v.y, v.w};
     }
+  for (int j = 0; j < nkb; ++j)
     if (wr == 0 && lane < 6) {
       double x = 0.0;
-      for (int w = 0; w < WR; ++w) x += part[rw][w][j][lane];
+      for (int w = 0; w < WR; ++w) x += part[w][j][lane];
       rowsum[((int64_t)(k0 + j) * N + i) * 6 + lane] = x;
     }
+}
+
+// Bulk assembly for meshes whose elements each carry one boundary condition on all six nodes
+// (every element of a sound-hard or sound-soft body), one wavenumber per thread ("mixed.asm_kb" 1).
+// Per element a lane carries the six nodal sums of the one kernel that enters A (dG/dnu on a hard
+// element, -G on a soft one), the right-hand-side sum against the interpolated known values kq, and
+// the two regularisation sums.  A row has ASM_W warps, which take consecutive elements of a colour.
+// grid (ceil(N / rows), nk); block 32 * rows * ASM_W.  Where a row accumulates:
+//   MODE 0: shared memory, rows * N cf;
+//   MODE 1 (large N): A itself, each row owned by one CTA and the row's warps ordered by the same
+//     barriers (scattered read-modify-writes in L2).
+template <int MODE>
+__global__ void __launch_bounds__(256, 2) k_asm32_bulk_u(
+    const double* __restrict__ nodes, const double* __restrict__ normals, const uint8_t* __restrict__ bc,
+    const int32_t* __restrict__ esort, int64_t N, int64_t E, int Q, const float4* __restrict__ qaos,
+    const float* __restrict__ qshape, const int32_t* __restrict__ color_off, int ncolors,
+    const double* __restrict__ kv, const cf* __restrict__ kq, cf* __restrict__ A, int64_t lda,
+    double* __restrict__ rowsum /* [nk][N][6] */, int rows, float far_r2) {
+  constexpr bool GROW = MODE == 1;
+  extern __shared__ cf acc32[];
+  __shared__ float shp[64 * 6];
+  __shared__ double part[8][ASM_W][6];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rw = warp / ASM_W, sub = warp % ASM_W;
+  const int kk = blockIdx.y;
+  const ff k = ff_from_double(kv[kk]);
+  const float kinv = kinv32(kv[kk]);
+  for (int t = threadIdx.x; t < Q * 6; t += blockDim.x) shp[t] = qshape[t];
+  const int64_t i = (int64_t)blockIdx.x * rows + rw;
+  const bool valid = i < N;
+  cf* Arow = A + ((int64_t)kk * N + (valid ? i : 0)) * lda;
+  cf* row = GROW ? Arow : acc32 + (int64_t)rw * N;
+  if constexpr (GROW) {
+    if (valid)
+      for (int64_t c2 = sub * 32 + lane; c2 < N; c2 += 32 * ASM_W) row[c2] = {0.f, 0.f};
+  } else {
+    for (int64_t t = threadIdx.x; t < (int64_t)rows * N; t += blockDim.x) acc32[t] = {0.f, 0.f};
+  }
+  __syncthreads();
+  ff xi[3], nui[3];
+  for (int d = 0; d < 3; ++d) {
+    xi[d] = ff_from_double(valid ? nodes[3 * i + d] : 0.0);
+    nui[d] = ff_from_double(valid ? normals[3 * i + d] : 0.0);
+  }
+  RowSums S;
+  for (int col = 0; col < ncolors; ++col) {
+    const int32_t cbeg = color_off[col], cend = color_off[col + 1];
+    for (int32_t t = cbeg + sub * 32 + lane; valid && t < cend; t += 32 * ASM_W) {
+      bool act = true;
+      int32_t el[6];
+#pragma unroll
+      for (int a = 0; a < 6; ++a) {
+        el[a] = esort[a * E + t];
+        if (el[a] == i) act = false;  // near pair: the near kernel's
+      }
+      if (!act) continue;
+      float ar[6], ai[6];
+#pragma unroll
+      for (int a = 0; a < 6; ++a) ar[a] = ai[a] = 0.f;
+      const bool soft = bc[el[0]] != 0;
+      float sr = 0.f, si = 0.f, ear = 0.f, eai = 0.f, ebr = 0.f, ebi = 0.f;
+      // the point's 64-byte record (colour-sorted, point-major: four 16-byte loads); the next
+      // point's is loaded while this one is computed
+      const float4* qp = qaos + (int64_t)t * 4;
+      float4 v0 = qp[0], v1 = qp[1], v2 = qp[2], v3 = qp[3];
+      const cf* kqp = kq + (int64_t)kk * Q * E + t;
+      cf kqn = kqp[0];
+      for (int qq = 0; qq < Q; ++qq) {
+        const float q[P32COUNT] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w, v2.x, v2.y, v2.z, v2.w, v3.x};
+        const cf kqv = kqn;
+        if (qq + 1 < Q) {
+          const float4* qn = qaos + ((int64_t)(qq + 1) * E + t) * 4;
+          v0 = qn[0]; v1 = qn[1]; v2 = qn[2]; v3 = qn[3];
+          kqn = kqp[(int64_t)(qq + 1) * E];
+        }
+        // float-float geometry with lazy tails (distance, 1/R, nu_i.r)
+        const ff rx = ff_diff_lazy(ff{q[0], q[3]}, xi[0]);
+        const ff ry = ff_diff_lazy(ff{q[1], q[4]}, xi[1]);
+        const ff rz = ff_diff_lazy(ff{q[2], q[5]}, xi[2]);
+        const ff R2 = ff_norm2_lazy(rx, ry, rz);
+        float invR;
+        const ff R = ff_sqrt_lazy(R2, invR);
+        const ff nr = ff_dot3_lazy(nui, rx, ry, rz);
+        float rnu;
+        if (R2.hi > far_r2) {
+          rnu = (rx.hi + rx.lo) * q[6] + (ry.hi + ry.lo) * q[7] + (rz.hi + rz.lo) * q[8];
+        } else {
+          const ff nq[3] = {ff{q[6], q[10]}, ff{q[7], q[11]}, ff{q[8], q[12]}};
+          const ff d = ff_dot3_lazy(nq, rx, ry, rz);
+          rnu = d.hi + d.lo;
+        }
+        const float nn = nui[0].hi * q[6] + nui[1].hi * q[7] + nui[2].hi * q[8];
+        const float wj = q[P32W];
+        // the weight rides on 1/R and on r.nu/R^3: G and dG/dnu below are w G and w dG/dnu
+        const float wiR = wj * invR, wrn = wj * (rnu * invR * invR * invR);
+        float c, s;
+        cis_ffprod(k, R, c, s);
+        const float kR = k.hi * R.hi;
+        const float Gr = c * wiR, Gi = s * wiR;
+        const float dGr = (-c - s * kR) * wrn, dGi = (c * kR - s) * wrn;
+        float cg, sg;
+        cis_ffprod(k, nr, cg, sg);
+        const float g = cg, f = kinv != 0.f ? sg * kinv : nr.hi, dg = -k.hi * sg * nn, df = cg * nn;
+        ear = __fmaf_rn(g, dGr, __fmaf_rn(-dg, Gr, ear));
+        eai = __fmaf_rn(g, dGi, __fmaf_rn(-dg, Gi, eai));
+        ebr = __fmaf_rn(f, dGr, __fmaf_rn(-df, Gr, ebr));
+        ebi = __fmaf_rn(f, dGi, __fmaf_rn(-df, Gi, ebi));
+        // into A: dG (hard) or -G (soft); into b: G kq (hard) or -dG kq (soft)
+        const float war = soft ? -Gr : dGr, wai = soft ? -Gi : dGi;
+        const float wbr = soft ? -dGr : Gr, wbi = soft ? -dGi : Gi;
+#pragma unroll
+        for (int a = 0; a < 6; ++a) {
+          const float sh = shp[qq * 6 + a];
+          ar[a] = __fmaf_rn(sh, war, ar[a]);
+          ai[a] = __fmaf_rn(sh, wai, ai[a]);
+        }
+        sr = __fmaf_rn(wbr, kqv.re, __fmaf_rn(-wbi, kqv.im, sr));
+        si = __fmaf_rn(wbr, kqv.im, __fmaf_rn(wbi, kqv.re, si));
+      }
+      S.ar.add(ear); S.ai.add(eai);
+      S.br.add(ebr); S.bi.add(ebi);
+      S.sr.add(sr); S.si.add(si);
+#pragma unroll
+      for (int a = 0; a < 6; ++a) {
+        row[el[a]].re += ar[a];
+        row[el[a]].im += ai[a];
+      }
+    }
+    bar_named(1 + rw, 32 * ASM_W);  // the row's warps finish the colour (rows <= 8: ids 1..8)
+  }
+  // reduce the compensated sums across the warp in FP64 (6 values per row)
+  const ksum* v[6] = {&S.ar, &S.ai, &S.br, &S.bi, &S.sr, &S.si};
+#pragma unroll
+  for (int u = 0; u < 6; ++u) {
+    double x = (double)v[u]->s + (double)v[u]->c;
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (lane == 0) part[rw][sub][u] = x;
+  }
+  __syncthreads();
+  if (!valid) return;
+  if constexpr (!GROW)
+    for (int64_t c2 = sub * 32 + lane; c2 < N; c2 += 32 * ASM_W) Arow[c2] = row[c2];
+  if (sub == 0 && lane < 6) {
+    double x = 0.0;
+    for (int w = 0; w < ASM_W; ++w) x += part[rw][w][lane];
+    rowsum[((int64_t)kk * N + i) * 6 + lane] = x;
   }
 }
 
@@ -689,6 +878,11 @@ static float4* sorted_aos(bie_ctx* c) { return reinterpret_cast<float4*>(c->qgeo
 static float4* near_aos(bie_ctx* c) {
   return reinterpret_cast<float4*>(c->qgeo32 + sorted_aos_offset(c) + 16 * (size_t)c->E * c->rule.Q);
 }
+// the colour-sorted elements' condition (of their first node), uint8 [E], after the near records
+static size_t sorted_soft_offset(bie_ctx* c) {
+  return sorted_aos_offset(c) + 16 * (size_t)(c->E * c->rule.Q + c->E * 6 * (int64_t)c->rule.QN);
+}
+static uint8_t* sorted_soft(bie_ctx* c) { return reinterpret_cast<uint8_t*>(c->qgeo32 + sorted_soft_offset(c)); }
 const float4* sorted_aos_ptr(bie_ctx* c) { return sorted_aos(c); }
 
 const float* sorted_table_ptr(bie_ctx* c) { return sorted_table(c); }
@@ -697,12 +891,13 @@ const int32_t* sorted_elems_ptr(bie_ctx* c) { return sorted_elems(c); }
 int ensure_mixed_tables(bie_ctx* c) {
   if (c->qgeo32) return BIE_OK;
   const int64_t nq = c->E * c->rule.Q, nn = c->E * 6 * (int64_t)c->rule.QN;
-  BIE_TRY(dev_alloc(c, (void**)&c->qgeo32, (sorted_aos_offset(c) + 16 * (size_t)(nq + nn)) * sizeof(float)));
+  BIE_TRY(dev_alloc(c, (void**)&c->qgeo32, sorted_soft_offset(c) * sizeof(float) + (size_t)c->E));
   BIE_LAUNCH(k_points_to32<<<(unsigned)((nq + 255) / 256), 256, 0, c->stream>>>(c->qgeo, nq, c->qgeo32, nullptr));
   BIE_LAUNCH(k_points_to32<<<(unsigned)((nn + 255) / 256), 256, 0, c->stream>>>(c->ngeo, nn, c->qgeo32 + P32COUNT * nq,
                                                                                 near_aos(c)));
   BIE_LAUNCH(k_points_to32_sorted<<<(unsigned)((nq + 255) / 256), 256, 0, c->stream>>>(
-      c->qgeo, c->elem_perm, c->elems, c->E, c->rule.Q, sorted_table(c), sorted_elems(c), sorted_aos(c)));
+      c->qgeo, c->elem_perm, c->elems, c->bc == c->bc_flip, c->bc, c->E, c->rule.Q, sorted_table(c), sorted_elems(c),
+      sorted_aos(c), sorted_soft(c)));
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
 }
@@ -748,41 +943,33 @@ int assemble32(bie_ctx* c, const double* kv, int nk, cf* A, int64_t lda, cd* b, 
       for (int a = 1; a < 6; ++a)
         if (c->h_bc[c->h_elems[6 * e + a]] != c->h_bc[c->h_elems[6 * e]]) c->uniform_bc = 0;
   }
-  // the uniform-condition kernel: KB = 2 wavenumbers per thread with the quadrature points of an
-  // element split over two warps (2 rows x 4 warps, 256 threads); its rows in shared memory while
-  // two CTAs fit an SM, else (large N) in A itself; KB = 1 (4 rows x 2 warps) on request
+  // the uniform-condition kernels: two wavenumbers per thread with the quadrature points of an
+  // element split over two warps (one row, 128 threads), the row in shared memory while four CTAs
+  // fit an SM, else (large N) window by window or in A itself; one per thread (4 rows x 2 warps) on
+  // request
   int kb = (kq && c->uniform_bc == 1) ? c->asm_kb : 0;
   if (kb >= 1) {
     const int64_t E = c->E;
     dim3 gq((unsigned)((E + 255) / 256), nk);
-    BIE_LAUNCH(k_known_q32<<<gq, 256, 0, c->stream>>>(sorted_elems(c), E, c->rule.Q, c->qshape32, known, N, kq));
+    BIE_LAUNCH(k_known_q32<<<gq, 256, 0, c->stream>>>(sorted_elems(c), E, c->rule.Q, c->qshape32, known, N, kq, kb == 2));
     if (kb == 2) {
-      const int urows = 2;
-      const bool grow = (size_t)urows * 2 * N * sizeof(cf) > 100 * 1024;
+      const size_t full = (size_t)N * sizeof(float4);
+      const bool grow = full > 50 * 1024;
       // large N: window by window in shared memory where the mesh has column windows
       // ("asm.windows" 0 keeps the rows in A)
-      const bool win = grow && c->nwin > 1 && c->asm_windows != 0 &&
-                       (size_t)urows * 2 * c->win_max * sizeof(cf) <= 100 * 1024;
-      const size_t usmem = win ? (size_t)urows * 2 * c->win_max * sizeof(cf) : grow ? 0 : (size_t)urows * 2 * N * sizeof(cf);
-      dim3 gu((unsigned)((N + urows - 1) / urows), (unsigned)((nk + 1) / 2));
-      if (win) {
-        BIE_TRY((set_smem_max(k_asm32_bulk_u<2, 2, 2>)));
-        BIE_LAUNCH(k_asm32_bulk_u<2, 2, 2><<<gu, 32 * urows * ASM_W * 2, usmem, c->stream>>>(
-            c->nodes, c->normals, c->bc, sorted_elems(c), N, E, c->rule.Q, sorted_aos(c), c->qshape32, c->color_off,
-            c->ncolors, kv, nk, kq, A, lda, rowsum, urows, tp, (float)c->far_r2, c->win_lo, c->wcol_off, c->nwin,
-            c->win_max));
-      } else if (grow) {
-        BIE_LAUNCH(k_asm32_bulk_u<2, 2, 1><<<gu, 32 * urows * ASM_W * 2, 0, c->stream>>>(
-            c->nodes, c->normals, c->bc, sorted_elems(c), N, E, c->rule.Q, sorted_aos(c), c->qshape32, c->color_off,
-            c->ncolors, kv, nk, kq, A, lda, rowsum, urows, tp, (float)c->far_r2, c->win_lo, c->wcol_off, c->nwin,
-            c->win_max));
-      } else {
-        BIE_TRY((set_smem_max(k_asm32_bulk_u<2, 2, 0>)));
-        BIE_LAUNCH(k_asm32_bulk_u<2, 2, 0><<<gu, 32 * urows * ASM_W * 2, usmem, c->stream>>>(
-            c->nodes, c->normals, c->bc, sorted_elems(c), N, E, c->rule.Q, sorted_aos(c), c->qshape32, c->color_off,
-            c->ncolors, kv, nk, kq, A, lda, rowsum, urows, tp, (float)c->far_r2, c->win_lo, c->wcol_off, c->nwin,
-            c->win_max));
-      }
+      const size_t part = (size_t)c->win_max * sizeof(float4);
+      const bool win = grow && c->nwin > 1 && c->asm_windows != 0 && part <= 50 * 1024;
+      dim3 gu((unsigned)N, (unsigned)((nk + 1) / 2));
+      auto go = [&](auto kernel, size_t usmem) -> int {
+        BIE_TRY(set_smem_max(kernel));
+        BIE_LAUNCH(kernel<<<gu, 32 * 2 * ASM_W, usmem, c->stream>>>(
+            c->nodes, c->normals, sorted_soft(c), c->bc == c->bc_flip, sorted_elems(c), N, E, c->rule.Q, sorted_aos(c),
+            c->qshape32, c->color_off, c->ncolors, kv, nk, kq, A, lda, rowsum, (float)c->far_r2, c->win_lo, c->wcol_off, c->nwin, c->win_max));
+        return BIE_OK;
+      };
+      if (win) BIE_TRY(go(k_asm32_pair<2>, part));
+      else if (grow) BIE_TRY(go(k_asm32_pair<1>, 0));
+      else BIE_TRY(go(k_asm32_pair<0>, full));
     } else {
       int urows = 4;
       while (urows > 1 && (size_t)urows * N * sizeof(cf) > 200 * 1024) urows /= 2;
@@ -790,18 +977,15 @@ int assemble32(bie_ctx* c, const double* kv, int nk, cf* A, int64_t lda, cd* b, 
       if (grow) urows = 4;
       const size_t usmem = grow ? 0 : (size_t)urows * N * sizeof(cf);
       dim3 gu((unsigned)((N + urows - 1) / urows), (unsigned)nk);
-      if (grow) {
-        BIE_LAUNCH(k_asm32_bulk_u<1, 1, 1><<<gu, 32 * urows * ASM_W, 0, c->stream>>>(
+      auto go = [&](auto kernel) -> int {
+        BIE_TRY(set_smem_max(kernel));
+        BIE_LAUNCH(kernel<<<gu, 32 * urows * ASM_W, usmem, c->stream>>>(
             c->nodes, c->normals, c->bc, sorted_elems(c), N, E, c->rule.Q, sorted_aos(c), c->qshape32, c->color_off,
-            c->ncolors, kv, nk, kq, A, lda, rowsum, urows, tp, (float)c->far_r2, c->win_lo, c->wcol_off, c->nwin,
-            c->win_max));
-      } else {
-        BIE_TRY((set_smem_max(k_asm32_bulk_u<1, 1, 0>)));
-        BIE_LAUNCH(k_asm32_bulk_u<1, 1, 0><<<gu, 32 * urows * ASM_W, usmem, c->stream>>>(
-            c->nodes, c->normals, c->bc, sorted_elems(c), N, E, c->rule.Q, sorted_aos(c), c->qshape32, c->color_off,
-            c->ncolors, kv, nk, kq, A, lda, rowsum, urows, tp, (float)c->far_r2, c->win_lo, c->wcol_off, c->nwin,
-            c->win_max));
-      }
+            c->ncolors, kv, kq, A, lda, rowsum, urows, (float)c->far_r2));
+        return BIE_OK;
+      };
+      if (grow) BIE_TRY(go(k_asm32_bulk_u<1>));
+      else BIE_TRY(go(k_asm32_bulk_u<0>));
     }
   }
   if (kb == 0) {

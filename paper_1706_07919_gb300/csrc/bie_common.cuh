@@ -462,6 +462,21 @@ __device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
 }
 __device__ __forceinline__ f2 f2_neg(f2 a) { return f2{a.v ^ 0x8000000080000000ull}; }
 
+// Both halves of cis_ffprod2's constants (2/pi negated, the rounding constant, pi/2 in three parts, the
+// Taylor coefficients of cis_split), read as operands from constant memory: packed instructions take
+// no immediates, and as literals they cost two moves each whenever registers run short.
+static __constant__ float2 kCis2[14] = {
+    {-0.636619772367581343f, -0.636619772367581343f}, {kRoundMagic, kRoundMagic},
+    {kHalfPi1, kHalfPi1}, {kHalfPi2, kHalfPi2}, {kHalfPi3, kHalfPi3},
+    {2.75573192239858907e-6f, 2.75573192239858907e-6f}, {-1.98412698412698413e-4f, -1.98412698412698413e-4f},
+    {8.33333333333333333e-3f, 8.33333333333333333e-3f}, {-1.66666666666666667e-1f, -1.66666666666666667e-1f},
+    {-2.75573192239858907e-7f, -2.75573192239858907e-7f}, {2.48015873015873016e-5f, 2.48015873015873016e-5f},
+    {-1.38888888888888889e-3f, -1.38888888888888889e-3f}, {4.16666666666666667e-2f, 4.16666666666666667e-2f},
+    {-0.5f, -0.5f}};
+__device__ __forceinline__ f2 cis2_const(int i) {
+  return f2{*reinterpret_cast<const unsigned long long*>(&kCis2[i])};
+}
+
 // cis_ffprod for two wavenumbers at one distance: k = -(nkh + nkl) per half (the negated float-float
 // wavenumbers: with them every subtraction of cis_ffprod and cis_split becomes a fused multiply-add
 // of the same magnitude, and the results are theirs bit for bit).
@@ -471,21 +486,21 @@ __device__ __forceinline__ void cis_ffprod2(f2 nkh, f2 nkl, ff R, f2& c, f2& s) 
   f2 e = f2_fma(nkh, Rh, f2_neg(np));  // -(tail)
   e = f2_fma(nkh, Rl, e);
   e = f2_fma(nkl, Rh, e);
-  const f2 qm = f2_fma(np, f2_dup(-0.636619772367581343f), f2_dup(kRoundMagic));
-  const f2 n = f2_sub(qm, f2_dup(kRoundMagic));
-  const f2 nh = f2_fma(n, f2_dup(kHalfPi1), np);  // -(p - n h1)
-  f2 t = f2_fma(n, f2_dup(kHalfPi2), e);          // -(e - n h2 - n h3)
-  t = f2_fma(n, f2_dup(kHalfPi3), t);
+  const f2 qm = f2_fma(np, cis2_const(0), cis2_const(1));
+  const f2 n = f2_sub(qm, cis2_const(1));
+  const f2 nh = f2_fma(n, cis2_const(2), np);  // -(p - n h1)
+  f2 t = f2_fma(n, cis2_const(3), e);          // -(e - n h2 - n h3)
+  t = f2_fma(n, cis2_const(4), t);
   const f2 nv = f2_add(nh, t);
   const f2 v2 = f2_mul(nv, nv);
-  f2 ps = f2_fma(v2, f2_dup(2.75573192239858907e-6f), f2_dup(-1.98412698412698413e-4f));  // 1/9!, -1/7!
-  ps = f2_fma(v2, ps, f2_dup(8.33333333333333333e-3f));                                   // 1/5!
-  ps = f2_fma(v2, ps, f2_dup(-1.66666666666666667e-1f));                                  // -1/3!
+  f2 ps = f2_fma(v2, cis2_const(5), cis2_const(6));  // 1/9!, -1/7!
+  ps = f2_fma(v2, ps, cis2_const(7));                                   // 1/5!
+  ps = f2_fma(v2, ps, cis2_const(8));                                  // -1/3!
   const f2 nsv = f2_fma(f2_mul(nv, v2), ps, nv);                                          // -sin
-  f2 pc = f2_fma(v2, f2_dup(-2.75573192239858907e-7f), f2_dup(2.48015873015873016e-5f));  // -1/10!, 1/8!
-  pc = f2_fma(v2, pc, f2_dup(-1.38888888888888889e-3f));                                  // -1/6!
-  pc = f2_fma(v2, pc, f2_dup(4.16666666666666667e-2f));                                   // 1/4!
-  pc = f2_fma(v2, pc, f2_dup(-0.5f));
+  f2 pc = f2_fma(v2, cis2_const(9), cis2_const(10));  // -1/10!, 1/8!
+  pc = f2_fma(v2, pc, cis2_const(11));                                  // -1/6!
+  pc = f2_fma(v2, pc, cis2_const(12));                                   // 1/4!
+  pc = f2_fma(v2, pc, cis2_const(13));
   const f2 cv = f2_fma(v2, pc, f2_dup(1.0f));
   float ns[2], co[2], q[2], cc[2], ss[2];
   f2_split(nsv, ns[0], ns[1]);
@@ -493,12 +508,13 @@ __device__ __forceinline__ void cis_ffprod2(f2 nkh, f2 nkl, ff R, f2& c, f2& s) 
   f2_split(qm, q[0], q[1]);
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    // quadrant i: (c, s) = (cv, sv), (-sv, cv), (-cv, -sv), (sv, -cv); signs by the sign bit
-    const unsigned i = __float_as_uint(q[h]);
-    const unsigned sv = __float_as_uint(ns[h]) ^ 0x80000000u, cu = __float_as_uint(co[h]);
-    const unsigned a = (i & 1u) ? sv : cu, b = (i & 1u) ? cu : sv;
-    cc[h] = __uint_as_float(a ^ (((i + 1u) << 30) & 0x80000000u));
-    ss[h] = __uint_as_float(b ^ ((i << 30) & 0x80000000u));
+    // quadrant i (mod 4): (c, s) = (cv, sv), (-sv, cv), (-cv, -sv), (sv, -cv) with sv = -ns; the sign
+    // of c flips with bit 1 of i and that of s with bit 1 of i + 3 once sv's own sign is counted
+    const unsigned i = __float_as_uint(q[h]), t = i << 30;
+    const unsigned nu = __float_as_uint(ns[h]), cu = __float_as_uint(co[h]);
+    const unsigned a = (i & 1u) ? nu : cu, b = (i & 1u) ? cu : nu;
+    cc[h] = __uint_as_float(a ^ (t & 0x80000000u));
+    ss[h] = __uint_as_float(b ^ ((t + 0xc0000000u) & 0x80000000u));
   }
   c = f2_make(cc[0], cc[1]);
   s = f2_make(ss[0], ss[1]);
