@@ -4,7 +4,8 @@
 //   spectrum:  S[p][m] = sum_n s[p][n] exp(+2 pi i m n / Nt) = conj(FFT(s))_m  (real s)
 //   synthesis: out[p][x][n] = (1/Nt) Re sum_m c_m exp(-2 pi i m n / Nt),  c_m = w_m S[p][m] T[m][x],
 //              w_0 = w_{Nt/2} = 1, else 2 (the m > Nt/2 half is the complex conjugate).
-// One CTA transforms one signal in shared memory with a Stockham (self-sorting) radix-2 FFT.
+// Spectra and the shortest signals: one CTA transforms one signal in shared memory with a Stockham
+// (self-sorting) radix-2 FFT; longer signals by k_synth_real.
 #include <mutex>
 
 #include "bie_common.cuh"
@@ -61,7 +62,7 @@ __global__ void k_pulse_spectrum(const double* __restrict__ s, int n, const doub
   for (int t = threadIdx.x; t <= n / 2; t += blockDim.x) o[t] = {(double)X[t].re, -(double)X[t].im};
 }
 
-// grid: (M, P); one signal per CTA.
+// Synthesis of signals of fewer than 32 samples; grid: (M, P), one signal per CTA.
 template <class S, class O>
 __global__ void k_synth(const cd* __restrict__ T, const int64_t* __restrict__ midx, int nk, int64_t M,
                         const cd* __restrict__ Sp, int n, const double2* __restrict__ tw, O* __restrict__ out) {
@@ -86,6 +87,323 @@ __global__ void k_synth(const cd* __restrict__ T, const int64_t* __restrict__ mi
   for (int t = threadIdx.x; t < n; t += blockDim.x) o[t] = (O)(X[t].re * inv);
 }
 
+// ---- synthesis of signals of 32 samples and more ------------------------------------------------
+// A real signal of n samples is one complex transform of h = n / 2 values,
+//   out[2 j] + i out[2 j + 1] = sum_k Z_k exp(-2 pi i j k / h),
+//   Z_k = (H_k + conj(H_{h-k})) + i exp(-2 pi i k / n) (H_k - conj(H_{h-k})),
+// H_m = S_m T_m / n for 0 < m < h, H_0 and H_h the real parts of theirs.  h / 16 threads take a
+// signal, 16 values each in registers: one pass of radix 2, 4 or 8 where log2 h leaves a
+// remainder, then radix-16 passes (Stockham order), exchanging through shared memory between
+// passes -- two exchanges for n = 4096, where the radix-2 kernel had twelve round trips through
+// shared memory, each with a division and a twiddle converted from FP64.  A CTA of about 256 threads holds
+// SB = 4096 / h neighbouring points, so that T is read in whole sectors, and takes PG pulses one
+// after the other with the points' T kept in shared memory.  FP32: S and T enter as float-float
+// (T split once per point, S once per call, `sp` or, without it, in the kernel) and their product
+// rounds once, as the FP64 product rounded to FP32 did: eight FP64 operations a frequency, point and
+// pulse would cost 0.4 ms below on this GPU's narrow FP64 pipe.
+// Bound: shared memory and the transforms' arithmetic in about equal parts (DRAM: 1.1 GB written).
+// Measured, 8 pulses x 8192 points x 4096 samples from 512 frequencies in FP32: 7.2 -> 1.06 ms (1.86
+// with the passes' factors read out of the plain table).
+// Relative error against FP64 1.2e-7 before and after.  128 registers (2 CTAs) measured 1.18 ms.
+template <class S> __device__ __forceinline__ C2<S> c2mul(C2<S> a, C2<S> b) {
+  return {a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re};
+}
+template <class S> __device__ __forceinline__ C2<S> c2add(C2<S> a, C2<S> b) { return {a.re + b.re, a.im + b.im}; }
+template <class S> __device__ __forceinline__ C2<S> c2sub(C2<S> a, C2<S> b) { return {a.re - b.re, a.im - b.im}; }
+
+template <class S> __device__ __forceinline__ void fft2(C2<S>& a, C2<S>& b) {
+  const C2<S> t = c2sub(a, b);
+  a = c2add(a, b);
+  b = t;
+}
+template <class S> __device__ __forceinline__ void fft4(C2<S>& a, C2<S>& b, C2<S>& c, C2<S>& d) {
+  const C2<S> t0 = c2add(a, c), t1 = c2sub(a, c), t2 = c2add(b, d), u = c2sub(b, d), t3 = {u.im, -u.re};
+  a = c2add(t0, t2);
+  b = c2add(t1, t3);
+  c = c2sub(t0, t2);
+  d = c2sub(t1, t3);
+}
+// Transforms of v[0 .. R-1]; output k is left at v[fft_at<R>(k)].
+template <int R, class S> __device__ __forceinline__ void fft_small(C2<S>* v) {
+  if constexpr (R == 2) {
+    fft2(v[0], v[1]);
+  } else if constexpr (R == 4) {
+    fft4(v[0], v[1], v[2], v[3]);
+  } else if constexpr (R == 8) {
+    const S h = (S)0.70710678118654752440;
+    fft4(v[0], v[2], v[4], v[6]);
+    fft4(v[1], v[3], v[5], v[7]);
+    v[3] = C2<S>{h * (v[3].re + v[3].im), h * (v[3].im - v[3].re)};
+    v[5] = C2<S>{v[5].im, -v[5].re};
+    v[7] = C2<S>{h * (v[7].im - v[7].re), -h * (v[7].re + v[7].im)};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) fft2(v[2 * q], v[2 * q + 1]);
+  } else {
+    const S h = (S)0.70710678118654752440, c = (S)0.92387953251128675613, s = (S)0.38268343236508977173;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) fft4(v[i], v[i + 4], v[i + 8], v[i + 12]);
+    v[5] = c2mul(v[5], C2<S>{c, -s});
+    v[9] = C2<S>{h * (v[9].re + v[9].im), h * (v[9].im - v[9].re)};
+    v[13] = c2mul(v[13], C2<S>{s, -c});
+    v[6] = C2<S>{h * (v[6].re + v[6].im), h * (v[6].im - v[6].re)};
+    v[10] = C2<S>{v[10].im, -v[10].re};
+    v[14] = C2<S>{h * (v[14].im - v[14].re), -h * (v[14].re + v[14].im)};
+    v[7] = c2mul(v[7], C2<S>{s, -c});
+    v[11] = C2<S>{h * (v[11].im - v[11].re), -h * (v[11].re + v[11].im)};
+    v[15] = c2mul(v[15], C2<S>{-c, s});
+#pragma unroll
+    for (int q = 0; q < 4; ++q) fft4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+  }
+}
+template <int R> __device__ __forceinline__ constexpr int fft_at(int k) {
+  return R == 16 ? 4 * (k & 3) + (k >> 2) : R == 8 ? 2 * (k & 3) + (k >> 2) : k;
+}
+// element i of a signal's buffer: one spare element after every 16 keeps the passes' strided writes
+// off the same banks
+__device__ __forceinline__ int fft_pad(int i) { return i + (i >> 4); }
+inline int fft_pad_len(int h) { return h + 1 + ((h + 1) >> 4) + 1; }
+
+// tw[j] = exp(-2 pi i j / n), j < n / 2, in the transform's own type (rounded from FP64).  With
+// `count` > n / 2 the radix-16 passes' factors follow in the order in which they are read: for a
+// pass after Ns values (Ns = R0, 16 R0, ... < h) the 16 Ns factors exp(-2 pi i r t / (16 Ns)) at
+// r Ns + t -- read from tw itself a warp's factors lie in up to 32 lines.
+inline int pass_radix0(int L) { return (L & 3) ? 1 << (L & 3) : 16; }
+inline int twiddle_count(int n) {  // table entries, pass factors included
+  int L = 0;
+  while ((2 << L) < n) ++L;
+  const int h = n / 2;
+  int c = h;
+  for (int Ns = pass_radix0(L); Ns < h; Ns <<= 4) c += 16 * Ns;
+  return c;
+}
+template <class S>
+__global__ void k_twiddles_of(int n, int R0, int count, C2<S>* tw) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= count) return;
+  const int h = n / 2;
+  double x = 2.0 * (double)i / (double)n;
+  int at = i - h, Ns = R0;
+  while (at >= 16 * Ns && at >= 0) {
+    at -= 16 * Ns;
+    Ns <<= 4;
+  }
+  if (at >= 0) x = 2.0 * (double)((at / Ns) * (at % Ns)) / (double)(16 * Ns);
+  double s, c;
+  sincospi(x, &s, &c);
+  tw[i] = {(S)c, (S)(-s)};
+}
+template <class S> __device__ __forceinline__ C2<S> twiddle(const C2<S>* __restrict__ tw, int i, int h) {
+  const C2<S> w = tw[i & (h - 1)];  // i < 2 h = n: the second half is the first negated
+  return (i & h) ? C2<S>{-w.re, -w.im} : w;
+}
+
+// (hi, lo) of a complex value: re hi, re lo, im hi, im lo
+__device__ __forceinline__ float4 split_cd(cd v) {
+  const ff r = ff_from_double(v.re), i = ff_from_double(v.im);
+  return make_float4(r.hi, r.lo, i.hi, i.lo);
+}
+__global__ void k_split_spectra(const cd* __restrict__ Sp, int64_t n, float4* __restrict__ out) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t < n) out[t] = split_cd(Sp[t]);
+}
+// a b - c d or a b + c d from float-float factors, rounded once
+__device__ __forceinline__ float ff_dot2(float ah, float al, float bh, float bl, float ch, float cl, float dh, float dl) {
+  const float p = __fmul_rn(ah, bh), q = __fmul_rn(ch, dh);
+  const float e = __fmaf_rn(ah, bl, __fmaf_rn(al, bh, __fmaf_rn(ah, bh, -p)));
+  const float f = __fmaf_rn(ch, dl, __fmaf_rn(cl, dh, __fmaf_rn(ch, dh, -q)));
+  const ff t = ff_two_sum(p, q);
+  return __fadd_rn(t.hi, __fadd_rn(t.lo, __fadd_rn(e, f)));
+}
+__device__ __forceinline__ C2<float> ff_cmul(float4 s, float4 t) {
+  return {ff_dot2(s.x, s.y, t.x, t.y, -s.z, -s.w, t.z, t.w), ff_dot2(s.x, s.y, t.z, t.w, s.z, s.w, t.x, t.y)};
+}
+
+// First pass of radix R0 (inputs made from the spectrum), then radix-16 passes; the last one leaves
+// its outputs in v (output fft_at<16>(r) of butterfly j is z[j + r Ns]).
+template <int L, class S>
+__device__ __forceinline__ void real_fft(C2<S>* __restrict__ buf, const C2<S>* __restrict__ tw, bool passes, int j,
+                                         C2<S>* v) {
+  constexpr int h = 1 << L, R0 = (L & 3) ? 1 << (L & 3) : 16, NT = h / 16;
+#pragma unroll
+  for (int b = 0; b < 16 / R0; ++b)
+#pragma unroll
+    for (int q = 0; q < R0; ++q) {
+      const int k = j + b * NT + q * (h / R0);
+      const C2<S> H = buf[fft_pad(k)], C = buf[fft_pad(h - k)];
+      C2<S> z;
+      if (k == 0) {
+        z = {H.re + C.re, H.re - C.re};
+      } else {
+        const C2<S> sum = {H.re + C.re, H.im - C.im}, dif = {H.re - C.re, H.im + C.im};
+        const C2<S> d = c2mul(tw[k], dif);
+        z = {sum.re - d.im, sum.im + d.re};
+      }
+      v[b * R0 + q] = z;
+    }
+#pragma unroll
+  for (int b = 0; b < 16 / R0; ++b) fft_small<R0, S>(v + b * R0);
+#pragma unroll
+  for (int Ns = R0; Ns < h; Ns <<= 4) {  // (Ns: product of the radices so far)
+    const int Np = Ns == R0 ? 1 : Ns >> 4;  // the previous pass's
+    __syncthreads();
+    if (Ns == R0) {
+#pragma unroll
+      for (int b = 0; b < 16 / R0; ++b)
+#pragma unroll
+        for (int r = 0; r < R0; ++r) buf[fft_pad((j + b * NT) * R0 + r)] = v[b * R0 + fft_at<R0>(r)];
+    } else {
+      const int at = (j / Np) * Np * 16 + (j & (Np - 1));
+#pragma unroll
+      for (int r = 0; r < 16; ++r) buf[fft_pad(at + r * Np)] = v[fft_at<16>(r)];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = buf[fft_pad(j + r * NT)];
+    if (passes) {
+      const C2<S>* pw = tw + h + (Ns == R0 ? 0 : 16 * R0 * ((Ns / R0 - 1) / 15)) + (j & (Ns - 1));
+#pragma unroll
+      for (int r = 1; r < 16; ++r) v[r] = c2mul(v[r], pw[r * Ns]);
+    } else {
+      const int step = (j & (Ns - 1)) * (2 * h / (Ns * 16));
+#pragma unroll
+      for (int r = 1; r < 16; ++r) v[r] = c2mul(v[r], twiddle<S>(tw, r * step, h));
+    }
+    fft_small<16, S>(v);
+  }
+}
+
+// grid (ceil(M / SB), ceil(P / PG)), block SB h / 16.  Dynamic shared memory: SB fft_pad_len(h)
+// values, then (KEEP: PG > 1) the points' T, [nk][SB] as float4 (FP32) or C2<double>.
+template <int L, class S, bool KEEP>
+__global__ void __launch_bounds__(256, sizeof(S) == 4 ? 3 : 1) k_synth_real(const cd* __restrict__ T, const int64_t* __restrict__ midx, int nk,
+                                                    int64_t M, const cd* __restrict__ Sp, const float4* __restrict__ sp,
+                                                    int P, int PG, const C2<S>* __restrict__ tw, bool passes,
+                                                    S* __restrict__ out, int wide) {
+  constexpr int h = 1 << L, n = 2 * h, NT = h / 16, SB = 4096 / h;
+  constexpr bool F32 = sizeof(S) == 4;
+  extern __shared__ float4 synth_smem[];
+  const int len = h + 1 + ((h + 1) >> 4) + 1;
+  C2<S>* bufs = reinterpret_cast<C2<S>*>(synth_smem);
+  float4* kept = reinterpret_cast<float4*>(reinterpret_cast<unsigned char*>(synth_smem) +
+                                           (((size_t)SB * len * sizeof(C2<S>) + 15) & ~(size_t)15));
+  const int tid = threadIdx.x, pt = tid / NT, j = tid - pt * NT;
+  const int64_t x0 = (int64_t)blockIdx.x * SB;
+  C2<S>* buf = bufs + pt * len;
+  if (KEEP)
+    for (int e = tid; e < nk * SB; e += SB * NT) {
+      const int r = e / SB, q = e - r * SB;
+      const cd t = x0 + q < M ? T[(int64_t)r * M + x0 + q] : cd{0.0, 0.0};
+      if constexpr (F32) kept[e] = split_cd(t);
+      else reinterpret_cast<cd*>(kept)[e] = t;
+    }
+  const int p1 = min(P, (int)(blockIdx.y + 1) * PG);
+  for (int p = blockIdx.y * PG; p < p1; ++p) {
+    __syncthreads();  // the kept values; the previous pulse's last reads of the buffers
+    for (int e = tid; e < SB * len; e += SB * NT) bufs[e] = {(S)0, (S)0};
+    __syncthreads();
+    const cd* Srow = Sp + (int64_t)p * (h + 1);
+    for (int e = tid; e < nk * SB; e += SB * NT) {
+      const int r = e / SB, q = e - r * SB;
+      const int m = (int)midx[r];
+      C2<S> v;
+      if constexpr (F32) {
+        const float4 s4 = sp ? sp[(int64_t)p * (h + 1) + m] : split_cd(Srow[m]);
+        float4 t4;
+        if (KEEP) t4 = kept[e];
+        else t4 = x0 + q < M ? split_cd(T[(int64_t)r * M + x0 + q]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        v = ff_cmul(s4, t4);
+        // outside a safe range of FP32 (zero, tiny, huge, not finite): the product in FP64
+        const float ta = fmaxf(fabsf(t4.x), fabsf(t4.z)), sa = fmaxf(fabsf(s4.x), fabsf(s4.z));
+        if (!(ta >= 1e-25f && ta <= 1e25f && sa >= 1e-25f && sa <= 1e25f) && x0 + q < M) {
+          const cd a = cmul(Srow[m], T[(int64_t)r * M + x0 + q]);
+          v = {(float)a.re, (float)a.im};
+        }
+      } else {
+        cd t;
+        if (KEEP) t = reinterpret_cast<cd*>(kept)[e];
+        else t = x0 + q < M ? T[(int64_t)r * M + x0 + q] : cd{0.0, 0.0};
+        const cd a = cmul(Srow[m], t);
+        v = {a.re, a.im};
+      }
+      constexpr S inv = (S)1 / (S)n;
+      bufs[q * len + fft_pad(m)] = {v.re * inv, v.im * inv};
+    }
+    __syncthreads();
+    C2<S> v[16];
+    real_fft<L, S>(buf, tw, passes, j, v);
+    if (x0 + pt < M) {
+      S* o = out + ((int64_t)p * M + x0 + pt) * n;
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        const C2<S> z = v[fft_at<16>(r)];
+        const int i = 2 * (j + r * NT);
+        if (wide) {  // the output is aligned to pairs
+          if constexpr (F32) *reinterpret_cast<float2*>(o + i) = make_float2(z.re, z.im);
+          else *reinterpret_cast<double2*>(o + i) = make_double2(z.re, z.im);
+        } else {
+          o[i] = z.re;
+          o[i + 1] = z.im;
+        }
+      }
+    }
+  }
+}
+
+// Twiddles of a transform of n samples: FP64 pairs for n < 32 (the radix-2 kernel), else in its type.
+// passes: the pass factors too.
+template <class S>
+static void launch_twiddles(int n, void* tw, bool passes, cudaStream_t st) {
+  int L = 0;
+  while ((2 << L) < n) ++L;
+  const int count = passes ? twiddle_count(n) : n / 2;
+  if (n < 32)
+    BIE_LAUNCH(k_twiddles<<<1, 256, 0, st>>>(n, (double2*)tw));
+  else
+    BIE_LAUNCH(k_twiddles_of<S><<<(count + 127) / 128, 128, 0, st>>>(n, pass_radix0(L), count, (C2<S>*)tw));
+}
+
+// sp: the spectra split into float-float (FP32 only; NULL: split in the kernel).
+template <class S>
+static int launch_synth(const cd* T, const int64_t* midx, int nk, int64_t M, const cd* Sp, const float4* sp, int64_t P,
+                        int n, const void* tw, bool passes, S* out, int nsm, cudaStream_t st) {
+  if (n < 32) {
+    const dim3 g((unsigned)M, (unsigned)P);
+    const size_t smem = 2 * (size_t)n * sizeof(C2<S>);
+    BIE_LAUNCH(k_synth<S, S><<<g, 32, smem, st>>>(T, midx, nk, M, Sp, n, (const double2*)tw, out));
+    return BIE_OK;
+  }
+  const int h = n / 2, SB = 4096 / h, wide = ((uintptr_t)out % (2 * sizeof(S))) == 0;
+  const int64_t bx = (M + SB - 1) / SB;
+  if (bx > 0x7fffffff) return fail(BIE_ERR_INVALID_ARG, "too many observation points");
+  const size_t bufs = ((size_t)SB * fft_pad_len(h) * sizeof(C2<S>) + 15) & ~(size_t)15;
+  const size_t kept = (size_t)nk * SB * 16;
+  // Pulses per CTA: all, with T kept, once the points alone give every SM a few CTAs; else one
+  // (more CTAs; T is read once per pulse).  The kept T must leave room for two CTAs.
+  const bool keep = P > 1 && bx >= 4 * nsm && bufs + kept <= 100 * 1024;
+  const int PG = keep ? (int)P : 1;
+  const dim3 g((unsigned)bx, (unsigned)(keep ? 1 : P));
+  auto go = [&](auto kernel) -> int {
+    BIE_TRY(set_smem_max(kernel));
+    BIE_LAUNCH(kernel<<<g, SB * (h / 16), bufs + (keep ? kept : 0), st>>>(T, midx, nk, M, Sp, sp, (int)P, PG,
+                                                                          (const C2<S>*)tw, passes, out, wide));
+    return BIE_OK;
+  };
+  switch (h) {
+#define BIE_SYNTH(L) \
+  case 1 << L: return keep ? go(k_synth_real<L, S, true>) : go(k_synth_real<L, S, false>)
+    BIE_SYNTH(4);
+    BIE_SYNTH(5);
+    BIE_SYNTH(6);
+    BIE_SYNTH(7);
+    BIE_SYNTH(8);
+    BIE_SYNTH(9);
+    BIE_SYNTH(10);
+    BIE_SYNTH(11);
+#undef BIE_SYNTH
+  }
+  return fail(BIE_ERR_INVALID_ARG, "Nt out of range");
+}
+
 static int twiddle_table(bie_ctx* c, int n, double2** tw) {
   BIE_TRY(ensure_buf(c, c->work2, (size_t)(n / 2 + 1) * sizeof(double2)));
   *tw = (double2*)c->work2.p;
@@ -106,18 +424,22 @@ int pulse_spectrum(bie_ctx* c, const double* s, int64_t P, int n, cd* Sout) {
 
 int synthesize(bie_ctx* c, const cd* T, const int64_t* midx_dev, int nk, int64_t M, const cd* Sp, int64_t P, int n,
                void* out, int out_dtype) {
-  double2* tw;
-  BIE_TRY(twiddle_table(c, n, &tw));
-  dim3 g((unsigned)M, (unsigned)P);
-  int threads = std::min(512, std::max(32, n / 2));
-  if (out_dtype == 0) {
-    size_t smem = 2 * (size_t)n * sizeof(C2<double>);
-    BIE_TRY((set_smem_max(k_synth<double, double>)));
-    BIE_LAUNCH(k_synth<double, double><<<g, threads, smem, c->stream>>>(T, midx_dev, nk, M, Sp, n, tw, (double*)out));
+  // twiddles (at most FP64 pairs), then the spectra in float-float (FP32)
+  const size_t twb = (size_t)(twiddle_count(n) + 16) * sizeof(double2);
+  const int64_t ns = P * (n / 2 + 1);
+  const bool f32 = out_dtype != 0;
+  BIE_TRY(ensure_buf(c, c->work2, twb + (f32 ? (size_t)ns * sizeof(float4) : 0)));
+  void* tw = c->work2.p;
+  int nsm = 0;
+  BIE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
+  if (f32) {
+    float4* sp = (float4*)((char*)tw + twb);
+    launch_twiddles<float>(n, tw, true, c->stream);
+    BIE_LAUNCH(k_split_spectra<<<(unsigned)((ns + 255) / 256), 256, 0, c->stream>>>(Sp, ns, sp));
+    BIE_TRY(launch_synth<float>(T, midx_dev, nk, M, Sp, sp, P, n, tw, true, (float*)out, nsm, c->stream));
   } else {
-    size_t smem = 2 * (size_t)n * sizeof(C2<float>);
-    BIE_TRY((set_smem_max(k_synth<float, float>)));
-    BIE_LAUNCH(k_synth<float, float><<<g, threads, smem, c->stream>>>(T, midx_dev, nk, M, Sp, n, tw, (float*)out));
+    launch_twiddles<double>(n, tw, true, c->stream);
+    BIE_TRY(launch_synth<double>(T, midx_dev, nk, M, Sp, nullptr, P, n, tw, true, (double*)out, nsm, c->stream));
   }
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
@@ -248,17 +570,15 @@ extern "C" int bie_synthesize_noalloc(const void* T, const int64_t* midx, int64_
   double2* tw = (double2*)base;  // n/2 entries, rewritten by every call
   int64_t* md = (int64_t*)((char*)base + kNoAllocScratchBytes / 2);
   if (Nk > 0) BIE_CUDA_TRY(cudaMemcpyAsync(md, midx, Nk * sizeof(int64_t), cudaMemcpyHostToDevice, st));
-  BIE_LAUNCH(k_twiddles<<<(n / 2 + 255) / 256, 256, 0, st>>>(n, tw));
-  dim3 g((unsigned)M, (unsigned)P);
-  const int threads = std::min(512, std::max(32, n / 2));
+  int dev = 0, nsm = 0;
+  BIE_CUDA_TRY(cudaGetDevice(&dev));
+  BIE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   if (out_dtype == 0) {
-    const size_t smem = 2 * (size_t)n * sizeof(C2<double>);
-    BIE_TRY((set_smem_max(k_synth<double, double>)));
-    BIE_LAUNCH(k_synth<double, double><<<g, threads, smem, st>>>((const cd*)T, md, (int)Nk, M, (const cd*)S, n, tw, (double*)out));
+    launch_twiddles<double>(n, tw, false, st);
+    BIE_TRY(launch_synth<double>((const cd*)T, md, (int)Nk, M, (const cd*)S, nullptr, P, n, tw, false, (double*)out, nsm, st));
   } else {
-    const size_t smem = 2 * (size_t)n * sizeof(C2<float>);
-    BIE_TRY((set_smem_max(k_synth<float, float>)));
-    BIE_LAUNCH(k_synth<float, float><<<g, threads, smem, st>>>((const cd*)T, md, (int)Nk, M, (const cd*)S, n, tw, (float*)out));
+    launch_twiddles<float>(n, tw, false, st);
+    BIE_TRY(launch_synth<float>((const cd*)T, md, (int)Nk, M, (const cd*)S, nullptr, P, n, tw, false, (float*)out, nsm, st));
   }
   BIE_CUDA_TRY(cudaGetLastError());
   // the host index array must outlive its asynchronous copy

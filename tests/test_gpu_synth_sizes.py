@@ -1,0 +1,64 @@
+"""Synthesis over every transform length, ragged point counts and pulse groupings, against the
+discrete Fourier sum of Eq. (inverseFourier) in FP64 (numpy).
+
+Tolerances: a transform of n samples makes log2 n additions and rotations of relative error a few eps
+each, so its relative 2-norm error is below 4 eps log2 n: 12 x 4 x 2^-24 = 2.9e-6 in FP32 and
+12 x 4 x 2^-53 = 5.4e-15 in FP64, plus eps of the result (and 2 eps of the reference)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _reference(T, midx, S, Nt):
+    H = np.zeros((S.shape[0], T.shape[1], Nt // 2 + 1), complex)
+    H[:, :, midx] = S[:, None, midx] * T.T[None]
+    return np.fft.irfft(np.conj(H), n=Nt, axis=2)
+
+
+def _case(Nt, M, P, seed, picked):
+    rng = np.random.default_rng(seed)
+    nm = Nt // 2 + 1
+    midx = np.sort(rng.choice(nm, max(1, nm // 3), replace=False)) if picked else np.arange(nm)
+    T = rng.standard_normal((len(midx), M)) + 1j * rng.standard_normal((len(midx), M))
+    S = rng.standard_normal((P, nm)) + 1j * rng.standard_normal((P, nm))
+    return T, midx.astype(np.int64), S
+
+
+@pytest.mark.parametrize("f32", [False, True])
+@pytest.mark.parametrize("Nt", [2 ** i for i in range(1, 13)])
+def test_synthesis_over_lengths(Nt, f32):
+    import torch
+    from paper_1706_07919_gb300 import Solver
+    from paper_1706_07919_gb300 import binding as B
+
+    sol = Solver(0)
+    dt = torch.float32 if f32 else torch.float64
+    eps = 2.0 ** -24 if f32 else 2.0 ** -53
+    # one point; ragged groups of points; enough points that a CTA keeps them for all pulses
+    for M, P, picked in ((1, 1, False), (3, 2, True), (41, 5, False), (4 * 152 * max(1, 8192 // Nt) + 1, 2, True)):
+        T, midx, S = _case(Nt, M, P, Nt + M, picked)
+        Td, Sd = torch.tensor(T, device="cuda:0"), torch.tensor(S, device="cuda:0")
+        ref = _reference(T, midx, S, Nt)
+        tol = (4 * np.log2(Nt) + 3) * eps
+        got = sol.synthesize(Td, midx, Sd, Nt, dt).cpu().numpy()
+        assert np.linalg.norm(got - ref) <= tol * np.linalg.norm(ref), (M, P)
+        out = torch.empty((P, M, Nt), dtype=dt, device="cuda:0")
+        B.bie_synthesize_noalloc(Td, midx, Sd, Nt, out, 1 if f32 else 0)
+        assert np.linalg.norm(out.cpu().numpy() - ref) <= tol * np.linalg.norm(ref), (M, P)
+    sol.close()
+
+
+def test_fp32_synthesis_takes_values_outside_fp32():
+    """Field spectra below and above FP32's range with pulses that bring the product back into it."""
+    import torch
+    from paper_1706_07919_gb300 import Solver
+
+    sol = Solver(0)
+    T, midx, S = _case(64, 5, 3, 1, False)
+    for scale in (1e-60, 1e-33, 1e33, 1e60):
+        got = sol.synthesize(torch.tensor(T * scale, device="cuda:0"), midx, torch.tensor(S / scale, device="cuda:0"), 64,
+                             torch.float32).cpu().numpy()
+        ref = _reference(T, midx, S, 64)
+        assert np.linalg.norm(got - ref) <= 27 * 2.0 ** -24 * np.linalg.norm(ref)
+    sol.close()
