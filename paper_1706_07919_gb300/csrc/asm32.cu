@@ -924,6 +924,8 @@ double far_radius2(bie_ctx* c) {
   return c->far_r2;
 }
 
+bool uniform_conditions(bie_ctx* c);
+
 int assemble32(bie_ctx* c, const double* kv, int nk, cf* A, int64_t lda, cd* b, cd* known, double* rowsum, cf* kq) {
   const int64_t N = c->N;
   BIE_TRY(ensure_mixed_tables(c));
@@ -937,17 +939,11 @@ int assemble32(bie_ctx* c, const double* kv, int nk, cf* A, int64_t lda, cd* b, 
   if (c->rule.Q > 64) return fail(BIE_ERR_INVALID_ARG, "standard rule too large");
   const TwoPi3 tp = two_pi3();
   far_radius2(c);
-  if (c->uniform_bc < 0) {  // does every element carry one condition on its six nodes?
-    c->uniform_bc = 1;
-    for (int64_t e = 0; e < c->E && c->uniform_bc; ++e)
-      for (int a = 1; a < 6; ++a)
-        if (c->h_bc[c->h_elems[6 * e + a]] != c->h_bc[c->h_elems[6 * e]]) c->uniform_bc = 0;
-  }
   // the uniform-condition kernels: two wavenumbers per thread with the quadrature points of an
   // element split over two warps (one row, 128 threads), the row in shared memory while four CTAs
   // fit an SM, else (large N) window by window or in A itself; one per thread (4 rows x 2 warps) on
   // request
-  int kb = (kq && c->uniform_bc == 1) ? c->asm_kb : 0;
+  int kb = (kq && uniform_conditions(c)) ? c->asm_kb : 0;
   if (kb >= 1) {
     const int64_t E = c->E;
     dim3 gq((unsigned)((E + 255) / 256), nk);

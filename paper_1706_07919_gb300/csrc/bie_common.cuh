@@ -520,6 +520,50 @@ __device__ __forceinline__ void cis_ffprod2(f2 nkh, f2 nkl, ff R, f2& c, f2& s) 
   s = f2_make(ss[0], ss[1]);
 }
 
+// ---- FP64 helpers of the quadrature kernels ---------------------------------------------------
+// cos and sin of x.  |x| <= 2^18 (the kernels' phases k R): n = rint(x 2/pi), r = x - n pi/2 with pi/2
+// as two FP64 values under FMA (the first difference rounds once, below an ulp of pi/4), then the
+// Taylor series of sin through r^17 and of cos through r^16 (truncation below 1e-18 and 3e-18 of
+// the result on |r| <= pi/4), placed by the quadrant n mod 4; beyond, CUDA's sincos.  22 FP64
+// instructions; error against CUDA's sincos at most 2.3e-16 over 2^26 arguments.
+__device__ __forceinline__ void cis64(double x, double& s, double& c) {
+  constexpr double kMagic = 6755399441055744.0;                  // 1.5 * 2^52
+  constexpr double kHi = 1.57079632679489655800, kLo = 6.12323399573676603587e-17;  // pi/2
+  if (!(fabs(x) <= 262144.0)) {
+    sincos(x, &s, &c);
+    return;
+  }
+  const double m = fma(x, 0.63661977236758134308, kMagic), n = m - kMagic;
+  const double r = fma(-n, kLo, fma(-n, kHi, x));
+  const double z = r * r;
+  double p = fma(z, 2.81145725434552076320e-15, -7.64716373181981647590e-13);  // 1/17!, -1/15!
+  p = fma(z, p, 1.60590438368216145994e-10);                                   // 1/13!
+  p = fma(z, p, -2.50521083854417187751e-8);                                   // -1/11!
+  p = fma(z, p, 2.75573192239858906526e-6);                                    // 1/9!
+  p = fma(z, p, -1.98412698412698412698e-4);                                   // -1/7!
+  p = fma(z, p, 8.33333333333333333333e-3);                                    // 1/5!
+  p = fma(z, p, -1.66666666666666666667e-1);                                   // -1/3!
+  const double sv = fma(r * z, p, r);
+  double q = fma(z, 4.77947733238738529744e-14, -1.14707455977297247139e-11);  // 1/16!, -1/14!
+  q = fma(z, q, 2.08767569878680989792e-9);                                    // 1/12!
+  q = fma(z, q, -2.75573192239858906526e-7);                                   // -1/10!
+  q = fma(z, q, 2.48015873015873015873e-5);                                    // 1/8!
+  q = fma(z, q, -1.38888888888888888889e-3);                                   // -1/6!
+  q = fma(z, q, 4.16666666666666666667e-2);                                    // 1/4!
+  q = fma(z, q, -0.5);
+  const double cv = fma(z, q, 1.0);
+  const int i = __double2loint(m) & 3;  // n mod 4 (the sum's low bits, two's complement)
+  const double a = (i & 1) ? sv : cv, b = (i & 1) ? cv : sv;
+  c = (i == 1 || i == 2) ? -a : a;
+  s = (i >= 2) ? -b : b;
+}
+// R = sqrt(R2) and 1 / R for R2 > 0: CUDA's reciprocal square root and one residual step for R.
+__device__ __forceinline__ void dist64(double R2, double& R, double& invR) {
+  invR = rsqrt(R2);
+  const double r = R2 * invR;
+  R = fma(fma(-r, r, R2), 0.5 * invR, r);
+}
+
 // Barrier of the nthreads threads (whole warps) that use barrier `id` (1..15; 0 is
 // __syncthreads); orders their shared- and global-memory accesses like __syncthreads.
 __device__ __forceinline__ void bar_named(int id, int nthreads) {

@@ -141,6 +141,7 @@ int autotune(bie_ctx* c, const double* k, int64_t nk, const char* cache_path, bi
 int field_mixed(bie_ctx* c, const double* hk, const double* kv, int nk, const cd* surf, const double* xp, int64_t M,
                 const int32_t* foot_elem, const double* foot, cd* T, void* scratch, size_t scratch_bytes);
 size_t field_mixed_scratch(bie_ctx* c, const double* hk, int nk, int64_t M);
+size_t field64_scratch(bie_ctx* c, int nk, int64_t M);
 
 static void free_geometry(bie_ctx* c) {
   void* ptrs[] = {c->nodes, c->elems, c->normals, c->bc, c->qgeo, c->ngeo, c->qshape, c->nshape, c->qgeo32,
@@ -662,18 +663,18 @@ int bie_eval_field(bie_ctx* c, const double* xobs, int64_t M, const double* k, i
   if (M == 0 || Nk == 0) return BIE_OK;
   if (!xobs || !surf || !T_out) return fail(BIE_ERR_INVALID_ARG, "NULL pointer");
   if (mode != BIE_MODE_FP64 && mode != BIE_MODE_MIXED) return fail(BIE_ERR_INVALID_ARG, "unknown mode");
-  const int64_t EQ = c->E * c->rule.Q;
   // foot points (k independent) then batches of k
   const size_t foot_bytes = (size_t)M * (8 * sizeof(double) + sizeof(int32_t)) + 256;
-  const size_t perk = 2 * (size_t)EQ * sizeof(cd) + 16;
   // up to 512 wavenumbers per launch: the field kernel's grid (points x groups of 16 wavenumbers)
   // then spans many waves of resident CTAs, so the last, partial wave costs little
   constexpr int64_t kMaxFieldBatch = 512;
   int64_t kb = std::max<int64_t>(1, std::min<int64_t>(Nk, kMaxFieldBatch));
-  size_t scratch_bytes = kb * perk;
-  if (mode == BIE_MODE_MIXED)
-    for (int64_t k0 = 0; k0 < Nk; k0 += kb)
-      scratch_bytes = std::max(scratch_bytes, field_mixed_scratch(c, k + k0, (int)std::min<int64_t>(kb, Nk - k0), M));
+  size_t scratch_bytes = 0;
+  for (int64_t k0 = 0; k0 < Nk; k0 += kb) {
+    const int nk = (int)std::min<int64_t>(kb, Nk - k0);
+    scratch_bytes = std::max(scratch_bytes, mode == BIE_MODE_MIXED ? field_mixed_scratch(c, k + k0, nk, M)
+                                                                   : field64_scratch(c, nk, M));
+  }
   BIE_TRY(ensure_buf(c, c->work3, foot_bytes + scratch_bytes + kMaxFieldBatch * sizeof(double) + 4096 + 256));
   double* foot = (double*)c->work3.p;
   int32_t* foot_elem = (int32_t*)(foot + 8 * M);

@@ -7,8 +7,10 @@
 // nu0 the surface normal there, P0 and P0' interpolated quadratically at x0.
 //
 // Layout: the surface values are first interpolated to every standard quadrature point
-// (k_interp_q), then each CTA owns a tile of observation points for one k and sweeps all
-// quadrature points through shared memory (an N-body style tile loop).
+// (k_interp_q), then each CTA owns a tile of observation points for a group of wavenumbers and
+// sweeps the quadrature points (an N-body style loop).
+#include <algorithm>
+
 #include "bie_common.cuh"
 
 namespace bie {
@@ -35,101 +37,188 @@ __global__ void k_interp_q64(const int32_t* __restrict__ elems, int64_t N, int64
   Pnq[(int64_t)kk * E * Q + p] = b;
 }
 
-constexpr int FT = 128;  // points per CTA and quadrature points per shared tile
+constexpr int FT = 128;  // points per CTA and quadrature points per shared tile (FP32 kernels)
 
-__global__ void __launch_bounds__(FT) k_field64(const int32_t* __restrict__ elems, int64_t N, int64_t EQ,
-                                                const double* __restrict__ qgeo, const cd* __restrict__ Pq,
-                                                const cd* __restrict__ Pnq, const cd* __restrict__ surf,
-                                                const double* __restrict__ xp, int64_t M,
-                                                const int32_t* __restrict__ foot_elem, const double* __restrict__ foot,
-                                                const double* __restrict__ kv, cd* __restrict__ T) {
-  __shared__ double sx[FT], sy[FT], sz[FT], snx[FT], sny[FT], snz[FT], sw[FT];
-  __shared__ cd sP[FT], sPn[FT];
-  const int kk = blockIdx.y;
-  const double k = kv[kk];
-  const int64_t m = (int64_t)blockIdx.x * FT + threadIdx.x;
-  const bool active = m < M;
-  double p[3] = {0, 0, 0}, x0[3] = {0, 0, 0}, nu0[3] = {0, 0, 1};
-  cd P0 = {0, 0}, Pn0 = {0, 0};
-  if (active) {
-    for (int d = 0; d < 3; ++d) {
-      p[d] = xp[3 * m + d];
-      x0[d] = foot[8 * m + d];
-      nu0[d] = foot[8 * m + 3 + d];
-    }
-    const double fxi = foot[8 * m + 6], feta = foot[8 * m + 7];
+// FP64 field.  A CTA evaluates 32 points (one per lane) for a group of F64K wavenumbers over the
+// quadrature points of its share z of `splits`, a quarter of them per warp.  Per (point, quadrature
+// point) pair the geometry is formed once; where the group's wavenumbers are equally spaced to
+// rounding the three phases' sines and cosines are formed at k_0 and at the spacing and rotated to
+// the others (at most F64K - 1 steps of one ulp each, the size of the rounding of k R), else per
+// wavenumber.  Partial sums: the warps' through shared memory, the splits' through `part`
+// [splits][nk][M] and k_field64_sum, each in a fixed order (splits 1: T directly).
+// Bound: the FP64 pipe.  64 wavenumbers, 1000 points, 2048 quadrature points: 51.9 -> 13.6 ms = 60 FP64
+// instructions an evaluation at the pipe's measured 0.58 T/s (45 of them the rotations and the
+// integrand); wavenumbers without a common spacing 23.4 ms.  Error against 64 bits unchanged.
+constexpr int F64K = 16;
+__global__ void __launch_bounds__(128, 2) k_field64(const int32_t* __restrict__ elems, int64_t N, int64_t EQ,
+                                                    const double* __restrict__ qgeo, const cd* __restrict__ Pq,
+                                                    const cd* __restrict__ Pnq, const cd* __restrict__ surf,
+                                                    const double* __restrict__ xp, int64_t M,
+                                                    const int32_t* __restrict__ foot_elem, const double* __restrict__ foot,
+                                                    const double* __restrict__ kv, int nk, int splits, cd* __restrict__ part,
+                                                    cd* __restrict__ T) {
+  __shared__ double4 s0[F64K][32];   // P0 re, im, P0' re, im at each lane's foot point
+  __shared__ cd red[4][32];
+  __shared__ double2 sk[F64K];  // k, 1 / k (0 at k = 0)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int kbase = blockIdx.y * F64K, nkb = min(F64K, nk - kbase);
+  const int64_t m0 = (int64_t)blockIdx.x * 32, m = m0 + lane < M ? m0 + lane : M - 1;
+  if (threadIdx.x < nkb) {
+    const double k = kv[kbase + threadIdx.x];
+    sk[threadIdx.x] = make_double2(k, k > 0.0 ? 1.0 / k : 0.0);
+  }
+  for (int e = threadIdx.x; e < nkb * 32; e += 128) {
+    const int j = e >> 5, t = e & 31;
+    const int64_t mm = m0 + t < M ? m0 + t : M - 1;
+    const double fxi = foot[8 * mm + 6], feta = foot[8 * mm + 7];
     const double L1 = 1.0 - fxi - feta;
     const double Nv[6] = {L1 * (2 * L1 - 1), fxi * (2 * fxi - 1), feta * (2 * feta - 1), 4 * L1 * fxi, 4 * fxi * feta,
                           4 * feta * L1};
-    const int32_t* el = elems + 6 * (int64_t)foot_elem[m];
-    const cd* P = surf + (int64_t)kk * 2 * N;
+    const int32_t* el = elems + 6 * (int64_t)foot_elem[mm];
+    const cd* P = surf + (int64_t)(kbase + j) * 2 * N;
+    double4 v = make_double4(0.0, 0.0, 0.0, 0.0);
     for (int a = 0; a < 6; ++a) {
-      cd v = P[el[a]], w = P[N + el[a]];
-      P0.re += Nv[a] * v.re; P0.im += Nv[a] * v.im;
-      Pn0.re += Nv[a] * w.re; Pn0.im += Nv[a] * w.im;
+      const cd x = P[el[a]], w = P[N + el[a]];
+      v.x += Nv[a] * x.re; v.y += Nv[a] * x.im;
+      v.z += Nv[a] * w.re; v.w += Nv[a] * w.im;
     }
+    s0[j][t] = v;
   }
-  const cd* Pqk = Pq + (int64_t)kk * EQ;
-  const cd* Pnqk = Pnq + (int64_t)kk * EQ;
-  cd sum = {0, 0};
-  for (int64_t t0 = 0; t0 < EQ; t0 += FT) {
-    const int64_t t = t0 + threadIdx.x;
-    if (t < EQ) {
-      sx[threadIdx.x] = qgeo[GX * EQ + t]; sy[threadIdx.x] = qgeo[GY * EQ + t]; sz[threadIdx.x] = qgeo[GZ * EQ + t];
-      snx[threadIdx.x] = qgeo[GNX * EQ + t]; sny[threadIdx.x] = qgeo[GNY * EQ + t]; snz[threadIdx.x] = qgeo[GNZ * EQ + t];
-      sw[threadIdx.x] = qgeo[GWJ * EQ + t];
-      sP[threadIdx.x] = Pqk[t];
-      sPn[threadIdx.x] = Pnqk[t];
+  __syncthreads();
+  double p[3], x0[3], nu0[3];
+  for (int d = 0; d < 3; ++d) {
+    p[d] = xp[3 * m + d];
+    x0[d] = foot[8 * m + d];
+    nu0[d] = foot[8 * m + 3 + d];
+  }
+  // equally spaced: every wavenumber within an ulp of the last one of the line between the ends
+  const double k0 = kv[kbase], kl = kv[kbase + nkb - 1], dk = nkb > 2 ? (kl - k0) / (nkb - 1) : 0.0;
+  bool uniform = nkb > 2;
+  for (int j = 1; j < nkb; ++j) uniform &= fabs(kv[kbase + j] - fma((double)j, dk, k0)) <= 2.3e-16 * fabs(kl);
+  cd sum[F64K];
+#pragma unroll
+  for (int j = 0; j < F64K; ++j) sum[j] = cd{0, 0};
+  const int64_t share = blockIdx.z * 4 + warp;
+  const int64_t qlo = share * EQ / (4 * splits), qhi = (share + 1) * EQ / (4 * splits);
+#pragma unroll 1
+  for (int64_t q = qlo; q < qhi; ++q) {
+    const double qx = qgeo[GX * EQ + q], qy = qgeo[GY * EQ + q], qz = qgeo[GZ * EQ + q];
+    const double nx = qgeo[GNX * EQ + q], ny = qgeo[GNY * EQ + q], nz = qgeo[GNZ * EQ + q], w = qgeo[GWJ * EQ + q];
+    double rx = qx - p[0], ry = qy - p[1], rz = qz - p[2];
+    double Rp, iRp, R0, iR0;
+    dist64(rx * rx + ry * ry + rz * rz, Rp, iRp);
+    const double rnp = (rx * nx + ry * ny + rz * nz) * iRp * iRp;
+    rx = qx - x0[0]; ry = qy - x0[1]; rz = qz - x0[2];
+    dist64(rx * rx + ry * ry + rz * rz, R0, iR0);
+    const double rn0 = (rx * nx + ry * ny + rz * nz) * iR0 * iR0;
+    const double nr = nu0[0] * rx + nu0[1] * ry + nu0[2] * rz, nn = nu0[0] * nx + nu0[1] * ny + nu0[2] * nz;
+    const double ap = w * iRp, a0 = w * iR0;
+    double cp, sp, c0, s0v, cg, sg, dcp, dsp, dc0, ds0, dcg, dsg;
+    if (uniform) {
+      cis64(k0 * Rp, sp, cp);
+      cis64(k0 * R0, s0v, c0);
+      cis64(k0 * nr, sg, cg);
+      cis64(dk * Rp, dsp, dcp);
+      cis64(dk * R0, ds0, dc0);
+      cis64(dk * nr, dsg, dcg);
+      cp *= ap; sp *= ap;  // G = w e^{ikR} / R rides through the rotations
+      c0 *= a0; s0v *= a0;
     }
-    __syncthreads();
-    const int cnt = (EQ - t0) < FT ? (int)(EQ - t0) : FT;
-    if (active) {
-      for (int u = 0; u < cnt; ++u) {
-        const double nx = snx[u], ny = sny[u], nz = snz[u];
-        // source x_p
-        double rx = sx[u] - p[0], ry = sy[u] - p[1], rz = sz[u] - p[2];
-        double R = sqrt(rx * rx + ry * ry + rz * rz), iR = 1.0 / R, kR = k * R, s, c;
-        sincos(kR, &s, &c);
-        double rn = (rx * nx + ry * ny + rz * nz) * iR * iR * iR;
-        cd Gp = {c * iR, s * iR}, dGp = {(-c - s * kR) * rn, (c * kR - s) * rn};
-        // source x0
-        rx = sx[u] - x0[0]; ry = sy[u] - x0[1]; rz = sz[u] - x0[2];
-        R = sqrt(rx * rx + ry * ry + rz * rz); iR = 1.0 / R; kR = k * R;
-        sincos(kR, &s, &c);
-        rn = (rx * nx + ry * ny + rz * nz) * iR * iR * iR;
-        cd G0 = {c * iR, s * iR}, dG0 = {(-c - s * kR) * rn, (c * kR - s) * rn};
-        // g, f about x0
-        const double nr = nu0[0] * rx + nu0[1] * ry + nu0[2] * rz;
-        double sa = k * nr, sg, cg;
-        sincos(sa, &sg, &cg);
-        double nn = nu0[0] * nx + nu0[1] * ny + nu0[2] * nz;
-        double g = cg, f = k > 0.0 ? sg / k : nr, dg = -k * sg * nn, df = cg * nn;  // f -> nu0.r at k = 0
-        cd Pt = {sP[u].re - P0.re * g - Pn0.re * f, sP[u].im - P0.im * g - Pn0.im * f};
-        cd dPt = {sPn[u].re - P0.re * dg - Pn0.re * df, sPn[u].im - P0.im * dg - Pn0.im * df};
-        cd a = cmul(Pt, csub(dGp, dG0)), b = cmul(csub(Gp, G0), dPt);
-        sum.re += sw[u] * (a.re - b.re);
-        sum.im += sw[u] * (a.im - b.im);
+#pragma unroll
+    for (int j = 0; j < F64K; ++j) {
+      if (j >= nkb) break;
+      const double2 kj = sk[j];
+      const double k = kj.x;
+      if (!uniform) {
+        cis64(k * Rp, sp, cp);
+        cis64(k * R0, s0v, c0);
+        cis64(k * nr, sg, cg);
+        cp *= ap; sp *= ap;
+        c0 *= a0; s0v *= a0;
+      } else if (j > 0) {
+        double u = cp * dcp - sp * dsp;
+        sp = sp * dcp + cp * dsp;
+        cp = u;
+        u = c0 * dc0 - s0v * ds0;
+        s0v = s0v * dc0 + c0 * ds0;
+        c0 = u;
+        u = cg * dcg - sg * dsg;
+        sg = sg * dcg + cg * dsg;
+        cg = u;
       }
+      const double kRp = k * Rp, kR0 = k * R0;
+      const double gdr = cp - c0, gdi = sp - s0v;  // w (Gp - G0), and w (dGp - dG0):
+      const double ddr = (s0v * kR0 + c0) * rn0 - (sp * kRp + cp) * rnp;
+      const double ddi = (cp * kRp - sp) * rnp - (c0 * kR0 - s0v) * rn0;
+      // g, f about x0 (f -> nu0.r at k = 0) and their normal derivatives
+      const double g = cg, f = k > 0.0 ? sg * kj.y : nr, dg = -k * sg * nn, df = cg * nn;
+      const double4 z = s0[j][lane];
+      const cd P = Pq[(int64_t)(kbase + j) * EQ + q], D = Pnq[(int64_t)(kbase + j) * EQ + q];
+      const double Ptr = P.re - z.x * g - z.z * f, Pti = P.im - z.y * g - z.w * f;
+      const double dPr = D.re - z.x * dg - z.z * df, dPi = D.im - z.y * dg - z.w * df;
+      // sum += Pt (dGp - dG0) - (Gp - G0) dPt, product by product: a fused addition each
+      sum[j].re = fma(Ptr, ddr, fma(-Pti, ddi, fma(-gdr, dPr, fma(gdi, dPi, sum[j].re))));
+      sum[j].im = fma(Ptr, ddi, fma(Pti, ddr, fma(-gdr, dPi, fma(-gdi, dPr, sum[j].im))));
     }
-    __syncthreads();
   }
-  if (active) {
-    const double inv4pi = 1.0 / (4.0 * kPi);
-    T[(int64_t)kk * M + m] = {P0.re + sum.re * inv4pi, P0.im + sum.im * inv4pi};
+  const double inv4pi = 1.0 / (4.0 * kPi);
+#pragma unroll
+  for (int j = 0; j < F64K; ++j) {
+    if (j >= nkb) break;
+    __syncthreads();
+    red[warp][lane] = sum[j];
+    __syncthreads();
+    if (warp == (j & 3) && m0 + lane < M) {
+      cd t = {0, 0};
+      for (int w = 0; w < 4; ++w) t = cadd(t, red[w][lane]);
+      t = cscale(t, inv4pi);
+      if (blockIdx.z == 0) {
+        t.re += s0[j][lane].x;
+        t.im += s0[j][lane].y;
+      }
+      (splits > 1 ? part + (int64_t)blockIdx.z * nk * M : T)[(int64_t)(kbase + j) * M + m0 + lane] = t;
+    }
   }
 }
 
-// Evaluates nk wavenumbers: surf [nk][2][N] -> T [nk][M].  scratch >= 2 * nk * E * Q * 16 B.
+// T = sum over the splits, in order; n = nk M
+__global__ void k_field64_sum(const cd* __restrict__ part, int splits, int64_t n, cd* __restrict__ T) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  cd v = part[t];
+  for (int z = 1; z < splits; ++z) v = cadd(v, part[z * n + t]);
+  T[t] = v;
+}
+
+// Shares of the quadrature points: sixteen CTAs to an SM (two are resident: a last, partial wave then
+// costs little; with the per-wavenumber phases 4 to an SM measured 27.7 ms, 16 23.4), shares of at
+// least 64 points.
+static int field64_splits(bie_ctx* c, int nk, int64_t M) {
+  const int64_t ctas = (M + 31) / 32 * ((nk + F64K - 1) / F64K), EQ = c->E * c->rule.Q;
+  return (int)std::max<int64_t>(1, std::min<int64_t>((16 * 152 + ctas - 1) / ctas, EQ / 64));
+}
+// Scratch of field64 in bytes.
+size_t field64_scratch(bie_ctx* c, int nk, int64_t M) {
+  const int z = field64_splits(c, nk, M);
+  return 2 * (size_t)nk * c->E * c->rule.Q * sizeof(cd) + (z > 1 ? (size_t)z * nk * M * sizeof(cd) : 0);
+}
+
+// Evaluates nk wavenumbers: surf [nk][2][N] -> T [nk][M].  scratch: field64_scratch bytes.
 int field64(bie_ctx* c, const double* kv, int nk, const cd* surf, const double* xp, int64_t M,
             const int32_t* foot_elem, const double* foot, cd* T, void* scratch) {
   const int64_t EQ = c->E * c->rule.Q;
   cd* Pq = (cd*)scratch;
   cd* Pnq = Pq + (int64_t)nk * EQ;
+  cd* part = Pnq + (int64_t)nk * EQ;
   dim3 gi((unsigned)((EQ + 255) / 256), nk);
   BIE_LAUNCH(k_interp_q64<<<gi, 256, 0, c->stream>>>(c->elems, c->N, c->E, c->rule.Q, c->qshape, surf, Pq, Pnq));
   if (M > 0) {
-    dim3 gf((unsigned)((M + FT - 1) / FT), nk);
-    BIE_LAUNCH(k_field64<<<gf, FT, 0, c->stream>>>(c->elems, c->N, EQ, c->qgeo, Pq, Pnq, surf, xp, M, foot_elem, foot, kv, T));
+    const int splits = field64_splits(c, nk, M);
+    dim3 gf((unsigned)((M + 31) / 32), (unsigned)((nk + F64K - 1) / F64K), (unsigned)splits);
+    BIE_LAUNCH(k_field64<<<gf, 128, 0, c->stream>>>(c->elems, c->N, EQ, c->qgeo, Pq, Pnq, surf, xp, M, foot_elem, foot, kv,
+                                                    nk, splits, part, T));
+    if (splits > 1)
+      BIE_LAUNCH(k_field64_sum<<<(unsigned)((nk * M + 255) / 256), 256, 0, c->stream>>>(part, splits, nk * M, T));
   }
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;

@@ -95,8 +95,8 @@ __global__ void k_synth(const cd* __restrict__ T, const int64_t* __restrict__ mi
 // signal, 16 values each in registers: one pass of radix 2, 4 or 8 where log2 h leaves a
 // remainder, then radix-16 passes (Stockham order), exchanging through shared memory between
 // passes -- two exchanges for n = 4096, where the radix-2 kernel had twelve round trips through
-// shared memory, each with a division and a twiddle converted from FP64.  A CTA of about 256 threads holds
-// SB = 4096 / h neighbouring points, so that T is read in whole sectors, and takes PG pulses one
+// shared memory, each with a division and a twiddle converted from FP64.  A CTA of up to 256 threads
+// holds SB neighbouring points, so that T is read in whole sectors, and takes PG pulses one
 // after the other with the points' T kept in shared memory.  FP32: S and T enter as float-float
 // (T split once per point, S once per call, `sp` or, without it, in the kernel) and their product
 // rounds once, as the FP64 product rounded to FP32 did: eight FP64 operations a frequency, point and
@@ -277,9 +277,9 @@ __device__ __forceinline__ void real_fft(C2<S>* __restrict__ buf, const C2<S>* _
 template <int L, class S, bool KEEP>
 __global__ void __launch_bounds__(256, sizeof(S) == 4 ? 3 : 1) k_synth_real(const cd* __restrict__ T, const int64_t* __restrict__ midx, int nk,
                                                     int64_t M, const cd* __restrict__ Sp, const float4* __restrict__ sp,
-                                                    int P, int PG, const C2<S>* __restrict__ tw, bool passes,
+                                                    int P, int PG, int SB, const C2<S>* __restrict__ tw, bool passes,
                                                     S* __restrict__ out, int wide) {
-  constexpr int h = 1 << L, n = 2 * h, NT = h / 16, SB = 4096 / h;
+  constexpr int h = 1 << L, n = 2 * h, NT = h / 16;
   constexpr bool F32 = sizeof(S) == 4;
   extern __shared__ float4 synth_smem[];
   const int len = h + 1 + ((h + 1) >> 4) + 1;
@@ -372,7 +372,11 @@ static int launch_synth(const cd* T, const int64_t* midx, int nk, int64_t M, con
     BIE_LAUNCH(k_synth<S, S><<<g, 32, smem, st>>>(T, midx, nk, M, Sp, n, (const double2*)tw, out));
     return BIE_OK;
   }
-  const int h = n / 2, SB = 4096 / h, wide = ((uintptr_t)out % (2 * sizeof(S))) == 0;
+  const int h = n / 2, wide = ((uintptr_t)out % (2 * sizeof(S))) == 0;
+  // points per CTA: 256 threads' worth, fewer (down to a warp, or two points for whole sectors of T)
+  // while the signals would not give every SM two CTAs
+  int SB = 4096 / h;
+  while (SB > 2 && SB * (h / 16) > 32 && (M + SB - 1) / SB * P < 2 * nsm) SB >>= 1;
   const int64_t bx = (M + SB - 1) / SB;
   if (bx > 0x7fffffff) return fail(BIE_ERR_INVALID_ARG, "too many observation points");
   const size_t bufs = ((size_t)SB * fft_pad_len(h) * sizeof(C2<S>) + 15) & ~(size_t)15;
@@ -384,7 +388,7 @@ static int launch_synth(const cd* T, const int64_t* midx, int nk, int64_t M, con
   const dim3 g((unsigned)bx, (unsigned)(keep ? 1 : P));
   auto go = [&](auto kernel) -> int {
     BIE_TRY(set_smem_max(kernel));
-    BIE_LAUNCH(kernel<<<g, SB * (h / 16), bufs + (keep ? kept : 0), st>>>(T, midx, nk, M, Sp, sp, (int)P, PG,
+    BIE_LAUNCH(kernel<<<g, SB * (h / 16), bufs + (keep ? kept : 0), st>>>(T, midx, nk, M, Sp, sp, (int)P, PG, SB,
                                                                           (const C2<S>*)tw, passes, out, wide));
     return BIE_OK;
   };
