@@ -224,9 +224,9 @@ int bie_set_incident_plane_wave(bie_ctx* ctx, const double* dir);
  *                          register-staged tcgen05 kernel, 0 FP32 on the CUDA cores.
  *   "mixed.lu_block"       columns of the deferred update of version 3: 128, 256, 512, or 0
  *                          (default): 512 from N = 8192 on, else 256
- *   "mixed.lu_coop"        1 (default): the panels of few tall matrices (at most half as many
- *                          matrices as SMs, more than 1536 rows) are factored by several CTAs per
- *                          matrix in one cooperative launch; 0: one CTA per matrix always
+ *   "mixed.lu_coop"        1 (default): panels are factored by a thread-block cluster per matrix (up
+ *                          to 16 CTAs) while as many clusters as matrices are resident at once;
+ *                          0: one CTA per matrix always
  *   "mixed.lu_panel"       panel width of version 3: 64 (default) or 32 (more, narrower panels:
  *                          shorter pivot chains per leaf, narrower K = 32 updates inside a block)
  *   "mixed.lu_tile"        tile of the tensor-core update (versions 2, 3): 128 rows x 256 real
@@ -303,7 +303,7 @@ int bie_assemble(bie_ctx* ctx, double k, void* A_out, void* b_out);
  *   rep      host bie_report [Nk] or NULL
  * Synchronises the stream before returning (the reports are read back).  Errors: INVALID_ARG,
  * STATE, OOM (scratch larger than free device memory), CUDA, TIMEOUT (a bounded wait of the
- * tensor-core factorisation or of a cooperative panel gave up: that factor is void). */
+ * tensor-core factorisation gave up: that factor is void). */
 int bie_solve_frequencies(bie_ctx* ctx, const double* k, int64_t Nk, int mode, void* surf_out,
                           bie_report* rep);
 

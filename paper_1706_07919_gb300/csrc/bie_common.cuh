@@ -135,7 +135,7 @@ struct bie_ctx {
                                      // with the update deferred over 256-column blocks
   int lu_block = 0;                  // mixed.tcgen05 3: columns over which the trailing update is
                                      // deferred (128, 256 or 512; 0: 512 from N = 8192 on, else 256)
-  int lu_coop = 1;                   // several CTAs per matrix in the panels of few tall matrices
+  int lu_coop = 1;                   // panels by a cluster of CTAs per matrix where enough clusters fit
   int lu_panel = 64;                 // mixed.tcgen05 3: panel width (32 or 64)
   int lu_tile = 256;                 // mixed.tcgen05 2, 3: update tile width in real columns (256 or 128)
   int mixed_batch = 256;             // wavenumbers per batch (capped by free memory; the tuner's

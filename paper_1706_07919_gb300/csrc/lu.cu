@@ -315,250 +315,193 @@ __global__ void __launch_bounds__(256) k_leaf_update(Cx<S>* __restrict__ A, int6
   }
 }
 
-// ---- cooperative panel: several CTAs per matrix for a few tall matrices ----------------------
-// With few matrices in a batch (at most half as many as co-resident CTAs) and panels taller than
-// a 16-column leaf that fits one CTA's shared memory, one CTA per matrix leaves most SMs idle and
-// has to narrow its leaves to a column or two.  Here `cpm` CTAs share each matrix: CTA j of
-// matrix z holds rows [p0 + j ch, p0 + (j + 1) ch) of a leaf of up to 16 columns in shared memory
-// (column by column), and the CTAs of one matrix agree on every pivot through records in global
-// memory, one exchange per column:
-//   each CTA posts its best candidate row (largest modulus, lowest row on ties) with the
-//   candidate's leaf entries (CTA 0 adds row c's), the record's tag written last with release
-//   semantics; one warp of every CTA polls the matrix's tags (acquire) until all carry this
-//   column's, which makes the exchange its own barrier; every CTA picks the same winner p, the
-//   holders of rows c and p exchange them in shared memory, and every CTA scales column c of its
-//   rows and applies the rank-1 update to the rest of its leaf, finding its next candidate on the
-//   way.  The records of consecutive columns alternate between two buffers, which is safe because
-//   no CTA can post column c + 2 before every CTA has posted column c + 1, after reading column c.
-// After a leaf, CTA 0 (its chunk holds the panel's diagonal rows: ch is a multiple of 64) applies
-// the leaf's row interchanges, as one gather of the at most 2 lw rows they touch, to the panel's
-// other columns and solves the leaf's U block L11^{-1} A12 for the panel columns right of the
-// leaf; after a barrier (a counter in global memory) every CTA updates its rows of those
-// columns, A -= L U (K = lw).
-// Launched cooperatively, so that all CTAs are resident together.  Every wait is bounded: a CTA
-// whose wait gives up raises the error word (bit 8) and an abort flag on which every other wait
-// ends, and all CTAs leave.  Data written by other CTAs is read with L2-coherent loads.
-namespace coop {
-constexpr int NT = 512;
-constexpr int LWMAX = 16;
-constexpr int WMAX = 64;                 // panel width
-constexpr uint32_t SPIN = 1u << 21;      // polls of one wait (about a second) before giving up
-struct alignas(16) Cand {                // one CTA's pivot candidate for one column
-  // |a|^2 of the candidate (bits of the float, -1: no row) << 32 | its row << 8 | tag: the column's
-  // place in the panel + 1 (1 .. 64; 0: not written in this launch), stored last with release
-  // semantics, so that one acquire load gives the whole verdict
-  unsigned long long head;
-  int pad[2];
-  Cx<float> v[LWMAX];                    // the candidate's leaf entries
-  Cx<float> d[LWMAX];                    // CTA 0: row c's leaf entries
+// ---- cluster panel: one panel of each matrix by a thread-block cluster ------------------------
+// The CTAs of a cluster (1, 2, 4, 8 or 16) share a matrix: CTA j holds rows [p0 + j ch, p0 + (j + 1) ch)
+// of a leaf of up to 16 columns in shared memory, column by column.  Per column each CTA finds its best
+// candidate row (largest modulus, lowest row on ties) during the rank-1 update of the column before,
+// one warp stores the candidate and its leaf entries (the holder of row c also row c's) into every
+// CTA's shared memory, and one cluster barrier later every warp picks the same winner p from its own
+// copy; the holders of rows c and p exchange them, every CTA scales column c of its rows and applies
+// the rank-1 update.  The records of consecutive columns alternate between two buffers: a CTA stores
+// column c + 2's only after the barrier of column c + 1, at which every CTA has read column c's.
+// After a leaf, CTA 0 (its chunk holds the panel's diagonal rows: ch >= 64) applies the leaf's
+// interchanges, as one gather of the at most 32 rows they touch, to the panel's other columns and
+// solves the leaf's U block L11^{-1} A12 for the panel columns right of the leaf; one barrier later
+// every CTA updates its rows of those columns, A -= L U.  Global data written by another CTA of the
+// cluster is read with L2-coherent loads after a cluster barrier (release / acquire).
+// Bound: the latency of a column (a CTA barrier, the remote stores, a cluster barrier).
+// Every entry goes through the operations of the one-CTA leaf (k_leaf) in its order, so that the
+// pivots and, for panels of up to 1536 rows (leaf, where that kernel takes 16 columns), the factor are
+// the same bit for bit whatever the cluster; sum_first: A -= (sum of L U), as k_leaf_update forms it
+// for small batches, instead of product by product.  (Taller panels of small batches fix the other
+// order of the U block's fused products, leaf 0.)  The refinement's result moves by up to 1e-9 with
+// the factor's rounding: which of the forms a panel takes depends on the batch, the rows and the
+// number of SMs alone (panel_cluster), not on the cluster.
+// The key of a candidate is |a|^2's leading 32 bits (FP32: all of them), 0 for none.
+namespace pcl {
+constexpr int NT = 512, LW = 16, PW = 64, MAXC = 16;
+template <class S> struct alignas(16) Rec {
+  unsigned long long head;  // key << 32 | row
+  unsigned long long pad;
+  Cx<S> v[LW];              // the candidate's leaf entries
 };
-// scratch: [nmat] barrier counters, abort flag, [2][grid] candidate records (zeroed before each
-// launch with the counters)
-inline size_t scratch_bytes(int nmat, int grid) {
-  return 256 + (size_t)(nmat + 1) * 4 + 256 + 2 * (size_t)grid * sizeof(Cand) + 256;
+template <class S> __host__ __device__ constexpr size_t smem_bytes(int lw, int ch) {
+  // leaf, gathered rows of the other columns (32 x 64), U block (16 x 64)
+  return ((size_t)lw * ch + 2 * LW * PW + LW * PW) * sizeof(Cx<S>);
 }
-}  // namespace coop
-constexpr int kCoopMaxGrid = 4096;  // CTAs of one cooperative panel launch (at most)
-
-__device__ __forceinline__ unsigned long long ld_acquire_gpu64(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];\n" : "=l"(v) : "l"(p) : "memory");
-  return v;
+__device__ __forceinline__ unsigned key_of(float m) { return __float_as_uint(m) + 1u; }
+__device__ __forceinline__ unsigned key_of(double m) { return (unsigned)__double2hiint(m) + 1u; }
+__device__ __forceinline__ uint32_t mapa(uint32_t a, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
 }
-__device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
-  return v;
+__device__ __forceinline__ void st_remote(uint32_t a, unsigned long long v) {
+  asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
 }
-__device__ __forceinline__ Cx<float> ldcg_cx(const Cx<float>* p) {
+__device__ __forceinline__ void st_remote(uint32_t a, Cx<float> v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.re), "f"(v.im) : "memory");
+}
+__device__ __forceinline__ void st_remote(uint32_t a, Cx<double> v) {
+  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(v.re), "d"(v.im) : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ Cx<float> ldcg(const Cx<float>* p) {
   const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
   return {v.x, v.y};
 }
+__device__ __forceinline__ Cx<double> ldcg(const Cx<double>* p) {
+  return {__ldcg(&p->re), __ldcg(&p->im)};
+}
+}  // namespace pcl
 
-__global__ void __launch_bounds__(coop::NT, 1) k_panel_coop(
-    Cx<float>* __restrict__ A, int64_t bstride, int n, int ld, int p0, int w, int lw, int cpm, int ch,
-    int32_t* __restrict__ piv, int32_t* __restrict__ info, unsigned* __restrict__ bar, unsigned* abort_flag,
-    coop::Cand* __restrict__ cand, int32_t* __restrict__ err) {
-  using coop::LWMAX;
-  using coop::NT;
-  extern __shared__ float4 coop_smem[];
-  Cx<float>* S = reinterpret_cast<Cx<float>*>(coop_smem);  // [lw][ch]: leaf entry (r, t) at t * ch + r - r_lo
-  Cx<float>* Ub = S + (size_t)lw * ch;                     // [LWMAX][WMAX]: the leaf's U block
-  __shared__ Cx<float> s_u[LWMAX], s_d[LWMAX];             // pivot row, former row c (leaf entries)
-  __shared__ float red_v[NT / 32];
-  __shared__ int red_i[NT / 32];
-  __shared__ int s_p, s_abort, s_m;
-  __shared__ int s_piv[LWMAX], s_rows[2 * LWMAX], s_src[2 * LWMAX];
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+// a -= l u, rounded as in the one-CTA leaf
+template <class S> __device__ __forceinline__ void cx_msub(Cx<S>& a, Cx<S> l, Cx<S> u) {
+  a.re -= l.re * u.re - l.im * u.im;
+  a.im -= l.re * u.im + l.im * u.re;
+}
+
+template <class S>
+__global__ void __launch_bounds__(pcl::NT, 1) k_panel_cluster(Cx<S>* __restrict__ A, int64_t bstride, int n, int ld,
+                                                              int p0, int w, int lw, int ch, int sum_first, int leaf,
+                                                              int32_t* __restrict__ piv, int32_t* __restrict__ info) {
+  using namespace pcl;
+  extern __shared__ float4 pcl_smem[];
+  Cx<S>* L = reinterpret_cast<Cx<S>*>(pcl_smem);  // [lw][ch]: leaf entry (r, t) at t * ch + r - r_lo
+  Cx<S>* X = L + (size_t)lw * ch;                 // [2 LW][PW]: gathered rows (CTA 0)
+  Cx<S>* Ub = X + 2 * LW * PW;                    // [LW][PW]: the leaf's U block
+  __shared__ Rec<S> rec[2][MAXC];
+  __shared__ Cx<S> drow[2][LW];                   // row c's leaf entries
+  __shared__ unsigned red_k[NT / 32], red_r[NT / 32];
+  __shared__ int s_piv[LW], s_rows[2 * LW], s_src[2 * LW], s_m;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int z = blockIdx.x / cpm, j = blockIdx.x - z * cpm;
-  Cx<float>* M = A + (int64_t)z * bstride;
-  const int r_lo = p0 + j * ch, r_hi = min(n, r_lo + ch);  // empty when r_lo >= n
+  uint32_t cl, rank;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(cl));
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  const int z = blockIdx.x / cl;
+  Cx<S>* M = A + (int64_t)z * bstride;
+  const int r_lo = p0 + (int)rank * ch, r_hi = min(n, r_lo + ch);  // empty when r_lo >= n
   const int pend = min(p0 + w, n);
-  unsigned gen = 0;
-  if (tid == 0) s_abort = 0;
-  __syncthreads();
-  // barrier of the cpm CTAs of matrix z; false when a wait gave up here or elsewhere.  The
-  // arrival is a release (it orders the CTA's writes, gathered by bar.sync, before it), the
-  // poll an acquire.
-  auto barrier = [&]() -> bool {
-    __syncthreads();
-    if (tid == 0) {
-      asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(bar + z) : "memory");
-      const unsigned target = (gen + 1) * (unsigned)cpm;
-      bool ok = false;
-      for (uint32_t it = 0; it < coop::SPIN; ++it) {
-        if (ld_acquire_gpu(bar + z) >= target) { ok = true; break; }
-        if (ld_acquire_gpu(abort_flag)) break;
-        if (it > 16) __nanosleep(32);
-      }
-      if (!ok) {
-        atomicOr(err, 8);
-        atomicExch(abort_flag, 1u);
-        s_abort = 1;
-      }
-      asm volatile("fence.acq_rel.gpu;\n" ::: "memory");
-    }
-    ++gen;
-    __syncthreads();
-    return s_abort == 0;
-  };
+  const uint32_t rec_a = (uint32_t)__cvta_generic_to_shared(&rec[0][0]);
+  const uint32_t drow_a = (uint32_t)__cvta_generic_to_shared(&drow[0][0]);
+  cluster_sync();  // every CTA of the cluster runs before the first remote store
   for (int c0 = p0; c0 < pend; c0 += lw) {
     const int l = min(lw, pend - c0);
-    const int a = max(r_lo, c0);       // first leaf row held here
+    const int a = max(r_lo, c0);  // first leaf row held here
     const int nr = max(0, r_hi - a);
+#pragma unroll 4
     for (int e = tid; e < nr * l; e += NT) {
       const int rr = e / l, t = e - rr * l;
-      S[t * ch + a - r_lo + rr] = ldcg_cx(M + (int64_t)(a + rr) * ld + c0 + t);
+      L[t * ch + a - r_lo + rr] = ldcg(M + (int64_t)(a + rr) * ld + c0 + t);
     }
     __syncthreads();
-    // this thread's candidate for the leaf's first column (later columns: found during the
-    // rank-1 update of the column before)
-    float best = -1.f;
+    // this thread's candidate for the leaf's first column
+    S best = -1;
     int bi = n;
     for (int r = a + tid; r < r_hi; r += NT) {
-      const Cx<float> v = S[r - r_lo];
-      const float m = v.re * v.re + v.im * v.im;
+      const Cx<S> v = L[r - r_lo];
+      const S m = v.re * v.re + v.im * v.im;
       if (m > best) { best = m; bi = r; }
     }
     for (int cc = 0; cc < l; ++cc) {
       const int c = c0 + cc, buf = c & 1;
-      const unsigned tag = (unsigned)(c - p0) + 1u;
-      for (int o = 16; o > 0; o >>= 1) {
-        const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+      {
+        const unsigned k = bi < n ? key_of(best) : 0u;
+        const unsigned K = __reduce_max_sync(0xffffffffu, k);
+        const unsigned R = __reduce_min_sync(0xffffffffu, k == K ? (unsigned)bi : 0xffffffffu);
+        if (lane == 0) { red_k[warp] = K; red_r[warp] = R; }
       }
-      if (lane == 0) { red_v[warp] = best; red_i[warp] = bi; }
       __syncthreads();
       if (warp == 0) {
-        best = lane < NT / 32 ? red_v[lane] : -1.f;
-        bi = lane < NT / 32 ? red_i[lane] : n;
-        for (int o = 16; o > 0; o >>= 1) {
-          const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-          const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-          if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-        }
-        coop::Cand* cd = cand + (int64_t)buf * gridDim.x + blockIdx.x;
-        if (lane == 0) {  // the whole record from one thread, its head last (release)
-          for (int t = 0; t < l; ++t) cd->v[t] = bi < r_hi ? S[t * ch + bi - r_lo] : Cx<float>{0.f, 0.f};
-          if (c >= r_lo && c < r_hi)
-            for (int t = 0; t < l; ++t) cd->d[t] = S[t * ch + c - r_lo];
-          const unsigned long long head = ((unsigned long long)__float_as_uint(best) << 32) |
-                                          ((unsigned long long)(unsigned)bi << 8) | tag;
-          asm volatile("st.release.gpu.global.u64 [%0], %1;\n" ::"l"(&cd->head), "l"(head) : "memory");
-        }
-        // wait for every record of this column (bounded; the abort flag, read every 32 polls,
-        // ends it too); the heads carry the candidates
-        const coop::Cand* cb = cand + (int64_t)buf * gridDim.x + (int64_t)z * cpm;
-        bool ok = false;
-        float b2 = -1.f;
-        int i2 = n, w2 = 0;
-        for (uint32_t it = 0; it < coop::SPIN; ++it) {
-          bool mine = true;
-          float bl = -1.f;
-          int il = n, wl = 0;
-          for (int q = lane; q < cpm; q += 32) {
-            const unsigned long long h = ld_acquire_gpu64(&cb[q].head);
-            if ((unsigned)(h & 0xffu) != tag) { mine = false; break; }
-            const float bq = __uint_as_float((unsigned)(h >> 32));
-            const int iq = (int)((h >> 8) & 0xffffffu);
-            if (bq > bl || (bq == bl && iq < il)) { bl = bq; il = iq; wl = q; }
-          }
-          if (__all_sync(0xffffffffu, mine)) {
-            ok = true;
-            b2 = bl;
-            i2 = il;
-            w2 = wl;
-            break;
-          }
-          if ((it & 31) == 31 && ld_acquire_gpu(abort_flag)) break;
-          if (it > 16) __nanosleep(32);
-        }
-        if (!ok) {
-          if (lane == 0) {
-            atomicOr(err, 8);
-            atomicExch(abort_flag, 1u);
-            s_abort = 1;
-          }
-        } else {
-          for (int o = 16; o > 0; o >>= 1) {
-            const float ob = __shfl_xor_sync(0xffffffffu, b2, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, i2, o);
-            const int ow = __shfl_xor_sync(0xffffffffu, w2, o);
-            if (ob > b2 || (ob == b2 && oi < i2)) { b2 = ob; i2 = oi; w2 = ow; }
-          }
-          if (i2 >= n) i2 = c;
-          if (lane == 0) {
-            s_p = i2;
-            s_piv[cc] = i2;
-            if (j == 0) {
-              piv[(int64_t)z * n + c] = i2;
-              if (!(b2 > 0) && info) atomicOr(info + z, 1);
-            }
-          }
-          if (lane < l) {
-            s_u[lane] = ldcg_cx(&cb[w2].v[lane]);
-            s_d[lane] = ldcg_cx(&cb[0].d[lane]);
-          }
+        const unsigned k = lane < NT / 32 ? red_k[lane] : 0u, r = lane < NT / 32 ? red_r[lane] : 0xffffffffu;
+        const unsigned K = __reduce_max_sync(0xffffffffu, k);
+        const unsigned R = __reduce_min_sync(0xffffffffu, k == K ? r : 0xffffffffu);
+        const int t = lane & 15;
+        const bool mine = c >= r_lo && c < r_hi;
+        const Cx<S> v = (K != 0u && t < l) ? L[t * ch + (int)R - r_lo] : Cx<S>{0, 0};
+        const Cx<S> d = (mine && t < l) ? L[t * ch + c - r_lo] : Cx<S>{0, 0};
+        const uint32_t ra = rec_a + (uint32_t)((buf * MAXC + (int)rank) * sizeof(Rec<S>));
+        for (uint32_t q = lane >> 4; q < cl; q += 2) {
+          const uint32_t rq = mapa(ra, q);
+          st_remote(rq + 16u + (uint32_t)(t * sizeof(Cx<S>)), v);
+          if (t == 0) st_remote(rq, ((unsigned long long)K << 32) | R);
+          if (mine) st_remote(mapa(drow_a, q) + (uint32_t)((buf * LW + t) * sizeof(Cx<S>)), d);
         }
       }
-      __syncthreads();
-      if (s_abort) return;
-      const int p = s_p;
-      // rows c and p exchange (row c takes the pivot row; the thread of row p, below, restores
-      // the former row c into it); rows below c are scaled and updated, and each thread keeps its
-      // best candidate for the next column
-      if (p != c && tid < l && c >= r_lo && c < r_hi) S[tid * ch + c - r_lo] = s_u[tid];
-      const Cx<float> d = s_u[cc];
-      const float dd = d.re * d.re + d.im * d.im;
-      const bool okd = dd > 0.f;
-      best = -1.f;
+      cluster_sync();
+      // the winner, from this CTA's copy of the records
+      const unsigned long long h = lane < (int)cl ? rec[buf][lane].head : 0ull;
+      const unsigned K = __reduce_max_sync(0xffffffffu, (unsigned)(h >> 32));
+      const unsigned R = __reduce_min_sync(0xffffffffu, (unsigned)(h >> 32) == K ? (unsigned)h : 0xffffffffu);
+      const unsigned who = __ballot_sync(0xffffffffu, (unsigned)(h >> 32) == K && (unsigned)h == R);
+      const bool found = K != 0u;
+      const int p = found ? (int)R : c;
+      const Cx<S>* u = found ? rec[buf][__ffs(who) - 1].v : drow[buf];  // the pivot row
+      const Cx<S> d = u[cc];
+      const S dd = d.re * d.re + d.im * d.im;
+      const bool okd = dd > 0;
+      if (tid == 0) {
+        s_piv[cc] = p;
+        if (rank == 0) {
+          piv[(int64_t)z * n + c] = p;
+          if (!okd && info) atomicOr(info + z, 1);
+        }
+      }
+      // row c takes the pivot row; the thread of row p, below, restores the former row c into it
+      if (p != c && tid < l && c >= r_lo && c < r_hi) L[tid * ch + c - r_lo] = u[tid];
+      best = -1;
       bi = n;
       for (int r = max(a, c + 1) + tid; r < r_hi; r += NT) {
+        Cx<S>* x = L + r - r_lo;
         if (r == p)
-          for (int t = 0; t < l; ++t) S[t * ch + r - r_lo] = s_d[t];
-        Cx<float> lv = S[cc * ch + r - r_lo];
+          for (int t = 0; t < l; ++t) x[t * ch] = drow[buf][t];
+        Cx<S> lv = x[cc * ch];
         if (okd) lv = cx_div(lv, d);
-        S[cc * ch + r - r_lo] = lv;
-        for (int t = cc + 1; t < l; ++t) {
-          const Cx<float> u = s_u[t];
-          Cx<float>& x = S[t * ch + r - r_lo];
-          x.re -= lv.re * u.re - lv.im * u.im;
-          x.im -= lv.re * u.im + lv.im * u.re;
-          if (t == cc + 1) {
-            const float m = x.re * x.re + x.im * x.im;
-            if (m > best) { best = m; bi = r; }
-          }
+        x[cc * ch] = lv;
+        if (cc + 1 < l) {
+          Cx<S> y = x[(cc + 1) * ch];
+          cx_msub(y, lv, u[cc + 1]);
+          x[(cc + 1) * ch] = y;
+          const S m = y.re * y.re + y.im * y.im;
+          if (m > best) { best = m; bi = r; }
+#pragma unroll 4
+          for (int t = cc + 2; t < l; ++t) cx_msub(x[t * ch], lv, u[t]);
         }
       }
-      // (the next column's first __syncthreads orders these updates before any read of them)
+      // (the next column's __syncthreads orders these updates before any other thread reads them)
     }
     __syncthreads();
+#pragma unroll 4
     for (int e = tid; e < nr * l; e += NT) {
       const int rr = e / l, t = e - rr * l;
-      M[(int64_t)(a + rr) * ld + c0 + t] = S[t * ch + a - r_lo + rr];
+      M[(int64_t)(a + rr) * ld + c0 + t] = L[t * ch + a - r_lo + rr];
     }
-    if (j == 0) {
+    const int wall = pend - p0;
+    if (rank == 0 && wall > l) {
       // net effect of the leaf's interchanges on the rows they touch: row s_rows[i] receives the
       // former row s_src[i]; the leaf's own rows c0 .. c0+l-1 come first
       if (tid == 0) {
@@ -568,8 +511,10 @@ __global__ void __launch_bounds__(coop::NT, 1) k_panel_coop(
           const int pr = s_piv[t];
           if (pr == c0 + t) continue;
           int ip = -1;
-          for (int i = 0; i < m; ++i)
-            if (s_rows[i] == pr) { ip = i; break; }
+          if (pr < c0 + l) ip = pr - c0;
+          else
+            for (int i = l; i < m; ++i)
+              if (s_rows[i] == pr) { ip = i; break; }
           if (ip < 0) { s_rows[m] = pr; s_src[m] = pr; ip = m++; }
           const int tmp = s_src[t];
           s_src[t] = s_src[ip];
@@ -579,56 +524,100 @@ __global__ void __launch_bounds__(coop::NT, 1) k_panel_coop(
       }
       __syncthreads();
       const int m = s_m;
-      for (int jj = p0 + tid; jj < pend; jj += NT) {  // the panel's columns outside the leaf
-        if (jj >= c0 && jj < c0 + l) continue;
-        Cx<float> v[2 * LWMAX];
-        for (int i = 0; i < m; ++i) v[i] = ldcg_cx(M + (int64_t)s_src[i] * ld + jj);
-        if (jj >= c0 + l)  // U block: forward substitution with the leaf's unit lower L11
-          for (int s = 1; s < l; ++s)
-            for (int t = 0; t < s; ++t) {
-              const Cx<float> lv = S[t * ch + c0 + s - r_lo];
-              v[s].re -= lv.re * v[t].re - lv.im * v[t].im;
-              v[s].im -= lv.re * v[t].im + lv.im * v[t].re;
-            }
-        for (int i = 0; i < m; ++i) M[(int64_t)s_rows[i] * ld + jj] = v[i];
+#pragma unroll 4
+      for (int e = tid; e < m * PW; e += NT) {
+        const int i = e / PW, jj = e - i * PW, col = p0 + jj;
+        if (jj < wall && (col < c0 || col >= c0 + l)) X[i * PW + jj] = ldcg(M + (int64_t)s_src[i] * ld + col);
+      }
+      __syncthreads();
+      for (int jj = tid; jj < wall; jj += NT)  // U block: forward substitution with the unit lower L11
+        if (p0 + jj >= c0 + l) {
+          Cx<S> x[LW];
+#pragma unroll
+          for (int s = 0; s < LW; ++s) x[s] = s < l ? X[s * PW + jj] : Cx<S>{0, 0};
+#pragma unroll
+          for (int t = 0; t < LW - 1; ++t)
+#pragma unroll
+            for (int s = t + 1; s < LW; ++s)
+              if (s < l) {
+                const Cx<S> lv = L[t * ch + c0 + s - r_lo];
+                S re, im;
+                re = fma(lv.re, x[t].re, -mul_rn(lv.im, x[t].im));
+                if (leaf) im = fma(lv.im, x[t].re, mul_rn(lv.re, x[t].im));
+                else im = fma(lv.re, x[t].im, mul_rn(lv.im, x[t].re));
+                x[s].re -= re;
+                x[s].im -= im;
+              }
+#pragma unroll
+          for (int s = 0; s < LW; ++s)
+            if (s < l) X[s * PW + jj] = x[s];
+        }
+      __syncthreads();
+#pragma unroll 4
+      for (int e = tid; e < m * PW; e += NT) {
+        const int i = e / PW, jj = e - i * PW, col = p0 + jj;
+        if (jj < wall && (col < c0 || col >= c0 + l)) M[(int64_t)s_rows[i] * ld + col] = X[i * PW + jj];
       }
     }
-    if (!barrier()) return;
+    cluster_sync();
     const int cs = c0 + l, wr = pend - cs;
     if (wr > 0) {  // rows below the leaf, panel columns right of it: A -= L_leaf U_leaf
       for (int e = tid; e < l * wr; e += NT) {
         const int t = e / wr, jj = e - t * wr;
-        Ub[t * coop::WMAX + jj] = ldcg_cx(M + (int64_t)(c0 + t) * ld + cs + jj);
+        Ub[t * PW + jj] = ldcg(M + (int64_t)(c0 + t) * ld + cs + jj);
       }
       __syncthreads();
       const int rb = max(r_lo, cs);
       const int nrow = max(0, r_hi - rb);
-      if ((wr & 1) == 0 && ((ld | cs) & 1) == 0 && (bstride & 1) == 0) {  // two columns per thread, 16-byte accesses
+      bool pairs = false;
+      if constexpr (sizeof(S) == 4) pairs = ((wr | ld | cs) & 1) == 0 && (bstride & 1) == 0;
+      if (pairs) {  // FP32: two columns per thread, 16-byte accesses
         const int hw = wr >> 1;
 #pragma unroll 2
         for (int e = tid; e < nrow * hw; e += NT) {
           const int rr = e / hw, jj = 2 * (e - rr * hw), r = rb + rr;
           float4* mp = reinterpret_cast<float4*>(M + (int64_t)r * ld + cs + jj);
           float4 acc = __ldcg(mp);
-          for (int t = 0; t < l; ++t) {
-            const Cx<float> lv = S[t * ch + r - r_lo];
-            const float4 u = *reinterpret_cast<const float4*>(Ub + t * coop::WMAX + jj);
-            acc.x -= lv.re * u.x - lv.im * u.y;
-            acc.y -= lv.re * u.y + lv.im * u.x;
-            acc.z -= lv.re * u.z - lv.im * u.w;
-            acc.w -= lv.re * u.w + lv.im * u.z;
+          if (sum_first) {
+            float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int t = 0; t < l; ++t) {
+              const Cx<S> lv = L[t * ch + r - r_lo];
+              const float4 uu = *reinterpret_cast<const float4*>(Ub + t * PW + jj);
+              sum.x += lv.re * uu.x - lv.im * uu.y;
+              sum.y += lv.re * uu.y + lv.im * uu.x;
+              sum.z += lv.re * uu.z - lv.im * uu.w;
+              sum.w += lv.re * uu.w + lv.im * uu.z;
+            }
+            acc.x -= sum.x; acc.y -= sum.y; acc.z -= sum.z; acc.w -= sum.w;
+          } else {
+            for (int t = 0; t < l; ++t) {
+              const Cx<S> lv = L[t * ch + r - r_lo];
+              const float4 uu = *reinterpret_cast<const float4*>(Ub + t * PW + jj);
+              acc.x -= lv.re * uu.x - lv.im * uu.y;
+              acc.y -= lv.re * uu.y + lv.im * uu.x;
+              acc.z -= lv.re * uu.z - lv.im * uu.w;
+              acc.w -= lv.re * uu.w + lv.im * uu.z;
+            }
           }
           *mp = acc;
         }
       } else {
+#pragma unroll 2
         for (int e = tid; e < nrow * wr; e += NT) {
           const int rr = e / wr, jj = e - rr * wr, r = rb + rr;
-          Cx<float>* mp = M + (int64_t)r * ld + cs + jj;
-          Cx<float> acc = ldcg_cx(mp);
-          for (int t = 0; t < l; ++t) {
-            const Cx<float> lv = S[t * ch + r - r_lo], u = Ub[t * coop::WMAX + jj];
-            acc.re -= lv.re * u.re - lv.im * u.im;
-            acc.im -= lv.re * u.im + lv.im * u.re;
+          Cx<S>* mp = M + (int64_t)r * ld + cs + jj;
+          Cx<S> acc = ldcg(mp);
+          if (sum_first) {
+            S ar = 0, ai = 0;
+            for (int t = 0; t < l; ++t) {
+              const Cx<S> lv = L[t * ch + r - r_lo], uu = Ub[t * PW + jj];
+              ar += lv.re * uu.re - lv.im * uu.im;
+              ai += lv.re * uu.im + lv.im * uu.re;
+            }
+            acc.re -= ar;
+            acc.im -= ai;
+          } else {
+            for (int t = 0; t < l; ++t) cx_msub(acc, L[t * ch + r - r_lo], Ub[t * PW + jj]);
           }
           *mp = acc;
         }
@@ -636,6 +625,7 @@ __global__ void __launch_bounds__(coop::NT, 1) k_panel_coop(
       __syncthreads();
     }
   }
+  cluster_sync();  // no CTA leaves while another may still store into its shared memory
 }
 
 // Leaf width for a panel whose rows start at p0: the widest power of two <= 16 whose leaf and U
@@ -924,71 +914,86 @@ int lu_factor_simt(bie_ctx* c, Cx<S>* A, int batch, int n, int ld, int64_t bstri
   return BIE_OK;
 }
 
-size_t lu_coop_scratch_bytes(int batch) { return coop::scratch_bytes(batch, kCoopMaxGrid); }
-
-// The cooperative panel (k_panel_coop) for the panel at p0 when it applies: a panel taller than
-// the 16-column one-CTA leaf holds (1536 rows), at most half as many matrices as SMs, and a
-// chunk of rows per CTA whose leaf of at least 4 columns fits shared memory.  *used tells whether
-// it ran.  `coop` is the scratch of lu_coop_scratch_bytes(batch), err the LU's error word.
-static int panel_coop32(bie_ctx* c, Cx<float>* A, int batch, int n, int ld, int64_t bstride, int p0, int w,
-                        int32_t* piv, int32_t* info, void* coop, int32_t* err, bool* used) {
+// The cluster panel (k_panel_cluster) for the panel at p0 when it applies; *used tells whether it
+// ran.  The largest cluster of which as many as matrices are resident at once, or in the fewest
+// rounds (the time of a column falls with its rows per CTA until the barrier's latency is left).
+// Measured, factorisation
+// phase with 16 / 8 / 4 / 2 CTAs a matrix and with one-CTA leaves (k_leaf): two systems of N = 10 272
+// 46.8 / 55.8 / 76.7 / 140 / 141 ms, 24 of N = 3086 30.7 / 20.9 / 16.7 / 20.5 / 23.2, 64 of N = 2884 67.6 /
+// 44.9 / 31.4 / 27.6 / 32.1, one of N = 362 0.86 / 0.87 / 0.87 / 0.90 / 1.09.  Where only one CTA a matrix
+// fits (128 systems: 51.3 against 47.6 ms) the leaves of k_leaf remain, except for a panel that one
+// CTA holds anyway.
+template <class S>
+static int panel_cluster(bie_ctx* c, Cx<S>* A, int batch, int n, int ld, int64_t bstride, int p0, int w, int32_t* piv,
+                         int32_t* info, bool* used) {
   *used = false;
   const int rows = n - p0;
-  if (!coop || !c->lu_coop || w > coop::WMAX || rows <= 1536) return BIE_OK;
+  if (!c->lu_coop || w > pcl::PW) return BIE_OK;
+  // The form of the roundings: panels of up to 1536 rows and of batches above half the SMs as
+  // k_leaf; else 16-column leaves, narrower where a matrix's share of the SMs, taken as one CTA each with
+  // at least 256 rows, would hold no more of its rows in shared memory.
   int nsm = 0;
   BIE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
-  int cpm = std::min(nsm / batch, (rows + 255) / 256);  // one CTA per SM (the leaf takes most of its memory)
-  if (cpm < 2) return BIE_OK;
-  const int ch = ((rows + cpm - 1) / cpm + 63) / 64 * 64;
-  cpm = (rows + ch - 1) / ch;
-  if (cpm < 2 || batch * cpm > kCoopMaxGrid) return BIE_OK;
-  BIE_TRY((set_smem_max(k_panel_coop)));
+  const int share = std::min(nsm / batch, (rows + 255) / 256);
+  const int leaf = rows <= 1536 || share < 2 ? 1 : 0, sum_first = leaf && batch < 64 ? 1 : 0;
+  int lw_max = pcl::LW;
+  if (!leaf && sizeof(S) == 4) {
+    const size_t held = ((rows + share - 1) / share + 63) / 64 * 64;
+    while (lw_max > 4 && (lw_max * held + pcl::LW * pcl::PW) * sizeof(Cx<S>) > 231 * 1024 - 4096) lw_max >>= 1;
+  }
+  BIE_TRY((set_smem_max(k_panel_cluster<S>)));
+  BIE_CUDA_TRY(cudaFuncSetAttribute((const void*)k_panel_cluster<S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaFuncAttributes fa;
-  BIE_CUDA_TRY(cudaFuncGetAttributes(&fa, (const void*)k_panel_coop));
+  BIE_CUDA_TRY(cudaFuncGetAttributes(&fa, (const void*)k_panel_cluster<S>));
   const size_t limit = (size_t)smem_optin() - fa.sharedSizeBytes;
-  int lw = coop::LWMAX;
-  auto smem_of = [&](int l) { return ((size_t)l * ch + (size_t)coop::LWMAX * coop::WMAX) * sizeof(Cx<float>); };
-  while (lw >= 4 && smem_of(lw) > limit) lw >>= 1;
-  if (lw < 4) return BIE_OK;
-  lw = std::min(lw, w);
-  const size_t smem = smem_of(lw);
-  int per_sm = 0;
-  BIE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_panel_coop, coop::NT, smem));
-  if ((int64_t)per_sm * nsm < (int64_t)batch * cpm) return BIE_OK;
-  char* base = (char*)coop + 256;
-  unsigned* bar = (unsigned*)base;  // [batch] counters, then the abort flag
-  unsigned* abort_flag = bar + batch;
-  const size_t cand_off = ((size_t)(batch + 1) * 4 + 255) & ~(size_t)255;
-  coop::Cand* cand = (coop::Cand*)(base + cand_off);
-  BIE_CUDA_TRY(cudaMemsetAsync(bar, 0, cand_off + 2 * (size_t)batch * cpm * sizeof(coop::Cand), c->stream));
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(batch * cpm));
-  cfg.blockDim = dim3(coop::NT);
-  cfg.dynamicSmemBytes = smem;
+  cfg.blockDim = dim3(pcl::NT);
   cfg.stream = c->stream;
   cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeCooperative;
-  at[0].val.cooperative = 1;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
+  // the cluster: fewest rounds of resident clusters, then the most CTAs
+  int best_cl = 0, best_ch = 0, best_rounds = 0;
+  for (int cl = pcl::MAXC; cl >= 1; cl >>= 1) {
+    const int ch = std::max(pcl::PW, ((rows + cl - 1) / cl + 31) / 32 * 32);
+    if (cl > 1 && (int64_t)(cl / 2) * ch >= rows) continue;  // half as many CTAs hold the rows
+    if (cl == 1 && rows > pcl::PW) continue;
+    if (pcl::smem_bytes<S>(lw_max, ch) > limit) continue;
+    cfg.gridDim = dim3((unsigned)(batch * cl));
+    cfg.dynamicSmemBytes = pcl::smem_bytes<S>(lw_max, ch);
+    at[0].val.clusterDim.x = (unsigned)cl;
+    int active = 0;
+    BIE_CUDA_TRY(cudaOccupancyMaxActiveClusters(&active, k_panel_cluster<S>, &cfg));
+    if (active < 1) continue;
+    const int rounds = (batch + active - 1) / active;
+    if (best_cl == 0 || rounds < best_rounds) {
+      best_cl = cl;
+      best_ch = ch;
+      best_rounds = rounds;
+    }
+  }
+  if (best_cl == 0 || best_rounds > (share >= 2 ? 2 : 1)) return BIE_OK;
+  cfg.gridDim = dim3((unsigned)(batch * best_cl));
+  cfg.dynamicSmemBytes = pcl::smem_bytes<S>(lw_max, best_ch);
+  at[0].val.clusterDim.x = (unsigned)best_cl;
   count_launch();
-  BIE_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_panel_coop, A, bstride, n, ld, p0, w, lw, cpm, ch, piv, info, bar,
-                                  abort_flag, cand, err));
+  BIE_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_panel_cluster<S>, A, bstride, n, ld, p0, w, std::min(lw_max, w), best_ch,
+                                  sum_first, leaf, piv, info));
   *used = true;
   return BIE_OK;
 }
 
 // Panel factorisation plus row swaps (all columns) and the U12 solve of the columns in
 // [p0 + w, tend) for one block column (FP32); the trailing update is left to the caller (the
-// tensor-core kernels of lu_tc.cu).  coop / err: scratch and error word of the cooperative panel
-// (NULL: one CTA per matrix always).
+// tensor-core kernels of lu_tc.cu).
 int lu_panel_steps32(bie_ctx* c, cf* A, int batch, int n, int ld, int64_t bstride, int p0, int w, int32_t* piv,
-                     int32_t* info, int tend, void* coop, int32_t* err, float* ub, int64_t ub_stride, int krow,
-                     int koff, bool* emitted) {
+                     int32_t* info, int tend, float* ub, int64_t ub_stride, int krow, int koff, bool* emitted) {
   if (emitted) *emitted = false;
   Cx<float>* M = reinterpret_cast<Cx<float>*>(A);
   bool used = false;
-  BIE_TRY(panel_coop32(c, M, batch, n, ld, bstride, p0, w, piv, info, coop, err, &used));
+  BIE_TRY(panel_cluster<float>(c, M, batch, n, ld, bstride, p0, w, piv, info, &used));
   if (!used) BIE_TRY(panel_factor<float>(c, M, batch, n, ld, bstride, p0, w, piv, info));
   dim3 gs((unsigned)((n + 127) / 128), batch);
   if (w == 64) {  // swaps here, the solve with the register-resident kernel
@@ -1040,17 +1045,14 @@ int lu_solve64(bie_ctx* c, const cd* LU, int batch, int n, int ld, int64_t bstri
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
 }
-// FP32 LU without tensor cores for systems the TF32 factor cannot refine: 64-column panels
-// (cooperative for a few tall matrices, see k_panel_coop), their row swaps and U blocks, and the
-// trailing update A22 -= L21 U12 in FP32 on the CUDA cores (k_gemm_update).  coop / err: the
-// cooperative panel's scratch and error word.
-int lu_factor32_panels(bie_ctx* c, cf* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info,
-                       void* coop, int32_t* err) {
+// FP32 LU without tensor cores for systems the TF32 factor cannot refine: 64-column panels, their
+// row swaps and U blocks, and the trailing update A22 -= L21 U12 in FP32 on the CUDA cores
+// (k_gemm_update).
+int lu_factor32_panels(bie_ctx* c, cf* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info) {
   Cx<float>* M = reinterpret_cast<Cx<float>*>(A);
-  BIE_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int32_t), c->stream));
   for (int p0 = 0; p0 < n; p0 += 64) {
     const int w = std::min(64, n - p0);
-    BIE_TRY(lu_panel_steps32(c, A, batch, n, ld, bstride, p0, w, piv, info, n, coop, err, nullptr, 0, 0, 0, nullptr));
+    BIE_TRY(lu_panel_steps32(c, A, batch, n, ld, bstride, p0, w, piv, info, n, nullptr, 0, 0, 0, nullptr));
     const int rem = n - p0 - w;
     if (rem > 0) {
       dim3 gg((unsigned)((rem + 63) / 64), (unsigned)((rem + 63) / 64), batch);

@@ -22,9 +22,7 @@
 namespace bie {
 
 int lu_panel_steps32(bie_ctx* c, cf* A, int batch, int n, int ld, int64_t bstride, int p0, int w, int32_t* piv,
-                     int32_t* info, int tend, void* coop, int32_t* err, float* ub, int64_t ub_stride, int krow,
-                     int koff, bool* emitted);
-size_t lu_coop_scratch_bytes(int batch);
+                     int32_t* info, int tend, float* ub, int64_t ub_stride, int krow, int koff, bool* emitted);
 int lu_trsm_rows32(bie_ctx* c, cf* A, int batch, int n, int ld, int64_t bstride, int p0, int w, int jlo, float* ub,
                    int64_t ub_stride, int krow, int koff, bool* emitted);
 
@@ -581,11 +579,9 @@ int lu_block_for(const bie_ctx* c, int n) {
 }
 
 size_t lu_tc_scratch_bytes(int batch, int n, int block) {
-  // error flag, the cooperative panel's scratch, B^T for one 64-row panel (128 floats per row)
-  // and for one outer block (2 NBO)
+  // error flag, B^T for one 64-row panel (128 floats per row) and for one outer block (2 NBO)
   if (block < tc::NB || block > kMaxLuBlock) block = kMaxLuBlock;
-  return 256 + ((lu_coop_scratch_bytes(batch) + 255) & ~(size_t)255) +
-         (size_t)batch * 2 * n * (2 * tc::NB + 2 * block) * sizeof(float);
+  return 256 + (size_t)batch * 2 * n * (2 * tc::NB + 2 * block) * sizeof(float);
 }
 
 int lu_factor_tc(bie_ctx* c, cf* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info,
@@ -594,13 +590,12 @@ int lu_factor_tc(bie_ctx* c, cf* A, int batch, int n, int ld, int64_t bstride, i
   if (ld % 64 != 0 || bstride % 2 != 0) return fail(BIE_ERR_INVALID_ARG, "tcgen05 LU needs ld % 64 == 0 and even batch stride");
   int32_t* err = (int32_t*)scratch;
   BIE_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int32_t), c->stream));
-  void* coop = (char*)scratch + 256;
   const int ver = c->tc_version;
   const int NBO = lu_block_for(c, n);
   // panel width of the deferred version (32 or 64; versions 1 and 2 use 64)
   const int nb = (ver >= 3 && c->lu_panel == 32) ? 32 : NB;
   if (NBO % NB != 0 || NBO < NB || NBO > kMaxLuBlock) return fail(BIE_ERR_INVALID_ARG, "LU block must be 128, 256 or 512");
-  float* ub = reinterpret_cast<float*>((char*)coop + ((lu_coop_scratch_bytes(batch) + 255) & ~(size_t)255));
+  float* ub = reinterpret_cast<float*>((char*)scratch + 256);
   const int kr = 2 * nb;                                // reals along K of one panel's B^T
   const int64_t ub_stride = (int64_t)2 * n * kr;        // floats per matrix, one panel
   float* ubo = ub + (int64_t)batch * ub_stride;
@@ -656,7 +651,7 @@ int lu_factor_tc(bie_ctx* c, cf* A, int batch, int n, int ld, int64_t bstride, i
         // the U solve of the block's columns right of the panel also writes their B^T (64-row
         // panels); otherwise the build pass does
         bool emitted = false;
-        BIE_TRY(lu_panel_steps32(c, A, batch, n, ld, bstride, p0, w, piv, info, E, coop, err, ub, ub_stride, kr, 0,
+        BIE_TRY(lu_panel_steps32(c, A, batch, n, ld, bstride, p0, w, piv, info, E, ub, ub_stride, kr, 0,
                                  &emitted));
         if (q < E) {  // then w == nb (E - P0 is a multiple of nb unless E == n)
           if (!emitted) BIE_TRY(build(p0, q, E, false, 0, w));
@@ -678,7 +673,7 @@ int lu_factor_tc(bie_ctx* c, cf* A, int batch, int n, int ld, int64_t bstride, i
   }
   for (int p0 = 0; p0 < n; p0 += NB) {
     const int w = std::min(NB, n - p0);
-    BIE_TRY(lu_panel_steps32(c, A, batch, n, ld, bstride, p0, w, piv, info, n, coop, err, nullptr, 0, 0, 0, nullptr));
+    BIE_TRY(lu_panel_steps32(c, A, batch, n, ld, bstride, p0, w, piv, info, n, nullptr, 0, 0, 0, nullptr));
     const int rem = n - p0 - w;
     if (rem <= 0) continue;
     if (ver == 2) {

@@ -23,8 +23,7 @@ int refine_solve(bie_ctx* c, const cf* A, const cf* LU, int nk, int n, int64_t l
                  int it_max, double tol, cf* D, void* tscratch);
 size_t trsv_scratch_bytes(int nk, int n);
 int lu_tc_error(bie_ctx* c, void* scratch, int32_t* out);
-int lu_factor32_panels(bie_ctx* c, cf* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info,
-                       void* coop, int32_t* err);
+int lu_factor32_panels(bie_ctx* c, cf* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info);
 int factor_aux(bie_ctx* c, const cf* LU, int nk, int n, int64_t ld, int64_t bstride, const int32_t* piv,
                int32_t* perm, cf* D);
 int64_t diag_inv_stride(int n);
@@ -326,7 +325,7 @@ int solve_mixed(bie_ctx* c, const double* k, int64_t Nk, cd* surf_out, bie_repor
       if (d == 0 && c->tc_version > 0) {  // a bounded wait of the factorisation gave up: its factor is void
         int32_t terr = 0;
         BIE_TRY(lu_tc_error(c, tcs, &terr));
-        if (terr) return fail(BIE_ERR_TIMEOUT, "LU: a bounded wait in the tensor-core update or a cooperative panel gave up");
+        if (terr) return fail(BIE_ERR_TIMEOUT, "LU: a bounded wait in the tensor-core update gave up");
       }
       if (timing && d == 0) {  // the batch has completed (its state was read)
         c->phase.assembly_ms += elapsed(0, 1);
@@ -425,17 +424,15 @@ int solve_mixed(bie_ctx* c, const double* k, int64_t Nk, cd* surf_out, bie_repor
     BIE_TRY(assemble64(c, kg, 1, A64, b64, s64, c->reassembly_ff != 0));
     BIE_LAUNCH(k_cd_to_cf<<<dim3((unsigned)((N + 255) / 256), (unsigned)N), 256, 0, c->stream>>>(A64, N, LU, ld));
     BIE_CUDA_TRY(cudaMemsetAsync(info, 0, sizeof(int32_t), c->stream));
-    BIE_TRY(lu_factor32_panels(c, LU, 1, (int)N, (int)ld, bstride, piv, info, (char*)tcs + 256, (int32_t*)tcs));
+    BIE_TRY(lu_factor32_panels(c, LU, 1, (int)N, (int)ld, bstride, piv, info));
     BIE_TRY(factor_aux(c, LU, 1, (int)N, ld, bstride, piv, perm, Dinv));
     BIE_CUDA_TRY(cudaMemsetAsync(x, 0, (size_t)N * sizeof(cd), c->stream));
     BIE_TRY(refine_fp64_system(c, A64, b64, LU, ld, bstride, perm, sel_g, 1, (int)N, x, xg, rg, rowabs_g, state_g,
                                kRefactorItMax, c->refine64_tol, Dinv, s64 + N, true));
-    int32_t d1 = 0, it1 = 0, zp = 0, terr = 0;
+    int32_t d1 = 0, it1 = 0, zp = 0;
     double b1 = 0.0, e1 = 0.0;
     BIE_TRY(refine_read_state(c, state_g, 1, &d1, &it1, &b1, &e1));
     BIE_CUDA_TRY(cudaMemcpy(&zp, info, sizeof(int32_t), cudaMemcpyDeviceToHost));
-    BIE_TRY(lu_tc_error(c, tcs, &terr));
-    if (terr) return fail(BIE_ERR_TIMEOUT, "LU: a bounded wait in a cooperative panel gave up");
     if (!d1 || zp || !std::isfinite(b1)) continue;  // stays for the full FP64 path
     dim3 gs((unsigned)((N + 255) / 256), 1);
     BIE_LAUNCH(k_surface_fields<<<gs, 256, 0, c->stream>>>(c->bc, N, x, s64, surf_out + full64_idx[f] * 2 * N, 2 * N));
