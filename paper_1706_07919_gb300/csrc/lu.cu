@@ -18,6 +18,17 @@ template <class S> __device__ __forceinline__ Cx<S> cx_div(Cx<S> a, Cx<S> b) {
   return {(a.re * b.re + a.im * b.im) / d, (a.im * b.re - a.re * b.im) / d};
 }
 
+// a -= l u: in FP32 rounded as the one-CTA leaf does, in FP64 every product fused (four instructions of
+// the narrow FP64 pipe instead of six).
+__device__ __forceinline__ void cx_msub(Cx<float>& a, Cx<float> l, Cx<float> u) {
+  a.re -= l.re * u.re - l.im * u.im;
+  a.im -= l.re * u.im + l.im * u.re;
+}
+__device__ __forceinline__ void cx_msub(Cx<double>& a, Cx<double> l, Cx<double> u) {
+  a.re = fma(-l.re, u.re, fma(l.im, u.im, a.re));
+  a.im = fma(-l.re, u.im, fma(-l.im, u.re, a.im));
+}
+
 // ---- panel factorisation: one CTA per matrix, columns p0 .. p0+nb-1, rows p0 .. n-1 ----------
 template <class S>
 __global__ void __launch_bounds__(512) k_panel(Cx<S>* __restrict__ A, int64_t bstride, int n, int ld, int p0,
@@ -273,8 +284,7 @@ __global__ void __launch_bounds__(1024) k_leaf(Cx<S>* __restrict__ A, int64_t bs
 
 // Rows below the leaf, panel columns right of it: A -= L_leaf U_leaf (K = lw <= 16), as its own
 // launch for small batches (the leaf kernel has one CTA per matrix).  One warp per row, lanes over the (<= 64) columns so that the read-modify-write of A coalesces;
-// the row's lw entries of L are broadcast.  grid (ceil(rows / 64), batch), block 256 (8 warps, 8
-// rows each).
+// the row's lw entries of L are broadcast.  grid (any, batch), block 256: 8 warps, a row each at a time.
 template <class S>
 __global__ void __launch_bounds__(256) k_leaf_update(Cx<S>* __restrict__ A, int64_t bstride, int n, int ld, int p0,
                                                      int w, int c0, int lw) {
@@ -288,8 +298,7 @@ __global__ void __launch_bounds__(256) k_leaf_update(Cx<S>* __restrict__ A, int6
   }
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int rbeg = c0 + lw + blockIdx.x * 64;
-  for (int r = rbeg + warp; r < min(rbeg + 64, n); r += 8) {
+  for (int r = c0 + lw + blockIdx.x * 8 + warp; r < n; r += gridDim.x * 8) {
     const Cx<S>* lrow = M + (int64_t)r * ld + c0;
     Cx<S> l[16];
 #pragma unroll
@@ -304,8 +313,13 @@ __global__ void __launch_bounds__(256) k_leaf_update(Cx<S>* __restrict__ A, int6
         for (int s = 0; s < 16; ++s)
           if (s < lw) {
             const Cx<S> u = U[s * 64 + j];
-            ar += l[s].re * u.re - l[s].im * u.im;
-            ai += l[s].re * u.im + l[s].im * u.re;
+            if constexpr (sizeof(S) == 4) {
+              ar += l[s].re * u.re - l[s].im * u.im;
+              ai += l[s].re * u.im + l[s].im * u.re;
+            } else {
+              ar = fma(l[s].re, u.re, fma(-l[s].im, u.im, ar));
+              ai = fma(l[s].re, u.im, fma(l[s].im, u.re, ai));
+            }
           }
         Cx<S>& m = M[(int64_t)r * ld + cs + j];
         m.re -= ar;
@@ -329,7 +343,9 @@ __global__ void __launch_bounds__(256) k_leaf_update(Cx<S>* __restrict__ A, int6
 // solves the leaf's U block L11^{-1} A12 for the panel columns right of the leaf; one barrier later
 // every CTA updates its rows of those columns, A -= L U.  Global data written by another CTA of the
 // cluster is read with L2-coherent loads after a cluster barrier (release / acquire).
-// Bound: the latency of a column (a CTA barrier, the remote stores, a cluster barrier).
+// Bound: the latency of a column (a CTA barrier, the remote stores, a cluster barrier); in FP64 the
+// rows' FP64 instructions.  N = 2884, two systems in FP64: 72.6 ms of one-CTA leaves and their updates ->
+// 19.9 ms, the panels' other columns updated over all SMs (29.3 ms inside the cluster).
 // Every entry goes through the operations of the one-CTA leaf (k_leaf) in its order, so that the
 // pivots and, for panels of up to 1536 rows (leaf, where that kernel takes 16 columns), the factor are
 // the same bit for bit whatever the cluster; sum_first: A -= (sum of L U), as k_leaf_update forms it
@@ -377,17 +393,11 @@ __device__ __forceinline__ Cx<double> ldcg(const Cx<double>* p) {
 }
 }  // namespace pcl
 
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-// a -= l u, rounded as in the one-CTA leaf
-template <class S> __device__ __forceinline__ void cx_msub(Cx<S>& a, Cx<S> l, Cx<S> u) {
-  a.re -= l.re * u.re - l.im * u.im;
-  a.im -= l.re * u.im + l.im * u.re;
-}
 
 template <class S>
 __global__ void __launch_bounds__(pcl::NT, 1) k_panel_cluster(Cx<S>* __restrict__ A, int64_t bstride, int n, int ld,
-                                                              int p0, int w, int lw, int ch, int sum_first, int leaf,
+                                                              int p0, int w, int c_lo, int c_hi, int lw, int ch,
+                                                              int sum_first, int leaf, int update,
                                                               int32_t* __restrict__ piv, int32_t* __restrict__ info) {
   using namespace pcl;
   extern __shared__ float4 pcl_smem[];
@@ -409,7 +419,7 @@ __global__ void __launch_bounds__(pcl::NT, 1) k_panel_cluster(Cx<S>* __restrict_
   const uint32_t rec_a = (uint32_t)__cvta_generic_to_shared(&rec[0][0]);
   const uint32_t drow_a = (uint32_t)__cvta_generic_to_shared(&drow[0][0]);
   cluster_sync();  // every CTA of the cluster runs before the first remote store
-  for (int c0 = p0; c0 < pend; c0 += lw) {
+  for (int c0 = c_lo; c0 < c_hi; c0 += lw) {
     const int l = min(lw, pend - c0);
     const int a = max(r_lo, c0);  // first leaf row held here
     const int nr = max(0, r_hi - a);
@@ -464,6 +474,15 @@ __global__ void __launch_bounds__(pcl::NT, 1) k_panel_cluster(Cx<S>* __restrict_
       const Cx<S> d = u[cc];
       const S dd = d.re * d.re + d.im * d.im;
       const bool okd = dd > 0;
+      Cx<S> inv = {0, 0};  // FP64: 1 / d once (a division's FP64 instructions for each row otherwise)
+      if constexpr (sizeof(S) == 8) {
+        double y;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(dd));
+        y = fma(y, fma(-dd, y, 1.0), y);
+        y = fma(y, fma(-dd, y, 1.0), y);
+        if (!(y - y == 0.0)) y = 1.0 / dd;  // outside the approximation's range
+        inv = {d.re * y, -d.im * y};
+      }
       if (tid == 0) {
         s_piv[cc] = p;
         if (rank == 0) {
@@ -480,7 +499,11 @@ __global__ void __launch_bounds__(pcl::NT, 1) k_panel_cluster(Cx<S>* __restrict_
         if (r == p)
           for (int t = 0; t < l; ++t) x[t * ch] = drow[buf][t];
         Cx<S> lv = x[cc * ch];
-        if (okd) lv = cx_div(lv, d);
+        if constexpr (sizeof(S) == 4) {
+          if (okd) lv = cx_div(lv, d);
+        } else {
+          if (okd) lv = cx_mul(lv, inv);
+        }
         x[cc * ch] = lv;
         if (cc + 1 < l) {
           Cx<S> y = x[(cc + 1) * ch];
@@ -541,12 +564,13 @@ __global__ void __launch_bounds__(pcl::NT, 1) k_panel_cluster(Cx<S>* __restrict_
             for (int s = t + 1; s < LW; ++s)
               if (s < l) {
                 const Cx<S> lv = L[t * ch + c0 + s - r_lo];
-                S re, im;
-                re = fma(lv.re, x[t].re, -mul_rn(lv.im, x[t].im));
-                if (leaf) im = fma(lv.im, x[t].re, mul_rn(lv.re, x[t].im));
-                else im = fma(lv.re, x[t].im, mul_rn(lv.im, x[t].re));
-                x[s].re -= re;
-                x[s].im -= im;
+                if constexpr (sizeof(S) == 4) {
+                  x[s].re -= fma(lv.re, x[t].re, -__fmul_rn(lv.im, x[t].im));
+                  x[s].im -= leaf ? fma(lv.im, x[t].re, __fmul_rn(lv.re, x[t].im))
+                                  : fma(lv.re, x[t].im, __fmul_rn(lv.im, x[t].re));
+                } else {
+                  cx_msub(x[s], lv, x[t]);
+                }
               }
 #pragma unroll
           for (int s = 0; s < LW; ++s)
@@ -559,6 +583,7 @@ __global__ void __launch_bounds__(pcl::NT, 1) k_panel_cluster(Cx<S>* __restrict_
         if (jj < wall && (col < c0 || col >= c0 + l)) M[(int64_t)s_rows[i] * ld + col] = X[i * PW + jj];
       }
     }
+    if (!update) continue;  // (one leaf per launch: its update is another kernel's)
     cluster_sync();
     const int cs = c0 + l, wr = pend - cs;
     if (wr > 0) {  // rows below the leaf, panel columns right of it: A -= L_leaf U_leaf
@@ -795,6 +820,66 @@ __global__ void __launch_bounds__(64) k_trsm64(Cx<float>* __restrict__ A, int64_
   }
 }
 
+// The same for FP64: 32 columns (lanes) per CTA, their 64 rows in the registers of four warps, four rows of
+// every 16 each: the owner of the next four rows solves them and leaves them in shared memory, then
+// every warp subtracts their products from its later rows.  Each SM quarter has its own FP64 lanes: one
+// warp alone reaches a quarter of the rate.  grid (ceil((j1 - j0) / 32), batch), block 128.
+// N = 2884, two systems (45 launches): 12.6 ms by k_swap_trsm<double>'s substitution through global
+// memory, 18.1 ms one warp per 32 columns, 4.7 ms this way.
+constexpr size_t kTrsm64dSmem = (64 * 64 + 4 * 32) * sizeof(Cx<double>);
+__global__ void __launch_bounds__(128) k_trsm64d(Cx<double>* __restrict__ A, int64_t bstride, int n, int ld, int p0, int j0,
+                                                 int j1) {
+  extern __shared__ double2 trsmd_smem[];
+  Cx<double>* LT = reinterpret_cast<Cx<double>*>(trsmd_smem);            // LT[t * 64 + s] = L11[s][t]
+  Cx<double>(*X)[32] = reinterpret_cast<Cx<double>(*)[32]>(LT + 64 * 64);  // the four rows just solved
+  Cx<double>* M = A + (int64_t)blockIdx.y * bstride;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll 8
+  for (int e = threadIdx.x; e < 64 * 64; e += 128) {
+    const int r = e >> 6, c = e & 63;
+    LT[c * 64 + r] = M[(int64_t)(p0 + r) * ld + p0 + c];
+  }
+  const int j = j0 + blockIdx.x * 32 + lane;
+  const bool act = j < j1 && j < n;
+  Cx<double> x[4][4];  // rows 16 b + 4 warp + r
+#pragma unroll
+  for (int b = 0; b < 4; ++b)
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      x[b][r] = act ? M[(int64_t)(p0 + 16 * b + 4 * warp + r) * ld + j] : Cx<double>{0.0, 0.0};
+  __syncthreads();
+#pragma unroll
+  for (int b = 0; b < 4; ++b)
+#pragma unroll 1
+    for (int w = 0; w < 4; ++w) {
+      const int t0 = 16 * b + 4 * w;
+      if (warp == w) {
+#pragma unroll
+        for (int t = 0; t < 3; ++t)
+#pragma unroll
+          for (int r = t + 1; r < 4; ++r) cx_msub(x[b][r], LT[(t0 + t) * 64 + t0 + r], x[b][t]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) X[r][lane] = x[b][r];
+      }
+      __syncthreads();
+#pragma unroll
+      for (int b2 = b; b2 < 4; ++b2)
+        if (b2 > b || warp > w)
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            const Cx<double> xt = X[t][lane];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) cx_msub(x[b2][r], LT[(t0 + t) * 64 + 16 * b2 + 4 * warp + r], xt);
+          }
+      __syncthreads();
+    }
+  if (act)
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) M[(int64_t)(p0 + 16 * b + 4 * warp + r) * ld + j] = x[b][r];
+}
+
 // ---- SIMT trailing update A22 -= L21 U12 (64 x 64 complex tile per CTA, 256 threads) ---------
 template <class S>
 __global__ void __launch_bounds__(256) k_gemm_update(Cx<S>* __restrict__ A, int64_t bstride, int n, int ld,
@@ -893,6 +978,71 @@ __global__ void __launch_bounds__(256) k_lu_solve(const Cx<S>* __restrict__ LU, 
   }
 }
 
+// The same in FP64 over all SMs: y = P b gathered, then for each 64-row block its triangular solve by
+// one CTA per system (k_solve_block) and the product with the rest of its columns by a warp per row
+// (k_solve_rows).  N = 2884, two systems: 35.6 ms of one CTA per system, row by row -> 2.5 ms.
+__global__ void k_gather_perm(const Cx<double>* __restrict__ b, int64_t bstride_b, int n, const int32_t* __restrict__ perm,
+                              Cx<double>* __restrict__ y) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) y[(int64_t)blockIdx.y * n + i] = b[(int64_t)blockIdx.y * bstride_b + perm[(int64_t)blockIdx.y * n + i]];
+}
+__global__ void k_copy_back(const Cx<double>* __restrict__ y, int n, Cx<double>* __restrict__ b, int64_t bstride_b) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) b[(int64_t)blockIdx.y * bstride_b + i] = y[(int64_t)blockIdx.y * n + i];
+}
+template <bool LOWER>
+__global__ void __launch_bounds__(256) k_solve_block(const Cx<double>* __restrict__ LU, int64_t bstride, int n, int ld,
+                                                     int j0, Cx<double>* __restrict__ yv) {
+  extern __shared__ double2 sblk_smem[];
+  Cx<double>* D = reinterpret_cast<Cx<double>*>(sblk_smem);  // [64][65], column t at t * 65
+  Cx<double>* x = D + 64 * 65;
+  const int bs = min(64, n - j0), tid = threadIdx.x;
+  const Cx<double>* M = LU + (int64_t)blockIdx.x * bstride + (int64_t)j0 * ld + j0;
+  Cx<double>* y = yv + (int64_t)blockIdx.x * n + j0;
+#pragma unroll 8
+  for (int e = tid; e < bs * 64; e += 256) {
+    const int r = e >> 6, t = e & 63;
+    if (t < bs) D[t * 65 + r] = M[(int64_t)r * ld + t];
+  }
+  if (tid < bs) x[tid] = y[tid];
+  __syncthreads();
+  if (tid >= 64) return;
+  Cx<double> v = tid < bs ? x[tid] : Cx<double>{0.0, 0.0};  // thread r holds row r
+  if (!LOWER && tid < bs) {  // 1 / U_rr, once
+    const Cx<double> d = D[tid * 65 + tid];
+    D[tid * 65 + tid] = cx_div(Cx<double>{1.0, 0.0}, d);
+  }
+  for (int k = 0; k < bs; ++k) {
+    const int s = LOWER ? k : bs - 1 - k;
+    if (tid == s) {
+      if (!LOWER) v = cx_mul(v, D[s * 65 + s]);
+      x[s] = v;
+    }
+    asm volatile("bar.sync 1, 64;" ::: "memory");
+    if (tid < bs && (LOWER ? tid > s : tid < s)) cx_msub(v, D[s * 65 + tid], x[s]);
+  }
+  if (tid < bs) y[tid] = v;
+}
+// y[r] -= sum over the block's columns of LU[r][c] y[c], rows [rlo, rhi): grid (ceil(rows / 8), batch), block 256
+__global__ void __launch_bounds__(256) k_solve_rows(const Cx<double>* __restrict__ LU, int64_t bstride, int n, int ld, int j0,
+                                                    int rlo, int rhi, Cx<double>* __restrict__ yv) {
+  const int lane = threadIdx.x & 31, r = rlo + blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (r >= rhi) return;
+  const Cx<double>* M = LU + (int64_t)blockIdx.y * bstride + (int64_t)r * ld + j0;
+  Cx<double>* y = yv + (int64_t)blockIdx.y * n;
+  const int bs = min(64, n - j0);
+  Cx<double> a = {0.0, 0.0};
+  for (int c = lane; c < bs; c += 32) cx_msub(a, M[c], y[j0 + c]);
+  for (int o = 16; o > 0; o >>= 1) {
+    a.re += __shfl_xor_sync(0xffffffffu, a.re, o);
+    a.im += __shfl_xor_sync(0xffffffffu, a.im, o);
+  }
+  if (lane == 0) {
+    y[r].re += a.re;
+    y[r].im += a.im;
+  }
+}
+
 // ---- host drivers -----------------------------------------------------------------------------
 template <class S>
 int lu_factor_simt(bie_ctx* c, Cx<S>* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info,
@@ -929,6 +1079,11 @@ static int panel_cluster(bie_ctx* c, Cx<S>* A, int batch, int n, int ld, int64_t
   *used = false;
   const int rows = n - p0;
   if (!c->lu_coop || w > pcl::PW) return BIE_OK;
+  BIE_TRY((set_smem_max(k_panel_cluster<S>)));
+  BIE_CUDA_TRY(cudaFuncSetAttribute((const void*)k_panel_cluster<S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaFuncAttributes fa;
+  BIE_CUDA_TRY(cudaFuncGetAttributes(&fa, (const void*)k_panel_cluster<S>));
+  const size_t limit = (size_t)smem_optin() - fa.sharedSizeBytes;
   // The form of the roundings: panels of up to 1536 rows and of batches above half the SMs as
   // k_leaf; else 16-column leaves, narrower where a matrix's share of the SMs, taken as one CTA each with
   // at least 256 rows, would hold no more of its rows in shared memory.
@@ -937,15 +1092,13 @@ static int panel_cluster(bie_ctx* c, Cx<S>* A, int batch, int n, int ld, int64_t
   const int share = std::min(nsm / batch, (rows + 255) / 256);
   const int leaf = rows <= 1536 || share < 2 ? 1 : 0, sum_first = leaf && batch < 64 ? 1 : 0;
   int lw_max = pcl::LW;
-  if (!leaf && sizeof(S) == 4) {
+  if (sizeof(S) == 8) {  // FP64: the widest leaf that 16 CTAs hold
+    const int ch16 = std::max(pcl::PW, ((rows + 15) / 16 + 31) / 32 * 32);
+    while (lw_max > 4 && pcl::smem_bytes<S>(lw_max, ch16) > limit) lw_max >>= 1;
+  } else if (!leaf) {
     const size_t held = ((rows + share - 1) / share + 63) / 64 * 64;
     while (lw_max > 4 && (lw_max * held + pcl::LW * pcl::PW) * sizeof(Cx<S>) > 231 * 1024 - 4096) lw_max >>= 1;
   }
-  BIE_TRY((set_smem_max(k_panel_cluster<S>)));
-  BIE_CUDA_TRY(cudaFuncSetAttribute((const void*)k_panel_cluster<S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  cudaFuncAttributes fa;
-  BIE_CUDA_TRY(cudaFuncGetAttributes(&fa, (const void*)k_panel_cluster<S>));
-  const size_t limit = (size_t)smem_optin() - fa.sharedSizeBytes;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(pcl::NT);
   cfg.stream = c->stream;
@@ -978,9 +1131,24 @@ static int panel_cluster(bie_ctx* c, Cx<S>* A, int batch, int n, int ld, int64_t
   cfg.gridDim = dim3((unsigned)(batch * best_cl));
   cfg.dynamicSmemBytes = pcl::smem_bytes<S>(lw_max, best_ch);
   at[0].val.clusterDim.x = (unsigned)best_cl;
-  count_launch();
-  BIE_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_panel_cluster<S>, A, bstride, n, ld, p0, w, std::min(lw_max, w), best_ch,
-                                  sum_first, leaf, piv, info));
+  const int lw = std::min(lw_max, w), pend = std::min(p0 + w, n);
+  if (sizeof(S) == 4) {
+    count_launch();
+    BIE_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_panel_cluster<S>, A, bstride, n, ld, p0, w, p0, pend, lw, best_ch, sum_first,
+                                    leaf, 1, piv, info));
+  } else {
+    // FP64: a launch per leaf, and the update of the panel's other columns over all SMs (the
+    // clusters' few SMs would take longer for its FP64 arithmetic than for the leaf)
+    for (int c0 = p0; c0 < pend; c0 += lw) {
+      const int l = std::min(lw, pend - c0), below = n - c0 - l;
+      count_launch();
+      BIE_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_panel_cluster<S>, A, bstride, n, ld, p0, w, c0, c0 + l, lw, best_ch,
+                                      sum_first, leaf, 0, piv, info));
+      if (below > 0 && c0 + l < pend)
+        BIE_LAUNCH(k_leaf_update<S><<<dim3((unsigned)((below + 7) / 8), batch), 256, 0, c->stream>>>(A, bstride, n, ld, p0, w,
+                                                                                                  c0, l));
+    }
+  }
   *used = true;
   return BIE_OK;
 }
@@ -1035,13 +1203,73 @@ int lu_trsm_rows32(bie_ctx* c, cf* A, int batch, int n, int ld, int64_t bstride,
   return BIE_OK;
 }
 
+size_t lu_split_scratch_bytes(int batch, int n);
+int lu_update_split64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int p0, void* scratch, int32_t* info);
+
+// FP64 LU: 64-column panels (clusters, else one CTA per matrix), their row swaps and U blocks, and the
+// trailing update: split into digits on the tensor cores (lu_split.cu), or on the FP64 pipe for matrices
+// of at most two panels and where the digits do not fit memory.
 int lu_factor64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info) {
-  return lu_factor_simt<double>(c, reinterpret_cast<Cx<double>*>(A), batch, n, ld, bstride, piv, info, 32);
+  Cx<double>* M = reinterpret_cast<Cx<double>*>(A);
+  const bool split = info && n > 128 && ensure_buf(c, c->work6, lu_split_scratch_bytes(batch, n)) == BIE_OK;
+  for (int p0 = 0; p0 < n; p0 += 64) {
+    const int w = std::min(64, n - p0);
+    bool used = false;
+    BIE_TRY(panel_cluster<double>(c, M, batch, n, ld, bstride, p0, w, piv, info, &used));
+    if (!used) BIE_TRY(panel_factor<double>(c, M, batch, n, ld, bstride, p0, w, piv, info));
+    dim3 gs((unsigned)((n + 127) / 128), batch);
+    BIE_LAUNCH(k_swap_trsm<double><<<gs, 128, 0, c->stream>>>(M, bstride, n, ld, p0, w, piv, 0, p0 + w, 1));
+    const int rem = n - p0 - w;
+    if (rem > 0) {
+      BIE_TRY((set_smem_max(k_trsm64d)));
+      BIE_LAUNCH(k_trsm64d<<<dim3((unsigned)((rem + 31) / 32), batch), 128, kTrsm64dSmem, c->stream>>>(M, bstride, n, ld, p0,
+                                                                                                     p0 + w, n));
+      if (split) {
+        BIE_TRY(lu_update_split64(c, A, batch, n, ld, bstride, p0, c->work6.p, info));
+        continue;
+      }
+      dim3 gg((unsigned)((rem + 63) / 64), (unsigned)((rem + 63) / 64), batch);
+      BIE_LAUNCH(k_gemm_update<double><<<gg, 256, 0, c->stream>>>(M, bstride, n, ld, p0, w));
+    }
+  }
+  BIE_CUDA_TRY(cudaGetLastError());
+  return BIE_OK;
 }
+
+__global__ void k_piv_to_perm(const int32_t* __restrict__ piv, int n, int32_t* __restrict__ perm);
+
 int lu_solve64(bie_ctx* c, const cd* LU, int batch, int n, int ld, int64_t bstride, const int32_t* piv, cd* b,
                int64_t bstride_b) {
-  BIE_LAUNCH(k_lu_solve<double, double><<<batch, 256, 0, c->stream>>>(reinterpret_cast<const Cx<double>*>(LU), bstride, n, ld,
-                                                           piv, reinterpret_cast<Cx<double>*>(b), bstride_b));
+  const Cx<double>* M = reinterpret_cast<const Cx<double>*>(LU);
+  Cx<double>* rhs = reinterpret_cast<Cx<double>*>(b);
+  if ((size_t)n * sizeof(int32_t) > 200 * 1024) {  // the permutation is formed in shared memory
+    BIE_LAUNCH(k_lu_solve<double, double><<<batch, 256, 0, c->stream>>>(M, bstride, n, ld, piv, rhs, bstride_b));
+    BIE_CUDA_TRY(cudaGetLastError());
+    return BIE_OK;
+  }
+  const size_t ysz = (size_t)batch * n * sizeof(Cx<double>);
+  BIE_TRY(ensure_buf(c, c->work6, ysz + (size_t)batch * n * sizeof(int32_t)));
+  Cx<double>* y = (Cx<double>*)c->work6.p;
+  int32_t* perm = (int32_t*)((char*)c->work6.p + ysz);
+  BIE_TRY((set_smem_max(k_piv_to_perm)));
+  BIE_LAUNCH(k_piv_to_perm<<<batch, 256, (size_t)n * sizeof(int32_t), c->stream>>>(piv, n, perm));
+  const dim3 gv((unsigned)((n + 255) / 256), batch);
+  BIE_LAUNCH(k_gather_perm<<<gv, 256, 0, c->stream>>>(rhs, bstride_b, n, perm, y));
+  const size_t smem = (64 * 65 + 64) * sizeof(Cx<double>);
+  BIE_TRY((set_smem_max(k_solve_block<true>)));
+  BIE_TRY((set_smem_max(k_solve_block<false>)));
+  const int nblk = (n + 63) / 64;
+  for (int pass = 0; pass < 2; ++pass)
+    for (int bi = 0; bi < nblk; ++bi) {
+      const int j0 = (pass == 0 ? bi : nblk - 1 - bi) * 64;
+      if (pass == 0) BIE_LAUNCH(k_solve_block<true><<<batch, 256, smem, c->stream>>>(M, bstride, n, ld, j0, y));
+      else BIE_LAUNCH(k_solve_block<false><<<batch, 256, smem, c->stream>>>(M, bstride, n, ld, j0, y));
+      const int rlo = pass == 0 ? j0 + 64 : 0, rhi = pass == 0 ? n : j0;
+      if (rhi > rlo)
+        BIE_LAUNCH(k_solve_rows<<<dim3((unsigned)((rhi - rlo + 7) / 8), batch), 256, 0, c->stream>>>(M, bstride, n, ld, j0,
+                                                                                                  rlo, rhi, y));
+    }
+  BIE_LAUNCH(k_copy_back<<<gv, 256, 0, c->stream>>>(y, n, rhs, bstride_b));
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
 }
