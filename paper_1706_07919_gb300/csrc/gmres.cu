@@ -10,10 +10,9 @@
 
 namespace bie {
 
-__global__ void k_trsv_lu(const cf* __restrict__ LU, int n, int64_t ld, int64_t bstride, const int32_t* __restrict__ perm,
-                          const cd* __restrict__ rhs, cd* __restrict__ out, int accumulate,
-                          const RefineState* __restrict__ st, const int32_t* __restrict__ sel, int64_t rstride,
-                          int64_t roff, int64_t ostride, int64_t ooff, const cf* __restrict__ Dinv, int64_t dstride);
+int trsv_launch(bie_ctx* c, const cf* LU, int nk, int n, int64_t ld, int64_t bstride, const int32_t* perm, const cd* rhs,
+                cd* out, int accumulate, const RefineState* st, const int32_t* sel, int64_t rstride, int64_t roff,
+                int64_t ostride, int64_t ooff, const cf* D, int64_t dstride);
 int64_t diag_inv_stride(int n);
 int residual_ff(bie_ctx* c, const cf* A, int n, int64_t ld, int64_t bstride, int nk, const cd* b, const cd* x, cd* r,
                 double* rowabs, const RefineState* st);
@@ -268,7 +267,6 @@ int gmres_solve(bie_ctx* c, const cf* A, int nk, int n, int64_t ld, int64_t bstr
   BIE_CUDA_TRY(cudaMemsetAsync(gs, 0, nk * sizeof(GmresState), c->stream));
   const size_t sm_trsv = (size_t)n * sizeof(cf), sm_mv = (size_t)n * sizeof(float2);
   if (sm_trsv > 200 * 1024) return fail(BIE_ERR_INVALID_ARG, "N too large for the shared-memory Krylov kernels");
-  BIE_TRY((set_smem_max(k_trsv_lu)));
   BIE_TRY((set_smem_max(k_gm_matvec)));
   dim3 gr((unsigned)((n + 15) / 16), nk);
   for (int cy = 0; cy <= cycles; ++cy) {
@@ -278,9 +276,8 @@ int gmres_solve(bie_ctx* c, const cf* A, int nk, int n, int64_t ld, int64_t bstr
     BIE_LAUNCH(k_gm_start<<<nk, 1024, 0, c->stream>>>(n, m, r, V, g, gs, rs, gate, tol));
     for (int j = 0; j < m; ++j) {
       // z_j = M^{-1} v_j
-      BIE_LAUNCH(k_trsv_lu<<<nk, 1024, sm_trsv, c->stream>>>(LU, n, ld, lu_bstride, perm, V, Z, 0, gate, sel,
-                                                             (int64_t)(m + 1) * n, (int64_t)j * n, (int64_t)m * n,
-                                                             (int64_t)j * n, Dinv, dstride));
+      BIE_TRY(trsv_launch(c, LU, nk, n, ld, lu_bstride, perm, V, Z, 0, gate, sel, (int64_t)(m + 1) * n, (int64_t)j * n,
+                          (int64_t)m * n, (int64_t)j * n, Dinv, dstride));
       BIE_LAUNCH(k_gm_matvec<<<gr, 512, sm_mv, c->stream>>>(A, n, ld, bstride, Z, V, m, j, gate));
       BIE_LAUNCH(k_gm_arnoldi<<<nk, 1024, 0, c->stream>>>(n, m, j, V, H, cs, sn, g, gs, gate, inner_tol));
     }

@@ -229,6 +229,262 @@ __global__ void __launch_bounds__(1024) k_trsv_lu(const cf* __restrict__ LU, int
   }
 }
 
+// ---- the same sweep by a thread-block cluster per system ---------------------------------------
+// The cl CTAs of a cluster own the 64-row blocks of a system in turn (block b: CTA b mod cl), each its
+// rows of y in its shared memory.  Per block the owner applies the diagonal block's inverse and stores
+// the solved entries into every CTA's shared memory; one cluster barrier later every CTA subtracts
+// their products from its later rows.  The owner of the next block takes that block first, applies its
+// inverse and arrives at the next barrier before its other rows, the others arrive at once: the rows'
+// products overlap the next block's way through the cluster.  Three buffers: entries of block b + 3 are
+// stored after every CTA has arrived at b + 2's barrier, that is, after its products with block b.
+// Factor entries needed right after a barrier are loaded before it.  Every product and sum is
+// k_trsv_lu's, in its order.
+// Bound: the latency of a block on its way through the cluster, or the factor's bytes.  Measured, the
+// refinement phase with 16 / 8 / 4 / 2 CTAs a system and with one (k_trsv_lu): 4 systems of N = 2884 2.31 / 2.82 /
+// 3.98 / 6.30 / 7.75 ms, 28 of N = 2562 5.99 / 5.07 / 4.94 / 6.81 / 8.05, 24 of N = 1002 1.93 / 1.41 / 1.27 / 1.60 /
+// 1.85, 64 of N = 2884 16.0 / 13.2 / 11.1 / 11.4 / 12.9, 256 of them 64 / 52 / 46 / 47 / 44.
+namespace trc {
+constexpr int NT = 512, NW = NT / 32;
+__device__ __forceinline__ void arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void st_remote(uint32_t a, uint32_t rank, cf v) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(r), "f"(v.re), "f"(v.im) : "memory");
+}
+
+// Factor entries of 8 rows r0.. (up to rhi) for this lane's two columns c0, c0 + 1 (< j1).
+__device__ __forceinline__ void load8(const cf* __restrict__ M, int64_t ld, int r0, int rhi, int c0, int j1, float4* v) {
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r0 + u < rhi) {
+      const cf* p = M + (int64_t)(r0 + u) * ld + c0;
+      if (c0 + 1 < j1) v[u] = *reinterpret_cast<const float4*>(p);
+      else if (c0 < j1) v[u] = make_float4(p[0].re, p[0].im, 0.f, 0.f);
+    }
+  }
+}
+// y[r0 + u] -= v[u] . (ya, yb) over the warp's lanes (halving exchanges, see trsv_sweep)
+__device__ __forceinline__ void sub8(const float4* v, cf ya, cf yb, int r0, int rhi, cf* y) {
+  const int lane = threadIdx.x & 31;
+  float t[16];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    t[2 * u] = v[u].x * ya.re - v[u].y * ya.im + v[u].z * yb.re - v[u].w * yb.im;
+    t[2 * u + 1] = v[u].x * ya.im + v[u].y * ya.re + v[u].z * yb.im + v[u].w * yb.re;
+  }
+#pragma unroll
+  for (int h = 8; h >= 1; h >>= 1) {
+    const bool up = (lane & (2 * h)) != 0;
+#pragma unroll
+    for (int j = 0; j < h; ++j) {
+      const float send = up ? t[j] : t[j + h];
+      const float keep = up ? t[j + h] : t[j];
+      t[j] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * h);
+    }
+  }
+  t[0] += __shfl_xor_sync(0xffffffffu, t[0], 1);
+  if ((lane & 1) == 0) {
+    const int idx = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
+    const int r = r0 + (idx >> 1);
+    if (r < rhi) {
+      if (idx & 1) y[r].im -= t[0];
+      else y[r].re -= t[0];
+    }
+  }
+}
+
+// y <- L^-1 y or U^-1 y for the n rows of a system (or of a diagonal range of it); y [n] holds this
+// CTA's blocks, xb [3][TB] the solved entries, ytmp [TB].  D: inverses of the diagonal blocks.
+template <bool LOWER>
+__device__ void sweep(const cf* __restrict__ M, int n, int64_t ld, cf* y, const cf* __restrict__ D, cf* xb, cf* ytmp,
+                      int cl, int rank) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nblk = (n + TB - 1) / TB;
+  const uint32_t xa = (uint32_t)__cvta_generic_to_shared(xb);
+  auto block = [&](int s) { return LOWER ? s : nblk - 1 - s; };
+  // rows of the inverse for this warp (rows warp, warp + NW, ...), two columns a lane
+  auto load_inv = [&](int blk, cf (*d)[2]) {
+    const cf* Db = D + ((int64_t)blk * 2 + (LOWER ? 0 : 1)) * TB * TB;
+    const int bs = min(TB, n - blk * TB);
+#pragma unroll
+    for (int i = 0; i < TB / NW; ++i)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int r = warp + i * NW, cc = lane + 32 * h;
+        d[i][h] = (r < bs && cc < bs) ? Db[r * TB + cc] : cf{0.f, 0.f};
+      }
+  };
+  // solves the owner's block, stores it here and into every CTA's buffer
+  auto solve = [&](int blk, int slot, const cf (*d)[2]) {
+    const int j0 = blk * TB, bs = min(TB, n - j0);
+#pragma unroll
+    for (int i = 0; i < TB / NW; ++i) {
+      const int r = warp + i * NW;
+      float sr = 0.f, si = 0.f;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int cc = lane + 32 * h;
+        if (cc < bs) {
+          const cf v = y[j0 + cc];
+          sr += d[i][h].re * v.re - d[i][h].im * v.im;
+          si += d[i][h].re * v.im + d[i][h].im * v.re;
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        sr += __shfl_xor_sync(0xffffffffu, sr, o);
+        si += __shfl_xor_sync(0xffffffffu, si, o);
+      }
+      if (lane == 0 && r < bs) ytmp[r] = {sr, si};
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < TB * cl; e += NT) {
+      const int t = e & (TB - 1), q = e / TB;
+      const cf v = t < bs ? ytmp[t] : cf{0.f, 0.f};
+      st_remote(xa + (uint32_t)((slot * TB + t) * sizeof(cf)), (uint32_t)q, v);
+      if (q == 0 && t < bs) y[j0 + t] = v;
+    }
+  };
+  cf inv[TB / NW][2];
+  if (block(0) % cl == rank) {
+    load_inv(block(0), inv);
+    solve(block(0), 0, inv);
+  }
+  arrive();
+  for (int s = 0; s < nblk; ++s) {
+    const int blk = block(s), j0 = blk * TB, j1 = min(j0 + TB, n), c0 = j0 + 2 * lane;
+    const int nb = s + 1 < nblk ? block(s + 1) : -1;
+    const bool next = nb >= 0 && nb % cl == rank;
+    // this CTA's other remaining blocks: first, first + cl, ... (count of them)
+    int first, count;
+    if (LOWER) {
+      first = blk + 1 + ((rank - (blk + 1)) % cl + cl) % cl;
+      count = first < nblk ? (nblk - 1 - first) / cl + 1 : 0;
+    } else {
+      first = rank;
+      count = first < blk ? (blk - 1 - first) / cl + 1 : 0;
+    }
+    // before the barrier: the next block's rows and inverse, or the first group of rows
+    float4 v[8];
+    const int g8 = count * 8;  // groups of eight rows; group g: block first + (g / 8) cl, rows 8 (g % 8)
+    if (next) {
+      load_inv(nb, inv);
+      if (warp < 8) load8(M, ld, nb * TB + warp * 8, min(n, nb * TB + TB), c0, j1, v);
+    } else if (warp < g8) {
+      const int b = first + (warp >> 3) * cl;
+      load8(M, ld, b * TB + (warp & 7) * 8, min(n, b * TB + TB), c0, j1, v);
+    }
+    wait();
+    __syncthreads();  // this CTA's products with the block before
+    const cf* x = xb + (s % 3) * TB;
+    const cf ya = x[2 * lane], yb = x[2 * lane + 1];  // (zero past the last row)
+    if (next) {
+      if (warp < 8) sub8(v, ya, yb, nb * TB + warp * 8, min(n, nb * TB + TB), y);
+      __syncthreads();
+      solve(nb, (s + 1) % 3, inv);
+    }
+    if (s + 1 < nblk) arrive();
+    for (int g = warp; g < g8; g += NW) {
+      const int b = first + (g >> 3) * cl;
+      if (next && b == nb) continue;
+      const int r0 = b * TB + (g & 7) * 8, rhi = min(n, b * TB + TB);
+      if (next || g != warp) load8(M, ld, r0, rhi, c0, j1, v);
+      sub8(v, ya, yb, r0, rhi, y);
+    }
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ void cluster_of(int& cl, int& rank) {
+  uint32_t a, b;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(a));
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(b));
+  cl = (int)a;
+  rank = (int)b;
+}
+}  // namespace trc
+
+// k_trsv_lu by clusters (Dinv given): grid nk * cl, cluster (cl), block 512, dynamic smem n cf.
+__global__ void __launch_bounds__(trc::NT) k_trsv_cluster(const cf* __restrict__ LU, int n, int64_t ld, int64_t bstride,
+                                                          const int32_t* __restrict__ perm, const cd* __restrict__ rhs,
+                                                          cd* __restrict__ out, int accumulate,
+                                                          const RefineState* __restrict__ st,
+                                                          const int32_t* __restrict__ sel, int64_t rstride, int64_t roff,
+                                                          int64_t ostride, int64_t ooff, const cf* __restrict__ Dinv,
+                                                          int64_t dstride) {
+  extern __shared__ cf yv[];
+  __shared__ cf ytmp[TB], xb[3 * TB];
+  __shared__ double s_scale;
+  int cl, rank;
+  trc::cluster_of(cl, rank);
+  const int kk = blockIdx.x / cl;
+  if (st && st[kk].done) return;  // the whole cluster
+  const int fk = sel ? sel[kk] : kk;
+  const cf* M = LU + (int64_t)fk * bstride;
+  const int32_t* pm = perm + (int64_t)fk * n;
+  const cd* r = rhs + (int64_t)kk * rstride + roff;
+  // scale the right-hand side to O(1) before rounding it to FP32
+  if (threadIdx.x == 0) s_scale = 0.0;
+  __syncthreads();
+  double mx = 0.0;
+  for (int i = threadIdx.x; i < n; i += trc::NT) mx = fmax(mx, fmax(fabs(r[i].re), fabs(r[i].im)));
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if ((threadIdx.x & 31) == 0) atomicMax((unsigned long long*)&s_scale, __double_as_longlong(mx));
+  __syncthreads();
+  const double sc = s_scale > 0.0 ? s_scale : 1.0;
+  for (int b = rank; b * TB < n; b += cl)
+    for (int i = b * TB + threadIdx.x; i < min(n, b * TB + TB); i += trc::NT) {
+      const cd v = r[pm[i]];
+      yv[i] = {(float)(v.re / sc), (float)(v.im / sc)};
+    }
+  __syncthreads();
+  trc::arrive();  // every CTA of the cluster runs before the first remote store
+  trc::wait();
+  const cf* Df = Dinv + (int64_t)fk * dstride;
+  trc::sweep<true>(M, n, ld, yv, Df, xb, ytmp, cl, rank);
+  trc::arrive();  // every CTA has read the last solved entries before the buffers are used again
+  trc::wait();
+  trc::sweep<false>(M, n, ld, yv, Df, xb, ytmp, cl, rank);
+  cd* o = out + (int64_t)kk * ostride + ooff;
+  for (int b = rank; b * TB < n; b += cl)
+    for (int i = b * TB + threadIdx.x; i < min(n, b * TB + TB); i += trc::NT) {
+      const cd v = {(double)yv[i].re * sc, (double)yv[i].im * sc};
+      o[i] = accumulate ? cadd(o[i], v) : v;
+    }
+  trc::arrive();  // no CTA leaves while another may still store into its shared memory
+  trc::wait();
+}
+
+// Launch of a cluster kernel of at most `cl` CTAs per system (8 where the device holds no larger cluster
+// of them: only clusters up to 8 are certain to fit).
+template <class... P, class... X>
+static int launch_cluster(bie_ctx* c, void (*f)(P...), int nk, int cl, size_t smem, X... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(nk * cl));
+  cfg.blockDim = dim3(trc::NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = c->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)cl;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  BIE_TRY(set_smem_max(f));
+  BIE_CUDA_TRY(cudaFuncSetAttribute((const void*)f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  if (cl > 8) {
+    int active = 0;
+    BIE_CUDA_TRY(cudaOccupancyMaxActiveClusters(&active, f, &cfg));
+    if (active < 1) {
+      cfg.gridDim = dim3((unsigned)(nk * 8));
+      at[0].val.clusterDim.x = 8;
+    }
+  }
+  count_launch();
+  BIE_CUDA_TRY(cudaLaunchKernelEx(&cfg, f, P(args)...));
+  return BIE_OK;
+}
+
 // ---- the same solves for a few large systems: diagonal super-blocks and wide products ---------
 // k_trsv_lu gives each system one CTA, whose bandwidth (about 180 GB/s) bounds a solve of a few
 // large systems (9 systems of N = 20 544: 9 of 152 SMs busy).  Here the factor is taken in
@@ -267,25 +523,32 @@ __global__ void __launch_bounds__(1024) k_trsv_begin(const int32_t* __restrict__
   }
 }
 
-// diagonal super-block [s0, s1) of system kk's L (LOWER) or U, in place on y; one CTA per system
+// diagonal super-block [s0, s1) of system kk's L (LOWER) or U, in place on y; a cluster per system
 template <bool LOWER>
-__global__ void __launch_bounds__(1024) k_trsv_super(const cf* __restrict__ LU, int n, int64_t ld, int64_t bstride,
-                                                     const RefineState* __restrict__ st,
-                                                     const int32_t* __restrict__ sel, cf* __restrict__ y, int s0,
-                                                     int s1, const cf* __restrict__ Dinv, int64_t dstride) {
+__global__ void __launch_bounds__(trc::NT) k_trsv_super(const cf* __restrict__ LU, int n, int64_t ld, int64_t bstride,
+                                                        const RefineState* __restrict__ st,
+                                                        const int32_t* __restrict__ sel, cf* __restrict__ y, int s0,
+                                                        int s1, const cf* __restrict__ Dinv, int64_t dstride) {
   __shared__ cf ys[kSuper];
-  __shared__ cf ytmp[TB];
-  const int kk = blockIdx.x;
-  if (st && st[kk].done) return;
+  __shared__ cf ytmp[TB], xb[3 * TB];
+  int cl, rank;
+  trc::cluster_of(cl, rank);
+  const int kk = blockIdx.x / cl;
+  if (st && st[kk].done) return;  // the whole cluster
   const int fk = sel ? sel[kk] : kk;
   const cf* M = LU + (int64_t)fk * bstride + (int64_t)s0 * ld + s0;
-  cf* yk = y + (int64_t)kk * n;
+  cf* yk = y + (int64_t)kk * n + s0;
   const int m = s1 - s0;
-  for (int i = threadIdx.x; i < m; i += blockDim.x) ys[i] = yk[s0 + i];
+  for (int b = rank; b * TB < m; b += cl)
+    for (int i = b * TB + threadIdx.x; i < min(m, b * TB + TB); i += trc::NT) ys[i] = yk[i];
   __syncthreads();
-  const cf* Df = Dinv ? Dinv + (int64_t)fk * dstride + (int64_t)(s0 / TB) * 2 * TB * TB : nullptr;
-  trsv_sweep<LOWER>(M, m, ld, ys, Df, ytmp);
-  for (int i = threadIdx.x; i < m; i += blockDim.x) yk[s0 + i] = ys[i];
+  trc::arrive();
+  trc::wait();
+  trc::sweep<LOWER>(M, m, ld, ys, Dinv + (int64_t)fk * dstride + (int64_t)(s0 / TB) * 2 * TB * TB, xb, ytmp, cl, rank);
+  for (int b = rank; b * TB < m; b += cl)
+    for (int i = b * TB + threadIdx.x; i < min(m, b * TB + TB); i += trc::NT) yk[i] = ys[i];
+  trc::arrive();
+  trc::wait();
 }
 
 // rows [r0, r1) of system kk: y[r] -= sum over c in [s0, s1) of F[r][c] y[c]; a warp takes 8 rows,
@@ -354,6 +617,28 @@ __global__ void k_trsv_end(const cf* __restrict__ y, const double* __restrict__ 
   o = accumulate ? cadd(o, w) : w;
 }
 
+// x (+)= (LU)^{-1} P rhs for nk systems by clusters, or one CTA per system (k_trsv_lu) without the
+// diagonal blocks' inverses or beyond the systems that two CTAs each would give every SM two of.
+int trsv_launch(bie_ctx* c, const cf* LU, int nk, int n, int64_t ld, int64_t bstride, const int32_t* perm, const cd* rhs,
+                cd* out, int accumulate, const RefineState* st, const int32_t* sel, int64_t rstride, int64_t roff,
+                int64_t ostride, int64_t ooff, const cf* D, int64_t dstride) {
+  int nsm = 0;
+  BIE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
+  // the most CTAs a system that two to an SM hold, not more than its blocks, four blocks each beyond one
+  // CTA to an SM
+  const int nblk = (n + TB - 1) / TB;
+  int cl = 16;
+  while (cl > 1 && (nk * cl > 2 * nsm || cl / 2 >= nblk || (nk * cl > nsm && 4 * cl > nblk))) cl >>= 1;
+  const size_t smem = (size_t)n * sizeof(cf);
+  if (D && cl > 1)
+    return launch_cluster(c, k_trsv_cluster, nk, cl, smem, LU, n, ld, bstride, perm, rhs, out, accumulate, st, sel, rstride,
+                          roff, ostride, ooff, D, dstride);
+  BIE_TRY((set_smem_max(k_trsv_lu)));
+  BIE_LAUNCH(k_trsv_lu<<<nk, 1024, smem, c->stream>>>(LU, n, ld, bstride, perm, rhs, out, accumulate, st, sel, rstride, roff,
+                                                      ostride, ooff, D, dstride));
+  return BIE_OK;
+}
+
 size_t trsv_scratch_bytes(int nk, int n) { return 256 + (size_t)nk * n * sizeof(cf) + (size_t)nk * sizeof(double); }
 
 // x (+)= (LU)^{-1} P rhs for nk systems (vectors [nk][n]; factor sel[kk] if sel); systems whose
@@ -366,18 +651,17 @@ int trsv_solve(bie_ctx* c, const cf* LU, int nk, int n, int64_t ld, int64_t bstr
   int nsm = 0;
   BIE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
   if (!scratch || !D || n < 4 * kSuper || 2 * nk > nsm) {
-    BIE_TRY((set_smem_max(k_trsv_lu)));
-    BIE_LAUNCH(k_trsv_lu<<<nk, 1024, (size_t)n * sizeof(cf), c->stream>>>(LU, n, ld, bstride, perm, rhs, out, accumulate,
-                                                                        st, sel, n, 0, n, 0, D, dstride));
-    return BIE_OK;
+    return trsv_launch(c, LU, nk, n, ld, bstride, perm, rhs, out, accumulate, st, sel, n, 0, n, 0, D, dstride);
   }
   double* scales = (double*)scratch;
   cf* y = (cf*)((char*)scratch + (((size_t)nk * sizeof(double) + 255) & ~(size_t)255));
   BIE_LAUNCH(k_trsv_begin<<<nk, 1024, 0, c->stream>>>(perm, rhs, n, st, sel, y, scales));
   const int ns = (n + kSuper - 1) / kSuper;
+  int cls = 8;  // (16 blocks of 64 rows in a super-block)
+  while (cls > 1 && nk * cls > 2 * nsm) cls >>= 1;
   for (int b = 0; b < ns; ++b) {  // L: super-blocks in order, then the rows below
     const int s0 = b * kSuper, s1 = std::min(n, s0 + kSuper);
-    BIE_LAUNCH(k_trsv_super<true><<<nk, 1024, 0, c->stream>>>(LU, n, ld, bstride, st, sel, y, s0, s1, D, dstride));
+    BIE_TRY(launch_cluster(c, k_trsv_super<true>, nk, cls, 0, LU, n, ld, bstride, st, sel, y, s0, s1, D, dstride));
     if (s1 < n) {
       dim3 g((unsigned)((n - s1 + 63) / 64), nk);
       BIE_LAUNCH(k_trsv_gemv<<<g, 256, 0, c->stream>>>(LU, n, ld, bstride, st, sel, y, s0, s1, s1, n));
@@ -385,7 +669,7 @@ int trsv_solve(bie_ctx* c, const cf* LU, int nk, int n, int64_t ld, int64_t bstr
   }
   for (int b = ns - 1; b >= 0; --b) {  // U: super-blocks in reverse, then the rows above
     const int s0 = b * kSuper, s1 = std::min(n, s0 + kSuper);
-    BIE_LAUNCH(k_trsv_super<false><<<nk, 1024, 0, c->stream>>>(LU, n, ld, bstride, st, sel, y, s0, s1, D, dstride));
+    BIE_TRY(launch_cluster(c, k_trsv_super<false>, nk, cls, 0, LU, n, ld, bstride, st, sel, y, s0, s1, D, dstride));
     if (s0 > 0) {
       dim3 g((unsigned)((s0 + 63) / 64), nk);
       BIE_LAUNCH(k_trsv_gemv<<<g, 256, 0, c->stream>>>(LU, n, ld, bstride, st, sel, y, s0, s1, 0, s0));
