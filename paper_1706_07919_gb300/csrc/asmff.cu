@@ -78,7 +78,7 @@ __device__ __forceinline__ void cis_ff(ff phi, const FFConst& K, ff& c, ff& s) {
   s = (q >= 2) ? ff_neg(b) : b;
 }
 
-// Same outputs and launch shape as k_asm32_bulk (rows per CTA x ASMF_W warps per row, colours
+// Elements of any conditions.  Same outputs and launch shape as k_asm32_bulk (rows per CTA x ASMF_W warps per row, colours
 // separated by block barriers), with a float-float row accumulator [rows][N] in shared memory, or
 // for large N (GROW) in the output rows of A themselves (each row belongs to one CTA; the elements
 // of a colour share no node, so the row's warps never touch the same entry between barriers),
@@ -236,6 +236,179 @@ __global__ void __launch_bounds__(256, 2) k_asmff_bulk(
   }
 }
 
+// ---- elements of one boundary condition ---------------------------------------------------------
+// 1 / a from the FP32 reciprocal square root of a^2 (as a head), corrected to second order
+__device__ __forceinline__ ff ffx_recip_of(ff a, float sq) {
+  const float y = rsqrtf(sq);
+  const float e = __fmaf_rn(-a.lo, y, __fmaf_rn(-a.hi, y, 1.0f));
+  return ff_fast_two_sum(y, __fmul_rn(y, __fmaf_rn(e, e, e)));
+}
+__device__ __forceinline__ ff ffx_dot3(const ff* a, ff x, ff y, ff z) {
+  return ff_add(ff_add(ff_mul(a[0], x), ff_mul(a[1], y)), ff_mul(a[2], z));
+}
+
+// k_asmff_bulk where every element carries one condition: of its two kernels (H hard, -Gm soft) one
+// enters the matrix, the other meets the known values at the quadrature points (kq), so that a point
+// takes 16 products into sums instead of 24 and 24 more per element.  A CTA of four warps takes a row;
+// two neighbouring lanes take an element, half of its points each, and then three of its nodes each.
+// Shared memory N float4, or (GROW) the row of A itself: beyond 4600 nodes fewer than three CTAs would
+// fit an SM.  Products and sums outside the six nodes' are renormalised: without (about 800 instructions a
+// point) 2884 nodes took 2.47 ms, but the error against FP64 doubled; as it is, it is k_asmff_bulk's.
+// Bound: FP32 instructions.  Measured, one wavenumber with its near pairs, k_asmff_bulk / here: 1002 nodes
+// 0.95 / 0.71 ms, 2884 nodes 3.95 / 3.11, 4842 nodes (rows in A here, two rows a CTA there) 16.6 / 7.9.
+template <bool GROW>
+__global__ void __launch_bounds__(128, 4) k_asmff_rows(
+    const double* __restrict__ nodes, const double* __restrict__ normals, const uint8_t* __restrict__ bc,
+    const int32_t* __restrict__ esort, int64_t N, int64_t E, int Q, const float4* __restrict__ qaos,
+    const double* __restrict__ qshape, const int32_t* __restrict__ color_off, int ncolors,
+    const double* __restrict__ kv, const float4* __restrict__ kq /* [nk][Q][E] */, cd* __restrict__ A,
+    cd* __restrict__ rowsum /* [nk][N][3] */, FFConst K) {
+  extern __shared__ float4 accf[];
+  __shared__ ff shp[64 * 6];
+  __shared__ double part[4][6];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = lane & 1;
+  const int kk = blockIdx.y;
+  if (kv[kk] < 0.0) return;  // an idle slot of a re-assembly round (stream-ordered solves)
+  const ff k = ff_from_double(kv[kk]);
+  const bool kzero = !(kv[kk] > 0.0);  // the zero-frequency term: f takes its limit nu_i.r
+  const ff kinv = ff_from_double(kzero ? 0.0 : 1.0 / kv[kk]);
+  const int64_t i = blockIdx.x;
+  cd* Arow = A + ((int64_t)kk * N + i) * N;
+  float4* row = GROW ? reinterpret_cast<float4*>(Arow) : accf;
+  for (int t = threadIdx.x; t < Q * 6; t += 128) shp[t] = ff_from_double(qshape[t]);
+  for (int64_t t = threadIdx.x; t < N; t += 128) row[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+  ff xi[3], nui[3];
+  for (int d = 0; d < 3; ++d) {
+    xi[d] = ff_from_double(nodes[3 * i + d]);
+    nui[d] = ff_from_double(normals[3 * i + d]);
+  }
+  const int qlo = h * Q / 2, qhi = (h + 1) * Q / 2;
+  kq += (int64_t)kk * Q * E;
+  ff rs[6];  // alpha, beta, right-hand side (re, im)
+#pragma unroll
+  for (int u = 0; u < 6; ++u) rs[u] = ff{0.f, 0.f};
+  for (int col = 0; col < ncolors; ++col) {
+    __syncthreads();  // the row's entries of the colour before
+    const int32_t cbeg = color_off[col], cend = color_off[col + 1];
+    for (int32_t t0 = cbeg + 16 * warp; t0 < cend; t0 += 64) {
+      const int32_t t = t0 + (lane >> 1);
+      bool act = t < cend;
+      int32_t el[6];
+#pragma unroll
+      for (int a = 0; a < 6; ++a) {
+        el[a] = act ? esort[a * E + t] : 0;
+        if (el[a] == i) act = false;  // near pair: the near kernel's
+      }
+      const bool hard = bc[el[0]] == 0;
+      ff er[6], ei[6];
+#pragma unroll
+      for (int a = 0; a < 6; ++a) er[a] = ei[a] = ff{0.f, 0.f};
+      for (int qq = qlo; act && qq < qhi; ++qq) {
+        const float4* qp = qaos + ((int64_t)qq * E + t) * 4;  // x hi, x lo, nu hi, w, nu lo, w lo
+        const float4 v0 = qp[0], v1 = qp[1], v2 = qp[2], v3 = qp[3];
+        const float4 k4 = kq[(int64_t)qq * E + t];
+        const ff nu[3] = {{v1.z, v2.z}, {v1.w, v2.w}, {v2.x, v3.x}};
+        const ff wj = {v2.y, v3.y};
+        const ff rx = ff_sub(ff{v0.x, v0.w}, xi[0]), ry = ff_sub(ff{v0.y, v1.x}, xi[1]),
+                 rz = ff_sub(ff{v0.z, v1.y}, xi[2]);
+        const ff R2 = ff_add(ff_add(ff_sqr(rx), ff_sqr(ry)), ff_sqr(rz));
+        const ff R = ff_sqrt(R2), invR = ffx_recip_of(R, R2.hi);
+        const ff kR = ff_mul(k, R);
+        ff c, s;
+        cis_ff(kR, K, c, s);
+        const ff rnu = ffx_dot3(nu, rx, ry, rz);
+        const ff nr = ffx_dot3(nui, rx, ry, rz);
+        const ff nn = ffx_dot3(nui, nu[0], nu[1], nu[2]);
+        // w J G = w J e^{ikR} / R;  w J dG/dnu = w J (r.nu) / R^3 (i kR - 1) e^{ikR}
+        const ff wi = ff_mul(wj, invR);
+        const ff wd = ff_mul(ff_mul(wi, rnu), ff_mul(invR, invR));
+        const ff Gr = ff_mul(c, wi), Gi = ff_mul(s, wi);
+        const ff dGr = ff_mul(ff_neg(ff_add(c, ff_mul(s, kR))), wd);
+        const ff dGi = ff_mul(ff_add(ff_mul(c, kR), ff_neg(s)), wd);
+        ff cg, sg;
+        cis_ff(ff_mul(k, nr), K, cg, sg);
+        const ff f = kzero ? nr : ff_mul(sg, kinv);
+        const ff dgm = ff_mul(ff_mul(k, sg), nn), dfm = ff_neg(ff_mul(cg, nn));  // -dg, -df
+        // row sums: w J [g dG - dg G], w J [f dG - df G]
+        ffx_mac(rs[0], cg, dGr);
+        ffx_mac(rs[0], dgm, Gr);
+        ffx_mac(rs[1], cg, dGi);
+        ffx_mac(rs[1], dgm, Gi);
+        ffx_mac(rs[2], f, dGr);
+        ffx_mac(rs[2], dfm, Gr);
+        ffx_mac(rs[3], f, dGi);
+        ffx_mac(rs[3], dfm, Gi);
+        // hard: A += H, b += Gm P'_known; soft: A -= Gm, b -= H P_known
+        const ff Er = hard ? dGr : ff_neg(Gr), Ei = hard ? dGi : ff_neg(Gi);
+        const ff Br = hard ? Gr : ff_neg(dGr), Bi = hard ? Gi : ff_neg(dGi);
+        const ff kr = {k4.x, k4.y}, ki = {k4.z, k4.w};
+        ffx_mac(rs[4], Br, kr);
+        ffx_mac(rs[4], ff_neg(Bi), ki);
+        ffx_mac(rs[5], Br, ki);
+        ffx_mac(rs[5], Bi, kr);
+#pragma unroll
+        for (int a = 0; a < 6; ++a) {
+          const ff sh = shp[qq * 6 + a];
+          ffx_mac_lazy(er[a], sh, Er);
+          ffx_mac_lazy(ei[a], sh, Ei);
+        }
+      }
+      // the lanes of an element exchange their halves: nodes 0..2 to the even one, 3..5 to the odd one
+      __syncwarp();
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        auto half = [&](const ff& lo, const ff& hi) {
+          const ff send = h ? lo : hi, keep = h ? hi : lo;
+          return ff_add(keep, ff{__shfl_xor_sync(0xffffffffu, send.hi, 1), __shfl_xor_sync(0xffffffffu, send.lo, 1)});
+        };
+        const ff sr = half(er[a], er[a + 3]), si = half(ei[a], ei[a + 3]);
+        if (act) {
+          const int32_t j = h ? el[a + 3] : el[a];
+          const float4 v = row[j];
+          const ff ar = ff_add(ff{v.x, v.y}, sr), ai = ff_add(ff{v.z, v.w}, si);
+          row[j] = make_float4(ar.hi, ar.lo, ai.hi, ai.lo);
+        }
+      }
+    }
+  }
+  // combine the lanes' and the warps' sums in FP64
+#pragma unroll
+  for (int u = 0; u < 6; ++u) {
+    double v = ff_to_double(rs[u]);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) part[warp][u] = v;
+  }
+  __syncthreads();
+  for (int64_t j = threadIdx.x; j < N; j += 128) {
+    const float4 v = row[j];
+    Arow[j] = {ff_to_double(ff{v.x, v.y}), ff_to_double(ff{v.z, v.w})};
+  }
+  if (threadIdx.x < 3) {
+    const int u = 2 * threadIdx.x;
+    rowsum[((int64_t)kk * N + i) * 3 + threadIdx.x] = {part[0][u] + part[1][u] + part[2][u] + part[3][u],
+                                                       part[0][u + 1] + part[1][u + 1] + part[2][u + 1] + part[3][u + 1]};
+  }
+}
+
+// known values at the quadrature points, sum_a N_a known, as float-float [nk][Q][E] (colour-sorted)
+__global__ void k_known_qff(const int32_t* __restrict__ esort, int64_t E, int Q, const double* __restrict__ qshape,
+                            const cd* __restrict__ known, int64_t N, float4* __restrict__ kq) {
+  const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (u >= E * Q) return;
+  const int64_t qq = u / E, t = u - qq * E;
+  const cd* kn = known + (int64_t)blockIdx.y * N;
+  double re = 0.0, im = 0.0;
+#pragma unroll
+  for (int a = 0; a < 6; ++a) {
+    const double w = qshape[qq * 6 + a];
+    const cd v = kn[esort[a * E + t]];
+    re += w * v.re;
+    im += w * v.im;
+  }
+  const ff r = ff_from_double(re), m = ff_from_double(im);
+  kq[(int64_t)blockIdx.y * E * Q + u] = make_float4(r.hi, r.lo, m.hi, m.lo);
+}
+
 static FFConst make_ffconst() {
   FFConst K;
   const double pio2 = 1.57079632679489661923132169163975144;
@@ -273,6 +446,7 @@ static FFConst make_ffconst() {
 }
 
 int ensure_mixed_tables(bie_ctx* c);
+bool uniform_conditions(bie_ctx* c);
 const float4* sorted_aos_ptr(bie_ctx* c);
 const int32_t* sorted_elems_ptr(bie_ctx* c);
 
@@ -289,6 +463,27 @@ __global__ void k_known_ff(const cd* __restrict__ known, int64_t n, float4* __re
 int assemble_ff_bulk(bie_ctx* c, const double* kv, int nk, cd* A, const cd* known, cd* rowsum) {
   const int64_t N = c->N;
   BIE_TRY(ensure_mixed_tables(c));
+  if (c->rule.Q > 64) return fail(BIE_ERR_INVALID_ARG, "standard rule too large");
+  static const FFConst K = make_ffconst();
+  if (uniform_conditions(c)) {
+    const int64_t E = c->E, EQ = E * c->rule.Q;
+    BIE_TRY(ensure_buf(c, c->work6, (size_t)nk * EQ * sizeof(float4)));
+    float4* kq = (float4*)c->work6.p;
+    BIE_LAUNCH(k_known_qff<<<dim3((unsigned)((EQ + 127) / 128), nk), 128, 0, c->stream>>>(
+        sorted_elems_ptr(c), E, c->rule.Q, c->qshape, known, N, kq));
+    const bool grow = (size_t)N * sizeof(float4) > 72 * 1024;
+    auto go = [&](auto kernel, size_t smem) -> int {
+      BIE_TRY(set_smem_max(kernel));
+      BIE_LAUNCH(kernel<<<dim3((unsigned)N, nk), 128, smem, c->stream>>>(
+          c->nodes, c->normals, c->bc, sorted_elems_ptr(c), N, E, c->rule.Q, sorted_aos_ptr(c), c->qshape, c->color_off,
+          c->ncolors, kv, kq, A, rowsum, K));
+      return BIE_OK;
+    };
+    if (grow) BIE_TRY(go(k_asmff_rows<true>, 0));
+    else BIE_TRY(go(k_asmff_rows<false>, (size_t)N * sizeof(float4)));
+    BIE_CUDA_TRY(cudaGetLastError());
+    return BIE_OK;
+  }
   BIE_TRY(ensure_buf(c, c->work6, (size_t)nk * N * sizeof(float4)));
   float4* knf = (float4*)c->work6.p;
   BIE_LAUNCH(k_known_ff<<<(unsigned)((nk * N + 255) / 256), 256, 0, c->stream>>>(known, nk * N, knf));
@@ -300,8 +495,6 @@ int assemble_ff_bulk(bie_ctx* c, const double* kv, int nk, cd* A, const cd* know
   const bool grow = (size_t)rows * N * sizeof(cd) > 200 * 1024;
   if (grow) rows = 4;
   const size_t smem = grow ? 0 : (size_t)rows * N * sizeof(cd);
-  if (c->rule.Q > 64) return fail(BIE_ERR_INVALID_ARG, "standard rule too large");
-  static const FFConst K = make_ffconst();
   dim3 gb((unsigned)((N + rows - 1) / rows), nk);
   if (grow) {
     BIE_LAUNCH(k_asmff_bulk<true, 1><<<gb, 32 * rows * ASMF_W, 0, c->stream>>>(
