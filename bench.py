@@ -641,7 +641,7 @@ def roofline_field(w, field_ms, M, Nk, variant, peaks):
     achieved = flops_per_eval * evals / (field_ms * 1e-3) / 1e12
     peak = peaks["ffma_tflops"]
     launches = (Nk + FIELD_BATCH - 1) // FIELD_BATCH
-    name = {1: "k_field32c<16,64,4,64>", 2: "k_field32c<16,128,3,32>"}.get(variant, "k_field32b")
+    name = {1: "k_field32c<16,64,4,64>", 2: "k_field_pair"}.get(variant, "k_field32b")
     return {"kernel": name + " (Eq. BRIEFdmn, float-float phases)", "bound": "alu",
             "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "traffic": FIELD_LAUNCH_DRAM_BYTES.get(variant), "traffic_unit": "bytes per launch",
@@ -894,7 +894,7 @@ def main():
     ap.add_argument("--lu-panel", type=int, default=64, help="panel width of the deferred LU update (64, 32)")
     ap.add_argument("--lu-tile", type=int, default=256, help="real columns of the LU update tile (256, 128)")
     ap.add_argument("--field-variant", type=int, default=2,
-                    help="mixed field kernel: 2 (128 points per CTA, 32-point tiles), 1 (64 points), 0 (k_field32b)")
+                    help="mixed field kernel: 2 (two groups of wavenumbers in packed arithmetic), 1 (k_field32c), 0 (k_field32b)")
     ap.add_argument("--asm-kb", type=int, default=2,
                     help="FP32 bulk assembly: wavenumbers per thread (2, 1) or 0 for the general kernel")
     ap.add_argument("--tc", type=int, default=3,
