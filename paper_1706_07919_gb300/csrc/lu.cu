@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(pcl::NT, 1) k_panel_cluster(Cx<S>* __restrict_
   Cx<S>* X = L + (size_t)lw * ch;                 // [2 LW][PW]: gathered rows (CTA 0)
   Cx<S>* Ub = X + 2 * LW * PW;                    // [LW][PW]: the leaf's U block
   __shared__ Rec<S> rec[2][MAXC];
-  __shared__ Cx<S> drow[2][LW];                   // row c's leaf entries
+  __shared__ alignas(16) Cx<S> drow[2][LW];       // row c's leaf entries (vector stores, as rec)
   __shared__ unsigned red_k[NT / 32], red_r[NT / 32];
   __shared__ int s_piv[LW], s_rows[2 * LW], s_src[2 * LW], s_m;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

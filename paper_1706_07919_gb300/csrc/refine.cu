@@ -413,7 +413,8 @@ __global__ void __launch_bounds__(trc::NT) k_trsv_cluster(const cf* __restrict__
                                                           int64_t ostride, int64_t ooff, const cf* __restrict__ Dinv,
                                                           int64_t dstride) {
   extern __shared__ cf yv[];
-  __shared__ cf ytmp[TB], xb[3 * TB];
+  __shared__ cf ytmp[TB];
+  __shared__ alignas(16) cf xb[3 * TB];  // (8-byte stores of a value, also from other CTAs)
   __shared__ double s_scale;
   int cl, rank;
   trc::cluster_of(cl, rank);
@@ -530,7 +531,8 @@ __global__ void __launch_bounds__(trc::NT) k_trsv_super(const cf* __restrict__ L
                                                         const int32_t* __restrict__ sel, cf* __restrict__ y, int s0,
                                                         int s1, const cf* __restrict__ Dinv, int64_t dstride) {
   __shared__ cf ys[kSuper];
-  __shared__ cf ytmp[TB], xb[3 * TB];
+  __shared__ cf ytmp[TB];
+  __shared__ alignas(16) cf xb[3 * TB];  // (8-byte stores of a value, also from other CTAs)
   int cl, rank;
   trc::cluster_of(cl, rank);
   const int kk = blockIdx.x / cl;
