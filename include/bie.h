@@ -265,6 +265,10 @@ int bie_set_incident_plane_wave(bie_ctx* ctx, const double* dir);
  *                          (default), 0: launch every kernel directly
  *   "mixed.phase_timing"   1: time the phases of each call with CUDA events (see
  *                          bie_get_phase_times; graphs are then not used), 0: off (default)
+ * FP64 factorisation:
+ *   "fp64.wait_polls"      polls of a bounded wait in its tensor-core update before the wait gives up
+ *                          and the call returns BIE_ERR_TIMEOUT (0..2^30, default 2^22: seconds; 0:
+ *                          every wait gives up at once)
  * Learned warm start and Krylov solve (BIE_MODE_LEARNED):
  *   "learned.stride"       every stride-th wavenumber of the call is an anchor (>= 2, default 8;
  *                          indices stride-1, 2 stride-1, ...; the last index if none)
@@ -303,7 +307,7 @@ int bie_assemble(bie_ctx* ctx, double k, void* A_out, void* b_out);
  *   rep      host bie_report [Nk] or NULL
  * Synchronises the stream before returning (the reports are read back).  Errors: INVALID_ARG,
  * STATE, OOM (scratch larger than free device memory), CUDA, TIMEOUT (a bounded wait of the
- * tensor-core factorisation gave up: that factor is void). */
+ * tensor-core factorisation gave up, in any mode and with or without rep: those factors are void). */
 int bie_solve_frequencies(bie_ctx* ctx, const double* k, int64_t Nk, int mode, void* surf_out,
                           bie_report* rep);
 

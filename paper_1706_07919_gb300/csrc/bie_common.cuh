@@ -177,6 +177,7 @@ struct bie_ctx {
   int mlp_epochs = 60;               // training epochs over the anchors' solutions
   int mlp_batch = 8192;              // rows per minibatch
   double mlp_lr = 2e-3, mlp_lr_min = 1e-4;  // Adam step size, cosine-decayed to lr_min
+  int64_t fp64_wait_polls = 1 << 22; // FP64 LU: polls of a bounded wait before it gives up
   int64_t mlp_seed = 1234;           // initial weights and minibatch order
   double mlp_kmax = 0.0;             // feature wavenumber scale (0: largest training wavenumber)
   int mlp_graph = 1;                 // replay training epochs from a captured CUDA graph

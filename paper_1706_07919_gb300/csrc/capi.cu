@@ -112,7 +112,7 @@ void build_quad_rule(QuadRule& r, int ng, int ng_near);
 int launch_foot_points(bie_ctx* c, const double* xp, int64_t M, int32_t* foot_elem, double* foot,
                        unsigned long long* first_inside);
 int assemble64(bie_ctx* c, const double* kv, int nk, cd* A, cd* b, void* scratch, bool ff_bulk);
-int lu_factor64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info);
+int lu_factor64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info, int32_t* err);
 int lu_solve64(bie_ctx* c, const cd* LU, int batch, int n, int ld, int64_t bstride, const int32_t* piv, cd* b,
                int64_t bstride_b);
 int field64(bie_ctx* c, const double* kv, int nk, const cd* surf, const double* xp, int64_t M,
@@ -213,6 +213,15 @@ __global__ void k_known64(const double* __restrict__ nodes, const double* __rest
                           const uint8_t* __restrict__ bc, int64_t N, const double* __restrict__ kv, double dx,
                           double dy, double dz, cd* __restrict__ known);
 
+// Waits for the stream; TIMEOUT if a bounded wait of the FP64 factorisations raised *err (device).
+int lu64_error(bie_ctx* c, const int32_t* err) {
+  int32_t e = 0;
+  BIE_CUDA_TRY(cudaMemcpyAsync(&e, err, sizeof(e), cudaMemcpyDeviceToHost, c->stream));
+  BIE_CUDA_TRY(cudaStreamSynchronize(c->stream));
+  if (e) return fail(BIE_ERR_TIMEOUT, "FP64 LU: a bounded wait in the tensor-core update gave up");
+  return BIE_OK;
+}
+
 // Several incident directions in FP64 (see solve_mixed): A and the known-column matrix B assembled
 // once per wavenumber, A factored once, b_d = -B known_d per direction.  surf_out [Nk][ndir][2][N].
 int solve_fp64_multi(bie_ctx* c, const double* k, int64_t Nk, const double* dirs, int ndir, cd* surf_out,
@@ -246,7 +255,9 @@ int solve_fp64_multi(bie_ctx* c, const double* k, int64_t Nk, const double* dirs
   double* rowabs = (double*)(known + kb * N);
   int32_t* piv = (int32_t*)(rowabs + kb * N);
   int32_t* info = piv + kb * N;
-  char* stp = (char*)(((uintptr_t)(info + kb) + 15) & ~(uintptr_t)15);
+  int32_t* err = info + kb;
+  char* stp = (char*)(((uintptr_t)(err + 1) + 15) & ~(uintptr_t)15);
+  BIE_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int32_t), c->stream));
   void* state = stp;
   double* kdev = (double*)(stp + kb * st_bytes);
   std::vector<int32_t> hinfo(kb);
@@ -261,7 +272,7 @@ int solve_fp64_multi(bie_ctx* c, const double* k, int64_t Nk, const double* dirs
     c->bc = bc_real;
     BIE_TRY(rc);
     BIE_TRY(assemble64(c, kdev, nk, A, b, scratch, false));
-    BIE_TRY(lu_factor64(c, A, nk, (int)N, (int)N, N * N, piv, info));
+    BIE_TRY(lu_factor64(c, A, nk, (int)N, (int)N, N * N, piv, info, err));
     for (int d = 0; d < ndir; ++d) {
       set_dir(d);
       dim3 gk((unsigned)((N + 255) / 256), nk);
@@ -282,8 +293,7 @@ int solve_fp64_multi(bie_ctx* c, const double* k, int64_t Nk, const double* dirs
           rep[(k0 + i) * ndir + d] = bie_report{0, BIE_MODE_FP64, hinfo[i] ? BIE_FLAG_ZERO_PIVOT : 0u, 0, 0.0, 0.0};
     }
   }
-  BIE_CUDA_TRY(cudaStreamSynchronize(c->stream));
-  return BIE_OK;
+  return lu64_error(c, err);
 }
 
 int solve_fp64(bie_ctx* c, const double* k, int64_t Nk, cd* surf_out, bie_report* rep) {
@@ -300,14 +310,16 @@ int solve_fp64(bie_ctx* c, const double* k, int64_t Nk, cd* surf_out, bie_report
   cd* scratch = b + kb * N;  // known [kb][N], rowsum [kb][N][3]
   int32_t* piv = (int32_t*)(scratch + kb * N * 4);
   int32_t* info = piv + kb * N;
-  double* kdev = (double*)(((uintptr_t)(info + kb) + 15) & ~(uintptr_t)15);
+  int32_t* err = info + kb;
+  double* kdev = (double*)(((uintptr_t)(err + 1) + 15) & ~(uintptr_t)15);
+  BIE_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int32_t), c->stream));
   std::vector<int32_t> hinfo(kb);
   for (int64_t k0 = 0; k0 < Nk; k0 += kb) {
     const int nk = (int)std::min<int64_t>(kb, Nk - k0);
     BIE_CUDA_TRY(cudaMemcpyAsync(kdev, k + k0, nk * sizeof(double), cudaMemcpyHostToDevice, c->stream));
     BIE_CUDA_TRY(cudaMemsetAsync(info, 0, nk * sizeof(int32_t), c->stream));
     BIE_TRY(assemble64(c, kdev, nk, A, b, scratch, false));
-    BIE_TRY(lu_factor64(c, A, nk, (int)N, (int)N, N * N, piv, info));
+    BIE_TRY(lu_factor64(c, A, nk, (int)N, (int)N, N * N, piv, info, err));
     BIE_TRY(lu_solve64(c, A, nk, (int)N, (int)N, N * N, piv, b, N));
     dim3 g((unsigned)((N + 255) / 256), nk);
     BIE_LAUNCH(k_surface_fields<<<g, 256, 0, c->stream>>>(c->bc, N, b, scratch, surf_out + k0 * 2 * N, 2 * N));
@@ -320,8 +332,7 @@ int solve_fp64(bie_ctx* c, const double* k, int64_t Nk, cd* surf_out, bie_report
       }
     }
   }
-  BIE_CUDA_TRY(cudaStreamSynchronize(c->stream));
-  return BIE_OK;
+  return lu64_error(c, err);
 }
 
 }  // namespace bie
@@ -464,6 +475,9 @@ int bie_set_option(bie_ctx* c, const char* name, double value) {
   } else if (n == "learned.lr_min") {
     if (!(value >= 0.0) || value > 1.0) return fail(BIE_ERR_INVALID_ARG, "learned.lr_min must be in [0, 1]");
     c->mlp_lr_min = value;
+  } else if (n == "fp64.wait_polls") {
+    if (value < 0 || value > 1073741824.0) return fail(BIE_ERR_INVALID_ARG, "fp64.wait_polls must be in [0, 2^30]");
+    c->fp64_wait_polls = (int64_t)value;
   } else if (n == "learned.seed") {
     if (value < 0 || value > 9.0e15) return fail(BIE_ERR_INVALID_ARG, "learned.seed must be in [0, 9e15]");
     c->mlp_seed = (int64_t)value;

@@ -22,7 +22,8 @@ extern "C" int set_geometry_impl(bie_ctx* c, const double* nodes, int64_t N, con
 namespace bie {
 
 int assemble64(bie_ctx* c, const double* kv, int nk, cd* A, cd* b, void* scratch, bool ff_bulk);
-int lu_factor64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info);
+int lu_factor64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info, int32_t* err);
+int lu64_error(bie_ctx* c, const int32_t* err);
 int lu_solve64(bie_ctx* c, const cd* LU, int batch, int n, int ld, int64_t bstride, const int32_t* piv, cd* b,
                int64_t bstride_b);
 int rhs_from_known64(bie_ctx* c, const cd* B, int nk, int n, const cd* known, cd* zero, cd* b, double* rowabs,
@@ -139,7 +140,9 @@ int solve_fp64_linear(bie_ctx* c, const double* k, int64_t Nk, cd* surf_out, bie
   cd* known = bl + kb * Nl;
   int32_t* piv = (int32_t*)(known + kb * Nl);
   int32_t* info = piv + kb * Nl;
-  double* kdev = (double*)(((uintptr_t)(info + kb) + 15) & ~(uintptr_t)15);
+  int32_t* err = info + kb;
+  double* kdev = (double*)(((uintptr_t)(err + 1) + 15) & ~(uintptr_t)15);
+  BIE_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int32_t), c->stream));
   char* scratch = (char*)(kdev + kb);
   std::vector<int32_t> hinfo(kb);
   for (int64_t k0 = 0; k0 < Nk; k0 += kb) {
@@ -147,7 +150,7 @@ int solve_fp64_linear(bie_ctx* c, const double* k, int64_t Nk, cd* surf_out, bie
     BIE_CUDA_TRY(cudaMemcpyAsync(kdev, k + k0, nk * sizeof(double), cudaMemcpyHostToDevice, c->stream));
     BIE_CUDA_TRY(cudaMemsetAsync(info, 0, nk * sizeof(int32_t), c->stream));
     BIE_TRY(assemble_linear(c, kdev, nk, Al, bl, known, scratch));
-    BIE_TRY(lu_factor64(c, Al, nk, (int)Nl, (int)Nl, Nl * Nl, piv, info));
+    BIE_TRY(lu_factor64(c, Al, nk, (int)Nl, (int)Nl, Nl * Nl, piv, info, err));
     BIE_TRY(lu_solve64(c, Al, nk, (int)Nl, (int)Nl, Nl * Nl, piv, bl, Nl));
     dim3 g((unsigned)((Nl + 255) / 256), nk);
     BIE_LAUNCH(k_surface_fields<<<g, 256, 0, c->stream>>>(c->bc, Nl, bl, known, surf_out + k0 * 2 * Nl, 2 * Nl));
@@ -159,8 +162,7 @@ int solve_fp64_linear(bie_ctx* c, const double* k, int64_t Nk, cd* surf_out, bie
         rep[k0 + i] = bie_report{0, BIE_MODE_FP64, hinfo[i] ? BIE_FLAG_ZERO_PIVOT : 0u, 0, 0.0, 0.0};
     }
   }
-  BIE_CUDA_TRY(cudaStreamSynchronize(c->stream));
-  return BIE_OK;
+  return lu64_error(c, err);
 }
 
 // bie_assemble on linear elements: A_out [Nl][Nl], b_out [Nl].

@@ -1207,14 +1207,15 @@ int lu_trsm_rows32(bie_ctx* c, cf* A, int batch, int n, int ld, int64_t bstride,
 }
 
 size_t lu_split_scratch_bytes(int batch, int n);
-int lu_update_split64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int p0, void* scratch, int32_t* info);
+int lu_update_split64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int p0, void* scratch, int32_t* err);
 
 // FP64 LU: 64-column panels (clusters, else one CTA per matrix), their row swaps and U blocks, and the
 // trailing update: split into digits on the tensor cores (lu_split.cu), or on the FP64 pipe for matrices
-// of at most two panels and where the digits do not fit memory.
-int lu_factor64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info) {
+// of at most two panels and where the digits do not fit memory.  info: zero pivots, per system; *err
+// (device, cleared by the caller): a bounded wait gave up, every factor of the batch is void.
+int lu_factor64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info, int32_t* err) {
   Cx<double>* M = reinterpret_cast<Cx<double>*>(A);
-  const bool split = info && n > 128 && ensure_buf(c, c->work6, lu_split_scratch_bytes(batch, n)) == BIE_OK;
+  const bool split = n > 128 && ensure_buf(c, c->work6, lu_split_scratch_bytes(batch, n)) == BIE_OK;
   for (int p0 = 0; p0 < n; p0 += 64) {
     const int w = std::min(64, n - p0);
     bool used = false;
@@ -1228,7 +1229,7 @@ int lu_factor64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, in
       BIE_LAUNCH(k_trsm64d<<<dim3((unsigned)((rem + 31) / 32), batch), 128, kTrsm64dSmem, c->stream>>>(M, bstride, n, ld, p0,
                                                                                                      p0 + w, n));
       if (split) {
-        BIE_TRY(lu_update_split64(c, A, batch, n, ld, bstride, p0, c->work6.p, info));
+        BIE_TRY(lu_update_split64(c, A, batch, n, ld, bstride, p0, c->work6.p, err));
         continue;
       }
       dim3 gg((unsigned)((rem + 63) / 64), (unsigned)((rem + 63) / 64), batch);

@@ -146,19 +146,25 @@ __device__ __forceinline__ double int_to_double(int64_t v) {  // |v| < 2^51
 
 // Persistent: grid min(tiles, SMs), block NT.  Warp 0 loads the tile's digits by TMA, one K half at a time
 // (168 KB), warp 1 issues the MMAs, warps 2-5 combine and subtract; the next tile's first half loads while
-// the epilogue runs.  Every wait is bounded: a failed one raises a system's info flag and ends all roles.
+// the epilogue runs.  Every wait is bounded: one that gives up after `polls` polls raises *err and ends its
+// role, the other roles' waits then give up too, and the copies and MMAs in flight are waited for (with
+// tcx::mbar_wait's own limit) before the CTA ends.  A launch that finds *err raised does nothing.
 __global__ void __launch_bounds__(NT, 1) k_update_split(const __grid_constant__ CUtensorMap ma,
                                                         const __grid_constant__ CUtensorMap mb, double* __restrict__ A,
                                                         int64_t bstride, int ld, int r0, int m, int batch,
                                                         const int32_t* __restrict__ ea, const int32_t* __restrict__ eb,
-                                                        int32_t* __restrict__ info) {
+                                                        int32_t* err, uint32_t polls) {
   extern __shared__ unsigned char sm_raw[];
   __shared__ Bars bars;
+  __shared__ int s_void;
   const uint32_t base = (tcx::smem_u32(sm_raw) + 1023u) & ~1023u;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int tm = (m + BM - 1) / BM, tn = (2 * m + BN - 1) / BN, per = tm * tn, tiles = per * batch;
   const uint32_t full = tcx::smem_u32(&bars.full), empty = tcx::smem_u32(&bars.empty);
   const uint32_t accf = tcx::smem_u32(&bars.acc_full), acce = tcx::smem_u32(&bars.acc_empty);
+  if (tid == 0) s_void = *(volatile int32_t*)err;
+  __syncthreads();
+  if (s_void) return;  // an earlier update of this factorisation gave up
   if (warp == 0) tcx::tmem_alloc(&bars.tmem_slot, 512);
   if (tid == 0) {
     tcx::mbar_init(full, 1);
@@ -178,7 +184,7 @@ __global__ void __launch_bounds__(NT, 1) k_update_split(const __grid_constant__ 
         const int z = t / per, u = t - z * per, im = u % tm, in = u / tm;
         bool ok = true;
         for (int kc = 0; kc < 2 && ok; ++kc, ++it) {
-          if (it > 0) ok = tcx::mbar_wait(empty, (it - 1) & 1, info + z, 2);
+          if (it > 0) ok = tcx::mbar_wait(empty, (it - 1) & 1, err, 1, polls);
           if (!ok) break;
           tcx::mbar_expect_tx(full, SL * (A_SL + B_SL));
           for (int s = 0; s < SL; ++s) {
@@ -188,20 +194,19 @@ __global__ void __launch_bounds__(NT, 1) k_update_split(const __grid_constant__ 
         }
         if (!ok) break;
       }
-      if (it > 0) tcx::mbar_wait(full, (it - 1) & 1, info, 2);  // no copy is in flight when the CTA ends
+      if (it > 0) tcx::mbar_wait(full, (it - 1) & 1, err, 1);  // no copy is in flight when the CTA ends
     }
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t idesc = tcx::idesc_bf16(BM, BN);
       uint32_t it = 0, n = 0;
       for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++n) {
-        int32_t* flag = info + t / per;
         bool ok = true;
-        if (n > 0) ok = tcx::mbar_wait(acce, (n - 1) & 1, flag, 2);
+        if (n > 0) ok = tcx::mbar_wait(acce, (n - 1) & 1, err, 1, polls);
         if (!ok) break;
         tcx::fence_after();
         for (int kc = 0; kc < 2 && ok; ++kc, ++it) {
-          ok = tcx::mbar_wait(full, it & 1, flag, 2);
+          ok = tcx::mbar_wait(full, it & 1, err, 1, polls);
           if (!ok) break;
           tcx::fence_after();
           for (int d = 0; d < SL; ++d)
@@ -216,14 +221,15 @@ __global__ void __launch_bounds__(NT, 1) k_update_split(const __grid_constant__ 
         if (!ok) break;
         tcx::mma_commit(accf);
       }
-      if (it > 0) tcx::mbar_wait(empty, (it - 1) & 1, info, 2);  // nor an MMA
+      if (it > 0) tcx::mbar_wait(empty, (it - 1) & 1, err, 1);  // nor an MMA
+      if (n > 0) tcx::mbar_wait(accf, (n - 1) & 1, err, 1);     // nor the last tile's arrival
     }
   } else {
     const int wl = warp & 3;  // TMEM lanes 32 wl .. 32 wl + 31
     uint32_t n = 0;
     for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++n) {
       const int z = t / per, u = t - z * per, im = u % tm, in = u / tm;
-      const bool ok = __all_sync(0xffffffffu, tcx::mbar_wait(accf, n & 1, info + z, 2));
+      const bool ok = __all_sync(0xffffffffu, tcx::mbar_wait(accf, n & 1, err, 1, polls));
       if (!ok) break;
       tcx::fence_after();
       const int r = im * BM + wl * 32 + lane;
@@ -284,8 +290,9 @@ size_t lu_split_scratch_bytes(int batch, int n) {
   return batch * (m * split::SL * split::KR * 2 * 3 + 2 * m * sizeof(int32_t)) + 1024;
 }
 
-// A22 -= L21 U12 for the 64-column panel at p0 (FP64, all rows and columns past it).
-int lu_update_split64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int p0, void* scratch, int32_t* info) {
+// A22 -= L21 U12 for the 64-column panel at p0 (FP64, all rows and columns past it).  *err (device) is
+// raised if a bounded wait gave up: the factors of the whole batch are void.
+int lu_update_split64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int p0, void* scratch, int32_t* err) {
   using namespace split;
   const int r0 = p0 + 64, m = n - r0;
   if (m <= 0) return BIE_OK;
@@ -304,7 +311,7 @@ int lu_update_split64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstri
   const int64_t tiles = (int64_t)((m + BM - 1) / BM) * ((2 * m + BN - 1) / BN) * batch;
   BIE_TRY(set_smem_max(k_update_split));
   BIE_LAUNCH(k_update_split<<<(unsigned)std::min<int64_t>(tiles, nsm), NT, SMEM, c->stream>>>(
-      ma, mb, reinterpret_cast<double*>(A), bstride, ld, r0, m, batch, ea, eb, info));
+      ma, mb, reinterpret_cast<double*>(A), bstride, ld, r0, m, batch, ea, eb, err, (uint32_t)c->fp64_wait_polls));
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
 }
