@@ -1,20 +1,34 @@
 // lu_split.cu -- the FP64 LU's trailing update A22 -= L21 U12 (panels of 64 columns) on the tensor cores,
-// exact to FP64 rounding, by splitting the operands into 8-bit digits (the error-free splitting of
+// within FP64's own error bound, by splitting the operands into 8-bit digits (the error-free splitting of
 // Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix multiplication by using fast
 // routines of matrix multiplication", 2012, with integer digits):
 //   a row of L (a column of U) is scaled by a power of two 2^-e to below one, and x 2^(7-e) is cut into
-//   SL = 7 integer digits |d| <= 128, x = 2^(e-7) sum_s d_s 2^(-8 s) up to 2^-56 of the row's largest;
-//   digits are exact in BF16, products below 2^14, and the sums of one weight 2^(-8 (s + t)) -- up to
-//   7 digit pairs x 128 products -- stay below 2^24: exact in the tensor cores' FP32 accumulators.
-// Digit pairs with s + t < SL are kept (28 of 49): the dropped ones are below 2^-56 a product, under the
-// rounding 2^-53 of the FP64 products they replace.  The seven accumulators of an entry are combined
-// as 64-bit integers and enter A22 with one FP64 fused multiply-add each.
+//   SL = 9 integer digits |d| <= 128, x = 2^(e-7) sum_s d_s 2^(-8 s) up to 2^-72 of 2^e; the digits are
+//   held as d_s 2^(-8 s), exact in BF16.  The products of one weight s + t, at most 2^14 each in units of
+//   2^(-8 (s + t)), 128 of each of up to 8 pairs, add up to at most 2^24 units: exact in the tensor
+//   cores' FP32 accumulators.  Seven accumulators hold the weights 0 .. 6, the eighth (tensor memory holds
+//   no more) the weights 7 and 8, where what is below weight 7's units rounds off.
+// Digit pairs with s + t < SL are kept (45 of 81).  In units of the leading digits' product, the 128 real
+// products of an entry lose at most 2^-48 with the eight dropped pairs of weight 9 (the rest is smaller
+// by 2^-8), 2^-50 with the operands' remainders and 2^-49 in the eighth accumulator (an ulp at each of
+// its 120 instructions): below 2^-46 together.  That is a bound relative to the scales 2^er 2^ec of the
+// entry's row and column; FP64 arithmetic's is 128 x 2^-53 sum |l||u|.  It is no smaller where the sum is at
+// least one unit, that is, where some k has |l_ik| |u_kj| >= 2^-14 of the scales.  So a row carries for
+// each of its 64 entries whether it is within 2^-3, 2^-7, 2^-11 of the scale, a column 2^-11, 2^-7, 2^-3, and an
+// entry whose row and column have no bit in common (graded panels), or whose scales leave the exponents'
+// range or are not finite, takes its 64 products in FP64, by the lanes of the warp together.  Share of
+// such entries over spheres, two spheres and ellipsoids of 258 .. 2884 nodes: 0.03 % at the lowest
+// wavenumbers, 0 .. 1e-6 above (eight digits, whose bound asks for 2^-8, with one level, 2^-4 on both
+// sides: up to 3 %, and 18 ms more for the systems below).
+// The accumulators of an entry are combined as 64-bit integers and enter A22 with one FP64 fused
+// multiply-add.
 // The complex product is a real one on the interleaved storage (as in lu_tc.cu): C (m x 2n) -= L (m x
 // 128) B with B^T rows 2 c and 2 c + 1 = [ur, -ui], [ui, ur].
 // Bound: the FP64 pipe of the epilogue (four instructions an entry) and the MMAs (one tile of 128 x 64
-// reals at a time: seven accumulators fill the tensor memory).  Two systems of N = 2884: the updates
-// 189 ms on the FP64 pipe (0.67 of 1.1 TFLOP/s) -> 13.2 ms with the splitting (9.7 TFLOP/s of the
-// products it replaces); error of the solutions against 64 bits 8.3e-15 -> 7.9e-15.
+// reals at a time: eight accumulators fill the tensor memory).  Two systems of N = 2884: the
+// updates 189 ms on the FP64 pipe (0.67 of 1.1 TFLOP/s) -> 16.3 ms with the splitting (7.8 TFLOP/s of the
+// products it replaces); error of the solutions against 64 bits 9.0e-15 -> 8.7e-15.  Seven digits without
+// the bits measured 13.2 ms, but lost 2^g on panels graded by 2^g.
 #include "tcgen05.cuh"
 
 #include <algorithm>
@@ -22,14 +36,16 @@
 namespace bie {
 namespace split {
 
-constexpr int SL = 7;              // digits
+constexpr int SL = 9;              // digits
+constexpr int NACC = 8;            // accumulators
+constexpr int NL = 3;              // levels of the bits: 2^-(3 + 4 i) of a row's scale, 2^-(11 - 4 i) of a column's
 constexpr int KR = 128;            // reals along K (64 complex)
 constexpr int BM = 128, BN = 64;   // tile: rows x real columns
 constexpr int KCH = 64;            // BF16 per 128-byte swizzle row
 constexpr int A_SL = BM * 128, B_SL = BN * 128;  // bytes of one digit's chunk
 constexpr int SMEM = SL * (A_SL + B_SL) + 1024;
 constexpr int NT = 192;
-constexpr int kBadExp = 5000;      // exponent of a row or column that is not finite
+constexpr int kBadExp = 5000;      // exponent of a row or column that is not finite (or above 1e308)
 
 // Digits of t (|t| <= 128): d = rint(t), t <- 256 (t - d).
 __device__ __forceinline__ int next_digit(double& t) {
@@ -38,7 +54,8 @@ __device__ __forceinline__ int next_digit(double& t) {
   t = (t - (m - M)) * 256.0;
   return __double2loint(m);
 }
-__device__ __forceinline__ uint32_t bf16_of(int d) { return __float_as_uint((float)d) >> 16; }  // exact, |d| <= 256
+// d w in BF16: exact for |d| <= 256 and a power of two w
+__device__ __forceinline__ uint32_t bf16_of(int d, float w) { return __float_as_uint((float)d * w) >> 16; }
 // exponent e with |x| < 2^e for the largest magnitude x of a row
 __device__ __forceinline__ int exp_of(double x) {
   if (!(x < 1e308)) return kBadExp;  // too large, infinite or NaN
@@ -46,14 +63,23 @@ __device__ __forceinline__ int exp_of(double x) {
   const int e = ((__double2hiint(x) >> 20) & 0x7ff) - 1022;
   return e > -1000 ? e : -1000;  // (2^(7 - e) stays finite)
 }
+// the least magnitude that counts for a row's or column's bits of one level: 2^(e - level), anything in one of
+// zeros, nothing in one that is not finite
+__device__ __forceinline__ double near_of(int e, double mx, int level) {
+  return e == kBadExp ? INFINITY : mx > 0.0 ? __hiloint2double((1023 - level + e) << 20, 0) : 0.0;
+}
+__device__ __forceinline__ int row_level(int i) { return 3 + 4 * i; }
+__device__ __forceinline__ int col_level(int i) { return 11 - 4 * i; }
 __device__ __forceinline__ double scale_of(int e) {  // 2^(7 - e)
   return e == kBadExp ? 0.0 : __hiloint2double((1030 - e) << 20, 0);
 }
 
-// L rows r0 + r (r < m) of columns [p0, p0 + 64): digits as [z][s][m][128] BF16, exponents [z][m].
+// L rows r0 + r (r < m) of columns [p0, p0 + 64): digits as [z][s][m][128] BF16, exponents [z][m], bits of
+// the entries near the row's scale [z][m][NL].
 // One warp per row; grid (ceil(m / 8), batch), block 256.
 __global__ void __launch_bounds__(256) k_split_rows(const double2* __restrict__ A, int64_t bstride, int ld, int p0, int r0,
-                                                    int m, uint32_t* __restrict__ da, int32_t* __restrict__ ea) {
+                                                    int m, uint32_t* __restrict__ da, int32_t* __restrict__ ea,
+                                                    uint64_t* __restrict__ na) {
   const int lane = threadIdx.x & 31, r = blockIdx.x * 8 + (threadIdx.x >> 5), z = blockIdx.y;
   if (r >= m) return;
   const double2* row = A + (int64_t)z * bstride + (int64_t)(r0 + r) * ld + p0;
@@ -62,6 +88,13 @@ __global__ void __launch_bounds__(256) k_split_rows(const double2* __restrict__ 
   if (!(v[0].x - v[0].x == 0.0 && v[0].y - v[0].y == 0.0 && v[1].x - v[1].x == 0.0 && v[1].y - v[1].y == 0.0)) mx = INFINITY;
   for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   const int e = exp_of(mx);
+#pragma unroll
+  for (int i = 0; i < NL; ++i) {
+    const double lim = near_of(e, mx, row_level(i));
+    const unsigned b0 = __ballot_sync(0xffffffffu, fmax(fabs(v[0].x), fabs(v[0].y)) >= lim);
+    const unsigned b1 = __ballot_sync(0xffffffffu, fmax(fabs(v[1].x), fabs(v[1].y)) >= lim);
+    if (lane == 0) na[((int64_t)z * m + r) * NL + i] = e == kBadExp ? 0ull : ((uint64_t)b1 << 32) | b0;
+  }
   if (lane == 0) ea[(int64_t)z * m + r] = e;
   const double sc = scale_of(e);
 #pragma unroll
@@ -70,18 +103,22 @@ __global__ void __launch_bounds__(256) k_split_rows(const double2* __restrict__ 
     uint32_t* o = da + ((int64_t)z * SL * m + r) * (KR / 2) + lane + 32 * h;
 #pragma unroll
     for (int s = 0; s < SL; ++s) {
-      const uint32_t a = bf16_of(next_digit(x)), b = bf16_of(next_digit(y));
+      const float w = ldexpf(1.f, -8 * s);
+      const uint32_t a = bf16_of(next_digit(x), w), b = bf16_of(next_digit(y), w);
       o[(int64_t)s * m * (KR / 2)] = a | (b << 16);
     }
   }
 }
 
-// U columns c0 + c (c < m) of rows [p0, p0 + 64): digits of B^T as [z][s][2 m][128] BF16, exponents [z][m].
+// U columns c0 + c (c < m) of rows [p0, p0 + 64): digits of B^T as [z][s][2 m][128] BF16, exponents [z][m]
+// and bits [z][m][NL] as for the rows.
 // CTA: 32 columns (lanes) x 8 warps of 8 rows; grid (ceil(m / 32), batch), block 256.
 __global__ void __launch_bounds__(256) k_split_cols(const double2* __restrict__ A, int64_t bstride, int ld, int p0, int c0,
-                                                    int m, uint32_t* __restrict__ db, int32_t* __restrict__ eb) {
+                                                    int m, uint32_t* __restrict__ db, int32_t* __restrict__ eb,
+                                                    uint64_t* __restrict__ nb) {
   __shared__ uint32_t t[64][65];  // [2 c, 2 c + 1][k] pairs of one digit
   __shared__ double smx[8][32];
+  __shared__ uint8_t sbit[NL][8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, z = blockIdx.y, cb = blockIdx.x * 32;
   const int c = cb + lane;
   const bool act = c < m;
@@ -97,6 +134,20 @@ __global__ void __launch_bounds__(256) k_split_cols(const double2* __restrict__ 
   __syncthreads();
   for (int w = 0; w < 8; ++w) mx = fmax(mx, smx[w][lane]);
   const int e = exp_of(mx);
+#pragma unroll
+  for (int l = 0; l < NL; ++l) {
+    const double lim = near_of(e, mx, col_level(l));
+    unsigned bits = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) bits |= (unsigned)(fmax(fabs(v[i].x), fabs(v[i].y)) >= lim) << i;
+    sbit[l][warp][lane] = (uint8_t)bits;
+  }
+  __syncthreads();
+  if (warp < NL && act) {
+    uint64_t all = 0;
+    for (int w = 0; w < 8; ++w) all |= (uint64_t)sbit[warp][w][lane] << (8 * w);
+    nb[((int64_t)z * m + c) * NL + warp] = e == kBadExp ? 0ull : all;
+  }
   if (warp == 0 && act) eb[(int64_t)z * m + c] = e;
   const double sc = scale_of(e);
 #pragma unroll
@@ -105,12 +156,13 @@ __global__ void __launch_bounds__(256) k_split_cols(const double2* __restrict__ 
     v[i].y = e == kBadExp ? 0.0 : v[i].y * sc;
   }
   const int rows = min(64, 2 * (m - cb));
-  for (int s = 0; s < SL; ++s) {
+  float wt = 1.f;  // 2^(-8 s)
+  for (int s = 0; s < SL; ++s, wt *= 0.00390625f) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const uint32_t a = bf16_of(next_digit(v[i].x)), b = bf16_of(next_digit(v[i].y));
-      const uint32_t nb = b == 0u ? 0u : b ^ 0x8000u;
-      t[2 * lane][warp * 8 + i] = a | (nb << 16);
+      const uint32_t a = bf16_of(next_digit(v[i].x), wt), b = bf16_of(next_digit(v[i].y), wt);
+      const uint32_t minus = b == 0u ? 0u : b ^ 0x8000u;
+      t[2 * lane][warp * 8 + i] = a | (minus << 16);
       t[2 * lane + 1][warp * 8 + i] = b | (a << 16);
     }
     __syncthreads();
@@ -145,7 +197,7 @@ __device__ __forceinline__ double int_to_double(int64_t v) {  // |v| < 2^51
 }
 
 // Persistent: grid min(tiles, SMs), block NT.  Warp 0 loads the tile's digits by TMA, one K half at a time
-// (168 KB), warp 1 issues the MMAs, warps 2-5 combine and subtract; the next tile's first half loads while
+// (216 KB), warp 1 issues the MMAs, warps 2-5 combine and subtract; the next tile's first half loads while
 // the epilogue runs.  Every wait is bounded: one that gives up after `polls` polls raises *err and ends its
 // role, the other roles' waits then give up too, and the copies and MMAs in flight are waited for (with
 // tcx::mbar_wait's own limit) before the CTA ends.  A launch that finds *err raised does nothing.
@@ -153,6 +205,7 @@ __global__ void __launch_bounds__(NT, 1) k_update_split(const __grid_constant__ 
                                                         const __grid_constant__ CUtensorMap mb, double* __restrict__ A,
                                                         int64_t bstride, int ld, int r0, int m, int batch,
                                                         const int32_t* __restrict__ ea, const int32_t* __restrict__ eb,
+                                                        const uint64_t* __restrict__ na, const uint64_t* __restrict__ nb,
                                                         int32_t* err, uint32_t polls) {
   extern __shared__ unsigned char sm_raw[];
   __shared__ Bars bars;
@@ -214,7 +267,8 @@ __global__ void __launch_bounds__(NT, 1) k_update_split(const __grid_constant__ 
               const uint64_t da = tcx::desc_sw128(base + s * A_SL), db = tcx::desc_sw128(base + SL * A_SL + (d - s) * B_SL);
 #pragma unroll
               for (int k = 0; k < KCH / 16; ++k)  // 32 bytes along K: two descriptor units
-                tcx::mma_bf16(tmem + d * BN, da + 2 * k, db + 2 * k, idesc, (kc | s | k) ? 1u : 0u);
+                tcx::mma_bf16(tmem + min(d, NACC - 1) * BN, da + 2 * k, db + 2 * k, idesc,
+                              (kc | s | k) || d >= NACC ? 1u : 0u);
             }
           tcx::mma_commit(empty);
         }
@@ -234,42 +288,80 @@ __global__ void __launch_bounds__(NT, 1) k_update_split(const __grid_constant__ 
       tcx::fence_after();
       const int r = im * BM + wl * 32 + lane;
       const int er = r < m ? ea[(int64_t)z * m + r] : 0;
+      uint64_t near_row[NL], near_col[NL];
+      // the tile's 32 complex columns: exponent and bits, one a lane
+      const int cl = in * (BN / 2) + lane;
+      const int ec = cl < m ? eb[(int64_t)z * m + cl] : 0;
+#pragma unroll
+      for (int i = 0; i < NL; ++i) {
+        near_row[i] = r < m ? na[((int64_t)z * m + r) * NL + i] : 0ull;
+        near_col[i] = cl < m ? nb[((int64_t)z * m + cl) * NL + i] : 0ull;
+      }
       double* row = A + 2 * ((int64_t)z * bstride + (int64_t)(r0 + (r < m ? r : 0)) * ld + r0);
+      const double2* L = reinterpret_cast<const double2*>(A) + (int64_t)z * bstride + (int64_t)(r0 + im * BM + wl * 32) * ld + r0 - 64;
+      const double2* U = reinterpret_cast<const double2*>(A) + (int64_t)z * bstride + (int64_t)(r0 - 64) * ld + r0;
       const uint32_t taddr = tmem + ((uint32_t)(wl * 32) << 16);
 #pragma unroll 1
       for (int j0 = 0; j0 < BN; j0 += 8) {
-        uint32_t a[SL][8];
+        uint32_t a[NACC][8];
 #pragma unroll
-        for (int d = 0; d < SL; ++d) tmem_ld8(taddr + d * BN + j0, a[d]);
+        for (int d = 0; d < NACC; ++d) tmem_ld8(taddr + d * BN + j0, a[d]);
         const int c = in * BN + j0;  // real column (even)
         double2 v[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q)
           v[q] = (r < m && c + 2 * q < 2 * m) ? *reinterpret_cast<double2*>(row + c + 2 * q) : make_double2(0.0, 0.0);
 #pragma unroll
-        for (int d = 0; d < SL; ++d) tmem_wait8(a[d]);
+        for (int d = 0; d < NACC; ++d) tmem_wait8(a[d]);
+        unsigned slow = 0;  // of the four complex columns, those where this row takes its products in FP64
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          if (c + 2 * q >= 2 * m) break;
-          // 2^(er + ec - 62): the digits' weights; not finite where a row or a column is not
-          const int ex = 1023 + er + eb[(int64_t)z * m + (c >> 1) + q] - 62;
-          const int hi = ex >= 2047 ? 0x7ff80000 : ex <= 0 ? 0 : ex << 20;
-          const double sc = __hiloint2double(hi, 0);
+          const int cq = j0 / 2 + q;  // column of the tile
+          // 2^(er + ec - 70): the digits' weights
+          const int ex = 1023 + er + __shfl_sync(0xffffffffu, ec, cq) - 70;
+          uint64_t both = 0ull;
+#pragma unroll
+          for (int i = 0; i < NL; ++i) both |= near_row[i] & __shfl_sync(0xffffffffu, near_col[i], cq);
+          const bool digits = ex > 0 && ex < 2047 && both != 0ull;
+          if (r < m && c + 2 * q < 2 * m && !digits) slow |= 1u << q;
+          const double sc = digits ? __hiloint2double(ex << 20, 0) : 0.0;
           double x[2];
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             const int i = 2 * q + h;
-            auto iv = [&](int d) { return (int64_t)__float2int_rn(__uint_as_float(a[d][i])); };
-            const int64_t top = (iv(0) << 16) + (iv(1) << 8) + iv(2);
-            const int64_t low = (iv(3) << 24) + (iv(4) << 16) + (iv(5) << 8) + iv(6);
+            auto iv = [&](int d) { return (int64_t)__float2int_rn(__uint_as_float(a[d][i]) * ldexpf(1.f, 8 * d)); };
+            const int64_t top = (iv(0) << 24) + (iv(1) << 16) + (iv(2) << 8) + iv(3);
+            const int64_t low = (iv(4) << 24) + (iv(5) << 16) + (iv(6) << 8) + iv(7);
             x[h] = fma(int_to_double(top), 4294967296.0, int_to_double(low));
           }
-          if (r < m) {
-            v[q].x = fma(-x[0], sc, v[q].x);
-            v[q].y = fma(-x[1], sc, v[q].y);
-            *reinterpret_cast<double2*>(row + c + 2 * q) = v[q];
-          }
+          v[q].x = fma(-x[0], sc, v[q].x);
+          v[q].y = fma(-x[1], sc, v[q].y);
         }
+        if (__any_sync(0xffffffffu, slow != 0u)) {  // each such entry by the whole warp, two of its products a lane
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            for (unsigned todo = __ballot_sync(0xffffffffu, (slow >> q) & 1u); todo; todo &= todo - 1u) {
+              const int src = __ffs(todo) - 1;
+              double2 p = make_double2(0.0, 0.0);
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                const double2 l = L[(int64_t)src * ld + lane + 32 * h], w = U[(int64_t)(lane + 32 * h) * ld + (c >> 1) + q];
+                p.x = fma(l.x, w.x, fma(-l.y, w.y, p.x));
+                p.y = fma(l.x, w.y, fma(l.y, w.x, p.y));
+              }
+              for (int o = 16; o > 0; o >>= 1) {
+                p.x += __shfl_xor_sync(0xffffffffu, p.x, o);
+                p.y += __shfl_xor_sync(0xffffffffu, p.y, o);
+              }
+              if (lane == src) {
+                v[q].x -= p.x;
+                v[q].y -= p.y;
+              }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (r < m && c + 2 * q < 2 * m) *reinterpret_cast<double2*>(row + c + 2 * q) = v[q];
       }
       tcx::fence_before();
       __syncwarp();
@@ -287,7 +379,7 @@ __global__ void __launch_bounds__(NT, 1) k_update_split(const __grid_constant__ 
 // Scratch of lu_update_split64 for matrices of n rows.
 size_t lu_split_scratch_bytes(int batch, int n) {
   const size_t m = (size_t)std::max(0, n - 64);
-  return batch * (m * split::SL * split::KR * 2 * 3 + 2 * m * sizeof(int32_t)) + 1024;
+  return batch * (m * split::SL * split::KR * 2 * 3 + 2 * m * (sizeof(int32_t) + split::NL * sizeof(uint64_t))) + 1024;
 }
 
 // A22 -= L21 U12 for the 64-column panel at p0 (FP64, all rows and columns past it).  *err (device) is
@@ -298,11 +390,13 @@ int lu_update_split64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstri
   if (m <= 0) return BIE_OK;
   uint32_t* da = (uint32_t*)(((uintptr_t)scratch + 255) & ~(uintptr_t)255);
   uint32_t* db = da + (size_t)batch * SL * m * (KR / 2);
-  int32_t* ea = (int32_t*)(db + (size_t)batch * SL * 2 * m * (KR / 2));
+  uint64_t* na = (uint64_t*)(db + (size_t)batch * SL * 2 * m * (KR / 2));
+  uint64_t* nb = na + (size_t)batch * m * NL;
+  int32_t* ea = (int32_t*)(nb + (size_t)batch * m * NL);
   int32_t* eb = ea + (size_t)batch * m;
   const double2* M = reinterpret_cast<const double2*>(A);
-  BIE_LAUNCH(k_split_rows<<<dim3((unsigned)((m + 7) / 8), batch), 256, 0, c->stream>>>(M, bstride, ld, p0, r0, m, da, ea));
-  BIE_LAUNCH(k_split_cols<<<dim3((unsigned)((m + 31) / 32), batch), 256, 0, c->stream>>>(M, bstride, ld, p0, r0, m, db, eb));
+  BIE_LAUNCH(k_split_rows<<<dim3((unsigned)((m + 7) / 8), batch), 256, 0, c->stream>>>(M, bstride, ld, p0, r0, m, da, ea, na));
+  BIE_LAUNCH(k_split_cols<<<dim3((unsigned)((m + 31) / 32), batch), 256, 0, c->stream>>>(M, bstride, ld, p0, r0, m, db, eb, nb));
   CUtensorMap ma, mb;
   BIE_TRY(tcx::make_map_bf16_2d(&ma, da, KR, (uint64_t)batch * SL * m, KR, KCH, BM));
   BIE_TRY(tcx::make_map_bf16_2d(&mb, db, KR, (uint64_t)batch * SL * 2 * m, KR, KCH, BN));
@@ -311,7 +405,7 @@ int lu_update_split64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstri
   const int64_t tiles = (int64_t)((m + BM - 1) / BM) * ((2 * m + BN - 1) / BN) * batch;
   BIE_TRY(set_smem_max(k_update_split));
   BIE_LAUNCH(k_update_split<<<(unsigned)std::min<int64_t>(tiles, nsm), NT, SMEM, c->stream>>>(
-      ma, mb, reinterpret_cast<double*>(A), bstride, ld, r0, m, batch, ea, eb, err, (uint32_t)c->fp64_wait_polls));
+      ma, mb, reinterpret_cast<double*>(A), bstride, ld, r0, m, batch, ea, eb, na, nb, err, (uint32_t)c->fp64_wait_polls));
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
 }
