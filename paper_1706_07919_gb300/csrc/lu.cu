@@ -29,6 +29,18 @@ __device__ __forceinline__ void cx_msub(Cx<double>& a, Cx<double> l, Cx<double> 
   a.im = fma(-l.re, u.im, fma(-l.im, u.re, a.im));
 }
 
+// x / d from y = 1 / d: one correction of the rounded product by its residual (Markstein's division), the
+// quotient rounded once as by a division; plain division where the residual could leave FP64's range.
+__device__ __forceinline__ bool quotient_safe(double d) { return d >= 0x1p-900 && d <= 0x1p900; }
+__device__ __forceinline__ double quotient(double x, double d, double y, bool safe) {
+  if (!safe) return x / d;
+  const double q = x * y;
+  return fma(fma(-q, d, x), y, q);
+}
+__device__ __forceinline__ Cx<double> cx_div_by(Cx<double> a, Cx<double> b, double bb, double y, bool safe) {  // bb = |b|^2
+  return {quotient(fma(a.re, b.re, a.im * b.im), bb, y, safe), quotient(fma(a.im, b.re, -(a.re * b.im)), bb, y, safe)};
+}
+
 // ---- panel factorisation: one CTA per matrix, columns p0 .. p0+nb-1, rows p0 .. n-1 ----------
 template <class S>
 __global__ void __launch_bounds__(512) k_panel(Cx<S>* __restrict__ A, int64_t bstride, int n, int ld, int p0,
@@ -330,7 +342,7 @@ __global__ void __launch_bounds__(256) k_leaf_update(Cx<S>* __restrict__ A, int6
 }
 
 // ---- cluster panel: one panel of each matrix by a thread-block cluster ------------------------
-// The CTAs of a cluster (1, 2, 4, 8 or 16) share a matrix: CTA j holds rows [p0 + j ch, p0 + (j + 1) ch)
+// The CTAs of a cluster (up to 16) share a matrix: CTA j holds rows [p0 + j ch, p0 + (j + 1) ch)
 // of a leaf of up to 16 columns in shared memory, column by column.  Per column each CTA finds its best
 // candidate row (largest modulus, lowest row on ties) during the rank-1 update of the column before,
 // one warp stores the candidate and its leaf entries (the holder of row c also row c's) into every
@@ -346,27 +358,43 @@ __global__ void __launch_bounds__(256) k_leaf_update(Cx<S>* __restrict__ A, int6
 // Bound: the latency of a column (a CTA barrier, the remote stores, a cluster barrier); in FP64 the
 // rows' FP64 instructions.  N = 2884, two systems in FP64: 72.6 ms of one-CTA leaves and their updates ->
 // 19.9 ms, the panels' other columns updated over all SMs (29.3 ms inside the cluster).
-// Every entry goes through the operations of the one-CTA leaf (k_leaf) in its order, so that the
-// pivots and, for panels of up to 1536 rows (leaf, where that kernel takes 16 columns), the factor are
-// the same bit for bit whatever the cluster; sum_first: A -= (sum of L U), as k_leaf_update forms it
+// The pivots and the factor do not depend on the cluster.  In FP32 every entry goes through the operations of
+// the one-CTA leaf (k_leaf) in its order, so that for panels of up to 1536 rows (leaf, where that kernel
+// takes 16 columns) the factor is its bit for bit; in FP64 the pivots are chosen as there, the products
+// fused.  sum_first: A -= (sum of L U), as k_leaf_update forms it
 // for small batches, instead of product by product.  (Taller panels of small batches fix the other
 // order of the U block's fused products, leaf 0.)  The refinement's result moves by up to 1e-9 with
 // the factor's rounding: which of the forms a panel takes depends on the batch, the rows and the
 // number of SMs alone (panel_cluster), not on the cluster.
-// The key of a candidate is |a|^2's leading 32 bits (FP32: all of them), 0 for none.
+// The key of a candidate is |a|^2's bits plus one, 0 for none.  In FP64 the record also carries 1 / |a|^2, formed
+// by the candidate's warp alone (every warp of every CTA would take the division's FP64 instructions
+// otherwise); the quotients take one correction each and round once.  Two FP64 solves of N = 2884 in all:
+// 72.1 ms with the keys' upper halves alone and 1 / |a|^2 by every warp, 69.0 this way.
 namespace pcl {
 constexpr int NT = 512, LW = 16, PW = 64, MAXC = 16;
-template <class S> struct alignas(16) Rec {
+template <class S> struct alignas(16) RecHead {
   unsigned long long head;  // key << 32 | row
-  unsigned long long pad;
-  Cx<S> v[LW];              // the candidate's leaf entries
+};
+template <> struct alignas(16) RecHead<double> {
+  unsigned long long head, row;  // key; row
+  double inv, mag;               // 1 / |a|^2, |a|^2
+};
+template <class S> struct alignas(16) Rec : RecHead<S> {
+  alignas(16) Cx<S> v[LW];  // the candidate's leaf entries
 };
 template <class S> __host__ __device__ constexpr size_t smem_bytes(int lw, int ch) {
   // leaf, gathered rows of the other columns (32 x 64), U block (16 x 64)
   return ((size_t)lw * ch + 2 * LW * PW + LW * PW) * sizeof(Cx<S>);
 }
 __device__ __forceinline__ unsigned key_of(float m) { return __float_as_uint(m) + 1u; }
-__device__ __forceinline__ unsigned key_of(double m) { return (unsigned)__double2hiint(m) + 1u; }
+__device__ __forceinline__ unsigned long long key_of(double m) { return (unsigned long long)__double_as_longlong(m) + 1ull; }
+__device__ __forceinline__ unsigned warp_max(unsigned k) { return __reduce_max_sync(0xffffffffu, k); }
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long k) {
+  const unsigned hi = (unsigned)(k >> 32), H = __reduce_max_sync(0xffffffffu, hi);
+  return ((unsigned long long)H << 32) | __reduce_max_sync(0xffffffffu, hi == H ? (unsigned)k : 0u);
+}
+template <class S> struct KeyOf { typedef unsigned type; };
+template <> struct KeyOf<double> { typedef unsigned long long type; };
 __device__ __forceinline__ uint32_t mapa(uint32_t a, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
@@ -406,7 +434,10 @@ __global__ void __launch_bounds__(pcl::NT, 1) k_panel_cluster(Cx<S>* __restrict_
   Cx<S>* Ub = X + 2 * LW * PW;                    // [LW][PW]: the leaf's U block
   __shared__ Rec<S> rec[2][MAXC];
   __shared__ alignas(16) Cx<S> drow[2][LW];       // row c's leaf entries (vector stores, as rec)
-  __shared__ unsigned red_k[NT / 32], red_r[NT / 32];
+  typedef typename KeyOf<S>::type Key;
+  constexpr bool F64 = sizeof(S) == 8;
+  __shared__ Key red_k[NT / 32];
+  __shared__ unsigned red_r[NT / 32];
   __shared__ int s_piv[LW], s_rows[2 * LW], s_src[2 * LW], s_m;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t cl, rank;
@@ -440,49 +471,70 @@ __global__ void __launch_bounds__(pcl::NT, 1) k_panel_cluster(Cx<S>* __restrict_
     for (int cc = 0; cc < l; ++cc) {
       const int c = c0 + cc, buf = c & 1;
       {
-        const unsigned k = bi < n ? key_of(best) : 0u;
-        const unsigned K = __reduce_max_sync(0xffffffffu, k);
+        const Key k = bi < n ? key_of(best) : (Key)0;
+        const Key K = warp_max(k);
         const unsigned R = __reduce_min_sync(0xffffffffu, k == K ? (unsigned)bi : 0xffffffffu);
         if (lane == 0) { red_k[warp] = K; red_r[warp] = R; }
       }
       __syncthreads();
       if (warp == 0) {
-        const unsigned k = lane < NT / 32 ? red_k[lane] : 0u, r = lane < NT / 32 ? red_r[lane] : 0xffffffffu;
-        const unsigned K = __reduce_max_sync(0xffffffffu, k);
+        const Key k = lane < NT / 32 ? red_k[lane] : (Key)0, K = warp_max(k);
+        const unsigned r = lane < NT / 32 ? red_r[lane] : 0xffffffffu;
         const unsigned R = __reduce_min_sync(0xffffffffu, k == K ? r : 0xffffffffu);
         const int t = lane & 15;
         const bool mine = c >= r_lo && c < r_hi;
-        const Cx<S> v = (K != 0u && t < l) ? L[t * ch + (int)R - r_lo] : Cx<S>{0, 0};
+        const Cx<S> v = (K != 0 && t < l) ? L[t * ch + (int)R - r_lo] : Cx<S>{0, 0};
         const Cx<S> d = (mine && t < l) ? L[t * ch + c - r_lo] : Cx<S>{0, 0};
+        double mag = 0.0, y = 0.0;
+        if constexpr (F64) {
+          if (K != 0) mag = __longlong_as_double((long long)(K - 1ull));
+          y = 1.0 / mag;
+        }
         const uint32_t ra = rec_a + (uint32_t)((buf * MAXC + (int)rank) * sizeof(Rec<S>));
         for (uint32_t q = lane >> 4; q < cl; q += 2) {
           const uint32_t rq = mapa(ra, q);
-          st_remote(rq + 16u + (uint32_t)(t * sizeof(Cx<S>)), v);
-          if (t == 0) st_remote(rq, ((unsigned long long)K << 32) | R);
+          st_remote(rq + (uint32_t)sizeof(RecHead<S>) + (uint32_t)(t * sizeof(Cx<S>)), v);
+          if constexpr (F64) {
+            if (t == 0) {
+              st_remote(rq, K);
+              st_remote(rq + 8u, (unsigned long long)R);
+              st_remote(rq + 16u, Cx<double>{y, mag});
+            }
+          } else {
+            if (t == 0) st_remote(rq, ((unsigned long long)K << 32) | R);
+          }
           if (mine) st_remote(mapa(drow_a, q) + (uint32_t)((buf * LW + t) * sizeof(Cx<S>)), d);
         }
       }
       cluster_sync();
       // the winner, from this CTA's copy of the records
       const unsigned long long h = lane < (int)cl ? rec[buf][lane].head : 0ull;
-      const unsigned K = __reduce_max_sync(0xffffffffu, (unsigned)(h >> 32));
-      const unsigned R = __reduce_min_sync(0xffffffffu, (unsigned)(h >> 32) == K ? (unsigned)h : 0xffffffffu);
-      const unsigned who = __ballot_sync(0xffffffffu, (unsigned)(h >> 32) == K && (unsigned)h == R);
-      const bool found = K != 0u;
-      const int p = found ? (int)R : c;
-      const Cx<S>* u = found ? rec[buf][__ffs(who) - 1].v : drow[buf];  // the pivot row
-      const Cx<S> d = u[cc];
-      const S dd = d.re * d.re + d.im * d.im;
-      const bool okd = dd > 0;
-      Cx<S> inv = {0, 0};  // FP64: 1 / d once (a division's FP64 instructions for each row otherwise)
-      if constexpr (sizeof(S) == 8) {
-        double y;
-        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(dd));
-        y = fma(y, fma(-dd, y, 1.0), y);
-        y = fma(y, fma(-dd, y, 1.0), y);
-        if (!(y - y == 0.0)) y = 1.0 / dd;  // outside the approximation's range
-        inv = {d.re * y, -d.im * y};
+      Key hk;
+      unsigned hr;
+      if constexpr (F64) {
+        hk = h;
+        hr = lane < (int)cl ? (unsigned)rec[buf][lane].row : 0u;
+      } else {
+        hk = (unsigned)(h >> 32);
+        hr = (unsigned)h;
       }
+      const Key K = warp_max(hk);
+      const unsigned R = __reduce_min_sync(0xffffffffu, hk == K ? hr : 0xffffffffu);
+      const unsigned who = __ballot_sync(0xffffffffu, hk == K && hr == R);
+      const bool found = K != 0;  // (else no candidate is a number: nor is row c's)
+      const int p = found ? (int)R : c;
+      const Rec<S>& win = rec[buf][found ? __ffs(who) - 1 : 0];
+      const Cx<S>* u = found ? win.v : drow[buf];  // the pivot row
+      const Cx<S> d = u[cc];
+      S dd = d.re * d.re + d.im * d.im;
+      bool safe = false;
+      double y = 0.0;
+      if constexpr (F64) {
+        dd = found ? win.mag : 0.0;
+        safe = quotient_safe(dd);
+        y = win.inv;
+      }
+      const bool okd = dd > 0;
       if (tid == 0) {
         s_piv[cc] = p;
         if (rank == 0) {
@@ -502,7 +554,7 @@ __global__ void __launch_bounds__(pcl::NT, 1) k_panel_cluster(Cx<S>* __restrict_
         if constexpr (sizeof(S) == 4) {
           if (okd) lv = cx_div(lv, d);
         } else {
-          if (okd) lv = cx_mul(lv, inv);
+          if (okd) lv = cx_div_by(lv, d, dd, y, safe);
         }
         x[cc * ch] = lv;
         if (cc + 1 < l) {
@@ -1008,14 +1060,18 @@ __global__ void __launch_bounds__(256) k_solve_block(const Cx<double>* __restric
   __syncthreads();
   if (tid >= 64) return;
   Cx<double> v = tid < bs ? x[tid] : Cx<double>{0.0, 0.0};  // thread r holds row r
-  if (!LOWER && tid < bs) {  // 1 / U_rr, once
-    const Cx<double> d = D[tid * 65 + tid];
-    D[tid * 65 + tid] = cx_div(Cx<double>{1.0, 0.0}, d);
+  Cx<double> d = {1.0, 0.0};
+  double dd = 1.0, inv = 1.0;  // |U_rr|^2 and its reciprocal, once
+  if (!LOWER && tid < bs) {
+    d = D[tid * 65 + tid];
+    dd = d.re * d.re + d.im * d.im;
+    inv = 1.0 / dd;
   }
+  const bool safe = quotient_safe(dd);
   for (int k = 0; k < bs; ++k) {
     const int s = LOWER ? k : bs - 1 - k;
     if (tid == s) {
-      if (!LOWER) v = cx_mul(v, D[s * 65 + s]);
+      if (!LOWER) v = cx_div_by(v, d, dd, inv, safe);
       x[s] = v;
     }
     asm volatile("bar.sync 1, 64;" ::: "memory");

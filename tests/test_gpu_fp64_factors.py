@@ -1,10 +1,10 @@
-"""FP64 LU of matrices whose factors are graded inside a panel: rows of L that rise over the panel's
-columns while the columns of U fall by as much.  The error of the digit-split update is relative to a row's
-and a column's largest entry, which such products do not reach; FP64 arithmetic's is relative to the
-products themselves.  Bound: Gaussian elimination computes |P A - L U| <= g |L||U| entrywise, g a
-complex product's and its sum's roundings, (n + 3) 2 sqrt(2) eps with eps = 2^-53 (Higham, Accuracy and
-Stability of Numerical Algorithms, ch. 3 and 9).  The residual is formed with 64-bit mantissas or more.
-The factorisation is called below the C entry points, which take meshes."""
+"""The FP64 LU by itself: pivots, factors, error bounds.  Graded matrices: rows of L that rise over a panel's
+columns while the columns of U fall by as much.  The digit-split update loses relative to a row's and a
+column's largest entry, which such products do not reach; FP64 arithmetic relative to the products
+themselves.  Bound: Gaussian elimination computes |P A - L U| <= g |L||U| entrywise, g a complex product's
+and its sum's roundings, (n + 3) 2 sqrt(2) eps with eps = 2^-53 (Higham, Accuracy and Stability of
+Numerical Algorithms, ch. 3 and 9).  The residual is formed with 64-bit mantissas or more.  The
+factorisation is called below the C entry points, which take meshes."""
 import ctypes
 import re
 import subprocess
@@ -15,8 +15,8 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-def _factor(sol, A):
-    """(LU, row order, zero-pivot word) of A [batch][n][n]"""
+def _factor_device(sol, d, info=None):
+    """(LU, pivots) of d [batch][n][n], which LU overwrites"""
     import torch
     from paper_1706_07919_gb300 import binding as B
 
@@ -25,20 +25,29 @@ def _factor(sol, A):
     f = getattr(lib, re.search(r"\sT\s(_ZN3bie11lu_factor64\S+)", names).group(1))
     f.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int64,
                   ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
-    nb, n, _ = A.shape
-    d = torch.tensor(A, device="cuda:0").contiguous()
-    words = torch.zeros((nb, n + 1), dtype=torch.int32, device="cuda:0")
-    piv, info = words[:, :n].contiguous(), torch.zeros(nb, dtype=torch.int32, device="cuda:0")
+    nb, n, _ = d.shape
+    piv = torch.zeros((nb, n), dtype=torch.int32, device="cuda:0")
+    info = torch.zeros(nb, dtype=torch.int32, device="cuda:0") if info is None else info
     err = torch.zeros(1, dtype=torch.int32, device="cuda:0")
     torch.cuda.synchronize()
     assert f(sol.ctx, d.data_ptr(), nb, n, n, n * n, piv.data_ptr(), info.data_ptr(), err.data_ptr()) == B.BIE_OK
     torch.cuda.synchronize()
     assert int(err) == 0
+    return d, piv
+
+
+def _factor(sol, A):
+    """(LU, row order, zero-pivot words) of A [batch][n][n]"""
+    import torch
+
+    nb, n, _ = A.shape
+    info = torch.zeros(nb, dtype=torch.int32, device="cuda:0")
+    LU, piv = _factor_device(sol, torch.tensor(A, device="cuda:0").contiguous(), info)
     order = np.tile(np.arange(n), (nb, 1))
     for z, p in enumerate(piv.cpu().numpy()):
         for c in range(n):
             order[z, [c, p[c]]] = order[z, [p[c], c]]
-    return d.cpu().numpy(), order, info.cpu().numpy()
+    return LU.cpu().numpy(), order, info.cpu().numpy()
 
 
 def _check(A, LU, order, cols=None):
@@ -99,4 +108,43 @@ def test_entries_that_are_not_finite():
     L, U = np.tril(LU[2], -1) + np.eye(n), np.triu(LU[2])
     res = np.abs(A[2][order[2]] - L @ U)[:, cols]
     assert np.all(res <= 2 * (n + 3) * 2 * np.sqrt(2.0) * 2.0 ** -53 * (np.abs(L) @ np.abs(U))[:, cols])
+    sol.close()
+
+
+def test_pivots_are_the_largest_entries():
+    """Entries of a column that differ by 1e-9: the pivot is the largest one, wherever it lies."""
+    from paper_1706_07919_gb300 import Solver
+
+    n = 700
+    rng = np.random.default_rng(11)
+    A = 1e-3 * (rng.standard_normal((2, n, n)) + 1j * rng.standard_normal((2, n, n)))
+    for z in range(2):
+        A[z, :, 0] = (1 + 1e-9 * rng.permutation(n)) * np.exp(2j * np.pi * rng.uniform(size=n))
+    sol = Solver(0)
+    LU, order, info = _factor(sol, A)
+    assert not info.any()
+    for z in range(2):
+        assert order[z][0] == np.argmax(np.abs(A[z, :, 0]))
+        assert np.max(np.abs(np.tril(LU[z], -1))) <= 1 + 4 * 2.0 ** -53
+    sol.close()
+
+
+@pytest.mark.parametrize("n", [1030, 1480])
+def test_factor_does_not_depend_on_the_cluster(n):
+    """The systems of a batch (which decide the CTAs of a cluster: 16 to 2, sizes between the powers of two
+    among them) have one system's factor, bit for bit; a cluster of few CTAs gives a thread several rows."""
+    import torch
+    from paper_1706_07919_gb300 import Solver
+
+    sol = Solver(0)
+    torch.manual_seed(n)
+    A = torch.randn((64, n, n), dtype=torch.complex128, device="cuda:0")
+    A[:, torch.arange(n), torch.arange(n)] += 8
+    one = {}
+    for batch in (1, 3, 10, 14, 20, 28, 40, 64):
+        LU, piv = _factor_device(sol, A[:batch].clone())
+        for z in range(batch):
+            if z not in one:
+                one[z] = (LU[z].clone(), piv[z].clone()) if batch == 1 else tuple(t[0] for t in _factor_device(sol, A[z:z + 1].clone()))
+            assert torch.equal(piv[z], one[z][1]) and torch.equal(torch.view_as_real(LU[z]), torch.view_as_real(one[z][0]))
     sol.close()
