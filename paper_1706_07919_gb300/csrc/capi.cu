@@ -113,6 +113,7 @@ int launch_foot_points(bie_ctx* c, const double* xp, int64_t M, int32_t* foot_el
                        unsigned long long* first_inside);
 int assemble64(bie_ctx* c, const double* kv, int nk, cd* A, cd* b, void* scratch, bool ff_bulk);
 int lu_factor64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info, int32_t* err);
+size_t fp64_scratch_bytes(bie_ctx* c, int batch, int n);
 int lu_solve64(bie_ctx* c, const cd* LU, int batch, int n, int ld, int64_t bstride, const int32_t* piv, cd* b,
                int64_t bstride_b);
 int field64(bie_ctx* c, const double* kv, int nk, const cd* surf, const double* xp, int64_t M,
@@ -241,7 +242,8 @@ int solve_fp64_multi(bie_ctx* c, const double* k, int64_t Nk, const double* dirs
                       (size_t)N * 4 + st_bytes + 64;
   size_t free_b = 0;
   BIE_TRY(device_free(c, &free_b));
-  int64_t kb = std::max<int64_t>(1, std::min<int64_t>(Nk, std::min<int64_t>(256, (int64_t)((free_b / 2) / perk))));
+  const size_t more = fp64_scratch_bytes(c, 1, (int)N);  // work6
+  int64_t kb = std::max<int64_t>(1, std::min<int64_t>(Nk, std::min<int64_t>(256, (int64_t)((free_b / 2) / (perk + more)))));
   if ((size_t)kb * perk > free_b) return fail(BIE_ERR_OOM, "two FP64 matrices of N = " + std::to_string(N) + " do not fit");
   BIE_TRY(ensure_buf(c, c->work, kb * perk + 4096));
   char* base = (char*)c->work.p;
@@ -301,7 +303,8 @@ int solve_fp64(bie_ctx* c, const double* k, int64_t Nk, cd* surf_out, bie_report
   const size_t perk = (size_t)N * N * sizeof(cd) + (size_t)N * sizeof(cd) * 6 + (size_t)N * 4 + 64;
   size_t free_b = 0;
   BIE_TRY(device_free(c, &free_b));
-  int64_t kb = std::max<int64_t>(1, std::min<int64_t>(Nk, std::min<int64_t>(256, (int64_t)((free_b / 2) / perk))));
+  const size_t more = fp64_scratch_bytes(c, 1, (int)N);  // work6
+  int64_t kb = std::max<int64_t>(1, std::min<int64_t>(Nk, std::min<int64_t>(256, (int64_t)((free_b / 2) / (perk + more)))));
   if ((size_t)kb * perk > free_b) return fail(BIE_ERR_OOM, "one FP64 system of N = " + std::to_string(N) + " does not fit in device memory");
   BIE_TRY(ensure_buf(c, c->work, kb * perk + 4096));
   char* base = (char*)c->work.p;

@@ -23,6 +23,7 @@ namespace bie {
 
 int assemble64(bie_ctx* c, const double* kv, int nk, cd* A, cd* b, void* scratch, bool ff_bulk);
 int lu_factor64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info, int32_t* err);
+size_t fp64_scratch_bytes(bie_ctx* c, int batch, int n);
 int lu64_error(bie_ctx* c, const int32_t* err);
 int lu_solve64(bie_ctx* c, const cd* LU, int batch, int n, int ld, int64_t bstride, const int32_t* piv, cd* b,
                int64_t bstride_b);
@@ -131,7 +132,8 @@ int solve_fp64_linear(bie_ctx* c, const double* k, int64_t Nk, cd* surf_out, bie
                       (size_t)Nl * 4 + 64;
   size_t free_b = 0;
   BIE_TRY(device_free(c, &free_b));
-  const int64_t kb = std::max<int64_t>(1, std::min<int64_t>(Nk, std::min<int64_t>(64, (int64_t)((free_b / 2) / perk))));
+  const size_t more = fp64_scratch_bytes(c, 1, (int)Nl);  // work6
+  const int64_t kb = std::max<int64_t>(1, std::min<int64_t>(Nk, std::min<int64_t>(64, (int64_t)((free_b / 2) / (perk + more)))));
   if ((size_t)kb * perk > free_b) return fail(BIE_ERR_OOM, "linear-element systems do not fit in device memory");
   BIE_TRY(ensure_buf(c, c->work, (size_t)kb * perk + 8192));
   char* base = (char*)c->work.p;

@@ -1265,9 +1265,18 @@ int lu_trsm_rows32(bie_ctx* c, cf* A, int batch, int n, int ld, int64_t bstride,
 size_t lu_split_scratch_bytes(int batch, int n);
 int lu_update_split64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int p0, void* scratch, int32_t* err);
 
+// Bytes of c->work6 for the FP64 assembly, factorisation and solves of `batch` systems of n rows (the
+// assembly's n may be the larger quadratic image's of a linear mesh: it is of the context's elements).
+size_t fp64_scratch_bytes(bie_ctx* c, int batch, int n) {
+  const size_t known = (size_t)batch * c->E * c->rule.Q * sizeof(cd);
+  const size_t solve = (size_t)batch * n * (sizeof(cd) + sizeof(int32_t));
+  return std::max(std::max(known, solve), n > 128 ? lu_split_scratch_bytes(batch, n) : (size_t)0);
+}
+
 // FP64 LU: 64-column panels (clusters, else one CTA per matrix), their row swaps and U blocks, and the
 // trailing update: split into digits on the tensor cores (lu_split.cu), or on the FP64 pipe for matrices
-// of at most two panels and where the digits do not fit memory.  info: zero pivots, per system; *err
+// of at most two panels.  Its callers size c->work6 with their batch (fp64_scratch_bytes); only where one
+// system alone fills the device's memory do the digits not fit beside it, and the FP64 pipe takes over.  info: zero pivots, per system; *err
 // (device, cleared by the caller): a bounded wait gave up, every factor of the batch is void.
 int lu_factor64(bie_ctx* c, cd* A, int batch, int n, int ld, int64_t bstride, int32_t* piv, int32_t* info, int32_t* err) {
   Cx<double>* M = reinterpret_cast<Cx<double>*>(A);

@@ -100,12 +100,14 @@ int solve_mixed(bie_ctx* c, const double* k, int64_t Nk, cd* surf_out, bie_repor
   // together when the pool is full and after the last batch, instead of batch by batch.
   const size_t pool1 = multi ? 0 : mat + align256((size_t)N * 4) + dsz + 2 * vec;
   const size_t fb1 = align256((size_t)N * N * sizeof(cd)) + 7 * vec + align256((size_t)N * 8) + 1024 + pool1;
+  const size_t known1 = (size_t)c->E * c->rule.Q * sizeof(cd);  // work6: known values at the quadrature points
   size_t free_b = 0;
   BIE_TRY(device_free(c, &free_b));
   const int G = (int)std::max<size_t>(
-      1, std::min<size_t>(std::min(kFallbackGroupMax, c->reassembly_group), (free_b / 8) / fb1));
+      1, std::min<size_t>(std::min(kFallbackGroupMax, c->reassembly_group), (free_b / 8) / (fb1 + known1)));
   const size_t fb = (size_t)G * fb1 + 4096;
-  const size_t avail = free_b > fb ? free_b - fb : 0;
+  const size_t aside = fb + (size_t)G * known1;
+  const size_t avail = free_b > aside ? free_b - aside : 0;
   int64_t kb = std::max<int64_t>(1, std::min<int64_t>(Nk, std::min<int64_t>(c->mixed_batch, (int64_t)((avail / 2) / perk))));
   size_t tc_scratch = lu_tc_scratch_bytes((int)kb, (int)N, lu_block_for(c, (int)N));
   if ((size_t)kb * perk + tc_scratch + fb > free_b)

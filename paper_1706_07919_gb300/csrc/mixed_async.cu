@@ -142,6 +142,7 @@ int solve_mixed_async(bie_ctx* c, const double* k, int64_t Nk, cd* surf_out, bie
                       2 * align256a((size_t)N * 4) + align256a(refine_state_bytes(1)) + 64 +
                       align256a(sizeof(bie_report)) + 16;
   const size_t fb1 = align256a((size_t)N * N * sizeof(cd)) + 7 * vec + align256a((size_t)N * 8) + 1024;
+  const size_t known1 = (size_t)c->E * c->rule.Q * sizeof(cd);  // work6: known values at the quadrature points
   if (rep && c->rep_pinned_bytes < (size_t)Nk * sizeof(bie_report)) {
     // report staging, grown before this call enqueues anything; a smaller earlier buffer is
     // retired, not freed, since an earlier call's host function may still read it (freed with
@@ -156,9 +157,10 @@ int solve_mixed_async(bie_ctx* c, const double* k, int64_t Nk, cd* surf_out, bie
   size_t free_b = 0;
   BIE_TRY(device_free(c, &free_b));
   const int G = (int)std::max<size_t>(
-      1, std::min<size_t>(std::min(kAsyncGroupMax, c->reassembly_group), (free_b / 8) / fb1));
+      1, std::min<size_t>(std::min(kAsyncGroupMax, c->reassembly_group), (free_b / 8) / (fb1 + known1)));
   const size_t fb = (size_t)G * fb1 + 4096;
-  const size_t avail = free_b > fb ? free_b - fb : 0;
+  const size_t aside = fb + (size_t)G * known1;
+  const size_t avail = free_b > aside ? free_b - aside : 0;
   int64_t kb = std::max<int64_t>(1, std::min<int64_t>(Nk, std::min<int64_t>(c->mixed_batch, (int64_t)((avail / 2) / perk))));
   const size_t fixed = align256a((size_t)Nk * sizeof(double)) + align256a((size_t)Nk * sizeof(bie_report)) + 4096;
   size_t tc_scratch = lu_tc_scratch_bytes((int)kb, (int)N, lu_block_for(c, (int)N));
