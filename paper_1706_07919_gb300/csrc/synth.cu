@@ -428,19 +428,25 @@ int pulse_spectrum(bie_ctx* c, const double* s, int64_t P, int n, cd* Sout) {
 
 int synthesize(bie_ctx* c, const cd* T, const int64_t* midx_dev, int nk, int64_t M, const cd* Sp, int64_t P, int n,
                void* out, int out_dtype) {
-  // twiddles (at most FP64 pairs), then the spectra in float-float (FP32)
+  // twiddles (at most FP64 pairs), then the spectra in float-float (FP32), of so many pulses at a time that
+  // they stay within 32 MB (1023 pulses of 4096 samples)
   const size_t twb = (size_t)(twiddle_count(n) + 16) * sizeof(double2);
-  const int64_t ns = P * (n / 2 + 1);
+  const int64_t nm = n / 2 + 1;
   const bool f32 = out_dtype != 0;
-  BIE_TRY(ensure_buf(c, c->work2, twb + (f32 ? (size_t)ns * sizeof(float4) : 0)));
+  const int64_t pc = f32 ? std::min(P, std::max<int64_t>(1, (int64_t)(32 << 20) / (nm * (int64_t)sizeof(float4)))) : P;
+  BIE_TRY(ensure_buf(c, c->work2, twb + (f32 ? (size_t)(pc * nm) * sizeof(float4) : 0)));
   void* tw = c->work2.p;
   int nsm = 0;
   BIE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
   if (f32) {
     float4* sp = (float4*)((char*)tw + twb);
     launch_twiddles<float>(n, tw, true, c->stream);
-    BIE_LAUNCH(k_split_spectra<<<(unsigned)((ns + 255) / 256), 256, 0, c->stream>>>(Sp, ns, sp));
-    BIE_TRY(launch_synth<float>(T, midx_dev, nk, M, Sp, sp, P, n, tw, true, (float*)out, nsm, c->stream));
+    for (int64_t p0 = 0; p0 < P; p0 += pc) {
+      const int64_t np = std::min(pc, P - p0), ns = np * nm;
+      const cd* S0 = Sp + p0 * nm;
+      BIE_LAUNCH(k_split_spectra<<<(unsigned)((ns + 255) / 256), 256, 0, c->stream>>>(S0, ns, sp));
+      BIE_TRY(launch_synth<float>(T, midx_dev, nk, M, S0, sp, np, n, tw, true, (float*)out + p0 * M * n, nsm, c->stream));
+    }
   } else {
     launch_twiddles<double>(n, tw, true, c->stream);
     BIE_TRY(launch_synth<double>(T, midx_dev, nk, M, Sp, nullptr, P, n, tw, true, (double*)out, nsm, c->stream));

@@ -62,3 +62,27 @@ def test_fp32_synthesis_takes_values_outside_fp32():
         ref = _reference(T, midx, S, 64)
         assert np.linalg.norm(got - ref) <= 27 * 2.0 ** -24 * np.linalg.norm(ref)
     sol.close()
+
+
+def test_many_pulses_take_bounded_scratch():
+    """FP32 output of 6000 pulses of 4096 samples: the device memory a context takes for their split spectra
+    stays below 64 MB (197 MB for all of them at once), and a pulse's signal is its own."""
+    import torch
+    from paper_1706_07919_gb300 import Solver
+
+    Nt, P = 4096, 6000
+    g = torch.Generator("cuda:0").manual_seed(3)
+    midx = np.arange(1, 40, dtype=np.int64)
+    T = torch.randn((len(midx), 1), dtype=torch.complex128, device="cuda:0", generator=g)
+    S = torch.randn((P, Nt // 2 + 1), dtype=torch.complex128, device="cuda:0", generator=g)
+    out = torch.empty((P, 1, Nt), dtype=torch.float32, device="cuda:0")
+    sol = Solver(0)
+    sol.synthesize(T, midx, S[:2], Nt, torch.float32, out=out[:2])  # (module and tables loaded)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    sol.synthesize(T, midx, S, Nt, torch.float32, out=out)
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] < 64 << 20
+    for p in (0, 1022, 1023, 1024, 2046, P - 1):
+        assert torch.equal(sol.synthesize(T, midx, S[p:p + 1], Nt, torch.float32)[0], out[p])
+    sol.close()
