@@ -394,7 +394,7 @@ int bie_top_frequencies(bie_ctx* ctx, const void* S, int64_t P, int64_t Nt, int6
  * hands out a fixed device-memory budget through its own pool, or a latency-bound pipeline in
  * which cudaMalloc/cudaFree would synchronise the device.  It needs no context and allocates
  * nothing: its scratch (the FFT twiddle table and the device copy of midx) lives in one
- * file-scope device array of 64 KB that every GPU loading the library holds until the process
+ * file-scope device array of 80 KB that every GPU loading the library holds until the process
  * exits.  Arguments and the result are those of bie_synthesize, on the caller's current device
  * and on `stream` (a cudaStream_t, NULL = legacy default stream); the call returns after the
  * stream has completed.

@@ -90,26 +90,42 @@ __global__ void k_synth(const cd* __restrict__ T, const int64_t* __restrict__ mi
 // ---- synthesis of signals of 32 samples and more ------------------------------------------------
 // A real signal of n samples is one complex transform of h = n / 2 values,
 //   out[2 j] + i out[2 j + 1] = sum_k Z_k exp(-2 pi i j k / h),
-//   Z_k = (H_k + conj(H_{h-k})) + i exp(-2 pi i k / n) (H_k - conj(H_{h-k})),
-// H_m = S_m T_m / n for 0 < m < h, H_0 and H_h the real parts of theirs.  h / 16 threads take a
-// signal, 16 values each in registers: one pass of radix 2, 4 or 8 where log2 h leaves a
-// remainder, then radix-16 passes (Stockham order), exchanging through shared memory between
-// passes -- two exchanges for n = 4096, where the radix-2 kernel had twelve round trips through
+//   Z_k = H_k (1 + i w_k) + conj(H_{h-k} (1 - i w_{h-k})),  w_k = exp(-2 pi i k / n),
+// H_m = S_m T_m / n for 0 < m < h, H_0 and H_h the real parts of theirs; a frequency thus adds to Z_m and to
+// Z_{h-m}.  h / 16 threads take a signal, 16 values each in registers: one pass of radix 2, 4 or 8
+// where log2 h leaves a remainder, then radix-16 passes (Stockham order), exchanging through shared memory
+// between passes -- two exchanges for n = 4096, where the radix-2 kernel had twelve round trips through
 // shared memory, each with a division and a twiddle converted from FP64.  A CTA of up to 256 threads
 // holds SB neighbouring points, so that T is read in whole sectors, and takes PG pulses one
-// after the other with the points' T kept in shared memory.  FP32: S and T enter as float-float
-// (T split once per point, S once per call, `sp` or, without it, in the kernel) and their product
-// rounds once, as the FP64 product rounded to FP32 did: eight FP64 operations a frequency, point and
-// pulse would cost 0.4 ms below on this GPU's narrow FP64 pipe.
+// after the other with the points' T kept in shared memory.  FP32: S (1 + i w) / n and S (1 - i w) / n
+// (`sp`, once per call) and T (once per point) enter as float-float and their products round once, as
+// the FP64 product rounded to FP32 did: eight FP64 operations a frequency, point and pulse would cost 0.4 ms
+// below on this GPU's narrow FP64 pipe.  Without `sp` the products are formed in FP64.
 // Bound: shared memory and the transforms' arithmetic in about equal parts (DRAM: 1.1 GB written).
-// Measured, 8 pulses x 8192 points x 4096 samples from 512 frequencies in FP32: 7.2 -> 1.06 ms (1.86
-// with the passes' factors read out of the plain table).
-// Relative error against FP64 1.2e-7 before and after.  128 registers (2 CTAs) measured 1.18 ms.
+// Measured, the call for 8 pulses x 8192 points x 4096 samples from 512 frequencies in FP32: 7.2 -> 0.67 ms
+// (with the factors 1 +- i w taken in the first pass, from rounded H, 0.84; with the passes' factors read
+// out of the plain table and that, 1.6); without `sp` 1.43.
+// Relative error against FP64 of 4096 / 512 samples, every frequency: 1.22e-7 / 1.03e-7 before (radix 2), 1.16e-7
+// / 0.98e-7 here; an eighth of the frequencies: 1.10e-7 / 0.89e-7 and 1.09e-7 / 0.90e-7 (at 64 samples 0.67e-7
+// and 0.70e-7: radix 2 adds exact zeros there).  That takes the products rounded once into Z and the fixed
+// factors with their rests: 1.25e-7 / 1.08e-7 without.
 template <class S> __device__ __forceinline__ C2<S> c2mul(C2<S> a, C2<S> b) {
   return {a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re};
 }
 template <class S> __device__ __forceinline__ C2<S> c2add(C2<S> a, C2<S> b) { return {a.re + b.re, a.im + b.im}; }
 template <class S> __device__ __forceinline__ C2<S> c2sub(C2<S> a, C2<S> b) { return {a.re - b.re, a.im - b.im}; }
+
+// a transform's fixed factors, each as a value of its type and the rest: rounded alone they would add an error
+// of the size of the products' own
+template <class S> struct Fix {
+  S hi, lo;
+  __host__ __device__ constexpr Fix(double v, double rest) : hi((S)v), lo((S)((v - (double)(S)v) + rest)) {}
+  __device__ __forceinline__ S operator()(S x) const { return fma(x, hi, x * lo); }
+};
+template <class S> __device__ __forceinline__ C2<S> c2fix(C2<S> a, Fix<S> c, Fix<S> s) {  // a (c + i s)
+  return {fma(a.re, c.hi, fma(-a.im, s.hi, fma(a.re, c.lo, -(a.im * s.lo)))),
+          fma(a.re, s.hi, fma(a.im, c.hi, fma(a.re, s.lo, a.im * c.lo)))};
+}
 
 template <class S> __device__ __forceinline__ void fft2(C2<S>& a, C2<S>& b) {
   const C2<S> t = c2sub(a, b);
@@ -130,27 +146,29 @@ template <int R, class S> __device__ __forceinline__ void fft_small(C2<S>* v) {
   } else if constexpr (R == 4) {
     fft4(v[0], v[1], v[2], v[3]);
   } else if constexpr (R == 8) {
-    const S h = (S)0.70710678118654752440;
+    constexpr Fix<S> h(0.70710678118654752440, -4.833646656726457e-17);  // sqrt(1/2)
     fft4(v[0], v[2], v[4], v[6]);
     fft4(v[1], v[3], v[5], v[7]);
-    v[3] = C2<S>{h * (v[3].re + v[3].im), h * (v[3].im - v[3].re)};
+    v[3] = C2<S>{h(v[3].re + v[3].im), h(v[3].im - v[3].re)};
     v[5] = C2<S>{v[5].im, -v[5].re};
-    v[7] = C2<S>{h * (v[7].im - v[7].re), -h * (v[7].re + v[7].im)};
+    v[7] = C2<S>{h(v[7].im - v[7].re), -h(v[7].re + v[7].im)};
 #pragma unroll
     for (int q = 0; q < 4; ++q) fft2(v[2 * q], v[2 * q + 1]);
   } else {
-    const S h = (S)0.70710678118654752440, c = (S)0.92387953251128675613, s = (S)0.38268343236508977173;
+    constexpr Fix<S> h(0.70710678118654752440, -4.833646656726457e-17);
+    constexpr Fix<S> c(0.92387953251128675613, 1.7645047084336677e-17), mc(-0.92387953251128675613, -1.7645047084336677e-17);
+    constexpr Fix<S> s(0.38268343236508977173, -1.0050772696461588e-17), ms(-0.38268343236508977173, 1.0050772696461588e-17);
 #pragma unroll
     for (int i = 0; i < 4; ++i) fft4(v[i], v[i + 4], v[i + 8], v[i + 12]);
-    v[5] = c2mul(v[5], C2<S>{c, -s});
-    v[9] = C2<S>{h * (v[9].re + v[9].im), h * (v[9].im - v[9].re)};
-    v[13] = c2mul(v[13], C2<S>{s, -c});
-    v[6] = C2<S>{h * (v[6].re + v[6].im), h * (v[6].im - v[6].re)};
+    v[5] = c2fix(v[5], c, ms);  // cos and sin of pi / 8
+    v[9] = C2<S>{h(v[9].re + v[9].im), h(v[9].im - v[9].re)};
+    v[13] = c2fix(v[13], s, mc);
+    v[6] = C2<S>{h(v[6].re + v[6].im), h(v[6].im - v[6].re)};
     v[10] = C2<S>{v[10].im, -v[10].re};
-    v[14] = C2<S>{h * (v[14].im - v[14].re), -h * (v[14].re + v[14].im)};
-    v[7] = c2mul(v[7], C2<S>{s, -c});
-    v[11] = C2<S>{h * (v[11].im - v[11].re), -h * (v[11].re + v[11].im)};
-    v[15] = c2mul(v[15], C2<S>{-c, s});
+    v[14] = C2<S>{h(v[14].im - v[14].re), -h(v[14].re + v[14].im)};
+    v[7] = c2fix(v[7], s, mc);
+    v[11] = C2<S>{h(v[11].im - v[11].re), -h(v[11].re + v[11].im)};
+    v[15] = c2fix(v[15], mc, s);
 #pragma unroll
     for (int q = 0; q < 4; ++q) fft4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
   }
@@ -202,9 +220,29 @@ __device__ __forceinline__ float4 split_cd(cd v) {
   const ff r = ff_from_double(v.re), i = ff_from_double(v.im);
   return make_float4(r.hi, r.lo, i.hi, i.lo);
 }
-__global__ void k_split_spectra(const cd* __restrict__ Sp, int64_t n, float4* __restrict__ out) {
+// a frequency's factors (1 +- i w) of an FP64 value a
+__device__ __forceinline__ cd plus_iw(cd a, double2 w) {
+  return {fma(-w.x, a.im, fma(-w.y, a.re, a.re)), fma(w.x, a.re, fma(-w.y, a.im, a.im))};
+}
+__device__ __forceinline__ cd minus_iw(cd a, double2 w) {
+  return {fma(w.x, a.im, fma(w.y, a.re, a.re)), fma(-w.x, a.re, fma(w.y, a.im, a.im))};
+}
+__device__ __forceinline__ double2 half_twiddle(int m, int n) {  // exp(-2 pi i m / n)
+  double s, c;
+  sincospi(2.0 * (double)m / (double)n, &s, &c);
+  return make_double2(c, -s);
+}
+// spectra of P pulses, [P][h + 1]: out[..][2] = S (1 + i w) / n, S (1 - i w) / n; for m = 0 and h: S / n, 0
+__global__ void k_split_spectra(const cd* __restrict__ Sp, int64_t count, int n, float4* __restrict__ out) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t < n) out[t] = split_cd(Sp[t]);
+  if (t >= count) return;
+  const int h = n / 2, m = (int)(t % (h + 1));
+  const double inv = 1.0 / n;  // a power of two
+  const cd a = {Sp[t].re * inv, Sp[t].im * inv};
+  const bool end = m == 0 || m == h;
+  const double2 w = half_twiddle(m, n);
+  out[2 * t] = split_cd(end ? a : plus_iw(a, w));
+  out[2 * t + 1] = end ? make_float4(0.f, 0.f, 0.f, 0.f) : split_cd(minus_iw(a, w));
 }
 // a b - c d or a b + c d from float-float factors, rounded once
 __device__ __forceinline__ float ff_dot2(float ah, float al, float bh, float bl, float ch, float cl, float dh, float dl) {
@@ -218,7 +256,7 @@ __device__ __forceinline__ C2<float> ff_cmul(float4 s, float4 t) {
   return {ff_dot2(s.x, s.y, t.x, t.y, -s.z, -s.w, t.z, t.w), ff_dot2(s.x, s.y, t.z, t.w, s.z, s.w, t.x, t.y)};
 }
 
-// First pass of radix R0 (inputs made from the spectrum), then radix-16 passes; the last one leaves
+// First pass of radix R0 (inputs Z in buf), then radix-16 passes; the last one leaves
 // its outputs in v (output fft_at<16>(r) of butterfly j is z[j + r Ns]).
 template <int L, class S>
 __device__ __forceinline__ void real_fft(C2<S>* __restrict__ buf, const C2<S>* __restrict__ tw, bool passes, int j,
@@ -229,16 +267,7 @@ __device__ __forceinline__ void real_fft(C2<S>* __restrict__ buf, const C2<S>* _
 #pragma unroll
     for (int q = 0; q < R0; ++q) {
       const int k = j + b * NT + q * (h / R0);
-      const C2<S> H = buf[fft_pad(k)], C = buf[fft_pad(h - k)];
-      C2<S> z;
-      if (k == 0) {
-        z = {H.re + C.re, H.re - C.re};
-      } else {
-        const C2<S> sum = {H.re + C.re, H.im - C.im}, dif = {H.re - C.re, H.im + C.im};
-        const C2<S> d = c2mul(tw[k], dif);
-        z = {sum.re - d.im, sum.im + d.re};
-      }
-      v[b * R0 + q] = z;
+      v[b * R0 + q] = buf[fft_pad(k)];
     }
 #pragma unroll
   for (int b = 0; b < 16 / R0; ++b) fft_small<R0, S>(v + b * R0);
@@ -277,7 +306,7 @@ __device__ __forceinline__ void real_fft(C2<S>* __restrict__ buf, const C2<S>* _
 template <int L, class S, bool KEEP>
 __global__ void __launch_bounds__(256, sizeof(S) == 4 ? 3 : 1) k_synth_real(const cd* __restrict__ T, const int64_t* __restrict__ midx, int nk,
                                                     int64_t M, const cd* __restrict__ Sp, const float4* __restrict__ sp,
-                                                    int P, int PG, int SB, const C2<S>* __restrict__ tw, bool passes,
+                                                    const double2* __restrict__ w64, int P, int PG, int SB, const C2<S>* __restrict__ tw, bool passes,
                                                     S* __restrict__ out, int wide) {
   constexpr int h = 1 << L, n = 2 * h, NT = h / 16;
   constexpr bool F32 = sizeof(S) == 4;
@@ -289,6 +318,16 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? 3 : 1) k_synth_real(cons
   const int tid = threadIdx.x, pt = tid / NT, j = tid - pt * NT;
   const int64_t x0 = (int64_t)blockIdx.x * SB;
   C2<S>* buf = bufs + pt * len;
+  __shared__ int s_low;  // frequencies below h / 2
+  if (tid == 0) {
+    int lo = 0, hi = nk;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (2 * midx[mid] < h) lo = mid + 1;
+      else hi = mid;
+    }
+    s_low = lo;
+  }
   if (KEEP)
     for (int e = tid; e < nk * SB; e += SB * NT) {
       const int r = e / SB, q = e - r * SB;
@@ -302,33 +341,56 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? 3 : 1) k_synth_real(cons
     for (int e = tid; e < SB * len; e += SB * NT) bufs[e] = {(S)0, (S)0};
     __syncthreads();
     const cd* Srow = Sp + (int64_t)p * (h + 1);
-    for (int e = tid; e < nk * SB; e += SB * NT) {
-      const int r = e / SB, q = e - r * SB;
-      const int m = (int)midx[r];
-      C2<S> v;
-      if constexpr (F32) {
-        const float4 s4 = sp ? sp[(int64_t)p * (h + 1) + m] : split_cd(Srow[m]);
-        float4 t4;
-        if (KEEP) t4 = kept[e];
-        else t4 = x0 + q < M ? split_cd(T[(int64_t)r * M + x0 + q]) : make_float4(0.f, 0.f, 0.f, 0.f);
-        v = ff_cmul(s4, t4);
-        // outside a safe range of FP32 (zero, tiny, huge, not finite): the product in FP64
-        const float ta = fmaxf(fabsf(t4.x), fabsf(t4.z)), sa = fmaxf(fabsf(s4.x), fabsf(s4.z));
-        if (!(ta >= 1e-25f && ta <= 1e25f && sa >= 1e-25f && sa <= 1e25f) && x0 + q < M) {
-          const cd a = cmul(Srow[m], T[(int64_t)r * M + x0 + q]);
-          v = {(float)a.re, (float)a.im};
+    // the frequencies below h / 2 store their shares of Z_m and Z_{h-m}, then those from h / 2 on add theirs
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+      const int e0 = half ? s_low * SB : 0, e1 = half ? nk * SB : s_low * SB;
+      for (int e = e0 + tid; e < e1; e += SB * NT) {
+        const int r = e / SB, q = e - r * SB;
+        const int m = (int)midx[r];
+        const bool end = m == 0 || m == h;
+        C2<S> za, zb;  // H (1 + i w), H (1 - i w); at the ends H
+        bool fp64 = true;
+        if constexpr (F32) {
+          if (sp) {
+            const float4 sa = sp[2 * ((int64_t)p * (h + 1) + m)], sb = sp[2 * ((int64_t)p * (h + 1) + m) + 1];
+            float4 t4;
+            if (KEEP) t4 = kept[e];
+            else t4 = x0 + q < M ? split_cd(T[(int64_t)r * M + x0 + q]) : make_float4(0.f, 0.f, 0.f, 0.f);
+            za = ff_cmul(sa, t4);
+            zb = ff_cmul(sb, t4);
+            // outside a safe range of FP32 (zero, tiny, huge, not finite): the product in FP64
+            const float tm = fmaxf(fabsf(t4.x), fabsf(t4.z)), sm = fmaxf(fabsf(sa.x), fabsf(sa.z));
+            fp64 = !(tm >= 1e-25f && tm <= 1e25f && sm >= 1e-25f && sm <= 1e25f);
+          }
         }
-      } else {
-        cd t;
-        if (KEEP) t = reinterpret_cast<cd*>(kept)[e];
-        else t = x0 + q < M ? T[(int64_t)r * M + x0 + q] : cd{0.0, 0.0};
-        const cd a = cmul(Srow[m], t);
-        v = {a.re, a.im};
+        if (fp64) {
+          cd t = {0.0, 0.0};
+          if constexpr (KEEP && !F32) t = reinterpret_cast<cd*>(kept)[e];
+          else if (x0 + q < M) t = T[(int64_t)r * M + x0 + q];
+          const cd a = cmul(Srow[m], t);
+          cd u = a, d = {0.0, 0.0};
+          if (!end) {
+            const double2 w = w64 ? w64[m] : half_twiddle(m, n);
+            u = plus_iw(a, w);
+            d = minus_iw(a, w);
+          }
+          constexpr S inv = (S)1 / (S)n;
+          za = {(S)u.re * inv, (S)u.im * inv};
+          zb = {(S)d.re * inv, (S)d.im * inv};
+        }
+        if (end) za = C2<S>{za.re, m == 0 ? za.re : -za.re};
+        C2<S>* z = bufs + q * len;
+        C2<S>& lo = z[fft_pad(m == h ? 0 : m)];
+        lo = half ? c2add(lo, za) : za;
+        if (!end && 2 * m != h) {  // (at h / 2, w = -i: 1 - i w = 0)
+          C2<S>& hi = z[fft_pad(h - m)];
+          const C2<S> b = {zb.re, -zb.im};
+          hi = half ? c2add(hi, b) : b;
+        }
       }
-      constexpr S inv = (S)1 / (S)n;
-      bufs[q * len + fft_pad(m)] = {v.re * inv, v.im * inv};
+      __syncthreads();
     }
-    __syncthreads();
     C2<S> v[16];
     real_fft<L, S>(buf, tw, passes, j, v);
     if (x0 + pt < M) {
@@ -362,10 +424,11 @@ static void launch_twiddles(int n, void* tw, bool passes, cudaStream_t st) {
     BIE_LAUNCH(k_twiddles_of<S><<<(count + 127) / 128, 128, 0, st>>>(n, pass_radix0(L), count, (C2<S>*)tw));
 }
 
-// sp: the spectra split into float-float (FP32 only; NULL: split in the kernel).
+// sp: the spectra's factors in float-float (k_split_spectra; FP32 only; NULL: products in FP64); w64:
+// exp(-2 pi i m / n), m < n / 2, in FP64 (NULL: formed where an FP64 product needs one).
 template <class S>
-static int launch_synth(const cd* T, const int64_t* midx, int nk, int64_t M, const cd* Sp, const float4* sp, int64_t P,
-                        int n, const void* tw, bool passes, S* out, int nsm, cudaStream_t st) {
+static int launch_synth(const cd* T, const int64_t* midx, int nk, int64_t M, const cd* Sp, const float4* sp,
+                        const double2* w64, int64_t P, int n, const void* tw, bool passes, S* out, int nsm, cudaStream_t st) {
   if (n < 32) {
     const dim3 g((unsigned)M, (unsigned)P);
     const size_t smem = 2 * (size_t)n * sizeof(C2<S>);
@@ -388,7 +451,7 @@ static int launch_synth(const cd* T, const int64_t* midx, int nk, int64_t M, con
   const dim3 g((unsigned)bx, (unsigned)(keep ? 1 : P));
   auto go = [&](auto kernel) -> int {
     BIE_TRY(set_smem_max(kernel));
-    BIE_LAUNCH(kernel<<<g, SB * (h / 16), bufs + (keep ? kept : 0), st>>>(T, midx, nk, M, Sp, sp, (int)P, PG, SB,
+    BIE_LAUNCH(kernel<<<g, SB * (h / 16), bufs + (keep ? kept : 0), st>>>(T, midx, nk, M, Sp, sp, w64, (int)P, PG, SB,
                                                                           (const C2<S>*)tw, passes, out, wide));
     return BIE_OK;
   };
@@ -429,12 +492,12 @@ int pulse_spectrum(bie_ctx* c, const double* s, int64_t P, int n, cd* Sout) {
 int synthesize(bie_ctx* c, const cd* T, const int64_t* midx_dev, int nk, int64_t M, const cd* Sp, int64_t P, int n,
                void* out, int out_dtype) {
   // twiddles (at most FP64 pairs), then the spectra in float-float (FP32), of so many pulses at a time that
-  // they stay within 32 MB (1023 pulses of 4096 samples)
+  // they stay within 32 MB (511 pulses of 4096 samples)
   const size_t twb = (size_t)(twiddle_count(n) + 16) * sizeof(double2);
   const int64_t nm = n / 2 + 1;
   const bool f32 = out_dtype != 0;
-  const int64_t pc = f32 ? std::min(P, std::max<int64_t>(1, (int64_t)(32 << 20) / (nm * (int64_t)sizeof(float4)))) : P;
-  BIE_TRY(ensure_buf(c, c->work2, twb + (f32 ? (size_t)(pc * nm) * sizeof(float4) : 0)));
+  const int64_t pc = f32 ? std::min(P, std::max<int64_t>(1, (int64_t)(32 << 20) / (nm * 2 * (int64_t)sizeof(float4)))) : P;
+  BIE_TRY(ensure_buf(c, c->work2, twb + (f32 ? (size_t)(2 * pc * nm) * sizeof(float4) : 0)));
   void* tw = c->work2.p;
   int nsm = 0;
   BIE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
@@ -444,12 +507,12 @@ int synthesize(bie_ctx* c, const cd* T, const int64_t* midx_dev, int nk, int64_t
     for (int64_t p0 = 0; p0 < P; p0 += pc) {
       const int64_t np = std::min(pc, P - p0), ns = np * nm;
       const cd* S0 = Sp + p0 * nm;
-      BIE_LAUNCH(k_split_spectra<<<(unsigned)((ns + 255) / 256), 256, 0, c->stream>>>(S0, ns, sp));
-      BIE_TRY(launch_synth<float>(T, midx_dev, nk, M, S0, sp, np, n, tw, true, (float*)out + p0 * M * n, nsm, c->stream));
+      BIE_LAUNCH(k_split_spectra<<<(unsigned)((ns + 255) / 256), 256, 0, c->stream>>>(S0, ns, n, sp));
+      BIE_TRY(launch_synth<float>(T, midx_dev, nk, M, S0, sp, nullptr, np, n, tw, true, (float*)out + p0 * M * n, nsm, c->stream));
     }
   } else {
     launch_twiddles<double>(n, tw, true, c->stream);
-    BIE_TRY(launch_synth<double>(T, midx_dev, nk, M, Sp, nullptr, P, n, tw, true, (double*)out, nsm, c->stream));
+    BIE_TRY(launch_synth<double>(T, midx_dev, nk, M, Sp, nullptr, (const double2*)tw, P, n, tw, true, (double*)out, nsm, c->stream));
   }
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
@@ -532,9 +595,10 @@ int top_frequencies(bie_ctx* c, const cd* S, int64_t P, int nm, int K, int64_t* 
 // scratch (the FFT twiddle table and the device copy of the frequency indices) lives in one
 // file-scope device array instead of context buffers, and no context is needed.
 // ------------------------------------------------------------------------------------------
-constexpr size_t kNoAllocScratchBytes = 64 * 1024;  // twiddles <= 32 KB (Nt <= 4096) + indices <= 32 KB
+constexpr size_t kNoAllocScratchBytes = 64 * 1024;  // FP64 twiddles <= 32 KB (Nt <= 4096) + indices <= 32 KB
+constexpr size_t kNoAllocTwiddle32Bytes = 16 * 1024;  // and the FP32 ones
 constexpr int kNoAllocMaxDevices = 64;
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes + kNoAllocTwiddle32Bytes];
 static std::mutex g_noalloc_mu;
 static void* g_noalloc_ptr[kNoAllocMaxDevices] = {};
 
@@ -585,10 +649,12 @@ extern "C" int bie_synthesize_noalloc(const void* T, const int64_t* midx, int64_
   BIE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   if (out_dtype == 0) {
     launch_twiddles<double>(n, tw, false, st);
-    BIE_TRY(launch_synth<double>((const cd*)T, md, (int)Nk, M, (const cd*)S, nullptr, P, n, tw, false, (double*)out, nsm, st));
+    BIE_TRY(launch_synth<double>((const cd*)T, md, (int)Nk, M, (const cd*)S, nullptr, tw, P, n, tw, false, (double*)out, nsm, st));
   } else {
-    launch_twiddles<float>(n, tw, false, st);
-    BIE_TRY(launch_synth<float>((const cd*)T, md, (int)Nk, M, (const cd*)S, nullptr, P, n, tw, false, (float*)out, nsm, st));
+    void* tw32 = (char*)base + kNoAllocScratchBytes;
+    launch_twiddles<double>(n, tw, false, st);
+    if (n >= 32) launch_twiddles<float>(n, tw32, false, st);
+    BIE_TRY(launch_synth<float>((const cd*)T, md, (int)Nk, M, (const cd*)S, nullptr, tw, P, n, n >= 32 ? tw32 : (void*)tw, false, (float*)out, nsm, st));
   }
   BIE_CUDA_TRY(cudaGetLastError());
   // the host index array must outlive its asynchronous copy
