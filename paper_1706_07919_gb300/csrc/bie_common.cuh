@@ -201,6 +201,7 @@ namespace bie {
 // Device memory of a context comes from the stream-ordered allocator on the context's stream
 // (cudaMallocAsync / cudaFreeAsync): freeing and growing buffers never synchronises the device,
 // so contexts on other streams (the scheduler's workers) keep running.
+constexpr int kMaxFieldBatch = 512;  // wavenumbers of one field launch, hence pairs of groups of one (field.cu)
 int dev_alloc(bie_ctx* c, void** p, size_t bytes);
 void dev_free(bie_ctx* c, void* p);
 int ensure_buf(bie_ctx* c, DeviceBuf& b, size_t bytes);

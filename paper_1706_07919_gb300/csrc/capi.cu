@@ -117,7 +117,7 @@ size_t fp64_scratch_bytes(bie_ctx* c, int batch, int n);
 int lu_solve64(bie_ctx* c, const cd* LU, int batch, int n, int ld, int64_t bstride, const int32_t* piv, cd* b,
                int64_t bstride_b);
 int field64(bie_ctx* c, const double* kv, int nk, const cd* surf, const double* xp, int64_t M,
-            const int32_t* foot_elem, const double* foot, cd* T, void* scratch);
+            const int32_t* foot_elem, const double* foot, cd* T, void* scratch, int nsm);
 int pulse_spectrum(bie_ctx* c, const double* s, int64_t P, int n, cd* Sout);
 int synthesize(bie_ctx* c, const cd* T, const int64_t* midx_dev, int nk, int64_t M, const cd* Sp, int64_t P, int n,
                void* out, int out_dtype);
@@ -140,9 +140,9 @@ int mlp_train(bie_ctx* c, const double* k, int64_t nk, const cd* surf, int epoch
 int mlp_predict_api(bie_ctx* c, const double* k, int64_t nk, cd* x0);
 int autotune(bie_ctx* c, const double* k, int64_t nk, const char* cache_path, bie_tune_result* out);
 int field_mixed(bie_ctx* c, const double* hk, const double* kv, int nk, const cd* surf, const double* xp, int64_t M,
-                const int32_t* foot_elem, const double* foot, cd* T, void* scratch, size_t scratch_bytes);
-size_t field_mixed_scratch(bie_ctx* c, const double* hk, int nk, int64_t M);
-size_t field64_scratch(bie_ctx* c, int nk, int64_t M);
+                const int32_t* foot_elem, const double* foot, cd* T, void* scratch, size_t scratch_bytes, int nsm);
+size_t field_mixed_scratch(bie_ctx* c, const double* hk, int nk, int64_t M, int nsm);
+size_t field64_scratch(bie_ctx* c, int nk, int64_t M, int nsm);
 
 static void free_geometry(bie_ctx* c) {
   void* ptrs[] = {c->nodes, c->elems, c->normals, c->bc, c->qgeo, c->ngeo, c->qshape, c->nshape, c->qgeo32,
@@ -684,13 +684,14 @@ int bie_eval_field(bie_ctx* c, const double* xobs, int64_t M, const double* k, i
   const size_t foot_bytes = (size_t)M * (8 * sizeof(double) + sizeof(int32_t)) + 256;
   // up to 512 wavenumbers per launch: the field kernel's grid (points x groups of 16 wavenumbers)
   // then spans many waves of resident CTAs, so the last, partial wave costs little
-  constexpr int64_t kMaxFieldBatch = 512;
+  int nsm = 0;
+  BIE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
   int64_t kb = std::max<int64_t>(1, std::min<int64_t>(Nk, kMaxFieldBatch));
   size_t scratch_bytes = 0;
   for (int64_t k0 = 0; k0 < Nk; k0 += kb) {
     const int nk = (int)std::min<int64_t>(kb, Nk - k0);
-    scratch_bytes = std::max(scratch_bytes, mode == BIE_MODE_MIXED ? field_mixed_scratch(c, k + k0, nk, M)
-                                                                   : field64_scratch(c, nk, M));
+    scratch_bytes = std::max(scratch_bytes, mode == BIE_MODE_MIXED ? field_mixed_scratch(c, k + k0, nk, M, nsm)
+                                                                   : field64_scratch(c, nk, M, nsm));
   }
   BIE_TRY(ensure_buf(c, c->work3, foot_bytes + scratch_bytes + kMaxFieldBatch * sizeof(double) + 4096 + 256));
   double* foot = (double*)c->work3.p;
@@ -720,9 +721,9 @@ int bie_eval_field(bie_ctx* c, const double* xobs, int64_t M, const double* k, i
     }
     cd* T = (cd*)T_out + k0 * M;
     if (mode == BIE_MODE_FP64)
-      BIE_TRY(field64(c, kdev, nk, s, xobs, M, foot_elem, foot, T, scratch));
+      BIE_TRY(field64(c, kdev, nk, s, xobs, M, foot_elem, foot, T, scratch, nsm));
     else
-      BIE_TRY(field_mixed(c, k + k0, kdev, nk, s, xobs, M, foot_elem, foot, T, scratch, scratch_bytes));
+      BIE_TRY(field_mixed(c, k + k0, kdev, nk, s, xobs, M, foot_elem, foot, T, scratch, scratch_bytes, nsm));
   }
   BIE_CUDA_TRY(cudaStreamSynchronize(c->stream));
   return BIE_OK;

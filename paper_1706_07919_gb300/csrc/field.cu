@@ -39,26 +39,62 @@ __global__ void k_interp_q64(const int32_t* __restrict__ elems, int64_t N, int64
 
 constexpr int FT = 128;  // points per CTA and quadrature points per shared tile (FP32 kernels)
 
-// FP64 field.  A CTA evaluates 32 points (one per lane) for a group of F64K wavenumbers over the
-// quadrature points of its share z of `splits`, a quarter of them per warp.  Per (point, quadrature
-// point) pair the geometry is formed once; where the group's wavenumbers are equally spaced to
-// rounding the three phases' sines and cosines are formed at k_0 and at the spacing and rotated to
-// the others (at most F64K - 1 steps of one ulp each, the size of the rounding of k R), else per
-// wavenumber.  Partial sums: the warps' through shared memory, the splits' through `part`
-// [splits][nk][M] and k_field64_sum, each in a fixed order (splits 1: T directly).
-// Bound: the FP64 pipe.  64 wavenumbers, 1000 points, 2048 quadrature points: 51.9 -> 13.6 ms = 60 FP64
+// FP64 field.  A CTA evaluates 32 points (one per lane) for a group of F64K wavenumbers over its share z of
+// `splits` of the quadrature points.  Per (point, quadrature point) pair the geometry is formed once; where
+// the group's wavenumbers are equally spaced to rounding the three phases' sines and cosines are formed at
+// k_0 and at the spacing and rotated to the others (at most F64K - 1 steps of one ulp each, the size of the
+// rounding of k R), else per wavenumber.  The order of the sums does not depend on the points and
+// wavenumbers of a call: the quadrature points are cut into `leaves` (a power of two, by the mesh alone),
+// each the sum of four warps' quarters through shared memory, and the leaves are added by pairs in one
+// binary tree -- the 2^b leaves of a CTA's share here (`stack`: the sums still waiting for their
+// partner, one a level), the shares, a power of two of them, from `part` [splits][nk][M] by
+// k_field64_sum.  With several shares the foot points' values come from k_foot_values64 (p0 [nk][M]), which
+// every share's CTA would otherwise gather anew.
+// Bound: the FP64 pipe.  64 wavenumbers, 1000 points, 2048 quadrature points: 51.9 -> 13.8 ms = 60 FP64
 // instructions an evaluation at the pipe's measured 0.58 T/s (45 of them the rotations and the
 // integrand); wavenumbers without a common spacing 23.4 ms.  Error against 64 bits unchanged.
 constexpr int F64K = 16;
+constexpr int kLeafLevels = 9;
+__device__ __forceinline__ cd field64_value(cd p0, cd sum) {  // P0 + sum / (4 pi)
+  const double inv4pi = 1.0 / (4.0 * kPi);
+  return {fma(sum.re, inv4pi, p0.re), fma(sum.im, inv4pi, p0.im)};
+}
+// P0 re, im, P0' re, im of one wavenumber (surface values P) at point m's foot point
+__device__ __forceinline__ double4 foot_value64(const int32_t* __restrict__ elems, int64_t N, const cd* __restrict__ P,
+                                                const int32_t* __restrict__ foot_elem, const double* __restrict__ foot,
+                                                int64_t m) {
+  const double fxi = foot[8 * m + 6], feta = foot[8 * m + 7];
+  const double L1 = 1.0 - fxi - feta;
+  const double Nv[6] = {L1 * (2 * L1 - 1), fxi * (2 * fxi - 1), feta * (2 * feta - 1), 4 * L1 * fxi, 4 * fxi * feta,
+                         4 * feta * L1};
+  const int32_t* el = elems + 6 * (int64_t)foot_elem[m];
+  double4 v = make_double4(0.0, 0.0, 0.0, 0.0);
+  for (int a = 0; a < 6; ++a) {
+    const cd x = P[el[a]], w = P[N + el[a]];
+    v.x += Nv[a] * x.re; v.y += Nv[a] * x.im;
+    v.z += Nv[a] * w.re; v.w += Nv[a] * w.im;
+  }
+  return v;
+}
+__global__ void k_foot_values64(const int32_t* __restrict__ elems, int64_t N, const cd* __restrict__ surf,
+                                const int32_t* __restrict__ foot_elem, const double* __restrict__ foot, int64_t M,
+                                double4* __restrict__ p0) {
+  const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (m < M) p0[(int64_t)blockIdx.y * M + m] = foot_value64(elems, N, surf + (int64_t)blockIdx.y * 2 * N, foot_elem, foot, m);
+}
+
 __global__ void __launch_bounds__(128, 2) k_field64(const int32_t* __restrict__ elems, int64_t N, int64_t EQ,
                                                     const double* __restrict__ qgeo, const cd* __restrict__ Pq,
                                                     const cd* __restrict__ Pnq, const cd* __restrict__ surf,
                                                     const double* __restrict__ xp, int64_t M,
                                                     const int32_t* __restrict__ foot_elem, const double* __restrict__ foot,
-                                                    const double* __restrict__ kv, int nk, int splits, cd* __restrict__ part,
+                                                    const double* __restrict__ kv, int nk, int splits, int leaves,
+                                                    const double4* __restrict__ p0, cd* __restrict__ part,
                                                     cd* __restrict__ T) {
   __shared__ double4 s0[F64K][32];   // P0 re, im, P0' re, im at each lane's foot point
   __shared__ cd red[4][32];
+  extern __shared__ double2 f64_smem[];
+  cd* stack = reinterpret_cast<cd*>(f64_smem);  // [levels][F64K][32]
   __shared__ double2 sk[F64K];  // k, 1 / k (0 at k = 0)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int kbase = blockIdx.y * F64K, nkb = min(F64K, nk - kbase);
@@ -70,18 +106,7 @@ __global__ void __launch_bounds__(128, 2) k_field64(const int32_t* __restrict__ 
   for (int e = threadIdx.x; e < nkb * 32; e += 128) {
     const int j = e >> 5, t = e & 31;
     const int64_t mm = m0 + t < M ? m0 + t : M - 1;
-    const double fxi = foot[8 * mm + 6], feta = foot[8 * mm + 7];
-    const double L1 = 1.0 - fxi - feta;
-    const double Nv[6] = {L1 * (2 * L1 - 1), fxi * (2 * fxi - 1), feta * (2 * feta - 1), 4 * L1 * fxi, 4 * fxi * feta,
-                          4 * feta * L1};
-    const int32_t* el = elems + 6 * (int64_t)foot_elem[mm];
-    const cd* P = surf + (int64_t)(kbase + j) * 2 * N;
-    double4 v = make_double4(0.0, 0.0, 0.0, 0.0);
-    for (int a = 0; a < 6; ++a) {
-      const cd x = P[el[a]], w = P[N + el[a]];
-      v.x += Nv[a] * x.re; v.y += Nv[a] * x.im;
-      v.z += Nv[a] * w.re; v.w += Nv[a] * w.im;
-    }
+    const double4 v = p0 ? p0[(int64_t)(kbase + j) * M + mm] : foot_value64(elems, N, surf + (int64_t)(kbase + j) * 2 * N, foot_elem, foot, mm);
     s0[j][t] = v;
   }
   __syncthreads();
@@ -95,11 +120,14 @@ __global__ void __launch_bounds__(128, 2) k_field64(const int32_t* __restrict__ 
   const double k0 = kv[kbase], kl = kv[kbase + nkb - 1], dk = nkb > 2 ? (kl - k0) / (nkb - 1) : 0.0;
   bool uniform = nkb > 2;
   for (int j = 1; j < nkb; ++j) uniform &= fabs(kv[kbase + j] - fma((double)j, dk, k0)) <= 2.3e-16 * fabs(kl);
+  const int own = leaves / splits;
+#pragma unroll 1
+  for (int leaf = 0; leaf < own; ++leaf) {
   cd sum[F64K];
 #pragma unroll
   for (int j = 0; j < F64K; ++j) sum[j] = cd{0, 0};
-  const int64_t share = blockIdx.z * 4 + warp;
-  const int64_t qlo = share * EQ / (4 * splits), qhi = (share + 1) * EQ / (4 * splits);
+  const int64_t quarter = ((int64_t)blockIdx.z * own + leaf) * 4 + warp;
+  const int64_t qlo = quarter * EQ / (4 * leaves), qhi = (quarter + 1) * EQ / (4 * leaves);
 #pragma unroll 1
   for (int64_t q = qlo; q < qhi; ++q) {
     const double qx = qgeo[GX * EQ + q], qy = qgeo[GY * EQ + q], qz = qgeo[GZ * EQ + q];
@@ -161,51 +189,84 @@ __global__ void __launch_bounds__(128, 2) k_field64(const int32_t* __restrict__ 
       sum[j].im = fma(Ptr, ddi, fma(Pti, ddr, fma(-gdr, dPi, fma(-gdi, dPr, sum[j].im))));
     }
   }
-  const double inv4pi = 1.0 / (4.0 * kPi);
 #pragma unroll
   for (int j = 0; j < F64K; ++j) {
     if (j >= nkb) break;
     __syncthreads();
     red[warp][lane] = sum[j];
     __syncthreads();
-    if (warp == (j & 3) && m0 + lane < M) {
+    if (warp == (j & 3)) {
       cd t = {0, 0};
       for (int w = 0; w < 4; ++w) t = cadd(t, red[w][lane]);
-      t = cscale(t, inv4pi);
-      if (blockIdx.z == 0) {
-        t.re += s0[j][lane].x;
-        t.im += s0[j][lane].y;
+      int l = 0;
+      for (; (leaf >> l) & 1; ++l) t = cadd(stack[(l * F64K + j) * 32 + lane], t);
+      stack[(l * F64K + j) * 32 + lane] = t;  // (the last leaf's: the share's sum)
+      if (leaf + 1 == own && m0 + lane < M) {
+        const int64_t at = (int64_t)(kbase + j) * M + m0 + lane, n = (int64_t)nk * M;
+        if (splits == 1) T[at] = field64_value(cd{s0[j][lane].x, s0[j][lane].y}, t);
+        else part[blockIdx.z * n + at] = t;
       }
-      (splits > 1 ? part + (int64_t)blockIdx.z * nk * M : T)[(int64_t)(kbase + j) * M + m0 + lane] = t;
     }
+  }
   }
 }
 
-// T = sum over the splits, in order; n = nk M
-__global__ void k_field64_sum(const cd* __restrict__ part, int splits, int64_t n, cd* __restrict__ T) {
+// The shares' sums added by pairs, and the value; n = nk M
+__global__ void k_field64_sum(const cd* __restrict__ part, const double4* __restrict__ p0, int splits, int64_t n,
+                              cd* __restrict__ T) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= n) return;
-  cd v = part[t];
-  for (int z = 1; z < splits; ++z) v = cadd(v, part[z * n + t]);
-  T[t] = v;
+  cd stack[kLeafLevels + 1];
+  for (int z = 0; z < splits; ++z) {
+    cd v = part[z * n + t];
+    bool put = false;
+#pragma unroll
+    for (int l = 0; l <= kLeafLevels; ++l)  // (unrolled: the stack stays in registers)
+      if (!put) {
+        if ((z >> l) & 1) {
+          v = cadd(stack[l], v);
+        } else {
+          stack[l] = v;
+          put = true;
+        }
+      }
+    if (z + 1 == splits) T[t] = field64_value(cd{p0[t].x, p0[t].y}, v);
+  }
 }
 
-// Shares of the quadrature points: sixteen CTAs to an SM (two are resident: a last, partial wave then
-// costs little; with the per-wavenumber phases 4 to an SM measured 27.7 ms, 16 23.4), shares of at
-// least 64 points.
-static int field64_splits(bie_ctx* c, int nk, int64_t M) {
-  const int64_t ctas = (M + 31) / 32 * ((nk + F64K - 1) / F64K), EQ = c->E * c->rule.Q;
-  return (int)std::max<int64_t>(1, std::min<int64_t>((16 * 152 + ctas - 1) / ctas, EQ / 64));
+// Leaves of the sums: as many as leave each 32 quadrature points, 2^kLeafLevels at most.
+static int field64_leaves(bie_ctx* c) {
+  const int64_t EQ = c->E * c->rule.Q;
+  int z = 1;
+  while (z < 1 << kLeafLevels && 2 * z * 32 <= EQ) z *= 2;
+  return z;
+}
+// Shares of the quadrature points: eight to sixty-four CTAs to an SM (two are resident), of the powers of two
+// in between the one whose last, partial wave leaves the least of the SMs idle (1000 points, 64
+// wavenumbers: 14 waves for 13.5 measured 15.8 ms, 27 for 26.9 15.4).
+static int field64_splits(int nk, int64_t M, int nsm, int leaves) {
+  const int64_t ctas = (M + 31) / 32 * ((nk + F64K - 1) / F64K), wave = 2 * nsm;
+  int best = 0;
+  double used = 0.0;
+  for (int z = 1; z <= leaves && (best == 0 || z * ctas <= 64 * nsm); z *= 2) {
+    if (z * ctas < 8 * nsm && z < leaves) continue;
+    const double u = (double)(z * ctas) / (double)((z * ctas + wave - 1) / wave * wave);
+    if (best == 0 || u > 1.01 * used) {
+      best = z;
+      used = u;
+    }
+  }
+  return best;
 }
 // Scratch of field64 in bytes.
-size_t field64_scratch(bie_ctx* c, int nk, int64_t M) {
-  const int z = field64_splits(c, nk, M);
-  return 2 * (size_t)nk * c->E * c->rule.Q * sizeof(cd) + (z > 1 ? (size_t)z * nk * M * sizeof(cd) : 0);
+size_t field64_scratch(bie_ctx* c, int nk, int64_t M, int nsm) {
+  const int z = field64_splits(nk, M, nsm, field64_leaves(c));
+  return 2 * (size_t)nk * c->E * c->rule.Q * sizeof(cd) + (z > 1 ? (size_t)(z + 2) * nk * M * sizeof(cd) : 0);
 }
 
 // Evaluates nk wavenumbers: surf [nk][2][N] -> T [nk][M].  scratch: field64_scratch bytes.
 int field64(bie_ctx* c, const double* kv, int nk, const cd* surf, const double* xp, int64_t M,
-            const int32_t* foot_elem, const double* foot, cd* T, void* scratch) {
+            const int32_t* foot_elem, const double* foot, cd* T, void* scratch, int nsm) {
   const int64_t EQ = c->E * c->rule.Q;
   cd* Pq = (cd*)scratch;
   cd* Pnq = Pq + (int64_t)nk * EQ;
@@ -213,12 +274,22 @@ int field64(bie_ctx* c, const double* kv, int nk, const cd* surf, const double* 
   dim3 gi((unsigned)((EQ + 255) / 256), nk);
   BIE_LAUNCH(k_interp_q64<<<gi, 256, 0, c->stream>>>(c->elems, c->N, c->E, c->rule.Q, c->qshape, surf, Pq, Pnq));
   if (M > 0) {
-    const int splits = field64_splits(c, nk, M);
+    const int leaves = field64_leaves(c), splits = field64_splits(nk, M, nsm, leaves);
+    double4* p0 = nullptr;
+    if (splits > 1) {  // (the foot points' values, then the shares' sums)
+      p0 = reinterpret_cast<double4*>(part);
+      part += 2 * (int64_t)nk * M;
+      BIE_LAUNCH(k_foot_values64<<<dim3((unsigned)((M + 127) / 128), nk), 128, 0, c->stream>>>(c->elems, c->N, surf, foot_elem,
+                                                                                              foot, M, p0));
+    }
+    int levels = 1;
+    while ((leaves / splits) >> levels) ++levels;  // of a share's leaves
     dim3 gf((unsigned)((M + 31) / 32), (unsigned)((nk + F64K - 1) / F64K), (unsigned)splits);
-    BIE_LAUNCH(k_field64<<<gf, 128, 0, c->stream>>>(c->elems, c->N, EQ, c->qgeo, Pq, Pnq, surf, xp, M, foot_elem, foot, kv,
-                                                    nk, splits, part, T));
+    BIE_TRY(set_smem_max(k_field64));
+    BIE_LAUNCH(k_field64<<<gf, 128, (size_t)levels * F64K * 32 * sizeof(cd), c->stream>>>(
+        c->elems, c->N, EQ, c->qgeo, Pq, Pnq, surf, xp, M, foot_elem, foot, kv, nk, splits, leaves, p0, part, T));
     if (splits > 1)
-      BIE_LAUNCH(k_field64_sum<<<(unsigned)((nk * M + 255) / 256), 256, 0, c->stream>>>(part, splits, nk * M, T));
+      BIE_LAUNCH(k_field64_sum<<<(unsigned)((nk * M + 255) / 256), 256, 0, c->stream>>>(part, p0, splits, nk * M, T));
   }
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
@@ -737,7 +808,6 @@ constexpr int FPP = 2 * FPG; // per pair
 
 // The pairs of one launch: pair y holds wavenumbers base[y] .. base[y] + n[y] - 1 (n <= FPP) of the
 // call's list, spaced by dk[y] where the launch takes the rotations.
-constexpr int kMaxFieldBatch = 512;  // wavenumbers of one field_mixed call, hence pairs of one launch
 struct PairList {
   ff dk[kMaxFieldBatch];
   int16_t base[kMaxFieldBatch];
@@ -1087,14 +1157,12 @@ int ensure_mixed_tables(bie_ctx* c);
 // that still give every SM one (M = 3000, 7 wavenumbers: 20 -> 4 ms; M = 1: 3.1 -> 0.1 ms).
 static int launch_pairs(bie_ctx* c, const cd* surf, const double* xp, int64_t M, const int32_t* foot_elem,
                         const double* foot, const double* kv, const PairList& l, int np, bool uni, cd* T,
-                        bool zero, float4* PQ) {
+                        bool zero, float4* PQ, int nsm) {
   if (np == 0) return BIE_OK;
   const int64_t EQ = c->E * c->rule.Q;
   const float far_r2 = (float)far_radius2(c);
   BIE_LAUNCH(k_interp_pair<<<dim3((unsigned)((EQ + 7) / 8), (unsigned)np), 128, 0, c->stream>>>(
       c->elems, c->N, EQ, c->rule.Q, c->qshape, surf, l, PQ));
-  int nsm = 0;
-  BIE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
   int P = 32, W = 4;
   auto ctas = [&](int p) { return (M + p - 1) / p * np; };
   if (ctas(32) < 2 * nsm) {
@@ -1150,10 +1218,9 @@ static std::vector<std::pair<int, int>> field_segments(const double* hk, int nk)
 
 // Whether a segment's single last group of n <= 16 wavenumbers takes the one-group kernel (k_field32c)
 // instead of a pair with an empty second half, whose packed instructions are half wasted.  The
-// one-group kernel's 128-point CTAs take as long for one point as for the 19456 that give every SM
-// one; measured on 23 040 quadrature points at M = 16 384: 26.2 ms against the pair's 28.3 for
+// one-group kernel's 128-point CTAs take as long for one point as for 128 on every SM; measured on 23 040 quadrature points at M = 16 384: 26.2 ms against the pair's 28.3 for
 // n = 16, 19.2 against 13.9 for n = 5 (equal near n = 13); M = 3000, n = 7: 20 against 4 ms.
-static bool scalar_tail(int64_t M, int n) { return M >= 2 * 152 * 128 || (M >= 100 * 152 && n > 12); }
+static bool scalar_tail(int64_t M, int n, int nsm) { return M >= (int64_t)2 * nsm * 128 || (M >= (int64_t)100 * nsm && n > 12); }
 
 // The pairs of wavenumber groups of a list (uniform segments' and the others'), and the scalar
 // kernel's groups (start, length, segment's step or 0).
@@ -1164,14 +1231,14 @@ struct FieldPlan {
   struct Tail { int start, n, uniform; double dk; };
   std::vector<Tail> tails;
 };
-static void field_plan(const double* hk, int nk, int64_t M, FieldPlan& f) {
+static void field_plan(const double* hk, int nk, int64_t M, int nsm, FieldPlan& f) {
   for (const auto& sg : field_segments(hk, nk)) {
     const int r0 = sg.first, n = sg.second > 0 ? sg.second : -sg.second;
     const bool uniform = sg.second > 0;
     const double dk = uniform ? hk[r0 + 1] - hk[r0] : 0.0;
     for (int i = 0; i < n; i += FPP) {
       const int m = std::min(FPP, n - i);
-      if (m <= FPG && scalar_tail(M, m)) {
+      if (m <= FPG && scalar_tail(M, m, nsm)) {
         f.tails.push_back({r0 + i, m, uniform ? 1 : 0, dk});
         continue;
       }
@@ -1187,12 +1254,12 @@ static void field_plan(const double* hk, int nk, int64_t M, FieldPlan& f) {
 }
 
 // Scratch of field_mixed in bytes for nk wavenumbers at M points.
-size_t field_mixed_scratch(bie_ctx* c, const double* hk, int nk, int64_t M) {
+size_t field_mixed_scratch(bie_ctx* c, const double* hk, int nk, int64_t M, int nsm) {
   const size_t EQ = (size_t)(c->E * c->rule.Q);
   size_t values = 2 * (size_t)nk * EQ * sizeof(cf);  // P and P' at the quadrature points
   if (c->field_accurate_phase && c->field_variant == 2) {
     FieldPlan f;
-    field_plan(hk, nk, M, f);
+    field_plan(hk, nk, M, nsm, f);
     values = (f.tails.empty() ? 0 : 2 * FPG * EQ * sizeof(cf)) + (size_t)std::max(f.nuni, f.ngen) * EQ * FPP * 2 * sizeof(cf);
   }
   return values + 512;
@@ -1200,10 +1267,10 @@ size_t field_mixed_scratch(bie_ctx* c, const double* hk, int nk, int64_t M) {
 
 // Evaluates nk <= kMaxFieldBatch wavenumbers (hk on the host, kv the same on the device).
 int field_mixed(bie_ctx* c, const double* hk, const double* kv, int nk, const cd* surf, const double* xp, int64_t M,
-                const int32_t* foot_elem, const double* foot, cd* T, void* scratch, size_t scratch_bytes) {
+                const int32_t* foot_elem, const double* foot, cd* T, void* scratch, size_t scratch_bytes, int nsm) {
   BIE_TRY(ensure_mixed_tables(c));
   const int64_t EQ = c->E * c->rule.Q;
-  if (nk > kMaxFieldBatch || field_mixed_scratch(c, hk, nk, M) > scratch_bytes)
+  if (nk > kMaxFieldBatch || field_mixed_scratch(c, hk, nk, M, nsm) > scratch_bytes)
     return fail(BIE_ERR_STATE, "field scratch too small");
   if (M <= 0) return BIE_OK;
   cf* Pq = (cf*)scratch;
@@ -1227,11 +1294,11 @@ int field_mixed(bie_ctx* c, const double* hk, const double* kv, int nk, const cd
                                                           foot, kv, T, tp));
   } else if (c->field_variant == 2) {
     FieldPlan f;
-    field_plan(hk, nk, M, f);
+    field_plan(hk, nk, M, nsm, f);
     float4* PQ = (float4*)scratch;
     if (!f.tails.empty()) PQ = (float4*)(((uintptr_t)(Pq + 2 * FPG * EQ) + 255) & ~(uintptr_t)255);
-    BIE_TRY(launch_pairs(c, surf, xp, M, foot_elem, foot, kv, f.uni, f.nuni, true, T, f.zuni, PQ));
-    BIE_TRY(launch_pairs(c, surf, xp, M, foot_elem, foot, kv, f.gen, f.ngen, false, T, f.zgen, PQ));
+    BIE_TRY(launch_pairs(c, surf, xp, M, foot_elem, foot, kv, f.uni, f.nuni, true, T, f.zuni, PQ, nsm));
+    BIE_TRY(launch_pairs(c, surf, xp, M, foot_elem, foot, kv, f.gen, f.ngen, false, T, f.zgen, PQ, nsm));
     for (const auto& t : f.tails) {
       const cf* Pnq = interp(t.start, t.n);
       bool zero = false;

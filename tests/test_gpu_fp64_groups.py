@@ -69,3 +69,28 @@ def test_fields_in_groups_match_single_fields(nk, M, uniform):
         ref = sol.eval_field(x, ks[i:i + 1], s[i:i + 1].contiguous(), B.BIE_MODE_FP64).cpu().numpy()[0]
         assert np.abs(got[i] - ref).max() <= 1e-12 * np.abs(ref).max() + 1e-12 * np.abs(surf).max()
     sol.close()
+
+
+@pytest.mark.parametrize("mesh", ["66 nodes", "258 nodes", "1002 nodes"])
+def test_fp64_field_of_a_point_is_its_own(mesh):
+    """A point's FP64 values do not depend on the other points of the call, nor on further groups of 16
+    wavenumbers: one order of the sums, whichever share of the quadrature points a CTA takes."""
+    import torch
+    from paper_1706_07919_gb300 import Solver
+    from paper_1706_07919_gb300 import binding as B
+    from workloads import ico_sphere, octa_sphere
+
+    m = {"66 nodes": octa_sphere(1), "258 nodes": octa_sphere(2), "1002 nodes": ico_sphere(5)}[mesh]
+    sol = Solver(0)
+    sol.set_geometry(m.nodes, m.elems, m.normals, m.bc)
+    g = torch.Generator("cuda:0").manual_seed(m.N)
+    x = torch.randn((3001, 3), dtype=torch.float64, device="cuda:0", generator=g)
+    x *= (1.05 + torch.rand((3001, 1), dtype=torch.float64, device="cuda:0", generator=g)) / x.norm(dim=1, keepdim=True)
+    ks = 0.4 + 0.07 * np.arange(48)
+    surf = torch.randn((48, 2, m.N), dtype=torch.complex128, device="cuda:0", generator=g)
+    full = sol.eval_field(x, ks, surf, B.BIE_MODE_FP64)
+    for M in (1, 2, 33, 500):
+        for nk in (16, 48):
+            part = sol.eval_field(x[:M].contiguous(), ks[:nk], surf[:nk].contiguous(), B.BIE_MODE_FP64)
+            assert torch.equal(torch.view_as_real(part), torch.view_as_real(full[:nk, :M]))
+    sol.close()
