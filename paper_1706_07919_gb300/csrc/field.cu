@@ -806,7 +806,7 @@ __global__ void __launch_bounds__(TP, MINB) k_field32c(const int32_t* __restrict
 constexpr int FPG = 16;      // wavenumbers per group
 constexpr int FPP = 2 * FPG; // per pair
 
-// The pairs of one launch: pair y holds wavenumbers base[y] .. base[y] + n[y] - 1 (n <= FPP) of the
+// The pairs of a call, launched from y0 on (field_pairs_max of them at a time): pair y holds wavenumbers base[y] .. base[y] + n[y] - 1 (n <= FPP) of the
 // call's list, spaced by dk[y] where the launch takes the rotations.
 struct PairList {
   ff dk[kMaxFieldBatch];
@@ -819,9 +819,9 @@ struct PairList {
 // grid (ceil(EQ / 8), pairs), block 128: 16 threads (j) per point.
 __global__ void k_interp_pair(const int32_t* __restrict__ elems, int64_t N, int64_t EQ, int Q,
                               const double* __restrict__ qshape, const cd* __restrict__ surf,
-                              const __grid_constant__ PairList pairs, float4* __restrict__ PQ) {
+                              const __grid_constant__ PairList pairs, int y0, float4* __restrict__ PQ) {
   const int j = threadIdx.x & (FPG - 1);
-  const int kbase = pairs.base[blockIdx.y], nk = pairs.n[blockIdx.y];
+  const int kbase = pairs.base[y0 + blockIdx.y], nk = pairs.n[y0 + blockIdx.y];
   const int64_t p = blockIdx.x * (int64_t)(blockDim.x / FPG) + threadIdx.x / FPG;
   if (p >= EQ) return;
   const int64_t e = p / Q;
@@ -1013,7 +1013,7 @@ __global__ void __launch_bounds__(384, 1) k_field_pair(const int32_t* __restrict
                                                        const cd* __restrict__ surf, const double* __restrict__ xp,
                                                        int64_t M, const int32_t* __restrict__ foot_elem,
                                                        const double* __restrict__ foot, const double* __restrict__ kv,
-                                                       const __grid_constant__ PairList pairs, int P_, cd* __restrict__ T,
+                                                       const __grid_constant__ PairList pairs, int y0, int P_, cd* __restrict__ T,
                                                        float far_r2) {
   constexpr int UT = 8;
   const int P = DIRECT ? P_ : 32;
@@ -1026,10 +1026,10 @@ __global__ void __launch_bounds__(384, 1) k_field_pair(const int32_t* __restrict
   float2* sr = skl + FPG;                                // [W][FPG][2][32]: the runs' sums
   float4* sg = (float4*)(sr + W * FPG * 2 * 32) + warp * UT * (4 + 2 * FPG);  // this warp's tile: [UT][4]
   float4* sq = sg + UT * 4;                              // [UT][FPG][2]
-  const int kbase = pairs.base[blockIdx.y], nk = pairs.n[blockIdx.y], nj = min(nk, FPG);
+  const int kbase = pairs.base[y0 + blockIdx.y], nk = pairs.n[y0 + blockIdx.y], nj = min(nk, FPG);
   const int64_t m0 = (int64_t)blockIdx.x * P;
   ff dk = {0.f, 0.f};
-  if (UNI) dk = pairs.dk[blockIdx.y];
+  if (UNI) dk = pairs.dk[y0 + blockIdx.y];
   if (tid < FPG) {
     ff k[2] = {{0.f, 0.f}, {0.f, 0.f}};
     float ki[2] = {0.f, 0.f};
@@ -1151,18 +1151,17 @@ static void launch_field32c(bie_ctx* c, int64_t EQ, const cf* Pq, const cf* Pnq,
 
 int ensure_mixed_tables(bie_ctx* c);
 
-// The pairs of `l` (np of them) by k_field_pair.  How the points and runs are laid out: with at least
+// The pairs y0 .. y0 + np - 1 of `l` by k_field_pair.  How the points and runs are laid out: with at least
 // two CTAs of 32 points and 4 warps to an SM (three are resident) that layout; fewer points leave
 // SMs without work, so a CTA takes 12 warps (one CTA fills its SM's registers) and the most points
 // that still give every SM one (M = 3000, 7 wavenumbers: 20 -> 4 ms; M = 1: 3.1 -> 0.1 ms).
 static int launch_pairs(bie_ctx* c, const cd* surf, const double* xp, int64_t M, const int32_t* foot_elem,
-                        const double* foot, const double* kv, const PairList& l, int np, bool uni, cd* T,
+                        const double* foot, const double* kv, const PairList& l, int y0, int np, bool uni, cd* T,
                         bool zero, float4* PQ, int nsm) {
-  if (np == 0) return BIE_OK;
   const int64_t EQ = c->E * c->rule.Q;
   const float far_r2 = (float)far_radius2(c);
   BIE_LAUNCH(k_interp_pair<<<dim3((unsigned)((EQ + 7) / 8), (unsigned)np), 128, 0, c->stream>>>(
-      c->elems, c->N, EQ, c->rule.Q, c->qshape, surf, l, PQ));
+      c->elems, c->N, EQ, c->rule.Q, c->qshape, surf, l, y0, PQ));
   int P = 32, W = 4;
   auto ctas = [&](int p) { return (M + p - 1) / p * np; };
   if (ctas(32) < 2 * nsm) {
@@ -1176,7 +1175,7 @@ static int launch_pairs(bie_ctx* c, const cd* surf, const double* xp, int64_t M,
   auto go = [&](auto kernel) -> int {
     BIE_TRY(set_smem_max(kernel));
     BIE_LAUNCH(kernel<<<g, 32 * W, smem, c->stream>>>(c->elems, c->N, EQ, c->qgeo32, PQ, surf, xp, M, foot_elem, foot, kv, l,
-                                                      P, T, far_r2));
+                                                      y0, P, T, far_r2));
     return BIE_OK;
   };
   if (P == 32) {
@@ -1253,6 +1252,11 @@ static void field_plan(const double* hk, int nk, int64_t M, int nsm, FieldPlan& 
   }
 }
 
+// Pairs of one launch: one for every 16 wavenumbers of the list, twice what full pairs take.  A list of short runs makes
+// more, each with a full pair's scratch however few its wavenumbers: they follow one another through
+// the same scratch.
+static int field_pairs_max(int nk) { return std::max(1, (nk + FPG - 1) / FPG); }
+
 // Scratch of field_mixed in bytes for nk wavenumbers at M points.
 size_t field_mixed_scratch(bie_ctx* c, const double* hk, int nk, int64_t M, int nsm) {
   const size_t EQ = (size_t)(c->E * c->rule.Q);
@@ -1260,7 +1264,7 @@ size_t field_mixed_scratch(bie_ctx* c, const double* hk, int nk, int64_t M, int 
   if (c->field_accurate_phase && c->field_variant == 2) {
     FieldPlan f;
     field_plan(hk, nk, M, nsm, f);
-    values = (f.tails.empty() ? 0 : 2 * FPG * EQ * sizeof(cf)) + (size_t)std::max(f.nuni, f.ngen) * EQ * FPP * 2 * sizeof(cf);
+    values = (f.tails.empty() ? 0 : 2 * FPG * EQ * sizeof(cf)) + (size_t)std::min(field_pairs_max(nk), std::max(f.nuni, f.ngen)) * EQ * FPP * 2 * sizeof(cf);
   }
   return values + 512;
 }
@@ -1297,8 +1301,11 @@ int field_mixed(bie_ctx* c, const double* hk, const double* kv, int nk, const cd
     field_plan(hk, nk, M, nsm, f);
     float4* PQ = (float4*)scratch;
     if (!f.tails.empty()) PQ = (float4*)(((uintptr_t)(Pq + 2 * FPG * EQ) + 255) & ~(uintptr_t)255);
-    BIE_TRY(launch_pairs(c, surf, xp, M, foot_elem, foot, kv, f.uni, f.nuni, true, T, f.zuni, PQ, nsm));
-    BIE_TRY(launch_pairs(c, surf, xp, M, foot_elem, foot, kv, f.gen, f.ngen, false, T, f.zgen, PQ, nsm));
+    const int most = field_pairs_max(nk);
+    for (int uni = 1; uni >= 0; --uni)
+      for (int y0 = 0, np = uni ? f.nuni : f.ngen; y0 < np; y0 += most)
+        BIE_TRY(launch_pairs(c, surf, xp, M, foot_elem, foot, kv, uni ? f.uni : f.gen, y0, std::min(most, np - y0), uni != 0, T,
+                             uni ? f.zuni : f.zgen, PQ, nsm));
     for (const auto& t : f.tails) {
       const cf* Pnq = interp(t.start, t.n);
       bool zero = false;

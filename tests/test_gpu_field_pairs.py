@@ -61,3 +61,30 @@ def test_one_group_tail_at_many_points():
         sol.set_option("field.variant", 2)
         assert torch.equal(a, sol.eval_field(x, k, surf, B.BIE_MODE_MIXED))
     sol.close()
+
+
+def test_many_short_runs_take_bounded_scratch():
+    """128 equally spaced runs of 4 wavenumbers: the scratch stays that of other lists of 512 (32 bytes a
+    wavenumber and quadrature point, and the rest below 64 MB), and the values are the one-group kernel's."""
+    import torch
+    from paper_1706_07919_gb300 import Solver
+    from paper_1706_07919_gb300 import binding as B
+    from workloads import ico_sphere
+
+    mesh = ico_sphere(8)  # 20 480 quadrature points
+    k = np.concatenate([i + 0.1 * np.arange(1, 5) for i in range(128)]) / 16
+    x = torch.tensor(shell_points(40, 1.3, 3.0, seed=2), dtype=torch.float64, device="cuda:0")
+    g = torch.Generator("cuda:0").manual_seed(1)
+    surf = torch.randn((len(k), 2, mesh.N), dtype=torch.complex128, device="cuda:0", generator=g)
+    out = torch.empty((len(k), 40), dtype=torch.complex128, device="cuda:0")
+    sol = Solver(0)
+    sol.set_geometry(mesh.nodes, mesh.elems, mesh.normals, mesh.bc)
+    sol.eval_field(x, k[:4], surf[:4], B.BIE_MODE_MIXED)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    sol.eval_field(x, k, surf, B.BIE_MODE_MIXED, out=out)
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] <= 32 * len(k) * 16 * mesh.elems.shape[0] + (64 << 20)
+    sol.set_option("field.variant", 1)
+    assert torch.equal(out, sol.eval_field(x, k, surf, B.BIE_MODE_MIXED))
+    sol.close()
