@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(256) k_leaf_update(Cx<S>* __restrict__ A, int6
 // for small batches, instead of product by product.  (Taller panels of small batches fix the other
 // order of the U block's fused products, leaf 0.)  The refinement's result moves by up to 1e-9 with
 // the factor's rounding: which of the forms a panel takes depends on the batch, the rows and the
-// number of SMs alone (panel_cluster), not on the cluster.
+// number of SMs alone (panel_cluster), not on the cluster; so does the width of the leaves.
 // The key of a candidate is |a|^2's bits plus one, 0 for none.  In FP64 the record also carries 1 / |a|^2, formed
 // by the candidate's warp alone (every warp of every CTA would take the division's FP64 instructions
 // otherwise); the quotients take one correction each and round once.  Two FP64 solves of N = 2884 in all:
@@ -1166,31 +1166,43 @@ static int panel_cluster(bie_ctx* c, Cx<S>* A, int batch, int n, int ld, int64_t
   // the cluster: fewest rounds of resident clusters, then the most CTAs; sizes between the powers of two
   // only where those take two rounds (a cluster stays within one group of SMs, which leaves some of them
   // idle beside 8 or 16 CTAs): 40 systems of N = 5010 72.0 -> 66.8 ms
-  int best_cl = 0, best_ch = 0, best_rounds = 0;
-  for (const int cl : {16, 8, 4, 2, 1, 12, 9, 7, 6, 5, 3}) {
-    if (cl == 12 && best_rounds == 1) break;
+  int best_cl = 0, best_ch = 0, best_lw = 0, best_rounds = 0;
+  auto consider = [&](int cl, int lw) -> int {
     const int ch = std::max(pcl::PW, ((rows + cl - 1) / cl + 31) / 32 * 32);
-    if (cl > 1 && (int64_t)(cl / 2) * ch >= rows) continue;  // half as many CTAs hold the rows
-    if (cl == 1 && rows > pcl::PW) continue;
-    if (pcl::smem_bytes<S>(lw_max, ch) > limit) continue;
+    if (cl > 1 && (int64_t)(cl / 2) * ch >= rows) return BIE_OK;  // half as many CTAs hold the rows
+    if (cl == 1 && rows > pcl::PW) return BIE_OK;
+    if (pcl::smem_bytes<S>(lw, ch) > limit) return BIE_OK;
     cfg.gridDim = dim3((unsigned)(batch * cl));
-    cfg.dynamicSmemBytes = pcl::smem_bytes<S>(lw_max, ch);
+    cfg.dynamicSmemBytes = pcl::smem_bytes<S>(lw, ch);
     at[0].val.clusterDim.x = (unsigned)cl;
     int active = 0;
     BIE_CUDA_TRY(cudaOccupancyMaxActiveClusters(&active, k_panel_cluster<S>, &cfg));
-    if (active < 1) continue;
+    if (active < 1) return BIE_OK;
     const int rounds = (batch + active - 1) / active;
     if (best_cl == 0 || rounds < best_rounds) {
       best_cl = cl;
       best_ch = ch;
+      best_lw = lw;
       best_rounds = rounds;
     }
-  }
+    return BIE_OK;
+  };
+  for (const int cl : {16, 8, 4, 2, 1}) BIE_TRY(consider(cl, lw_max));
+  if (best_rounds != 1)
+    for (const int cl : {12, 9, 7, 6, 5, 3}) BIE_TRY(consider(cl, lw_max));
+  // FP32 panels in two rounds: one round of clusters that hold eight columns of their rows costs less (a
+  // leaf's own costs, twice as often, are 5 % of a panel's time): 9 / 18 systems of N = 20 544, whose sixteen
+  // columns only 13 CTAs and more hold, 509 / 1019 -> 493 / 985 ms; 14 of N = 16 050 375.9 -> 373.6
+  if (sizeof(S) == 4 && !leaf && best_rounds > 1 && lw_max > 8)
+    for (const int cl : {12, 10, 9, 8, 7, 6, 5, 4, 3}) {
+      if (best_rounds == 1) break;
+      BIE_TRY(consider(cl, 8));
+    }
   if (best_cl == 0 || best_rounds > (share >= 2 ? 2 : 1)) return BIE_OK;
   cfg.gridDim = dim3((unsigned)(batch * best_cl));
-  cfg.dynamicSmemBytes = pcl::smem_bytes<S>(lw_max, best_ch);
+  cfg.dynamicSmemBytes = pcl::smem_bytes<S>(best_lw, best_ch);
   at[0].val.clusterDim.x = (unsigned)best_cl;
-  const int lw = std::min(lw_max, w), pend = std::min(p0 + w, n);
+  const int lw = std::min(best_lw, w), pend = std::min(p0 + w, n);
   if (sizeof(S) == 4) {
     count_launch();
     BIE_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_panel_cluster<S>, A, bstride, n, ld, p0, w, p0, pend, lw, best_ch, sum_first,
