@@ -550,7 +550,7 @@ def run_large(args, dev, stream, peaks=None):
                 "frac": ph["systems"] * (8.0 / 3.0) * float(w.mesh.N) ** 3 / (ph["factor_ms"] * 1e-3) / 1e12
                         / peaks["tf32_tflops"],
                 "note": "(8/3) N^3 per system over the factorisation phase (CUDA events), blocked LU with "
-                        "cooperative panels, against the tcgen05 TF32 rate measured in the same run"},
+                        "cluster panels, against the tcgen05 TF32 rate measured in the same run"},
             "solve_kernel_launches": int(solve_launches)}
 
 
@@ -761,7 +761,7 @@ def run_case(args):
     `step` runs one benchmark step once (cold: the geometry tables are built inside it); `lattice`
     solves one batch of the lattice (k = 0 and 8 wavenumbers, N = 20 544) with phase timing;
     `lu_n8004` solves two wavenumbers on two spheres of 4002 nodes (N = 8004, deferred block 512,
-    cooperative panels; a few GB on the device)."""
+    cluster panels; a few GB on the device)."""
     import torch
 
     import __graft_entry__

@@ -190,7 +190,7 @@ __global__ void k_known_q64(const int32_t* __restrict__ elems, const int32_t* __
 // Bound: the FP64 pipe (one warp instruction in 16 cycles of an SM).  64 wavenumbers at N = 258
 // (KB = 4): 27.6 -> 5.4 ms = 92 FP64 instructions an evaluation, where the one-wavenumber kernel had
 // 180 and two thirds of its lanes idle (colours of a dozen elements); two at N = 2884 (KB = 2) 39.0 ->
-// 27.5 ms.
+// 26.3 ms.
 // grid (N, ceil(nk / KB)); block 128.  The rows accumulate in shared memory, KB * N cd, or with GROW
 // (large N, KB = 1) in A.
 template <int KB, bool GROW>

@@ -224,7 +224,7 @@ int upload_geometry_tables(bie_ctx* c) {
 // one element shares a node with) in conflict, a colour is always free once C > E / cap + D, so
 // the retry loop (C + 1 after a failure) ends.
 constexpr int kColourCap = 64;
-constexpr int64_t kWinMax = 3200;  // nodes of a column window: 2 rows x 2 wavenumbers x 3200 x 8 B = 100 KB
+constexpr int64_t kWinMax = 3200;  // nodes of a column window: one row, 2 wavenumbers x 3200 x 8 B = 50 KB, four CTAs an SM
 int build_colouring(bie_ctx* c) {
   const int64_t N = c->N, E = c->E;
   std::vector<std::vector<int32_t>> n2e(N);

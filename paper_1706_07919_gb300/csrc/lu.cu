@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(256) k_leaf_update(Cx<S>* __restrict__ A, int6
 // cluster is read with L2-coherent loads after a cluster barrier (release / acquire).
 // Bound: the latency of a column (a CTA barrier, the remote stores, a cluster barrier); in FP64 the
 // rows' FP64 instructions.  N = 2884, two systems in FP64: 72.6 ms of one-CTA leaves and their updates ->
-// 19.9 ms, the panels' other columns updated over all SMs (29.3 ms inside the cluster).
+// 17.1 ms, the panels' other columns updated over all SMs (29.3 ms inside the cluster).
 // The pivots and the factor do not depend on the cluster.  In FP32 every entry goes through the operations of
 // the one-CTA leaf (k_leaf) in its order, so that for panels of up to 1536 rows (leaf, where that kernel
 // takes 16 columns) the factor is its bit for bit; in FP64 the pivots are chosen as there, the products
