@@ -119,7 +119,8 @@ int lu_solve64(bie_ctx* c, const cd* LU, int batch, int n, int ld, int64_t bstri
 int field64(bie_ctx* c, const double* kv, int nk, const cd* surf, const double* xp, int64_t M,
             const int32_t* foot_elem, const double* foot, cd* T, void* scratch, int nsm);
 int pulse_spectrum(bie_ctx* c, const double* s, int64_t P, int n, cd* Sout);
-int synthesize(bie_ctx* c, const cd* T, const int64_t* midx_dev, int nk, int64_t M, const cd* Sp, int64_t P, int n,
+int low_frequencies(const int64_t* midx, int64_t nk, int64_t n);
+int synthesize(bie_ctx* c, const cd* T, const int64_t* midx_dev, int nk, int low, int64_t M, const cd* Sp, int64_t P, int n,
                void* out, int out_dtype);
 int top_frequencies(bie_ctx* c, const cd* S, int64_t P, int nm, int K, int64_t* midx_dev);
 int solve_fp64_linear(bie_ctx* c, const double* k, int64_t Nk, cd* surf_out, bie_report* rep);
@@ -756,7 +757,7 @@ int bie_synthesize(bie_ctx* c, const void* T, const int64_t* midx, int64_t Nk, i
   BIE_TRY(ensure_buf(c, c->work3, (size_t)std::max<int64_t>(Nk, 1) * sizeof(int64_t)));
   int64_t* md = (int64_t*)c->work3.p;
   if (Nk > 0) BIE_CUDA_TRY(cudaMemcpyAsync(md, midx, Nk * sizeof(int64_t), cudaMemcpyHostToDevice, c->stream));
-  BIE_TRY(synthesize(c, (const cd*)T, md, (int)Nk, M, (const cd*)S, P, (int)Nt, out, out_dtype));
+  BIE_TRY(synthesize(c, (const cd*)T, md, (int)Nk, low_frequencies(midx, Nk, Nt), M, (const cd*)S, P, (int)Nt, out, out_dtype));
   BIE_CUDA_TRY(cudaStreamSynchronize(c->stream));
   return BIE_OK;
 }

@@ -26,9 +26,10 @@
 // 128) B with B^T rows 2 c and 2 c + 1 = [ur, -ui], [ui, ur].
 // Bound: the chain of a tile of 128 x 64 reals -- operands, 360 MMAs, the epilogue's FP64 instructions (four
 // an entry) and rows of A22 -- of which only the next operands overlap (eight accumulators fill the tensor
-// memory): FP64 pipe 30 % busy, tensor pipe 21 %.  Two systems of N = 2884: the updates 189 ms on the FP64 pipe (0.67 of 1.1 TFLOP/s) -> 16.3 ms with the splitting (7.8 TFLOP/s of the
-// products it replaces); error of the solutions against 64 bits 9.0e-15 -> 8.7e-15.  Seven digits without
-// the bits measured 13.2 ms, but lost 2^g on panels graded by 2^g.
+// memory): FP64 pipe 30 % busy, tensor pipe 21 %.  Two systems of N = 2884: the updates 189 ms on the FP64
+// pipe (0.67 of 1.1 TFLOP/s) -> 16.3 ms with the splitting (7.8 TFLOP/s of the products it replaces); error
+// of the solutions against 64 bits 9.0e-15 -> 8.7e-15.  Seven digits without the bits measured 13.2 ms, but
+// lost 2^g on panels graded by 2^g.
 #include "tcgen05.cuh"
 
 #include <algorithm>

@@ -4,8 +4,9 @@
 //   spectrum:  S[p][m] = sum_n s[p][n] exp(+2 pi i m n / Nt) = conj(FFT(s))_m  (real s)
 //   synthesis: out[p][x][n] = (1/Nt) Re sum_m c_m exp(-2 pi i m n / Nt),  c_m = w_m S[p][m] T[m][x],
 //              w_0 = w_{Nt/2} = 1, else 2 (the m > Nt/2 half is the complex conjugate).
-// Spectra and the shortest signals: one CTA transforms one signal in shared memory with a Stockham
-// (self-sorting) radix-2 FFT; longer signals by k_synth_real.
+// Spectra, and the shortest or fewest signals: one CTA transforms one signal in shared memory with a Stockham
+// (self-sorting) radix-2 FFT; others by k_synth_real.
+#include <algorithm>
 #include <mutex>
 
 #include "bie_common.cuh"
@@ -62,7 +63,7 @@ __global__ void k_pulse_spectrum(const double* __restrict__ s, int n, const doub
   for (int t = threadIdx.x; t <= n / 2; t += blockDim.x) o[t] = {(double)X[t].re, -(double)X[t].im};
 }
 
-// Synthesis of signals of fewer than 32 samples; grid: (M, P), one signal per CTA.
+// Synthesis of the shortest or fewest signals (synth_radix2); grid: (M, P), one signal per CTA.
 template <class S, class O>
 __global__ void k_synth(const cd* __restrict__ T, const int64_t* __restrict__ midx, int nk, int64_t M,
                         const cd* __restrict__ Sp, int n, const double2* __restrict__ tw, O* __restrict__ out) {
@@ -87,7 +88,7 @@ __global__ void k_synth(const cd* __restrict__ T, const int64_t* __restrict__ mi
   for (int t = threadIdx.x; t < n; t += blockDim.x) o[t] = (O)(X[t].re * inv);
 }
 
-// ---- synthesis of signals of 32 samples and more ------------------------------------------------
+// ---- synthesis of many or long signals ------------------------------------------------
 // A real signal of n samples is one complex transform of h = n / 2 values,
 //   out[2 j] + i out[2 j + 1] = sum_k Z_k exp(-2 pi i j k / h),
 //   Z_k = H_k (1 + i w_k) + conj(H_{h-k} (1 - i w_{h-k})),  w_k = exp(-2 pi i k / n),
@@ -194,21 +195,10 @@ inline int twiddle_count(int n) {  // table entries, pass factors included
   for (int Ns = pass_radix0(L); Ns < h; Ns <<= 4) c += 16 * Ns;
   return c;
 }
-template <class S>
-__global__ void k_twiddles_of(int n, int R0, int count, C2<S>* tw) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  const int h = n / 2;
-  double x = 2.0 * (double)i / (double)n;
-  int at = i - h, Ns = R0;
-  while (at >= 16 * Ns && at >= 0) {
-    at -= 16 * Ns;
-    Ns <<= 4;
-  }
-  if (at >= 0) x = 2.0 * (double)((at / Ns) * (at % Ns)) / (double)(16 * Ns);
+__device__ __forceinline__ double2 half_twiddle(int m, int n) {  // exp(-2 pi i m / n)
   double s, c;
-  sincospi(x, &s, &c);
-  tw[i] = {(S)c, (S)(-s)};
+  sincospi(2.0 * (double)m / (double)n, &s, &c);
+  return make_double2(c, -s);
 }
 template <class S> __device__ __forceinline__ C2<S> twiddle(const C2<S>* __restrict__ tw, int i, int h) {
   const C2<S> w = tw[i & (h - 1)];  // i < 2 h = n: the second half is the first negated
@@ -227,22 +217,43 @@ __device__ __forceinline__ cd plus_iw(cd a, double2 w) {
 __device__ __forceinline__ cd minus_iw(cd a, double2 w) {
   return {fma(w.x, a.im, fma(w.y, a.re, a.re)), fma(-w.x, a.re, fma(w.y, a.im, a.im))};
 }
-__device__ __forceinline__ double2 half_twiddle(int m, int n) {  // exp(-2 pi i m / n)
-  double s, c;
-  sincospi(2.0 * (double)m / (double)n, &s, &c);
-  return make_double2(c, -s);
-}
-// spectra of P pulses, [P][h + 1]: out[..][2] = S (1 + i w) / n, S (1 - i w) / n; for m = 0 and h: S / n, 0
-__global__ void k_split_spectra(const cd* __restrict__ Sp, int64_t count, int n, float4* __restrict__ out) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= count) return;
-  const int h = n / 2, m = (int)(t % (h + 1));
+// What a call prepares, in one launch: `count` entries of tw; w64 (unless NULL) [h]; and of `ns` values of
+// Sp, spectra [..][h + 1], the factors sp[..][2] = S (1 + i w) / n, S (1 - i w) / n -- for m = 0 and h: S / n, 0.
+template <class S>
+__global__ void k_synth_tables(int n, int R0, int count, C2<S>* __restrict__ tw, double2* __restrict__ w64,
+                               const cd* __restrict__ Sp, int64_t ns, float4* __restrict__ sp) {
+  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int h = n / 2;
+  if (i < count) {
+    int m = (int)i, N = n, at = (int)i - h, Ns = R0;
+    while (at >= 16 * Ns) {
+      at -= 16 * Ns;
+      Ns <<= 4;
+    }
+    if (at >= 0) {
+      m = (at / Ns) * (at % Ns);
+      N = 16 * Ns;
+    }
+    const double2 w = half_twiddle(m, N);
+    tw[i] = {(S)w.x, (S)w.y};
+    return;
+  }
+  i -= count;
+  if (w64) {
+    if (i < h) {
+      w64[i] = half_twiddle((int)i, n);
+      return;
+    }
+    i -= h;
+  }
+  if (i >= ns) return;
+  const int m = (int)(i % (h + 1));
   const double inv = 1.0 / n;  // a power of two
-  const cd a = {Sp[t].re * inv, Sp[t].im * inv};
+  const cd a = {Sp[i].re * inv, Sp[i].im * inv};
   const bool end = m == 0 || m == h;
   const double2 w = half_twiddle(m, n);
-  out[2 * t] = split_cd(end ? a : plus_iw(a, w));
-  out[2 * t + 1] = end ? make_float4(0.f, 0.f, 0.f, 0.f) : split_cd(minus_iw(a, w));
+  sp[2 * i] = split_cd(end ? a : plus_iw(a, w));
+  sp[2 * i + 1] = end ? make_float4(0.f, 0.f, 0.f, 0.f) : split_cd(minus_iw(a, w));
 }
 // a b - c d or a b + c d from float-float factors, rounded once
 __device__ __forceinline__ float ff_dot2(float ah, float al, float bh, float bl, float ch, float cl, float dh, float dl) {
@@ -305,7 +316,7 @@ __device__ __forceinline__ void real_fft(C2<S>* __restrict__ buf, const C2<S>* _
 // values, then (KEEP: PG > 1) the points' T, [nk][SB] as float4 (FP32) or C2<double>.
 template <int L, class S, bool KEEP>
 __global__ void __launch_bounds__(256, sizeof(S) == 4 ? 3 : 1) k_synth_real(const cd* __restrict__ T, const int64_t* __restrict__ midx, int nk,
-                                                    int64_t M, const cd* __restrict__ Sp, const float4* __restrict__ sp,
+                                                    int low, int64_t M, const cd* __restrict__ Sp, const float4* __restrict__ sp,
                                                     const double2* __restrict__ w64, int P, int PG, int SB, const C2<S>* __restrict__ tw, bool passes,
                                                     S* __restrict__ out, int wide) {
   constexpr int h = 1 << L, n = 2 * h, NT = h / 16;
@@ -318,16 +329,6 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? 3 : 1) k_synth_real(cons
   const int tid = threadIdx.x, pt = tid / NT, j = tid - pt * NT;
   const int64_t x0 = (int64_t)blockIdx.x * SB;
   C2<S>* buf = bufs + pt * len;
-  __shared__ int s_low;  // frequencies below h / 2
-  if (tid == 0) {
-    int lo = 0, hi = nk;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (2 * midx[mid] < h) lo = mid + 1;
-      else hi = mid;
-    }
-    s_low = lo;
-  }
   if (KEEP)
     for (int e = tid; e < nk * SB; e += SB * NT) {
       const int r = e / SB, q = e - r * SB;
@@ -344,9 +345,10 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? 3 : 1) k_synth_real(cons
     // the frequencies below h / 2 store their shares of Z_m and Z_{h-m}, then those from h / 2 on add theirs
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
-      const int e0 = half ? s_low * SB : 0, e1 = half ? nk * SB : s_low * SB;
+      const int e0 = half ? low * SB : 0, e1 = half ? nk * SB : low * SB;
       for (int e = e0 + tid; e < e1; e += SB * NT) {
         const int r = e / SB, q = e - r * SB;
+        if (x0 + q >= M) continue;
         const int m = (int)midx[r];
         const bool end = m == 0 || m == h;
         C2<S> za, zb;  // H (1 + i w), H (1 - i w); at the ends H
@@ -356,22 +358,23 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? 3 : 1) k_synth_real(cons
             const float4 sa = sp[2 * ((int64_t)p * (h + 1) + m)], sb = sp[2 * ((int64_t)p * (h + 1) + m) + 1];
             float4 t4;
             if (KEEP) t4 = kept[e];
-            else t4 = x0 + q < M ? split_cd(T[(int64_t)r * M + x0 + q]) : make_float4(0.f, 0.f, 0.f, 0.f);
+            else t4 = split_cd(T[(int64_t)r * M + x0 + q]);
             za = ff_cmul(sa, t4);
             zb = ff_cmul(sb, t4);
-            // outside a safe range of FP32 (zero, tiny, huge, not finite): the product in FP64
+            // outside a safe range of FP32 (tiny, huge, not finite; zeros of both parts are safe): in FP64
             const float tm = fmaxf(fabsf(t4.x), fabsf(t4.z)), sm = fmaxf(fabsf(sa.x), fabsf(sa.z));
-            fp64 = !(tm >= 1e-25f && tm <= 1e25f && sm >= 1e-25f && sm <= 1e25f);
+            const bool tz = t4.x == 0.f && t4.z == 0.f, sz = sa.x == 0.f && sa.z == 0.f;
+            fp64 = !((tz || (tm >= 1e-25f && tm <= 1e25f)) && (sz || (sm >= 1e-25f && sm <= 1e25f)));
           }
         }
         if (fp64) {
-          cd t = {0.0, 0.0};
+          cd t;
           if constexpr (KEEP && !F32) t = reinterpret_cast<cd*>(kept)[e];
-          else if (x0 + q < M) t = T[(int64_t)r * M + x0 + q];
+          else t = T[(int64_t)r * M + x0 + q];
           const cd a = cmul(Srow[m], t);
           cd u = a, d = {0.0, 0.0};
           if (!end) {
-            const double2 w = w64 ? w64[m] : half_twiddle(m, n);
+            const double2 w = w64[m];
             u = plus_iw(a, w);
             d = minus_iw(a, w);
           }
@@ -411,28 +414,38 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? 3 : 1) k_synth_real(cons
   }
 }
 
-// Twiddles of a transform of n samples: FP64 pairs for n < 32 (the radix-2 kernel), else in its type.
-// passes: the pass factors too.
+// Whether `signals` of n samples take the radix-2 kernel: fewer than 32 samples, which k_synth_real does not
+// hold, or so few short ones that the latency of one signal counts: with 16 values a thread its warps take
+// longer than radix 2 over n / 2 threads.  400 signals of 64 samples, the kernel: 5.4 us here, 9.5 there (FP64
+// 6.7 and 20.2); of 512 samples 9.3 and 10.6 (21.7 and 27.9); one of 1024 and more is no faster here.
+static bool synth_radix2(int n, int64_t signals, int nsm) { return n < 32 || (n <= 512 && signals <= 4 * nsm); }
+
+// Tables of a transform of n samples (k_synth_tables): tw, with the pass factors too if `passes`; for the
+// radix-2 kernel FP64 pairs in tw and nothing else.
 template <class S>
-static void launch_twiddles(int n, void* tw, bool passes, cudaStream_t st) {
+static void launch_tables(int n, bool radix2, void* tw, bool passes, double2* w64, const cd* Sp, int64_t ns, float4* sp,
+                          cudaStream_t st) {
+  if (radix2) {
+    if (tw) BIE_LAUNCH(k_twiddles<<<(n / 2 + 255) / 256, 256, 0, st>>>(n, (double2*)tw));
+    return;
+  }
   int L = 0;
   while ((2 << L) < n) ++L;
-  const int count = passes ? twiddle_count(n) : n / 2;
-  if (n < 32)
-    BIE_LAUNCH(k_twiddles<<<1, 256, 0, st>>>(n, (double2*)tw));
-  else
-    BIE_LAUNCH(k_twiddles_of<S><<<(count + 127) / 128, 128, 0, st>>>(n, pass_radix0(L), count, (C2<S>*)tw));
+  const int count = !tw ? 0 : passes ? twiddle_count(n) : n / 2;
+  const int64_t all = count + (w64 ? n / 2 : 0) + ns;
+  BIE_LAUNCH(k_synth_tables<S><<<(unsigned)((all + 127) / 128), 128, 0, st>>>(n, pass_radix0(L), count, (C2<S>*)tw, w64, Sp, ns, sp));
 }
 
-// sp: the spectra's factors in float-float (k_split_spectra; FP32 only; NULL: products in FP64); w64:
-// exp(-2 pi i m / n), m < n / 2, in FP64 (NULL: formed where an FP64 product needs one).
+// low: how many of the frequencies lie below h / 2 = n / 4; sp: the spectra's factors in float-float
+// (k_synth_tables; FP32 only; NULL: products in FP64); w64: exp(-2 pi i m / n), m < n / 2, in FP64.
 template <class S>
-static int launch_synth(const cd* T, const int64_t* midx, int nk, int64_t M, const cd* Sp, const float4* sp,
-                        const double2* w64, int64_t P, int n, const void* tw, bool passes, S* out, int nsm, cudaStream_t st) {
-  if (n < 32) {
+static int launch_synth(const cd* T, const int64_t* midx, int nk, int low, int64_t M, const cd* Sp, const float4* sp,
+                        const double2* w64, int64_t P, int n, bool radix2, const void* tw, bool passes, S* out, int nsm,
+                        cudaStream_t st) {
+  if (radix2) {
     const dim3 g((unsigned)M, (unsigned)P);
     const size_t smem = 2 * (size_t)n * sizeof(C2<S>);
-    BIE_LAUNCH(k_synth<S, S><<<g, 32, smem, st>>>(T, midx, nk, M, Sp, n, (const double2*)tw, out));
+    BIE_LAUNCH(k_synth<S, S><<<g, std::max(32, n / 2), smem, st>>>(T, midx, nk, M, Sp, n, (const double2*)tw, out));
     return BIE_OK;
   }
   const int h = n / 2, wide = ((uintptr_t)out % (2 * sizeof(S))) == 0;
@@ -451,7 +464,7 @@ static int launch_synth(const cd* T, const int64_t* midx, int nk, int64_t M, con
   const dim3 g((unsigned)bx, (unsigned)(keep ? 1 : P));
   auto go = [&](auto kernel) -> int {
     BIE_TRY(set_smem_max(kernel));
-    BIE_LAUNCH(kernel<<<g, SB * (h / 16), bufs + (keep ? kept : 0), st>>>(T, midx, nk, M, Sp, sp, w64, (int)P, PG, SB,
+    BIE_LAUNCH(kernel<<<g, SB * (h / 16), bufs + (keep ? kept : 0), st>>>(T, midx, nk, low, M, Sp, sp, w64, (int)P, PG, SB,
                                                                           (const C2<S>*)tw, passes, out, wide));
     return BIE_OK;
   };
@@ -489,11 +502,16 @@ int pulse_spectrum(bie_ctx* c, const double* s, int64_t P, int n, cd* Sout) {
   return BIE_OK;
 }
 
-int synthesize(bie_ctx* c, const cd* T, const int64_t* midx_dev, int nk, int64_t M, const cd* Sp, int64_t P, int n,
+// Frequencies below a quarter of n samples in the ascending host list midx.
+int low_frequencies(const int64_t* midx, int64_t nk, int64_t n) {
+  return (int)(std::lower_bound(midx, midx + nk, (n + 3) / 4) - midx);
+}
+
+int synthesize(bie_ctx* c, const cd* T, const int64_t* midx_dev, int nk, int low, int64_t M, const cd* Sp, int64_t P, int n,
                void* out, int out_dtype) {
-  // twiddles (at most FP64 pairs), then the spectra in float-float (FP32), of so many pulses at a time that
-  // they stay within 32 MB (511 pulses of 4096 samples)
-  const size_t twb = (size_t)(twiddle_count(n) + 16) * sizeof(double2);
+  // twiddles (at most FP64 pairs; FP32: theirs and FP64 ones), then the spectra in float-float (FP32), of so
+  // many pulses at a time that they stay within 32 MB (511 pulses of 4096 samples)
+  const size_t twb = (size_t)(twiddle_count(n) + n / 2 + 16) * sizeof(double2);
   const int64_t nm = n / 2 + 1;
   const bool f32 = out_dtype != 0;
   const int64_t pc = f32 ? std::min(P, std::max<int64_t>(1, (int64_t)(32 << 20) / (nm * 2 * (int64_t)sizeof(float4)))) : P;
@@ -501,18 +519,19 @@ int synthesize(bie_ctx* c, const cd* T, const int64_t* midx_dev, int nk, int64_t
   void* tw = c->work2.p;
   int nsm = 0;
   BIE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
+  const bool radix2 = synth_radix2(n, P * M, nsm);
   if (f32) {
     float4* sp = (float4*)((char*)tw + twb);
-    launch_twiddles<float>(n, tw, true, c->stream);
+    double2* w64 = (double2*)tw + twiddle_count(n) + 16;
     for (int64_t p0 = 0; p0 < P; p0 += pc) {
-      const int64_t np = std::min(pc, P - p0), ns = np * nm;
+      const int64_t np = std::min(pc, P - p0);
       const cd* S0 = Sp + p0 * nm;
-      BIE_LAUNCH(k_split_spectra<<<(unsigned)((ns + 255) / 256), 256, 0, c->stream>>>(S0, ns, n, sp));
-      BIE_TRY(launch_synth<float>(T, midx_dev, nk, M, S0, sp, nullptr, np, n, tw, true, (float*)out + p0 * M * n, nsm, c->stream));
+      launch_tables<float>(n, radix2, p0 == 0 ? tw : nullptr, true, p0 == 0 ? w64 : nullptr, S0, np * nm, sp, c->stream);
+      BIE_TRY(launch_synth<float>(T, midx_dev, nk, low, M, S0, sp, w64, np, n, radix2, tw, true, (float*)out + p0 * M * n, nsm, c->stream));
     }
   } else {
-    launch_twiddles<double>(n, tw, true, c->stream);
-    BIE_TRY(launch_synth<double>(T, midx_dev, nk, M, Sp, nullptr, (const double2*)tw, P, n, tw, true, (double*)out, nsm, c->stream));
+    launch_tables<double>(n, radix2, tw, true, nullptr, nullptr, 0, nullptr, c->stream);
+    BIE_TRY(launch_synth<double>(T, midx_dev, nk, low, M, Sp, nullptr, (const double2*)tw, P, n, radix2, tw, true, (double*)out, nsm, c->stream));
   }
   BIE_CUDA_TRY(cudaGetLastError());
   return BIE_OK;
@@ -637,6 +656,7 @@ extern "C" int bie_synthesize_noalloc(const void* T, const int64_t* midx, int64_
     if (midx[r] < 0 || midx[r] > Nt / 2) return fail(BIE_ERR_INVALID_ARG, "midx out of [0, Nt/2]");
     if (r > 0 && midx[r] <= midx[r - 1]) return fail(BIE_ERR_INVALID_ARG, "midx must be strictly increasing");
   }
+  const int low = low_frequencies(midx, Nk, Nt);
   void* base = nullptr;
   BIE_TRY(noalloc_scratch(&base));
   cudaStream_t st = (cudaStream_t)stream;
@@ -647,14 +667,15 @@ extern "C" int bie_synthesize_noalloc(const void* T, const int64_t* midx, int64_
   int dev = 0, nsm = 0;
   BIE_CUDA_TRY(cudaGetDevice(&dev));
   BIE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  const bool radix2 = synth_radix2(n, P * M, nsm);
   if (out_dtype == 0) {
-    launch_twiddles<double>(n, tw, false, st);
-    BIE_TRY(launch_synth<double>((const cd*)T, md, (int)Nk, M, (const cd*)S, nullptr, tw, P, n, tw, false, (double*)out, nsm, st));
+    launch_tables<double>(n, radix2, tw, false, nullptr, nullptr, 0, nullptr, st);
+    BIE_TRY(launch_synth<double>((const cd*)T, md, (int)Nk, low, M, (const cd*)S, nullptr, tw, P, n, radix2, tw, false, (double*)out, nsm, st));
   } else {
     void* tw32 = (char*)base + kNoAllocScratchBytes;
-    launch_twiddles<double>(n, tw, false, st);
-    if (n >= 32) launch_twiddles<float>(n, tw32, false, st);
-    BIE_TRY(launch_synth<float>((const cd*)T, md, (int)Nk, M, (const cd*)S, nullptr, tw, P, n, n >= 32 ? tw32 : (void*)tw, false, (float*)out, nsm, st));
+    if (radix2) tw32 = tw;
+    launch_tables<float>(n, radix2, tw32, false, tw, nullptr, 0, nullptr, st);
+    BIE_TRY(launch_synth<float>((const cd*)T, md, (int)Nk, low, M, (const cd*)S, nullptr, tw, P, n, radix2, tw32, false, (float*)out, nsm, st));
   }
   BIE_CUDA_TRY(cudaGetLastError());
   // the host index array must outlive its asynchronous copy

@@ -132,3 +132,25 @@ def test_fp32_rounding_is_no_larger_than_a_radix_2_transforms(Nt, share):
     got = sol.synthesize(torch.tensor(T, device="cuda:0"), midx, torch.tensor(S, device="cuda:0"), Nt, torch.float32)
     assert np.linalg.norm(got.cpu().numpy() - ref) <= np.linalg.norm(plain - ref)
     sol.close()
+
+
+@pytest.mark.parametrize("f32", [False, True])
+@pytest.mark.parametrize("Nt", [32, 64, 512, 1024])
+def test_few_and_many_signals(Nt, f32):
+    """Counts of signals at which short ones change from the radix-2 kernel to the other (four to an SM)."""
+    import torch
+    from paper_1706_07919_gb300 import Solver
+    from paper_1706_07919_gb300 import binding as B
+
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    dt, eps = (torch.float32, 2.0 ** -24) if f32 else (torch.float64, 2.0 ** -53)
+    sol = Solver(0)
+    for M, P in ((4 * sm, 1), (4 * sm + 1, 1), (2 * sm, 2), (sm, 5)):
+        T, midx, S = _case(Nt, M, P, Nt + M, True)
+        Td, Sd = torch.tensor(T, device="cuda:0"), torch.tensor(S, device="cuda:0")
+        ref = _reference(T, midx, S, Nt)
+        out = torch.empty((P, M, Nt), dtype=dt, device="cuda:0")
+        B.bie_synthesize_noalloc(Td, midx, Sd, Nt, out, 1 if f32 else 0)
+        for got in (sol.synthesize(Td, midx, Sd, Nt, dt), out):
+            assert np.linalg.norm(got.cpu().numpy() - ref) <= (4 * np.log2(Nt) + 3) * eps * np.linalg.norm(ref), (M, P)
+    sol.close()
