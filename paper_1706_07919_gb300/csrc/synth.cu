@@ -361,10 +361,9 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? 3 : 1) k_synth_real(cons
             else t4 = split_cd(T[(int64_t)r * M + x0 + q]);
             za = ff_cmul(sa, t4);
             zb = ff_cmul(sb, t4);
-            // outside a safe range of FP32 (tiny, huge, not finite; zeros of both parts are safe): in FP64
+            // outside a safe range of FP32 (zero there, tiny, huge, not finite): the product in FP64
             const float tm = fmaxf(fabsf(t4.x), fabsf(t4.z)), sm = fmaxf(fabsf(sa.x), fabsf(sa.z));
-            const bool tz = t4.x == 0.f && t4.z == 0.f, sz = sa.x == 0.f && sa.z == 0.f;
-            fp64 = !((tz || (tm >= 1e-25f && tm <= 1e25f)) && (sz || (sm >= 1e-25f && sm <= 1e25f)));
+            fp64 = !(tm >= 1e-25f && tm <= 1e25f && sm >= 1e-25f && sm <= 1e25f);
           }
         }
         if (fp64) {

@@ -154,3 +154,18 @@ def test_few_and_many_signals(Nt, f32):
         for got in (sol.synthesize(Td, midx, Sd, Nt, dt), out):
             assert np.linalg.norm(got.cpu().numpy() - ref) <= (4 * np.log2(Nt) + 3) * eps * np.linalg.norm(ref), (M, P)
     sol.close()
+
+
+def test_fp32_synthesis_keeps_products_of_values_that_vanish_in_fp32():
+    """Field spectra that round to zero in FP32 with pulses near the upper end of its safe range."""
+    import torch
+    from paper_1706_07919_gb300 import Solver
+
+    sol = Solver(0)
+    T, midx, S = _case(1024, 700, 3, 2, False)
+    for a, b in ((1e-47, 1e24), (1e24, 1e-47)):
+        got = sol.synthesize(torch.tensor(T * a, device="cuda:0"), midx, torch.tensor(S * b, device="cuda:0"), 1024,
+                             torch.float32).cpu().numpy()
+        ref = _reference(T * a, midx, S * b, 1024)
+        assert np.linalg.norm(got - ref) <= 43 * 2.0 ** -24 * np.linalg.norm(ref)
+    sol.close()
