@@ -666,7 +666,7 @@ __global__ void __launch_bounds__(kFootNT) k_foot_points(
     __syncthreads();
   }
   if (tid >= pts || !valid) return;
-  foot_elem[m] = be;
+  foot_elem[m] = max(be, 0);  // (no element is nearest to a point that is not finite: its field is NaN)
   double x0[3] = {0, 0, 0}, nu[3] = {0, 0, 0}, J = 0.0;
   if (be >= 0) iso_point(nodes, elems + 6 * (int64_t)be, bxi, beta, x0, nu, &J);
   double* o = foot + 8 * m;

@@ -40,3 +40,33 @@ def test_closest_points_do_not_depend_on_the_batch(mesh, M):
         if i.any():
             assert np.linalg.norm(T[i] - ref[i]) <= 1e-12 * np.linalg.norm(ref[i])
     sol.close()
+
+
+@pytest.mark.parametrize("mode", ["mixed", "fp64"])
+@pytest.mark.parametrize("variant", [0, 1, 2])
+def test_points_that_are_not_finite(mode, variant):
+    """A NaN or infinite observation point has no nearest element: its field is not finite, the other points'
+    are their own."""
+    import torch
+    from paper_1706_07919_gb300 import Solver
+    from paper_1706_07919_gb300 import binding as B
+    from workloads import octa_sphere, shell_points
+
+    m = octa_sphere(1)
+    sol = Solver(0)
+    sol.set_geometry(m.nodes, m.elems, m.normals, m.bc)
+    sol.set_option("field.variant", variant)
+    md = B.BIE_MODE_MIXED if mode == "mixed" else B.BIE_MODE_FP64
+    x = torch.tensor(shell_points(70, 1.2, 3.0, seed=4), device="cuda:0")
+    k = 0.3 * np.arange(1, 21)
+    g = torch.Generator("cuda:0").manual_seed(2)
+    surf = torch.randn((20, 2, m.N), dtype=torch.complex128, device="cuda:0", generator=g)
+    good = sol.eval_field(x, k, surf, md)
+    bad = x.clone()
+    bad[3, 1], bad[40, 0], bad[69] = float("nan"), float("inf"), float("nan")
+    got = sol.eval_field(bad, k, surf, md)
+    keep = torch.ones(70, dtype=torch.bool, device="cuda:0")
+    keep[[3, 40, 69]] = False
+    assert torch.equal(torch.view_as_real(got[:, keep]), torch.view_as_real(good[:, keep]))
+    assert not torch.isfinite(torch.view_as_real(got[:, ~keep])).all(dim=2).any()
+    sol.close()
